@@ -1,4 +1,4 @@
-"""ctypes binding of libfathom.so: argument marshalling only, every step runs in the CUDA kernels.
+"""Binding of libfathom.so: argument marshalling only, every step runs in the CUDA kernels.
 
 The function names are those of the C ABI (include/fathom.h).  Tensors are torch tensors used as
 plain device (or pinned host) buffers; their data pointers are passed through unchanged.  There is
@@ -127,18 +127,58 @@ def _dtype_code(t: torch.Tensor) -> int:
     raise TypeError(f"unsupported dtype {t.dtype}")
 
 
-class Context:
-    """Owns one fathom_ctx (scratch arena + status word) on one device."""
+def _load_native():
+    """The compiled call layer (csrc/native_binding.cpp), bound to the libfathom.so loaded above."""
+    try:
+        from . import _native
+    except ImportError as e:
+        raise ImportError(f"the extension module beside {LIB_PATH} is missing or does not load ({e}): run "
+                          "`python -m paper_2609_17652_b200.build` (needs nvcc and g++); there is no fallback path") from e
+    _native._setup(torch.float32, torch.bfloat16, torch._C._cuda_getDevice, torch._C._cuda_getCurrentRawStream,
+                   torch.cuda.current_stream, _raise)
+    return _native
+
+
+def _raise(status: int, ctx: int):
+    raise FathomError(status, C.c_void_p(ctx) if ctx else None)
+
+
+_native = _load_native()
+
+
+class Context(_native.ContextCalls):
+    """Owns one fathom_ctx (scratch arena + status word) on one device.
+
+    The enqueueing calls are methods of the compiled base class, with the C ABI's names (stream=None: torch's current
+    stream; buffers: tensors, plain addresses or None):
+        fathom_build_planes(layout, K, planes, scales, stream=None, k_dtype=None)
+        fathom_alloc_depth(layout, q, var, mode, budget, heads_per_plan, depth, stream=None)
+        fathom_scan(layout, planes, scales, q, depth, heads_per_plan, scores, stream=None)
+        fathom_scan_batch(items, heads_per_plan, stream=None)       items: (layout, planes, scales, q, depth, scores) each
+        fathom_topk(layout, scores, k, n_sink, n_local, idx, stream=None)
+        fathom_sparse_attend(layout, q, Krows, Vrows, idx, k, softmax_scale, out, stream=None, row_dtype=None)
+        fathom_calibrate(layout, K, mean, cov, stream=None)
+        fathom_channel_variance(layout, K, mean, var, stream=None)
+        fathom_klt_basis(layout, cov, basis, eigenvalues, stream=None)
+        fathom_rotate_keys(layout, K, mean, basis, K_rot, stream=None)
+        fathom_build_planes_rotated(layout, K, mean, basis, planes, scales, stream=None)
+        fathom_rotate_query(layout, q, basis, q_rot, stream=None)
+        fathom_scan_topk(layout, planes, scales, q, depth, heads_per_plan, k, n_sink, n_local, idx, stream=None)
+        fathom_gather_union(layout, idx, k, Krows, Vrows, K_stage, V_stage, idx_local, union_count, stream=None,
+                            row_dtype=None)
+    """
 
     def __init__(self, device: int = 0, scratch_bytes: int = 0):
         self._h = C.c_void_p()
         rc = lib.fathom_create(C.byref(self._h), device, scratch_bytes)
         if rc != 0:
             raise FathomError(rc)
+        self._attach(self._h.value)
         self.device, self.scratch_bytes = device, scratch_bytes
 
     def close(self):
         if self._h:
+            self._attach(0)
             lib.fathom_destroy(self._h)
             self._h = C.c_void_p()
 
@@ -151,66 +191,6 @@ class Context:
     def _check(self, rc: int):
         if rc != 0:
             raise FathomError(rc, self._h)
-
-    # ---- the five calls (raw status returned by the *_rc variants is used by the error-path tests)
-    def fathom_build_planes(self, layout, K, planes, scales, stream=None, k_dtype=None):
-        self._check(lib.fathom_build_planes(self._h, C.byref(layout), _ptr(K), _dtype_code(K) if k_dtype is None else k_dtype,
-                                            _ptr(planes), _ptr(scales), _stream(stream)))
-
-    def fathom_alloc_depth(self, layout, q, var, mode, budget, heads_per_plan, depth, stream=None):
-        self._check(lib.fathom_alloc_depth(self._h, C.byref(layout), _ptr(q), _ptr(var), mode, budget, heads_per_plan,
-                                           _ptr(depth), _stream(stream)))
-
-    def fathom_scan(self, layout, planes, scales, q, depth, heads_per_plan, scores, stream=None):
-        self._check(lib.fathom_scan(self._h, C.byref(layout), _ptr(planes), _ptr(scales), _ptr(q), _ptr(depth),
-                                    heads_per_plan, _ptr(scores), _stream(stream)))
-
-    def fathom_scan_batch(self, items, heads_per_plan, stream=None):
-        """items: sequence of (layout, planes, scales, q, depth, scores)."""
-        arr = (ScanItem * len(items))()
-        for i, (lay, planes, scales, q, depth, scores) in enumerate(items):
-            arr[i].layout = lay
-            arr[i].planes, arr[i].scales, arr[i].q = _ptr(planes), _ptr(scales), _ptr(q)
-            arr[i].depth, arr[i].scores = _ptr(depth), _ptr(scores)
-        self._check(lib.fathom_scan_batch(self._h, arr, len(items), heads_per_plan, _stream(stream)))
-
-    def fathom_topk(self, layout, scores, k, n_sink, n_local, idx, stream=None):
-        self._check(lib.fathom_topk(self._h, C.byref(layout), _ptr(scores), k, n_sink, n_local, _ptr(idx), _stream(stream)))
-
-    def fathom_sparse_attend(self, layout, q, Krows, Vrows, idx, k, softmax_scale, out, stream=None, row_dtype=None):
-        self._check(lib.fathom_sparse_attend(self._h, C.byref(layout), _ptr(q), _ptr(Krows), _ptr(Vrows),
-                                             _dtype_code(Krows) if row_dtype is None else row_dtype, _ptr(idx), k,
-                                             C.c_float(softmax_scale), _ptr(out), _stream(stream)))
-
-    def fathom_calibrate(self, layout, K, mean, cov, stream=None):
-        self._check(lib.fathom_calibrate(self._h, C.byref(layout), _ptr(K), _dtype_code(K), _ptr(mean), _ptr(cov), _stream(stream)))
-
-    def fathom_channel_variance(self, layout, K, mean, var, stream=None):
-        self._check(lib.fathom_channel_variance(self._h, C.byref(layout), _ptr(K), _dtype_code(K), _ptr(mean), _ptr(var), _stream(stream)))
-
-    def fathom_klt_basis(self, layout, cov, basis, eigenvalues, stream=None):
-        self._check(lib.fathom_klt_basis(self._h, C.byref(layout), _ptr(cov), _ptr(basis), _ptr(eigenvalues), _stream(stream)))
-
-    def fathom_rotate_keys(self, layout, K, mean, basis, K_rot, stream=None):
-        self._check(lib.fathom_rotate_keys(self._h, C.byref(layout), _ptr(K), _dtype_code(K), _ptr(mean), _ptr(basis),
-                                           _ptr(K_rot), _stream(stream)))
-
-    def fathom_build_planes_rotated(self, layout, K, mean, basis, planes, scales, stream=None):
-        self._check(lib.fathom_build_planes_rotated(self._h, C.byref(layout), _ptr(K), _dtype_code(K), _ptr(mean), _ptr(basis),
-                                                    _ptr(planes), _ptr(scales), _stream(stream)))
-
-    def fathom_rotate_query(self, layout, q, basis, q_rot, stream=None):
-        self._check(lib.fathom_rotate_query(self._h, C.byref(layout), _ptr(q), _ptr(basis), _ptr(q_rot), _stream(stream)))
-
-    def fathom_scan_topk(self, layout, planes, scales, q, depth, heads_per_plan, k, n_sink, n_local, idx, stream=None):
-        self._check(lib.fathom_scan_topk(self._h, C.byref(layout), _ptr(planes), _ptr(scales), _ptr(q), _ptr(depth),
-                                         heads_per_plan, k, n_sink, n_local, _ptr(idx), _stream(stream)))
-
-    def fathom_gather_union(self, layout, idx, k, Krows, Vrows, K_stage, V_stage, idx_local, union_count, stream=None,
-                            row_dtype=None):
-        self._check(lib.fathom_gather_union(self._h, C.byref(layout), _ptr(idx), k, _ptr(Krows), _ptr(Vrows),
-                                            _dtype_code(Krows) if row_dtype is None else row_dtype, _ptr(K_stage),
-                                            _ptr(V_stage), _ptr(idx_local), _ptr(union_count), _stream(stream)))
 
     def fathom_selftest_wait_expiry(self, tries: int = 200, stream=None):
         self._check(lib.fathom_selftest_wait_expiry(self._h, tries, _stream(stream)))
