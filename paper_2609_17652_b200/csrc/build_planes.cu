@@ -2,14 +2,11 @@
 //
 // Two threads own one channel of a 64-token block (32 tokens each): the 128 threads of a token half read
 // every token row as 512 contiguous bytes, keep their 32 values in registers, exchange the two half maxima
-// through shared memory, round a/8 to fp16 and derive the four plane bits of every code by comparing k
-// with exact multiples of the stored scale, most significant bit first:
-//     bit0 = k >= 0;  bit1 = k >= (bit0 ? 4 : -4) s;  bit2 = k >= thr1 + (bit1 ? 2 : -2) s;  ...
-// m * s (|m| <= 7, s an fp16 value) is exact in fp32, so the four comparisons give exactly
-// clip(floor(k / s), -8, 7) + 8 with no division.  A CTA walks BLOCKS_PER_CTA consecutive blocks and
+// through shared memory, round a/8 to fp16 and take the codes and their plane words from fathom_quantise32
+// (quantise.cuh).  A CTA walks BLOCKS_PER_CTA consecutive blocks and
 // collects their plane words and scales in shared memory, then writes every (channel, plane) row segment
 // as whole 32-byte sectors (partial-sector writes cost a fill read each).
-#include "fathom_common.cuh"
+#include "quantise.cuh"
 
 namespace {
 
@@ -57,32 +54,13 @@ build_planes_kernel(const T* __restrict__ K, uint32_t* __restrict__ planes32, ui
 
     const __half sh = __float2half_rn(a * 0.125f);             // a/8 is exact; one rounding to fp16
     const float sc = __half2float(sh);
-    const float s2 = sc * 2.0f, s4 = sc * 4.0f;
 
-    uint32_t w[FATHOM_NPLANES] = {0u, 0u, 0u, 0u};
     const uint32_t keep = (valid >= HALF) ? ~0u : (valid <= 0 ? 0u : (~0u >> (32 - valid)));   // absent tail tokens carry 0 bits
-    if (sc > 0.0f) {
+    uint32_t w[FATHOM_NPLANES];
+    fathom_quantise32(v, sc, 1.0f / sc, w);
+    if (!(sc > 0.0f)) { w[0] = ~0u; w[1] = w[2] = w[3] = 0u; }  // zero scale: every code is 8 = 0b1000
 #pragma unroll
-      for (int i = 0; i < HALF; ++i) {
-        const float k = v[i];
-        const uint32_t m = 1u << i;
-        const bool c0 = k >= 0.0f;
-        float thr = c0 ? s4 : -s4;
-        const bool c1 = k >= thr;
-        thr += c1 ? s2 : -s2;
-        const bool c2 = k >= thr;
-        thr += c2 ? sc : -sc;
-        const bool c3 = k >= thr;
-        if (c0) w[0] |= m;
-        if (c1) w[1] |= m;
-        if (c2) w[2] |= m;
-        if (c3) w[3] |= m;
-      }
-#pragma unroll
-      for (int p = 0; p < FATHOM_NPLANES; ++p) w[p] &= keep;
-    } else {                                                   // zero scale: every code is 8 = 0b1000
-      w[0] = keep;
-    }
+    for (int p = 0; p < FATHOM_NPLANES; ++p) w[p] &= keep;
     // little-endian halves of the 64-bit plane word: tokens 0..31 in the low 32 bits
 #pragma unroll
     for (int p = 0; p < FATHOM_NPLANES; ++p) s_out[j][(p * BLOCKS_PER_CTA + bb) * 2 + half] = w[p];
