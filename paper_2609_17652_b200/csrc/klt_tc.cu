@@ -1,44 +1,65 @@
-// fathom_rotate_keys on the 5th-generation tensor cores: K' = (K - mu) V  (Sec. 3.5 "Basis rule").
+// fathom_rotate_keys and fathom_build_planes_rotated on the 5th-generation tensor cores: K' = (K - mu) V  (Sec. 3.5 "Basis
+// rule"), and the covariance of fathom_calibrate.
 //
 // The rotation is the one dense contraction next to the decode path (n x 128 by 128 x 128 per KV head), so it runs
 // as tcgen05.mma with the accumulator in tensor memory.  The rotated keys feed a quantiser, so tf32's 11 significant
 // bits are not enough; both operands are split into a tf32 head and a tf32 tail, x = xh + xl, v = vh + vl, and three
 // products are accumulated in fp32:  xh vh + xh vl + xl vh  (the dropped xl vl term is below 2^-22 of |x||v|).
 //
-// One persistent CTA per SM walks a contiguous range of 128-token tiles.  Per tile and per chunk of 32 channels
-// (128 bytes of tf32: one row of the 128-byte swizzle) all 256 threads take the chunk from registers (loaded one
-// tile ahead), subtract the mean, split, and store head and tail into shared memory in the K-major 128-byte-swizzled
-// layout the MMA descriptors describe; one thread then issues the 4 x 3 MMAs of the chunk (M = 128 tokens, N = 128
-// rotated channels, K = 8) and commits them to the mbarrier that frees the chunk buffer (two buffers).  The split
-// basis (transposed, K-major) stays in shared memory for the whole tile range.  Two 128 x 128 fp32 accumulators
-// alternate: while the tensor cores work on tile t, the accumulator of tile t - 1 is read back with tcgen05.ld (warp
-// w: lanes 32 (w mod 4).., columns 64 (w div 4)..), staged per warp in shared memory and written to global memory in
-// 128-byte rows.
+// The BASIS is the left operand (M = 128 rotated channels) and the tokens are the right one (N = 128):
+//   * the split basis stays in tensor memory (256 columns) for all of a head's tiles, so an MMA reads only the tokens from
+//     shared memory: 4 KB per 64 cycles.  With both operands in shared memory (8 KB per 64 cycles) the MMAs alone took the whole
+//     128 bytes per cycle of the shared-memory data path, and the 128 KB of split keys per tile came on top: 4.1 us a tile;
+//   * the accumulator has a rotated channel per lane and a token per column, which is what both epilogues want: a thread
+//     holds 64 tokens = one block of ONE channel.  A warp writes 128 contiguous bytes of a rotated key per store straight from
+//     registers, and the quantiser's block maximum and plane words need no exchange between threads (with a token per
+//     lane they took a redux, four ballots and a shuffle per element: 9.5 us a tile).
+//
+// One persistent CTA per SM walks a contiguous range of 128-token tiles in three roles:
+//   16 producer warps  fetch a tile of keys one tile ahead into registers, subtract the mean, split, and store head and
+//                      tail of 32 channels (128 bytes of tf32: one row of the 128-byte swizzle) into a stage of a ring;
+//   1 MMA thread       issues a stage's 4 x 3 MMAs (M = N = 128, K = 8), commits them to the stage's barrier and, after a tile's last,
+//                      to its accumulator's (two accumulators alternate);
+//   8 epilogue warps   read the accumulator with tcgen05.ld (warp w: lanes 32 (w mod 4).., block w div 4 of the tile), hand it
+//                      back, and store or quantise.
+// Measured on 8 heads of 262,144 tokens, per 128-token tile and SM: fp32 keys to fp32 keys 4.2 -> 3.2 us (2.95 = its bytes at
+// the copy bandwidth), bf16 keys 4.2 -> 2.8 us, quantising 9.5 -> 2.65 us; the 48 MMAs alone, with nothing else running, take 2.0 us.
 //
 // Every wait on an mbarrier is bounded; a wait that runs out sets FATHOM_DEV_WAIT_EXPIRED in the context status and
-// the CTA stops waiting, finishes its loops, frees its tensor memory and returns.
-#include "fathom_common.cuh"
+// the thread stops waiting; every role still finishes its loops, and the CTA frees its tensor memory and returns.
+#include "quantise.cuh"
 
 namespace {
 
-constexpr int TC_THREADS = 256;
-constexpr int TILE_M = 128;                                  // tokens per tile (MMA M)
+constexpr int TC_THREADS = 256;                              // covariance kernel
+constexpr int TILE_M = 128;                                  // tokens per tile
 constexpr int KC = 32;                                       // channels per chunk = 128 bytes of tf32
 constexpr int NCHUNK = FATHOM_D / KC;                        // 4
 constexpr int SLAB = TILE_M * KC * 4;                        // 16 KB: 128 rows of 128 bytes
 constexpr int UMMA_K = 8;                                    // tf32 elements per MMA along K (32 bytes)
-constexpr uint32_t TMEM_COLS = 256;                          // two fp32 accumulators of 128 columns
 constexpr uint32_t WAIT_TRIES = 1u << 22;
 
-// shared-memory map (bytes from a 1024-byte aligned base)
-constexpr int OFF_VH = 0;                                    // 4 slabs: basis head, [chunk][rotated channel][32 channels]
-constexpr int OFF_VL = OFF_VH + NCHUNK * SLAB;               // 4 slabs: basis tail
-constexpr int OFF_XH = OFF_VL + NCHUNK * SLAB;               // 2 slabs: key head (double buffer)
-constexpr int OFF_XL = OFF_XH + 2 * SLAB;                    // 2 slabs: key tail
-constexpr int OFF_STAGE = OFF_XL + 2 * SLAB;                 // 8 warps x 32 x 32 floats
-constexpr int OFF_MU = OFF_STAGE + 8 * 32 * 32 * 4;          // 128 floats
-constexpr int OFF_BAR = OFF_MU + FATHOM_D * 4;               // 4 mbarriers + tensor-memory base
-constexpr int TC_SMEM = OFF_BAR + 64 + 1024;                 // + slack for the manual 1024-byte alignment
+// rotation kernel: roles, ring of stages, shared-memory map (bytes from a 1024-byte aligned base)
+constexpr int PRODUCERS = 512, EPILOGUE = 256;
+constexpr int RT_THREADS = PRODUCERS + EPILOGUE + 32;        // the last warp issues the MMAs
+constexpr int ROWS_PER_LANE = TILE_M * NCHUNK / (PRODUCERS / 32) / 4;       // 8
+constexpr int STAGE_BYTES = 2 * SLAB;                        // head and tail of 32 channels of 128 tokens
+constexpr int UNIT_BLOCKS = 4;                               // quantiser: blocks whose plane words are written together (32 bytes a row)
+constexpr int OUT_PITCH = FATHOM_NPLANES * UNIT_BLOCKS * 2 + 1;             // words per channel of staged plane words, odd: no bank conflicts
+template <bool BUILD>
+struct Map {
+  static constexpr int STAGES = BUILD ? 4 : 5;                // shared memory left over is L1, and the keys in flight need it: with seven stages
+                                                              // (fp32 keys) storing took 3.9 us a tile against 3.2, with six quantising 3.1 against 2.6
+  static constexpr int OUT = STAGES * STAGE_BYTES;            // BUILD: 128 x OUT_PITCH words
+  static constexpr int SCALE = OUT + (BUILD ? FATHOM_D * OUT_PITCH * 4 : 0);   // BUILD: 128 x 4 fp16
+  static constexpr int MU = SCALE + (BUILD ? FATHOM_D * UNIT_BLOCKS * 2 : 0);  // 128 floats
+  static constexpr int BAR = MU + FATHOM_D * 4;               // full and empty barriers of the stages, full and empty of the accumulators
+  static constexpr int BARS = 2 * STAGES + 4;
+  static constexpr int BYTES = BAR + BARS * 8 + 16 + 1024;    // + tensor-memory base, slack for the manual 1024-byte alignment
+  static_assert(BYTES <= 227 * 1024, "shared memory");
+};
+constexpr uint32_t COL_VH = 0, COL_VL = COL_VH + FATHOM_D, COL_ACC = 256;  // tensor memory: basis head, basis tail, two accumulators
+constexpr uint32_t RT_TMEM_COLS = 512;
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 __device__ __forceinline__ float tf32_head(float x) { return __uint_as_float(__float_as_uint(x) & 0xffffe000u); }
@@ -54,11 +75,12 @@ __device__ __forceinline__ uint64_t umma_desc(uint32_t saddr) {
 // fp32 accumulator, tf32 A and B, both K-major, N = 128, M = 128
 constexpr uint32_t UMMA_IDESC = (1u << 4) | (2u << 7) | (2u << 10) | ((128u >> 3) << 17) | ((128u >> 4) << 24);
 
-__device__ __forceinline__ void umma_tf32(uint32_t tmem_d, uint64_t a, uint64_t b, uint32_t accumulate) {
+// left operand in tensor memory (lane = row, one tf32 element per column), right operand in shared memory
+__device__ __forceinline__ void umma_tf32_ts(uint32_t tmem_d, uint32_t tmem_a, uint64_t b, uint32_t accumulate) {
   asm volatile(
       "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, {%5, %5, %5, %5}, p;\n\t}\n"
-      :: "r"(tmem_d), "l"(a), "l"(b), "r"(UMMA_IDESC), "r"(accumulate), "r"(0u) : "memory");
+      "tcgen05.mma.cta_group::1.kind::tf32 [%0], [%1], %2, %3, {%5, %5, %5, %5}, p;\n\t}\n"
+      :: "r"(tmem_d), "r"(tmem_a), "l"(b), "r"(UMMA_IDESC), "r"(accumulate), "r"(0u) : "memory");
 }
 __device__ __forceinline__ void umma_commit(uint32_t bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" :: "r"(bar) : "memory");
@@ -66,13 +88,16 @@ __device__ __forceinline__ void umma_commit(uint32_t bar) {
 __device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" :: "r"(bar), "r"(count) : "memory");
 }
+__device__ __forceinline__ bool mbar_test(uint32_t bar, uint32_t parity) {
+  uint32_t done;
+  asm volatile("{\n\t.reg .pred p;\n\tmbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}\n"
+               : "=r"(done) : "r"(bar), "r"(parity) : "memory");
+  return done != 0;
+}
 // Bounded wait for the phase with the given parity; false when the limit ran out.
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, uint32_t tries = WAIT_TRIES) {
   for (uint32_t i = 0; i < tries; ++i) {
-    uint32_t done;
-    asm volatile("{\n\t.reg .pred p;\n\tmbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}\n"
-                 : "=r"(done) : "r"(bar), "r"(parity) : "memory");
-    if (done) return true;
+    if (mbar_test(bar, parity)) return true;
     if (i > 64) __nanosleep(32);
   }
   return false;
@@ -90,16 +115,45 @@ __global__ void wait_expiry_selftest_kernel(uint32_t* dev_status, uint32_t tries
   }
 }
 
-// ---- basis prepared for the MMA: transposed (K-major for the B operand) and split into tf32 head and tail
-__global__ void __launch_bounds__(FATHOM_D)
-split_basis_kernel(const float* __restrict__ basis, float* __restrict__ vh_t, float* __restrict__ vl_t) {
-  const int kv = blockIdx.y, j = blockIdx.x, c = threadIdx.x;                 // out[kv][j][c] = basis[kv][c][j]
-  const float v = basis[((size_t)kv * FATHOM_D + c) * FATHOM_D + j];
-  const float h = tf32_head(v);
-  vh_t[((size_t)kv * FATHOM_D + j) * FATHOM_D + c] = h;
-  vl_t[((size_t)kv * FATHOM_D + j) * FATHOM_D + c] = tf32_head(v - h);
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}\n" : "=r"(p));
+  return p != 0;
 }
+__device__ __forceinline__ void mbar_arrive(uint32_t bar) {
+  asm volatile("mbarrier.arrive.release.cta.shared::cta.b64 _, [%0];" :: "r"(bar) : "memory");
+}
+// 32 columns of the warp's 32 lanes
+__device__ __forceinline__ void tmem_load32(uint32_t taddr, float (&r)[32]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
+      "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];\n"
+      : "=f"(r[0]), "=f"(r[1]), "=f"(r[2]), "=f"(r[3]), "=f"(r[4]), "=f"(r[5]), "=f"(r[6]), "=f"(r[7]), "=f"(r[8]),
+        "=f"(r[9]), "=f"(r[10]), "=f"(r[11]), "=f"(r[12]), "=f"(r[13]), "=f"(r[14]), "=f"(r[15]), "=f"(r[16]),
+        "=f"(r[17]), "=f"(r[18]), "=f"(r[19]), "=f"(r[20]), "=f"(r[21]), "=f"(r[22]), "=f"(r[23]), "=f"(r[24]),
+        "=f"(r[25]), "=f"(r[26]), "=f"(r[27]), "=f"(r[28]), "=f"(r[29]), "=f"(r[30]), "=f"(r[31])
+      : "r"(taddr) : "memory");
+}
+__device__ __forceinline__ void tmem_store32(uint32_t taddr, const uint32_t (&r)[32]) {
+  asm volatile(
+      "tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16, "
+      "%17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31, %32};\n"
+      :: "r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]), "r"(r[9]),
+         "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15]), "r"(r[16]), "r"(r[17]), "r"(r[18]), "r"(r[19]),
+         "r"(r[20]), "r"(r[21]), "r"(r[22]), "r"(r[23]), "r"(r[24]), "r"(r[25]), "r"(r[26]), "r"(r[27]), "r"(r[28]), "r"(r[29]),
+         "r"(r[30]), "r"(r[31]) : "memory");
+}
+__device__ __forceinline__ void epilogue_barrier() { asm volatile("bar.sync 1, %0;" :: "n"(EPILOGUE) : "memory"); }
 
+// 16 bytes of a key row: four fp32 or eight bf16 channels
+__device__ __forceinline__ void unpack16(const uint4& u, float (&x)[4]) {
+  x[0] = __uint_as_float(u.x); x[1] = __uint_as_float(u.y); x[2] = __uint_as_float(u.z); x[3] = __uint_as_float(u.w);
+}
+__device__ __forceinline__ void unpack16(const uint4& u, float (&x)[8]) {
+  const uint32_t w[4] = {u.x, u.y, u.z, u.w};
+#pragma unroll
+  for (int c = 0; c < 4; ++c) { x[2 * c] = __uint_as_float(w[c] << 16); x[2 * c + 1] = __uint_as_float(w[c] & 0xffff0000u); }
+}
 template <typename T> __device__ __forceinline__ float4 load_row4(const T* p);
 template <> __device__ __forceinline__ float4 load_row4<float>(const float* p) { return __ldg(reinterpret_cast<const float4*>(p)); }
 template <> __device__ __forceinline__ float4 load_row4<__nv_bfloat16>(const __nv_bfloat16* p) {
@@ -108,408 +162,286 @@ template <> __device__ __forceinline__ float4 load_row4<__nv_bfloat16>(const __n
                      __uint_as_float(u.y & 0xffff0000u));
 }
 
-template <typename T>
-__global__ void __launch_bounds__(TC_THREADS, 1)
-rotate_keys_tc_kernel(const T* __restrict__ K, const float* __restrict__ mean, const float* __restrict__ vh_t,
-                      const float* __restrict__ vl_t, float* __restrict__ K_rot, long long n, long long tiles_per_head,
-                      long long total_tiles, uint32_t* __restrict__ dev_status) {
+// One kernel for both entry points (so that every accumulator is bit for bit the same in both).  BUILD: planes and scales of the
+// rotated keys, tiles in pairs (a unit of 256 tokens = four blocks = 32 bytes of every plane row, written together:
+// partial-sector writes cost a fill read each); otherwise the rotated keys themselves.
+template <typename T, bool BUILD>
+__global__ void __launch_bounds__(RT_THREADS, 1)
+rotate_tc_kernel(const T* __restrict__ K, const float* __restrict__ mean, const float* __restrict__ basis, float* __restrict__ K_rot,
+                 uint64_t* __restrict__ planes, uint16_t* __restrict__ scales, long long n, long long plane_stride, long long scale_stride,
+                 long long tiles_per_head, long long total_tiles, uint32_t* __restrict__ dev_status) {
   extern __shared__ unsigned char smem_raw[];
   unsigned char* sm = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);   // 1024-byte aligned in the shared window
   const uint32_t sm_base = smem_u32(sm);
-  float* s_mu = reinterpret_cast<float*>(sm + OFF_MU);
-  float* s_stage = reinterpret_cast<float*>(sm + OFF_STAGE);
-  uint32_t* s_tmem = reinterpret_cast<uint32_t*>(sm + OFF_BAR + 32);
-  const uint32_t bar_empty0 = sm_base + OFF_BAR, bar_empty1 = sm_base + OFF_BAR + 8, bar_acc0 = sm_base + OFF_BAR + 16,
-                 bar_acc1 = sm_base + OFF_BAR + 24;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  using MP = Map<BUILD>;
+  constexpr int STAGES = MP::STAGES;
+  float* s_mu = reinterpret_cast<float*>(sm + MP::MU);
+  uint32_t* s_tmem = reinterpret_cast<uint32_t*>(sm + MP::BAR + MP::BARS * 8);
+  const uint32_t bar_full = sm_base + MP::BAR, bar_empty = bar_full + STAGES * 8, bar_acc_full = bar_empty + STAGES * 8,
+                 bar_acc_empty = bar_acc_full + 16;
+  const int tid = threadIdx.x, lane = tid & 31, warp = __shfl_sync(0xffffffffu, tid >> 5, 0);   // (uniform)
+  constexpr int MMA_WARP = (PRODUCERS + EPILOGUE) / 32;
 
   // contiguous range of tiles of this CTA over the (KV head, tile) space
-  const long long g0 = total_tiles * blockIdx.x / gridDim.x, g1 = total_tiles * (blockIdx.x + 1) / gridDim.x;
+  constexpr long long UNIT = BUILD ? UNIT_BLOCKS * FATHOM_BLOCK / TILE_M : 1;
+  const long long units = total_tiles / UNIT;
+  const long long g0 = units * blockIdx.x / gridDim.x * UNIT, g1 = units * (blockIdx.x + 1) / gridDim.x * UNIT;
 
   if (tid == 0) {
-    mbar_init(bar_empty0, 1);
-    mbar_init(bar_empty1, 1);
-    mbar_init(bar_acc0, 1);
-    mbar_init(bar_acc1, 1);
+    for (int s = 0; s < STAGES; ++s) {
+      mbar_init(bar_full + 8 * s, PRODUCERS / 32 / NCHUNK);
+      mbar_init(bar_empty + 8 * s, 1);
+    }
+    for (int a = 0; a < 2; ++a) {
+      mbar_init(bar_acc_full + 8 * a, 1);
+      mbar_init(bar_acc_empty + 8 * a, EPILOGUE / 32);
+    }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  if (warp == 0) {                                            // one warp owns the tensor-memory allocation
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" :: "r"(smem_u32(s_tmem)), "r"(TMEM_COLS) : "memory");
+  if (warp == MMA_WARP) {                                     // one warp owns the tensor-memory allocation
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" :: "r"(smem_u32(s_tmem)), "r"(RT_TMEM_COLS) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-  const uint32_t tmem_d = *s_tmem;
-
-  // the thread's share of a chunk: four 16-byte pieces, rows row0 + 32 i, piece c4 of the row
-  const int c4 = tid & 7, row0 = tid >> 3;
-  const int x_off = slab_offset(row0, c4);
-  float4 xr[NCHUNK][4];                                       // one tile ahead, in registers
-  // rows r_first + row0 + 32 i of the head whose keys start at Kh (nullptr: no such tile, zeros)
-  auto load_tile = [&](const T* Kh, long long r_first, int kc) {
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const long long r = r_first + row0 + 32 * i;
-      xr[kc][i] = (Kh != nullptr && r < n) ? load_row4<T>(Kh + (size_t)r * FATHOM_D + kc * KC + c4 * 4) : make_float4(0.f, 0.f, 0.f, 0.f);
-    }
-  };
-  auto head_keys = [&](long long kv) { return K + (size_t)kv * (size_t)n * FATHOM_D; };
-  if (g0 < g1) {
-#pragma unroll
-    for (int kc = 0; kc < NCHUNK; ++kc) load_tile(head_keys(g0 / tiles_per_head), (g0 % tiles_per_head) * TILE_M, kc);
-  }
+  const uint32_t tmem = *s_tmem;
 
   bool alive = true;                                          // false once a bounded wait ran out
-  uint32_t q = 0, tcount = 0;                                 // chunks and tiles handled so far (mbarrier phases)
-  long long cur_kv = -1;
-
-  // accumulator `acc` (tile number t, rows r0.. of head kv) -> registers -> per-warp staging -> 128-byte rows in global
-  // memory.  It runs one tile late, while the tensor cores work on the next tile in the other accumulator.
-  auto epilogue = [&](long long kv, long long r0, uint32_t t) {
-    const uint32_t acc = t & 1u;
-    if (alive && !mbar_wait(acc ? bar_acc1 : bar_acc0, (t >> 1) & 1u)) alive = false;
-    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    const int lq = warp & 3, cb = (warp >> 2) * 64;
-    float4* st4 = reinterpret_cast<float4*>(s_stage + warp * 1024);     // 32 rows of 8 16-byte pieces, piece f of row r at f ^ (r & 7)
-    float* out = K_rot + ((size_t)kv * (size_t)n + (size_t)r0 + lq * 32) * FATHOM_D + cb;
-    const int rows_valid = (int)min((long long)32, n - r0 - lq * 32);  // rows of this warp inside the sequence (may be <= 0)
-#pragma unroll
-    for (int p = 0; p < 2; ++p) {
-      uint32_t r[32];
-      const uint32_t taddr = tmem_d + ((uint32_t)(lq * 32) << 16) + acc * 128u + (uint32_t)(cb + p * 32);
-      asm volatile(
-          "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
-          "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];\n"
-          : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
-            "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]),
-            "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]),
-            "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-          : "r"(taddr) : "memory");
-      asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-      __syncwarp();
-#pragma unroll
-      for (int f = 0; f < 8; ++f)                                        // lane = row: its 32 columns as eight pieces
-        st4[lane * 8 + (f ^ (lane & 7))] = make_float4(__uint_as_float(r[4 * f]), __uint_as_float(r[4 * f + 1]),
-                                                        __uint_as_float(r[4 * f + 2]), __uint_as_float(r[4 * f + 3]));
-      __syncwarp();
-#pragma unroll
-      for (int it = 0; it < 8; ++it) {                                   // four rows of 128 bytes per store instruction
-        const int rr = it * 4 + (lane >> 3), f = lane & 7;
-        if (rr < rows_valid)
-          *reinterpret_cast<float4*>(out + (size_t)rr * FATHOM_D + p * 32 + f * 4) = st4[rr * 8 + (f ^ (rr & 7))];
-      }
-    }
-    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");   // a later MMA overwrites this accumulator
-  };
-
-  long long prev_kv = -1, prev_r0 = 0;                        // tile whose epilogue is still due
-  long long kv = g0 / tiles_per_head, tile_in_head = g0 % tiles_per_head;
-  for (long long g = g0; g < g1; ++g, ++tcount) {
-    const long long r0 = tile_in_head * TILE_M;
-    long long kv_next = kv, tile_next = tile_in_head + 1;     // the tile after this one (fetched while this one is handled)
-    if (tile_next == tiles_per_head) { tile_next = 0; ++kv_next; }
-    const T* K_next = (g + 1 < g1) ? head_keys(kv_next) : nullptr;
-    const long long r_next = tile_next * TILE_M;
-    if (kv != cur_kv) {                                       // new head: its split basis and mean into shared memory
-      if (prev_kv >= 0) { epilogue(prev_kv, prev_r0, tcount - 1); prev_kv = -1; }   // also waits for every MMA issued so far
-      __syncthreads();                                        // nobody reads the old basis any more
-      const float4* gh = reinterpret_cast<const float4*>(vh_t + (size_t)kv * FATHOM_D * FATHOM_D);
-      const float4* gl = reinterpret_cast<const float4*>(vl_t + (size_t)kv * FATHOM_D * FATHOM_D);
-      for (int e = tid; e < FATHOM_D * (FATHOM_D / 4); e += TC_THREADS) {
-        const int j = e >> 5, f = e & 31, kc = f >> 3, p = f & 7;       // row j, 16-byte piece f of the row
-        const int off = kc * SLAB + slab_offset(j, p);
-        *reinterpret_cast<float4*>(sm + OFF_VH + off) = __ldg(gh + e);
-        *reinterpret_cast<float4*>(sm + OFF_VL + off) = __ldg(gl + e);
-      }
-      if (tid < FATHOM_D) s_mu[tid] = mean[(size_t)kv * FATHOM_D + tid];
-      cur_kv = kv;
-      __syncthreads();
-    }
-    const uint32_t acc_col = tmem_d + (tcount & 1u) * 128u;
-#pragma unroll
-    for (int kc = 0; kc < NCHUNK; ++kc, ++q) {
-      const int buf = q & 1;
-      const uint32_t bar_empty = buf ? bar_empty1 : bar_empty0;
-      if (q >= 2 && alive && !mbar_wait(bar_empty, ((q >> 1) - 1) & 1)) alive = false;   // the MMAs that read this buffer are done
-      const float4 mu = *reinterpret_cast<const float4*>(s_mu + kc * KC + c4 * 4);
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const float4 x = xr[kc][i];
-        const float a0 = x.x - mu.x, a1 = x.y - mu.y, a2 = x.z - mu.z, a3 = x.w - mu.w;
-        const float h0 = tf32_head(a0), h1 = tf32_head(a1), h2 = tf32_head(a2), h3 = tf32_head(a3);
-        const int off = buf * SLAB + x_off + i * 4096;        // row0 + 32 i: four 8-row groups further, same place in the group
-        // (rows past the end of the sequence give rows of the accumulator that are never written out)
-        *reinterpret_cast<float4*>(sm + OFF_XH + off) = make_float4(h0, h1, h2, h3);
-        *reinterpret_cast<float4*>(sm + OFF_XL + off) = make_float4(tf32_head(a0 - h0), tf32_head(a1 - h1), tf32_head(a2 - h2), tf32_head(a3 - h3));
-      }
-      load_tile(K_next, r_next, kc);                          // the registers are free: fetch the next tile's chunk
-      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // generic-proxy stores -> visible to the MMA
-      asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-      __syncthreads();
-      if (tid == 0) {
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        const uint32_t xh = sm_base + OFF_XH + buf * SLAB, xl = sm_base + OFF_XL + buf * SLAB;
-        const uint32_t vh = sm_base + OFF_VH + kc * SLAB, vl = sm_base + OFF_VL + kc * SLAB;
-#pragma unroll
-        for (int ks = 0; ks < KC / UMMA_K; ++ks) {
-          const uint32_t ko = ks * UMMA_K * 4;                // bytes along K inside the swizzled row
-          umma_tf32(acc_col, umma_desc(xl + ko), umma_desc(vh + ko), (kc | ks) ? 1u : 0u);
-          umma_tf32(acc_col, umma_desc(xh + ko), umma_desc(vl + ko), 1u);
-          umma_tf32(acc_col, umma_desc(xh + ko), umma_desc(vh + ko), 1u);
-        }
-        umma_commit(bar_empty);
-        if (kc == NCHUNK - 1) umma_commit((tcount & 1u) ? bar_acc1 : bar_acc0);
-      }
-    }
-    if (prev_kv >= 0) epilogue(prev_kv, prev_r0, tcount - 1);  // the previous tile, while this one's MMAs run
-    prev_kv = kv;
-    prev_r0 = r0;
-    kv = kv_next;
-    tile_in_head = tile_next;
-  }
-  if (prev_kv >= 0) epilogue(prev_kv, prev_r0, tcount - 1);
-
-  // ---- all MMAs issued by this CTA are complete (their commits were waited for) unless a wait ran out
-  if (!alive && dev_status) atomicOr(dev_status, FATHOM_DEV_WAIT_EXPIRED);
-  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-  __syncthreads();
-  if (warp == 0) {
-    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" :: "r"(tmem_d), "r"(TMEM_COLS) : "memory");
-  }
-}
-
-// ---- rotation fused with the plane builder: planes and scales of (K - mu) V without ever storing the rotated keys ----
-// Same tile pipeline and the same sequence of MMAs as rotate_keys_tc_kernel (so every accumulator value is bit for bit
-// the rotated key that kernel would store), but the epilogue quantises instead of storing: a CTA takes 256 tokens at a
-// time (two tiles, one per accumulator = four 64-token blocks), and per block and channel forms a = max |k'| (one
-// redux per channel over the warp's 32 tokens, the two halves of a block meet in shared memory), the fp16 scale a/8,
-// the four plane bits of every code by the plane builder's comparisons with exact multiples of the stored scale, and
-// the plane words by warp ballots.  The four blocks' words of a (channel, plane) row are one 32-byte sector, written whole.
-constexpr int FB_PITCH = FATHOM_NPLANES * 4 * 2 + 1;         // words per channel in the staging: [plane][block][half], padded
-constexpr int FB_OFF_OUT = OFF_XL + 2 * SLAB;                // 128 x FB_PITCH words
-constexpr int FB_OFF_SCALE = FB_OFF_OUT + FATHOM_D * FB_PITCH * 4;          // 128 x 4 fp16
-constexpr int FB_OFF_AMAX = FB_OFF_SCALE + FATHOM_D * 4 * 2;                // [2 blocks][2 halves][128] floats
-constexpr int FB_OFF_MU = FB_OFF_AMAX + 2 * 2 * FATHOM_D * 4;
-constexpr int FB_OFF_BAR = FB_OFF_MU + FATHOM_D * 4;
-constexpr int FB_SMEM = FB_OFF_BAR + 64 + 1024;
-
-template <typename T>
-__global__ void __launch_bounds__(TC_THREADS, 1)
-rotate_build_tc_kernel(const T* __restrict__ K, const float* __restrict__ mean, const float* __restrict__ vh_t,
-                       const float* __restrict__ vl_t, uint32_t* __restrict__ planes32, uint16_t* __restrict__ scales,
-                       long long n, long long plane_stride, long long scale_stride, uint32_t* __restrict__ dev_status) {
-  extern __shared__ unsigned char smem_raw[];
-  unsigned char* sm = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
-  const uint32_t sm_base = smem_u32(sm);
-  float* s_mu = reinterpret_cast<float*>(sm + FB_OFF_MU);
-  uint32_t* s_out = reinterpret_cast<uint32_t*>(sm + FB_OFF_OUT);
-  uint16_t* s_scale = reinterpret_cast<uint16_t*>(sm + FB_OFF_SCALE);
-  float* s_amax = reinterpret_cast<float*>(sm + FB_OFF_AMAX);
-  uint32_t* s_tmem = reinterpret_cast<uint32_t*>(sm + FB_OFF_BAR + 32);
-  const uint32_t bar_empty0 = sm_base + FB_OFF_BAR, bar_empty1 = sm_base + FB_OFF_BAR + 8, bar_acc0 = sm_base + FB_OFF_BAR + 16,
-                 bar_acc1 = sm_base + FB_OFF_BAR + 24;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, kv = blockIdx.y;
-  const long long nb = (n + FATHOM_BLOCK - 1) / FATHOM_BLOCK;
-  const long long supers = (n + 255) / 256;                   // 256-token units of this head
-  const long long u0 = supers * blockIdx.x / gridDim.x, u1 = supers * (blockIdx.x + 1) / gridDim.x;
-  const T* Kh = K + (size_t)kv * (size_t)n * FATHOM_D;
-
-  if (tid == 0) {
-    mbar_init(bar_empty0, 1);
-    mbar_init(bar_empty1, 1);
-    mbar_init(bar_acc0, 1);
-    mbar_init(bar_acc1, 1);
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-  }
-  if (warp == 0) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" :: "r"(smem_u32(s_tmem)), "r"(TMEM_COLS) : "memory");
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-  }
-  {                                                           // the head's split basis and mean
-    const float4* gh = reinterpret_cast<const float4*>(vh_t + (size_t)kv * FATHOM_D * FATHOM_D);
-    const float4* gl = reinterpret_cast<const float4*>(vl_t + (size_t)kv * FATHOM_D * FATHOM_D);
-    for (int e = tid; e < FATHOM_D * (FATHOM_D / 4); e += TC_THREADS) {
-      const int j = e >> 5, f = e & 31, kc = f >> 3, p = f & 7;
-      const int off = kc * SLAB + slab_offset(j, p);
-      *reinterpret_cast<float4*>(sm + OFF_VH + off) = __ldg(gh + e);
-      *reinterpret_cast<float4*>(sm + OFF_VL + off) = __ldg(gl + e);
-    }
-    if (tid < FATHOM_D) s_mu[tid] = mean[(size_t)kv * FATHOM_D + tid];
-  }
-  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-  __syncthreads();
-  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-  const uint32_t tmem_d = *s_tmem;
-
-  const int c4 = tid & 7, row0 = tid >> 3;
-  const int x_off = slab_offset(row0, c4);
-  float4 xr[NCHUNK][4];                                       // one 128-token tile ahead, in registers
-  const long long tile_end = u1 * 2;                          // tiles of this CTA: [2 u0, 2 u1)
-  auto load_tile = [&](long long tile, int kc) {
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const long long r = tile * TILE_M + row0 + 32 * i;
-      xr[kc][i] = (tile < tile_end && r < n) ? load_row4<T>(Kh + (size_t)r * FATHOM_D + kc * KC + c4 * 4) : make_float4(0.f, 0.f, 0.f, 0.f);
+  // one lane polls for its warp
+  auto wait = [&](uint32_t bar, uint32_t parity) {
+    if (alive) {
+      bool ok = true;
+      if (lane == 0) ok = mbar_wait(bar, parity);
+      alive = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
     }
   };
-  if (u0 < u1) {
-#pragma unroll
-    for (int kc = 0; kc < NCHUNK; ++kc) load_tile(2 * u0, kc);
-  }
+  uint32_t stage = 0, phase = 0;                              // MMA thread: ring position and its round's parity
+  uint32_t tcount = 0;                                        // tiles so far: accumulator and its parity
 
-  bool alive = true;
-  uint32_t q = 0, ucount = 0;
-  for (long long u = u0; u < u1; ++u, ++ucount) {
-    // ---- both tiles of the unit: chunks -> shared memory -> MMAs into accumulator 0 / 1
-#pragma unroll
-    for (int sub = 0; sub < 2; ++sub) {
-      const long long tile = 2 * u + sub;
-      const uint32_t acc_col = tmem_d + (uint32_t)sub * 128u;
-#pragma unroll
-      for (int kc = 0; kc < NCHUNK; ++kc, ++q) {
-        const int buf = q & 1;
-        const uint32_t bar_empty = buf ? bar_empty1 : bar_empty0;
-        if (q >= 2 && alive && !mbar_wait(bar_empty, ((q >> 1) - 1) & 1)) alive = false;
-        const float4 mu = *reinterpret_cast<const float4*>(s_mu + kc * KC + c4 * 4);
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          const float4 x = xr[kc][i];
-          const float a0 = x.x - mu.x, a1 = x.y - mu.y, a2 = x.z - mu.z, a3 = x.w - mu.w;
-          const float h0 = tf32_head(a0), h1 = tf32_head(a1), h2 = tf32_head(a2), h3 = tf32_head(a3);
-          const int off = buf * SLAB + x_off + i * 4096;
-          *reinterpret_cast<float4*>(sm + OFF_XH + off) = make_float4(h0, h1, h2, h3);
-          *reinterpret_cast<float4*>(sm + OFF_XL + off) = make_float4(tf32_head(a0 - h0), tf32_head(a1 - h1), tf32_head(a2 - h2), tf32_head(a3 - h3));
-        }
-        load_tile(tile + 1, kc);
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-        __syncthreads();
-        if (tid == 0) {
-          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-          const uint32_t xh = sm_base + OFF_XH + buf * SLAB, xl = sm_base + OFF_XL + buf * SLAB;
-          const uint32_t vh = sm_base + OFF_VH + kc * SLAB, vl = sm_base + OFF_VL + kc * SLAB;
-#pragma unroll
-          for (int ks = 0; ks < KC / UMMA_K; ++ks) {
-            const uint32_t ko = ks * UMMA_K * 4;
-            umma_tf32(acc_col, umma_desc(xl + ko), umma_desc(vh + ko), (kc | ks) ? 1u : 0u);
-            umma_tf32(acc_col, umma_desc(xh + ko), umma_desc(vl + ko), 1u);
-            umma_tf32(acc_col, umma_desc(xh + ko), umma_desc(vh + ko), 1u);
-          }
-          umma_commit(bar_empty);
-          if (kc == NCHUNK - 1) umma_commit(sub ? bar_acc1 : bar_acc0);
-        }
-      }
-    }
-    // ---- quantising epilogue, tile by tile.  Warp w: tokens 32 (w & 3) .. + 31 of the tile, channels 64 (w >> 2) .. + 63.
-    const int lq = warp & 3, blk = lq >> 1, half = lq & 1, cb = (warp >> 2) * 64;
+  for (long long g = g0; g < g1;) {                           // head by head
+    const long long kv = g / tiles_per_head, tile0 = g - kv * tiles_per_head;
+    const long long count = min(g1, (kv + 1) * tiles_per_head) - g;
+    g += count;
+    // ---- the head's split basis into tensor memory (lane = rotated channel j, column = channel c), its mean into shared memory
+    if (warp < 4) {
+      const float* V = basis + (size_t)kv * FATHOM_D * FATHOM_D + tid;
 #pragma unroll 1
-    for (int sub = 0; sub < 2; ++sub) {
-      if (alive && !mbar_wait(sub ? bar_acc1 : bar_acc0, ucount & 1)) alive = false;
-      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      const long long tok = (2 * u + sub) * TILE_M + lq * 32 + lane;          // this lane's token
-      const bool present = tok < n;
-      const uint32_t keep = __ballot_sync(0xffffffffu, present);             // absent tail tokens carry 0 bits
-      uint32_t r[2][32];
-#pragma unroll
-      for (int p = 0; p < 2; ++p) {
-        const uint32_t taddr = tmem_d + ((uint32_t)(lq * 32) << 16) + (uint32_t)sub * 128u + (uint32_t)(cb + p * 32);
-        asm volatile(
-            "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
-            "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];\n"
-            : "=r"(r[p][0]), "=r"(r[p][1]), "=r"(r[p][2]), "=r"(r[p][3]), "=r"(r[p][4]), "=r"(r[p][5]), "=r"(r[p][6]), "=r"(r[p][7]),
-              "=r"(r[p][8]), "=r"(r[p][9]), "=r"(r[p][10]), "=r"(r[p][11]), "=r"(r[p][12]), "=r"(r[p][13]), "=r"(r[p][14]),
-              "=r"(r[p][15]), "=r"(r[p][16]), "=r"(r[p][17]), "=r"(r[p][18]), "=r"(r[p][19]), "=r"(r[p][20]), "=r"(r[p][21]),
-              "=r"(r[p][22]), "=r"(r[p][23]), "=r"(r[p][24]), "=r"(r[p][25]), "=r"(r[p][26]), "=r"(r[p][27]), "=r"(r[p][28]),
-              "=r"(r[p][29]), "=r"(r[p][30]), "=r"(r[p][31])
-            : "r"(taddr) : "memory");
-      }
-      asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-      // block maximum per channel: |k'| of non-negative floats orders like its bit pattern, so one integer redux per
-      // channel gives the warp's maximum; lane c keeps channel c's
-#pragma unroll
-      for (int p = 0; p < 2; ++p) {
-        uint32_t mine = 0u;
+      for (int c0 = 0; c0 < 2 * FATHOM_D; c0 += 32) {         // heads, then tails (32 registers at a time)
+        uint32_t part[32];
 #pragma unroll
         for (int c = 0; c < 32; ++c) {
-          if (!present) r[p][c] = 0u;                         // an absent token counts as 0 everywhere
-          const uint32_t m = __reduce_max_sync(0xffffffffu, r[p][c] & 0x7fffffffu);
-          if (lane == c) mine = m;
+          const float v = __ldg(V + ((c0 & (FATHOM_D - 1)) + c) * FATHOM_D), vh = tf32_head(v);
+          part[c] = __float_as_uint(c0 < FATHOM_D ? vh : tf32_head(v - vh));
         }
-        s_amax[(blk * 2 + half) * FATHOM_D + cb + p * 32 + lane] = __uint_as_float(mine);
+        tmem_store32(tmem + ((uint32_t)(warp * 32) << 16) + COL_VH + c0, part);
       }
-      __syncthreads();                                        // the two halves of every block have met
-#pragma unroll
-      for (int p = 0; p < 2; ++p) {
-        const int ch = cb + p * 32 + lane;                    // the channel whose scale and plane words this lane keeps
-        const float a = fmaxf(s_amax[(blk * 2 + 0) * FATHOM_D + ch], s_amax[(blk * 2 + 1) * FATHOM_D + ch]);
-        const __half sh = __float2half_rn(a * 0.125f);        // a/8 is exact; one rounding to fp16
-        const float my_sc = __half2float(sh);
-        uint32_t w0 = 0u, w1 = 0u, w2 = 0u, w3 = 0u;
-#pragma unroll
-        for (int c = 0; c < 32; ++c) {
-          const float sc = __shfl_sync(0xffffffffu, my_sc, c);               // scale of channel cb + 32 p + c
-          const float k = __uint_as_float(r[p][c]);
-          const float s2 = sc * 2.0f, s4 = sc * 4.0f;
-          const bool c0 = k >= 0.0f;
-          float thr = c0 ? s4 : -s4;
-          const bool c1 = k >= thr;
-          thr += c1 ? s2 : -s2;
-          const bool c2 = k >= thr;
-          thr += c2 ? sc : -sc;
-          const bool c3 = k >= thr;
-          const uint32_t b0 = __ballot_sync(0xffffffffu, c0), b1 = __ballot_sync(0xffffffffu, c1);
-          const uint32_t b2 = __ballot_sync(0xffffffffu, c2), b3 = __ballot_sync(0xffffffffu, c3);
-          if (lane == c) { w0 = b0; w1 = b1; w2 = b2; w3 = b3; }
-        }
-        if (my_sc > 0.0f) { w0 &= keep; w1 &= keep; w2 &= keep; w3 &= keep; }
-        else { w0 = keep; w1 = 0u; w2 = 0u; w3 = 0u; }        // zero scale: every code is 8 = 0b1000
-        const int bu = 2 * sub + blk;                         // block within the 256-token unit
-        uint32_t* o = s_out + ch * FB_PITCH;
-        o[(0 * 4 + bu) * 2 + half] = w0;
-        o[(1 * 4 + bu) * 2 + half] = w1;
-        o[(2 * 4 + bu) * 2 + half] = w2;
-        o[(3 * 4 + bu) * 2 + half] = w3;
-        if (half == 0) s_scale[ch * 4 + bu] = __half_as_ushort(sh);
-      }
-      asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-      __syncthreads();                                        // s_amax is reused by the next tile
+      asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+    } else if (warp < 8) {
+      s_mu[tid - 128] = mean[(size_t)kv * FATHOM_D + tid - 128];
     }
-    // ---- flush: the unit's four blocks of every (channel, plane) row are 32 contiguous bytes
-    {
-      const long long b0 = 4 * u;
-      const int nblk = (int)min((long long)4, nb - b0);
-      uint64_t* planes64 = reinterpret_cast<uint64_t*>(planes32);
-      for (int e = tid; e < FATHOM_D * FATHOM_NPLANES; e += TC_THREADS) {
-        const int ch = e >> 2, p = e & 3;
-        const uint32_t* src = s_out + ch * FB_PITCH + p * 8;
-        uint64_t* dst = planes64 + (((size_t)kv * FATHOM_D + ch) * FATHOM_NPLANES + p) * (size_t)plane_stride + b0;
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+
+    if (tid < PRODUCERS) {
+      // ---- producers: warp = (chunk kc, 32 rows of the tile), lane = (16 bytes of a row, every fourth or eighth row).  The warps of a tile
+      //      work on its four chunks side by side: a warp goes through wait - store - fence - arrive once per tile (all warps
+      //      on one chunk after the other went through it four times, and that chain was the longest of the kernel)
+      constexpr int CH = 16 / sizeof(T);                      // channels per 16-byte load: one or two 16-byte pieces of a tf32 row
+      constexpr int LANES = KC / CH, STEP = 32 / LANES, LOADS = 4 * ROWS_PER_LANE / STEP;
+      const int kc = warp & (NCHUNK - 1), row0 = (warp / NCHUNK) * (4 * ROWS_PER_LANE) + lane / LANES, c0 = (lane % LANES) * CH;
+      const T* Kh = K + (size_t)kv * (size_t)n * FATHOM_D + kc * KC + c0;
+      float mu[CH];
 #pragma unroll
-        for (int pair = 0; pair < 2; ++pair) {
-          if (2 * pair + 1 < nblk) {
-            *reinterpret_cast<uint4*>(dst + 2 * pair) = make_uint4(src[4 * pair], src[4 * pair + 1], src[4 * pair + 2], src[4 * pair + 3]);
-          } else if (2 * pair < nblk) {
-            dst[2 * pair] = ((uint64_t)src[4 * pair + 1] << 32) | src[4 * pair];
+      for (int c = 0; c < CH; ++c) mu[c] = s_mu[kc * KC + c0 + c];
+      uint4 xr[LOADS];                                        // one tile ahead, in registers, as loaded
+      auto load_tile = [&](long long tile) {
+        const long long r0 = tile * TILE_M + row0;
+        const uint4* p = reinterpret_cast<const uint4*>(Kh + (size_t)r0 * FATHOM_D);
+        constexpr int PITCH = STEP * FATHOM_D / CH;
+        if (r0 + STEP * (LOADS - 1) < n) {
+#pragma unroll
+          for (int i = 0; i < LOADS; ++i) xr[i] = __ldg(p + i * PITCH);
+        } else {
+#pragma unroll
+          for (int i = 0; i < LOADS; ++i) xr[i] = r0 + STEP * i < n ? __ldg(p + i * PITCH) : make_uint4(0u, 0u, 0u, 0u);
+        }
+      };
+      load_tile(tile0);
+      for (long long t = 0; t < count; ++t, ++tcount) {
+        const uint32_t q = tcount * NCHUNK + kc, stage = q % STAGES, round = q / STAGES;
+        wait(bar_empty + 8 * stage, (round & 1u) ^ 1u);       // (a fresh barrier lets the first round through)
+        unsigned char* xs = sm + stage * STAGE_BYTES;
+#pragma unroll
+        for (int i = 0; i < LOADS; ++i) {
+          float x[CH];
+          unpack16(xr[i], x);
+#pragma unroll
+          for (int f = 0; f < CH / 4; ++f) {
+            float h[4], l[4];
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+              const float a = x[4 * f + c] - mu[4 * f + c];
+              h[c] = tf32_head(a);
+              l[c] = tf32_head(a - h[c]);
+            }
+            // (rows past the end of the sequence give columns of the accumulator that are never used)
+            const int off = slab_offset(row0 + STEP * i, c0 / 4 + f);
+            *reinterpret_cast<float4*>(xs + off) = make_float4(h[0], h[1], h[2], h[3]);
+            *reinterpret_cast<float4*>(xs + SLAB + off) = make_float4(l[0], l[1], l[2], l[3]);
+          }
+        }
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // generic-proxy stores -> visible to the MMA
+        __syncwarp();
+        if (lane == 0) mbar_arrive(bar_full + 8 * stage);
+        if (t + 1 < count) load_tile(tile0 + t + 1);          // (not before the fence, which would wait for the loads' issue)
+      }
+    } else if (warp == MMA_WARP) {
+      // (the whole warp runs the loop, one elected lane issues: addresses and descriptors then stay in uniform registers; issued
+      // from a divergent branch an MMA took 66 to 80 cycles to issue, as long as it takes to run)
+      const uint32_t base = __shfl_sync(0xffffffffu, sm_base, 0), tm = __shfl_sync(0xffffffffu, tmem, 0);
+      bool ready = false;                                     // what a barrier said when it was asked ahead of time: an answer takes
+                                                              // ~300 cycles while the other warps store, four MMAs' worth
+      for (long long t = 0; t < count; ++t, ++tcount) {
+        const uint32_t buf = tcount & 1u, acc = tm + COL_ACC + buf * 128u;
+        if (alive && !mbar_wait(bar_acc_empty + 8 * buf, ((tcount >> 1) & 1u) ^ 1u)) alive = false;
+#pragma unroll
+        for (int kc = 0; kc < NCHUNK; ++kc) {
+          if (alive && !ready && !mbar_wait(bar_full + 8 * stage, phase)) alive = false;
+          const uint32_t next = stage + 1 == STAGES ? 0u : stage + 1;
+          ready = mbar_test(bar_full + 8 * next, phase ^ (next == 0u ? 1u : 0u));
+          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+          const uint64_t xh = umma_desc(base + stage * STAGE_BYTES), xl = umma_desc(base + stage * STAGE_BYTES + SLAB);
+          if (elect_one()) {
+#pragma unroll
+            for (int ks = 0; ks < KC / UMMA_K; ++ks) {
+              const uint32_t vh = tm + COL_VH + kc * KC + ks * UMMA_K, vl = tm + COL_VL + kc * KC + ks * UMMA_K;
+              const uint64_t ko = ks * UMMA_K * 4 >> 4;       // 16-byte units along K inside the swizzled row
+              umma_tf32_ts(acc, vh, xl + ko, (kc | ks) ? 1u : 0u);
+              umma_tf32_ts(acc, vl, xh + ko, 1u);
+              umma_tf32_ts(acc, vh, xh + ko, 1u);
+            }
+            umma_commit(bar_empty + 8 * stage);
+            if (kc == NCHUNK - 1) umma_commit(bar_acc_full + 8 * buf);
+          }
+          __syncwarp();
+          if (++stage == STAGES) { stage = 0; phase ^= 1u; }
+        }
+      }
+    } else {
+      // ---- epilogue: my channel, my block of every tile
+      const int lq = warp & 3, blk = (warp - PRODUCERS / 32) >> 2, ch = lq * 32 + lane;
+      for (long long t = 0; t < count; ++t, ++tcount) {
+        const long long tile = tile0 + t;
+        const uint32_t buf = tcount & 1u;
+        float r[32];
+        wait(bar_acc_full + 8 * buf, (tcount >> 1) & 1u);
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        const uint32_t taddr = tmem + ((uint32_t)(lq * 32) << 16) + COL_ACC + buf * 128u + (uint32_t)(blk * FATHOM_BLOCK);
+        auto load_half = [&](int half) {                      // 32 tokens at a time: 64 would spill
+          tmem_load32(taddr + 32 * half, r);
+          asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+        };
+        auto hand_back = [&]() {                              // a later MMA overwrites the accumulator
+          asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+          __syncwarp();
+          if (lane == 0) mbar_arrive(bar_acc_empty + 8 * buf);
+        };
+        const long long tok0 = tile * TILE_M + blk * FATHOM_BLOCK;
+        const int valid = (int)min((long long)FATHOM_BLOCK, n - tok0);       // tokens of this block (may be <= 0)
+        if (!BUILD) {
+          float* out = K_rot + ((size_t)kv * (size_t)n + (size_t)tok0) * FATHOM_D + ch;
+#pragma unroll
+          for (int half = 0; half < 2; ++half) {
+            load_half(half);
+            if (half == 1) hand_back();
+            if (valid == FATHOM_BLOCK) {
+#pragma unroll
+              for (int i = 0; i < 32; ++i) out[(32 * half + i) * FATHOM_D] = r[i];
+            } else {
+#pragma unroll
+              for (int i = 0; i < 32; ++i)
+                if (32 * half + i < valid) out[(32 * half + i) * FATHOM_D] = r[i];
+            }
+          }
+        } else {
+          // the plane builder's quantiser (build_planes.cu) on one thread's block; absent tail tokens count as 0
+          float a = 0.0f;
+          auto largest = [&](int half) {
+            if (valid < 32 * half + 32) {
+#pragma unroll
+              for (int i = 0; i < 32; ++i)
+                if (32 * half + i >= valid) r[i] = 0.0f;
+            }
+#pragma unroll
+            for (int i = 0; i < 32; i += 2) a = fmaxf(a, fmaxf(fabsf(r[i]), fabsf(r[i + 1])));
+          };
+          load_half(1);
+          largest(1);
+          load_half(0);
+          largest(0);
+          const __half sh = __float2half_rn(a * 0.125f);      // a/8 is exact; one rounding to fp16
+          const float sc = __half2float(sh), inv = 1.0f / sc;
+          const int bu = (int)(tile % UNIT) * (TILE_M / FATHOM_BLOCK) + blk;
+          uint32_t* o = reinterpret_cast<uint32_t*>(sm + MP::OUT) + ch * OUT_PITCH + bu * 2;
+#pragma unroll
+          for (int half = 0; half < 2; ++half) {
+            if (half == 1) {
+              load_half(1);
+              hand_back();
+            }
+            const int left = valid - 32 * half;
+            const uint32_t keep = left >= 32 ? ~0u : (left <= 0 ? 0u : (~0u >> (32 - left)));   // absent tail tokens carry 0 bits
+            uint32_t w[FATHOM_NPLANES];
+            fathom_quantise32(r, sc, inv, w);
+            if (!(sc > 0.0f)) { w[0] = ~0u; w[1] = w[2] = w[3] = 0u; }      // zero scale: every code is 8 = 0b1000
+#pragma unroll
+            for (int p = 0; p < FATHOM_NPLANES; ++p) o[p * UNIT_BLOCKS * 2 + half] = w[p] & keep;
+          }
+          reinterpret_cast<uint16_t*>(sm + MP::SCALE)[ch * UNIT_BLOCKS + bu] = __half_as_ushort(sh);
+          if ((tile + 1) % UNIT == 0) {
+            // ---- flush: the unit's four blocks of every (channel, plane) row are 32 contiguous bytes
+            epilogue_barrier();
+            const int et = tid - PRODUCERS;
+            const long long nb = (n + FATHOM_BLOCK - 1) / FATHOM_BLOCK, b0 = tile / UNIT * UNIT_BLOCKS;
+            const int nblk = (int)min((long long)UNIT_BLOCKS, nb - b0);
+            const uint32_t* staged = reinterpret_cast<const uint32_t*>(sm + MP::OUT);
+            for (int e = et; e < FATHOM_D * FATHOM_NPLANES; e += EPILOGUE) {
+              const uint32_t* src = staged + (e >> 2) * OUT_PITCH + (e & 3) * UNIT_BLOCKS * 2;
+              uint64_t* dst = planes + ((size_t)kv * FATHOM_D * FATHOM_NPLANES + e) * (size_t)plane_stride + b0;
+#pragma unroll
+              for (int pair = 0; pair < UNIT_BLOCKS / 2; ++pair) {
+                if (2 * pair + 1 < nblk) {
+                  *reinterpret_cast<uint4*>(dst + 2 * pair) = make_uint4(src[4 * pair], src[4 * pair + 1], src[4 * pair + 2], src[4 * pair + 3]);
+                } else if (2 * pair < nblk) {
+                  dst[2 * pair] = ((uint64_t)src[4 * pair + 1] << 32) | src[4 * pair];
+                }
+              }
+            }
+            if (et < FATHOM_D) {
+              const uint16_t* src = reinterpret_cast<const uint16_t*>(sm + MP::SCALE) + et * UNIT_BLOCKS;
+              uint16_t* dst = scales + ((size_t)kv * FATHOM_D + et) * (size_t)scale_stride + b0;
+              if (nblk == UNIT_BLOCKS) {
+                *reinterpret_cast<uint2*>(dst) = *reinterpret_cast<const uint2*>(src);
+              } else {
+                for (int x = 0; x < nblk; ++x) dst[x] = src[x];
+              }
+            }
+            epilogue_barrier();                               // the staging is rewritten by the next unit
           }
         }
       }
-      if (tid < FATHOM_D) {
-        uint16_t* dst = scales + ((size_t)kv * FATHOM_D + tid) * (size_t)scale_stride + b0;
-        for (int x = 0; x < nblk; ++x) dst[x] = s_scale[tid * 4 + x];
-      }
     }
-    __syncthreads();                                          // the staging is rewritten by the next unit
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();                                          // the epilogue has waited for every MMA of the head: basis and mean may change
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   }
 
   if (!alive && dev_status) atomicOr(dev_status, FATHOM_DEV_WAIT_EXPIRED);
-  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
-  if (warp == 0) {
-    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" :: "r"(tmem_d), "r"(TMEM_COLS) : "memory");
-  }
+  if (warp == MMA_WARP)
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" :: "r"(tmem), "r"(RT_TMEM_COLS) : "memory");
 }
 
 // ---- covariance partials on the tensor cores: C = sum_t (x_t - mu)(x_t - mu)^T ----------------------------------------
@@ -706,32 +638,40 @@ cov_partial_tc_kernel(const T* __restrict__ K, const float* __restrict__ shift, 
 
 }  // namespace
 
-size_t fathom_rotate_tc_scratch_bytes(int Hkv) { return fathom_round_up((size_t)2 * Hkv * FATHOM_D * FATHOM_D * 4, 256); }
-
-// Enqueues the tensor-core rotation; scratch holds the split, transposed basis (fathom_rotate_tc_scratch_bytes).
-int fathom_launch_rotate_tc(fathom_ctx* ctx, const fathom_layout* L, const void* K, int k_dtype, const float* mean,
-                            const float* basis, float* K_rot, void* scratch, cudaStream_t st) {
-  const int Hkv = L->n_kv_heads;
-  const long long n = L->n;
-  float* vh_t = static_cast<float*>(scratch);
-  float* vl_t = vh_t + (size_t)Hkv * FATHOM_D * FATHOM_D;
-  split_basis_kernel<<<dim3(FATHOM_D, Hkv), FATHOM_D, 0, st>>>(basis, vh_t, vl_t);
-  int dev = 0, sms = 0;
+namespace {
+template <typename T, bool BUILD>
+int launch_rotate(fathom_ctx* ctx, const fathom_layout* L, const void* K, const float* mean, const float* basis, float* K_rot,
+                  uint64_t* planes, uint16_t* scales, cudaStream_t st) {
+  static bool configured[64] = {};
+  static int sms[64] = {};
+  int dev = 0;
   FATHOM_CUDA_TRY(ctx, cudaGetDevice(&dev));
-  FATHOM_CUDA_TRY(ctx, cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-  const long long tiles_per_head = (n + TILE_M - 1) / TILE_M, total = tiles_per_head * Hkv;
-  const unsigned grid = (unsigned)(total < sms ? total : sms);
-  if (k_dtype == FATHOM_F32) {
-    FATHOM_CUDA_TRY(ctx, cudaFuncSetAttribute(rotate_keys_tc_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, TC_SMEM));
-    rotate_keys_tc_kernel<float><<<grid, TC_THREADS, TC_SMEM, st>>>(static_cast<const float*>(K), mean, vh_t, vl_t, K_rot, n,
-                                                                     tiles_per_head, total, ctx->dev_status);
-  } else {
-    FATHOM_CUDA_TRY(ctx, cudaFuncSetAttribute(rotate_keys_tc_kernel<__nv_bfloat16>, cudaFuncAttributeMaxDynamicSharedMemorySize, TC_SMEM));
-    rotate_keys_tc_kernel<__nv_bfloat16><<<grid, TC_THREADS, TC_SMEM, st>>>(static_cast<const __nv_bfloat16*>(K), mean, vh_t, vl_t,
-                                                                             K_rot, n, tiles_per_head, total, ctx->dev_status);
+  const int slot = dev >= 0 && dev < 64 ? dev : 0;
+  if (!configured[slot] || slot != dev) {
+    FATHOM_CUDA_TRY(ctx, cudaDeviceGetAttribute(&sms[slot], cudaDevAttrMultiProcessorCount, dev));
+    FATHOM_CUDA_TRY(ctx, cudaFuncSetAttribute(rotate_tc_kernel<T, BUILD>, cudaFuncAttributeMaxDynamicSharedMemorySize, Map<BUILD>::BYTES));
+    configured[slot] = true;
   }
+  constexpr int UNIT = BUILD ? UNIT_BLOCKS * FATHOM_BLOCK / TILE_M : 1;
+  const long long per_head = (L->n + TILE_M * UNIT - 1) / (TILE_M * UNIT) * UNIT, total = per_head * L->n_kv_heads;
+  const unsigned grid = (unsigned)(total / UNIT < sms[slot] ? total / UNIT : sms[slot]);
+  rotate_tc_kernel<T, BUILD><<<grid, RT_THREADS, Map<BUILD>::BYTES, st>>>(static_cast<const T*>(K), mean, basis, K_rot, planes, scales, L->n,
+                                                                L->plane_stride_words, L->scale_stride, per_head, total, ctx->dev_status);
   FATHOM_CUDA_TRY(ctx, cudaGetLastError());
   return FATHOM_OK;
+}
+}  // namespace
+
+int fathom_launch_rotate_tc(fathom_ctx* ctx, const fathom_layout* L, const void* K, int k_dtype, const float* mean,
+                            const float* basis, float* K_rot, cudaStream_t st) {
+  return k_dtype == FATHOM_F32 ? launch_rotate<float, false>(ctx, L, K, mean, basis, K_rot, nullptr, nullptr, st)
+                               : launch_rotate<__nv_bfloat16, false>(ctx, L, K, mean, basis, K_rot, nullptr, nullptr, st);
+}
+
+int fathom_launch_rotate_build_tc(fathom_ctx* ctx, const fathom_layout* L, const void* K, int k_dtype, const float* mean,
+                                  const float* basis, uint64_t* planes, uint16_t* scales, cudaStream_t st) {
+  return k_dtype == FATHOM_F32 ? launch_rotate<float, true>(ctx, L, K, mean, basis, nullptr, planes, scales, st)
+                               : launch_rotate<__nv_bfloat16, true>(ctx, L, K, mean, basis, nullptr, planes, scales, st);
 }
 
 // CTAs per KV head of the tensor-core covariance pass (one 128 x 128 partial each)
@@ -757,36 +697,6 @@ int fathom_launch_cov_tc(fathom_ctx* ctx, const fathom_layout* L, const void* K,
     cov_shift_kernel<__nv_bfloat16><<<L->n_kv_heads, FATHOM_D, 0, st>>>(static_cast<const __nv_bfloat16*>(K), L->n, shift);
     cov_partial_tc_kernel<__nv_bfloat16><<<grid, TC_THREADS, CV_SMEM, st>>>(static_cast<const __nv_bfloat16*>(K), shift, partial,
                                                                              partial_sum, L->n, ctx->dev_status);
-  }
-  FATHOM_CUDA_TRY(ctx, cudaGetLastError());
-  return FATHOM_OK;
-}
-
-// Enqueues the fused rotation + plane builder; scratch holds the split, transposed basis (fathom_rotate_tc_scratch_bytes).
-int fathom_launch_rotate_build_tc(fathom_ctx* ctx, const fathom_layout* L, const void* K, int k_dtype, const float* mean,
-                                  const float* basis, uint64_t* planes, uint16_t* scales, void* scratch, cudaStream_t st) {
-  const int Hkv = L->n_kv_heads;
-  const long long n = L->n;
-  float* vh_t = static_cast<float*>(scratch);
-  float* vl_t = vh_t + (size_t)Hkv * FATHOM_D * FATHOM_D;
-  split_basis_kernel<<<dim3(FATHOM_D, Hkv), FATHOM_D, 0, st>>>(basis, vh_t, vl_t);
-  int dev = 0, sms = 0;
-  FATHOM_CUDA_TRY(ctx, cudaGetDevice(&dev));
-  FATHOM_CUDA_TRY(ctx, cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-  const long long supers = (n + 255) / 256;
-  long long per_head = sms / Hkv > 0 ? sms / Hkv : 1;
-  if (per_head > supers) per_head = supers;
-  dim3 grid((unsigned)per_head, (unsigned)Hkv);
-  uint32_t* p32 = reinterpret_cast<uint32_t*>(planes);
-  if (k_dtype == FATHOM_F32) {
-    FATHOM_CUDA_TRY(ctx, cudaFuncSetAttribute(rotate_build_tc_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, FB_SMEM));
-    rotate_build_tc_kernel<float><<<grid, TC_THREADS, FB_SMEM, st>>>(static_cast<const float*>(K), mean, vh_t, vl_t, p32, scales, n,
-                                                                      L->plane_stride_words, L->scale_stride, ctx->dev_status);
-  } else {
-    FATHOM_CUDA_TRY(ctx, cudaFuncSetAttribute(rotate_build_tc_kernel<__nv_bfloat16>, cudaFuncAttributeMaxDynamicSharedMemorySize, FB_SMEM));
-    rotate_build_tc_kernel<__nv_bfloat16><<<grid, TC_THREADS, FB_SMEM, st>>>(static_cast<const __nv_bfloat16*>(K), mean, vh_t, vl_t, p32,
-                                                                              scales, n, L->plane_stride_words, L->scale_stride,
-                                                                              ctx->dev_status);
   }
   FATHOM_CUDA_TRY(ctx, cudaGetLastError());
   return FATHOM_OK;
