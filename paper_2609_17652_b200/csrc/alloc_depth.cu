@@ -39,19 +39,28 @@ alloc_depth_kernel(const float* __restrict__ q, const float* __restrict__ var, i
   if (tid < FATHOM_D) {                                       // thread = channel: its four priorities
     const int j = tid;
     double acc = 0.0;
-    if (mode == FATHOM_DEPTH_WATERFILL) {
-      for (int h = h0; h < h0 + heads_per_plan; ++h) {
-        const double x = (double)q[(size_t)h * FATHOM_D + j];
-        acc = __dadd_rn(acc, __dmul_rn(x, x));                // Eq. 3, heads in ascending order
+    const float* qj = q + (size_t)h0 * FATHOM_D + j;
+    auto add_heads = [&](auto term) {                         // ascending order; up to four loads in flight
+      int h = 0;
+      for (; h + 4 <= heads_per_plan; h += 4) {
+        float x[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) x[u] = qj[(h + u) * FATHOM_D];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) acc = __dadd_rn(acc, term((double)x[u]));
       }
-      const double g = __dmul_rn(acc, (double)var[(size_t)kv * FATHOM_D + j]);
+      for (; h < heads_per_plan; ++h) acc = __dadd_rn(acc, term((double)qj[h * FATHOM_D]));
+    };
+    if (mode == FATHOM_DEPTH_WATERFILL) {
+      const float v = var[(size_t)kv * FATHOM_D + j];
+      add_heads([](double x) { return __dmul_rn(x, x); });    // Eq. 3
+      const double g = __dmul_rn(acc, (double)v);
       pri[4 * j + 0] = (unsigned long long)__double_as_longlong(fabs(__dmul_rn(g, 0.25)));        // g_j 4^-m
       pri[4 * j + 1] = (unsigned long long)__double_as_longlong(fabs(__dmul_rn(g, 0.0625)));
       pri[4 * j + 2] = (unsigned long long)__double_as_longlong(fabs(__dmul_rn(g, 0.015625)));
       pri[4 * j + 3] = (unsigned long long)__double_as_longlong(fabs(__dmul_rn(g, 0.00390625)));
     } else {                                                  // fixed top-r channels by sum_h |q_j|
-      for (int h = h0; h < h0 + heads_per_plan; ++h)
-        acc = __dadd_rn(acc, fabs((double)q[(size_t)h * FATHOM_D + j]));
+      add_heads([](double x) { return fabs(x); });
       const unsigned long long key = (unsigned long long)__double_as_longlong(acc);
       pri[4 * j + 0] = key; pri[4 * j + 1] = key; pri[4 * j + 2] = key; pri[4 * j + 3] = key;
     }
@@ -102,7 +111,7 @@ extern "C" int fathom_alloc_depth(fathom_ctx* ctx, const fathom_layout* L, const
   const int G = L->n_q_heads / L->n_kv_heads;
   if (heads_per_plan < 1 || G % heads_per_plan != 0) return FATHOM_ERR_INVALID_ARG;
   const int plans = L->n_q_heads / heads_per_plan;
-  alloc_depth_kernel<<<plans * CTAS_PER_PLAN, AD_THREADS, 0, static_cast<cudaStream_t>(stream)>>>(q, var, mode, budget, heads_per_plan, G, depth);
-  FATHOM_CUDA_TRY(ctx, cudaGetLastError());
+  FATHOM_CUDA_TRY(ctx, fathom_launch_dependent(alloc_depth_kernel, dim3(plans * CTAS_PER_PLAN), dim3(AD_THREADS), 0,
+                                               static_cast<cudaStream_t>(stream), q, var, mode, budget, heads_per_plan, G, depth));
   return FATHOM_OK;
 }

@@ -6,22 +6,23 @@
 // (quantise.cuh).  A CTA walks BLOCKS_PER_CTA consecutive blocks and
 // collects their plane words and scales in shared memory, then writes every (channel, plane) row segment
 // as whole 32-byte sectors (partial-sector writes cost a fill read each).
+// A short sequence - appended tokens - takes one block per CTA instead: there the serial walk is what costs.
 #include "quantise.cuh"
 
 namespace {
 
 constexpr int BP_THREADS = 2 * FATHOM_D;
-constexpr int BLOCKS_PER_CTA = 8;
 constexpr int HALF = FATHOM_BLOCK / 2;                         // tokens per thread
-constexpr int OUT_PITCH = FATHOM_NPLANES * BLOCKS_PER_CTA * 2 + 1;
 
 __device__ __forceinline__ float load_k(const float* p) { return __ldg(p); }
 __device__ __forceinline__ float load_k(const __nv_bfloat16* p) { return __bfloat162float(__ldg(p)); }
 
-template <typename T>
+// BLOCKS_PER_CTA: 8, or 1 for short sequences
+template <typename T, int BLOCKS_PER_CTA>
 __global__ void __launch_bounds__(BP_THREADS)
 build_planes_kernel(const T* __restrict__ K, uint32_t* __restrict__ planes32, uint16_t* __restrict__ scales,
                     long long n, long long nb, long long plane_stride, long long scale_stride) {
+  constexpr int OUT_PITCH = FATHOM_NPLANES * BLOCKS_PER_CTA * 2 + 1;
   __shared__ float s_amax[2][2][FATHOM_D];                     // [parity of block][token half][channel]
   __shared__ uint32_t s_out[FATHOM_D][OUT_PITCH];              // [channel][plane][block][half], padded against bank conflicts
   __shared__ uint16_t s_scale[FATHOM_D][BLOCKS_PER_CTA];
@@ -30,6 +31,8 @@ build_planes_kernel(const T* __restrict__ K, uint32_t* __restrict__ planes32, ui
   const int h = blockIdx.y;                                    // KV head
   const long long b0 = (long long)blockIdx.x * BLOCKS_PER_CTA;
   const T* Kh = K + (size_t)h * (size_t)n * FATHOM_D;
+  FATHOM_PDL_WAIT();                                           // the keys may come from the previous kernel
+  FATHOM_PDL_RELEASE();
 
   for (int bb = 0; bb < BLOCKS_PER_CTA; ++bb) {
     const long long b = b0 + bb;
@@ -68,13 +71,22 @@ build_planes_kernel(const T* __restrict__ K, uint32_t* __restrict__ planes32, ui
   }
   __syncthreads();
 
-  // ---- flush: each (channel, plane) row segment is BLOCKS_PER_CTA words = 64 contiguous bytes
+  // ---- flush: each (channel, plane) row segment is BLOCKS_PER_CTA words (64 contiguous bytes)
   const int nblk = (int)min((long long)BLOCKS_PER_CTA, nb - b0);
   uint64_t* planes64 = reinterpret_cast<uint64_t*>(planes32);
-  for (int e = threadIdx.x; e < FATHOM_D * FATHOM_NPLANES * (BLOCKS_PER_CTA / 2); e += BP_THREADS) {
-    const int pair = e % (BLOCKS_PER_CTA / 2);                 // two words = one 16-byte store
-    const int p = (e / (BLOCKS_PER_CTA / 2)) % FATHOM_NPLANES;
-    const int c = e / (BLOCKS_PER_CTA / 2 * FATHOM_NPLANES);
+  if (BLOCKS_PER_CTA == 1) {
+    for (int e = threadIdx.x; e < FATHOM_D * FATHOM_NPLANES; e += BP_THREADS) {
+      const uint32_t* src = &s_out[e / FATHOM_NPLANES][e % FATHOM_NPLANES * 2];
+      planes64[((size_t)h * FATHOM_D * FATHOM_NPLANES + e) * (size_t)plane_stride + b0] = ((uint64_t)src[1] << 32) | src[0];
+    }
+    if (threadIdx.x < FATHOM_D) scales[((size_t)h * FATHOM_D + threadIdx.x) * (size_t)scale_stride + b0] = s_scale[threadIdx.x][0];
+    return;
+  }
+  constexpr int PAIRS = BLOCKS_PER_CTA / 2 > 0 ? BLOCKS_PER_CTA / 2 : 1;
+  for (int e = threadIdx.x; e < FATHOM_D * FATHOM_NPLANES * PAIRS; e += BP_THREADS) {
+    const int pair = e % PAIRS;                                // two words = one 16-byte store
+    const int p = (e / PAIRS) % FATHOM_NPLANES;
+    const int c = e / (PAIRS * FATHOM_NPLANES);
     const uint32_t* src = &s_out[c][(p * BLOCKS_PER_CTA + 2 * pair) * 2];
     uint64_t* dst = planes64 + (((size_t)h * FATHOM_D + c) * FATHOM_NPLANES + p) * (size_t)plane_stride + b0 + 2 * pair;
     if (2 * pair + 1 < nblk) {
@@ -86,24 +98,34 @@ build_planes_kernel(const T* __restrict__ K, uint32_t* __restrict__ planes32, ui
   for (int e = threadIdx.x; e < FATHOM_D; e += BP_THREADS) {
     uint16_t* dst = scales + ((size_t)h * FATHOM_D + e) * (size_t)scale_stride + b0;
     if (nblk == BLOCKS_PER_CTA) {
-      const uint16_t* sp = s_scale[e];
-      *reinterpret_cast<uint4*>(dst) = make_uint4(sp[0] | ((uint32_t)sp[1] << 16), sp[2] | ((uint32_t)sp[3] << 16),
-                                                  sp[4] | ((uint32_t)sp[5] << 16), sp[6] | ((uint32_t)sp[7] << 16));
+      uint32_t w[4] = {0u, 0u, 0u, 0u};
+#pragma unroll
+      for (int x = 0; x < BLOCKS_PER_CTA; ++x) w[x / 2] |= (uint32_t)s_scale[e][x] << (16 * (x & 1));
+      *reinterpret_cast<uint4*>(dst) = make_uint4(w[0], w[1], w[2], w[3]);
     } else {
       for (int x = 0; x < nblk; ++x) dst[x] = s_scale[e][x];
     }
   }
 }
 
-template <typename T>
-int launch_build(fathom_ctx* ctx, const fathom_layout* L, const T* K, uint64_t* planes, uint16_t* scales,
-                 cudaStream_t st) {
+template <typename T, int BLOCKS_PER_CTA>
+int launch_blocks(fathom_ctx* ctx, const fathom_layout* L, const T* K, uint64_t* planes, uint16_t* scales, cudaStream_t st) {
   const long long nb = fathom_nblocks(L->n);
   dim3 grid((unsigned)((nb + BLOCKS_PER_CTA - 1) / BLOCKS_PER_CTA), (unsigned)L->n_kv_heads);
-  build_planes_kernel<T><<<grid, BP_THREADS, 0, st>>>(K, reinterpret_cast<uint32_t*>(planes), scales, L->n, nb,
-                                                      L->plane_stride_words, L->scale_stride);
-  FATHOM_CUDA_TRY(ctx, cudaGetLastError());
+  FATHOM_CUDA_TRY(ctx, fathom_launch_dependent(build_planes_kernel<T, BLOCKS_PER_CTA>, grid, dim3(BP_THREADS), 0, st, K,
+                                               reinterpret_cast<uint32_t*>(planes), scales, (long long)L->n, nb,
+                                               (long long)L->plane_stride_words, (long long)L->scale_stride));
   return FATHOM_OK;
+}
+
+// A CTA per block while that is less than one wave of CTAs (four of 64 registers x 256 threads are resident per SM): the partial
+// sectors it writes are few then, and the walk over eight blocks is a chain of eight load latencies (one head, 424 tokens of
+// fp32: 5.9 -> 2.9 us).
+constexpr long long SHORT_BLOCKS = 148 * 4;
+template <typename T>
+int launch_build(fathom_ctx* ctx, const fathom_layout* L, const T* K, uint64_t* planes, uint16_t* scales, cudaStream_t st) {
+  if (fathom_nblocks(L->n) * L->n_kv_heads <= SHORT_BLOCKS) return launch_blocks<T, 1>(ctx, L, K, planes, scales, st);
+  return launch_blocks<T, 8>(ctx, L, K, planes, scales, st);
 }
 
 }  // namespace

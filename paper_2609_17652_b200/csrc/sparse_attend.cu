@@ -47,6 +47,7 @@ attend_partial_kernel(const float* __restrict__ q, const T* __restrict__ Krows, 
   const int split = blockIdx.x, head = blockIdx.y, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int kv = head / G;
   FATHOM_PDL_WAIT();                                          // the indices come from the previous kernel
+  FATHOM_PDL_RELEASE();                                       // (the next step's first kernel may become resident)
   const T* Kh = Krows + (size_t)kv * (size_t)n * FATHOM_D;
   const T* Vh = Vrows + (size_t)kv * (size_t)n * FATHOM_D;
   s_q[tid] = q[(size_t)head * FATHOM_D + tid];
