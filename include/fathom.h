@@ -174,18 +174,19 @@ int fathom_scan_set_ctas_per_plan(int ctas);
  *   scores  in   [Hq][score_stride] fp32 (finite)
  *   idx     out  [Hq][k] int32, ascending token indices
  * Uses the context scratch (fathom_scratch_bytes).
- * Long rows (at least 64 chunks of 1024 scores, k - forced >= 256) are read once: a histogram of every 16th chunk
+ * Rows of up to 131,072 scores are selected by one kernel that holds them in registers.  Longer rows are read once: a histogram of every 16th chunk
  * gives an estimated threshold bin (and a bound: the bin of the sample's own k-th largest score), one pass collects
  * the tokens above the estimate, and the exact selection runs among them, head by head.  A head that collected fewer
  * than it needs is served instead by a second launch, enqueued behind the first, in which the head's CTA collects
- * above the bound and selects; the decision is taken on the device and the result is the same either way.  Shorter
- * rows take two passes (histogram of all scores, filter).
+ * above the bound and selects; the decision is taken on the device and the result is the same either way.  Rows of
+ * which more than a thirty-second is wanted take two passes (histogram of all scores, filter).
  * Environment: FATHOM_TOPK_PATH=two_pass (read once) always takes the two-pass selection. */
 #define FATHOM_MAX_K 16384
 int fathom_topk(fathom_ctx* ctx, const fathom_layout* layout, const float* scores, int k,
                 int n_sink, int n_local, int32_t* idx, void* stream);
-/* How many times fathom_topk reads the scores for these arguments (host only, no GPU work): 1 or 2, or a negative
- * status for arguments fathom_topk would reject. */
+/* How many times fathom_topk reads the scores for these arguments at most (host only, no GPU work): 1 where at least 256
+ * tokens are wanted of a row long enough to estimate their threshold from a sample, else 2; or a negative status for
+ * arguments fathom_topk would reject. */
 int fathom_topk_passes(const fathom_layout* layout, int k, int n_sink, int n_local);
 
 /* ---- (3+4) fused scan and top-k, scores never materialised — Sec. 9 Conclusion (fusing the scan with what follows it) ------

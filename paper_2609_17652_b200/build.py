@@ -15,7 +15,7 @@ CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libfathom.so")
 NATIVE = os.path.join(HERE, "_native" + sysconfig.get_config_var("EXT_SUFFIX"))
 NATIVE_SOURCE = os.path.join(CSRC, "native_binding.cpp")
-SOURCES = ["fathom_api.cu", "build_planes.cu", "alloc_depth.cu", "scan.cu", "scan_simt.cu", "topk.cu", "sparse_attend.cu", "gather_union.cu", "klt.cu", "klt_tc.cu", "klt_eig.cu", "layer_plan.cu"]
+SOURCES = ["fathom_api.cu", "build_planes.cu", "alloc_depth.cu", "scan.cu", "scan_simt.cu", "topk.cu", "topk_resident.cu", "sparse_attend.cu", "gather_union.cu", "klt.cu", "klt_tc.cu", "klt_eig.cu", "layer_plan.cu"]
 
 
 def nvcc_path() -> str:

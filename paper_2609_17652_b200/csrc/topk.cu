@@ -1,9 +1,11 @@
 // fathom_topk: per-query-head top-k over n scores with deterministic ties (Sec. 2 "Top-k decoding").
 //
-// Both paths select on the order-preserving integer image of the fp32 score (-0 folded onto +0), and both give the
+// All paths select on the order-preserving integer image of the fp32 score (-0 folded onto +0), and all give the
 // one set the definition fixes (ties to the lower token index), in ascending token order.
 //
-// Single pass (rows of 64K scores or more, at least 256 wanted): one read of the scores.
+// Rows of up to 131,072 scores are held in registers by a cluster per head and selected in one kernel (topk_resident.cu).
+//
+// Single pass (longer rows, when a sixteenth of the row holds enough of what is wanted): one read of the scores.
 //   a. a cluster of four CTAs per head histograms every 16th 1024-score chunk (12 leading key bits, shared memory,
 //      merged through distributed shared memory) and finds two bins:
 //      the ESTIMATE, whose suffix count in the sample reaches the expected rank plus four standard deviations, and
@@ -20,7 +22,7 @@
 //      shorter than wanted (the estimate was too high) collects again itself above the bound bin, which cannot fall
 //      short.
 //
-// Two passes (short rows, or FATHOM_TOPK_PATH=two_pass): bucket select.
+// Two passes (more than a thirty-second of the row wanted, or FATHOM_TOPK_PATH=two_pass): bucket select.
 //   1. histogram of the 12 leading key bits over all eligible tokens (one read of the scores); the CTA that
 //      finishes a head's histogram last (ticket counter) finds
 //   2. the threshold bin b* whose suffix count first reaches the number wanted;
@@ -34,7 +36,7 @@
 //      counts the filter left behind, whose prefix sum gives every tile its place in the output;
 //   5. one small CTA per 8192-token tile emits its indices in ascending order (popcount prefix in the tile).
 // The selected set is unique, so neither the append order nor atomics can show in the output.
-#include "fathom_common.cuh"
+#include "topk_shared.cuh"
 
 #include <cooperative_groups.h>
 
@@ -54,24 +56,6 @@ constexpr int FILT_TILE = (FILT_THREADS / 32) * FILT_WARP_TOKENS;   // 8192 toke
 constexpr int FIN_THREADS = 1024;
 constexpr int FIN_CACHE = 8192;                              // candidate composites kept in shared memory: two-pass select (64 KB)
 constexpr int FIN_CACHE_MAX = 16384;                         // ... direct select, when k leaves room (128 KB)
-
-__device__ __forceinline__ uint32_t ordered_key(float f) {
-  uint32_t u = __float_as_uint(f);
-  if ((u << 1) == 0u) u = 0u;                                // -0 -> +0
-  return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
-}
-
-// fp32 value whose ordered key is `key` (the inverse of ordered_key for non-NaN patterns)
-__device__ __forceinline__ float key_to_float(uint32_t key) {
-  return __uint_as_float((key & 0x80000000u) ? (key & 0x7fffffffu) : ~key);
-}
-// Lower edge of a histogram bin as a score: the bins below -inf's (no finite score lies there) stand for "every score",
-// a bin past the last for "none" (a comparison with NaN is false).
-__device__ __forceinline__ float edge_of_bin(uint32_t bin) {
-  return bin >= FATHOM_TOPK_BINS ? __uint_as_float(0x7fc00000u) : (bin <= 7u ? -INFINITY : key_to_float(bin << 20));
-}
-
-struct Forced { long long sink_end, local_begin; };          // eligible tokens: sink_end <= i < local_begin
 
 using Gate = fathom_gate;
 
@@ -1189,7 +1173,7 @@ static bool single_pass_plan(long long n, int k, uint32_t want, uint32_t* rank_o
   const long long n_sample = sampled * 1024;
   const uint32_t rank = estimate_rank(want, n_sample, n) + (uint32_t)(k - want);
   *rank_out = rank;
-  return !force_two_pass() && want >= 256 && chunks >= 64 && (long long)rank * 8 <= n_sample && (long long)k * 2 <= n_sample;
+  return !force_two_pass() && want > 0 && chunks >= 64 && (long long)rank * 8 <= n_sample && (long long)k * 2 <= n_sample;
 }
 
 // log2 of the token range per counting-sort bucket of the direct select: the smallest that maps n tokens to SORT_BUCKETS
@@ -1238,6 +1222,8 @@ static int launch_direct_select(fathom_ctx* ctx, long long n, int Hq, int k, For
 
 static int run_dense_topk(fathom_ctx* ctx, const float* scores, long long n, long long score_stride, int Hq, int k,
                           Forced F, uint32_t want, const fathom_topk_scratch& S, int32_t* idx, cudaStream_t st) {
+  if (n <= FATHOM_TOPK_RESIDENT_MAX && !force_two_pass())
+    return fathom_launch_topk_resident(ctx, scores, n, score_stride, Hq, k, F, want, idx, st);
   const int ntiles = (int)((n + FILT_TILE - 1) / FILT_TILE);
   dim3 fgrid((unsigned)ntiles, (unsigned)Hq);
   Gate always = {nullptr, 0u, 0, 0};
@@ -1336,7 +1322,7 @@ extern "C" int fathom_topk_passes(const fathom_layout* L, int k, int n_sink, int
   const long long n_forced = sink_end + (n - local_begin);
   if (n_forced > k) return FATHOM_ERR_INVALID_ARG;
   uint32_t rank;
-  return single_pass_plan(n, k, (uint32_t)(k - n_forced), &rank) ? 1 : 2;
+  return k - n_forced >= 256 && single_pass_plan(n, k, (uint32_t)(k - n_forced), &rank) ? 1 : 2;
 }
 
 // Tile step of the sample scan for (n, k): every 16th scan tile when that sample still holds at least 2 k tokens,
@@ -1347,6 +1333,8 @@ int fathom_fused_tile_step(long long n, int k) {
   const long long sampled = (ntiles + 15) / 16;                       // tiles 0, 16, 32, ...
   const long long last_start = (sampled - 1) * 16 * tile;             // first token of the last sampled tile (< n)
   const long long valid = (sampled - 1) * tile + ((n - last_start) < tile ? (n - last_start) : tile);
+  // rows that the top-k holds in registers are scanned whole: one scan and one selection against the five kernels of the sampled path
+  if (n <= FATHOM_TOPK_RESIDENT_MAX && !force_two_pass()) return 1;
   return (ntiles >= 16 && valid >= 2LL * k) ? 16 : 1;
 }
 

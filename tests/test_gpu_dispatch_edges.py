@@ -1,0 +1,36 @@
+"""Kernels that a size rule picks, at the sizes where they can go wrong: the smallest and largest of their range, remainders
+of their tiles, and inputs that leave their common path.  Oracle or sibling kernel as the reference, exact where the result is."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import fathom_oracle as O
+
+pytestmark = pytest.mark.gpu
+
+
+# (tokens, k, sink, local): one CTA and clusters of 2, 4 and 8; 8, 16 and 32 scores per thread; one past each; up to the longest row
+@pytest.mark.parametrize("n,k,n_sink,n_local", [(1, 1, 0, 0), (31, 7, 0, 0), (64, 64, 4, 32), (4096, 64, 0, 0), (4097, 1000, 4, 32), (8193, 8193, 0, 0),
+                                                (16385, 5, 0, 0), (32768, 2048, 0, 0), (32769, 9000, 4, 32), (65536, 36, 4, 32),
+                                                (65537, 512, 0, 0), (131071, 4096, 4, 32), (131072, 16384, 0, 0)])
+@pytest.mark.parametrize("scores", ["spread", "ties", "equal", "negative"])
+def test_topk_of_rows_held_in_registers(n, k, n_sink, n_local, scores):
+    from paper_2609_17652_b200 import binding as fb
+    Hq = 3
+    lay = fb.make_layout(1, Hq, n)
+    ctx = fb.Context(0, fb.fathom_scratch_bytes(lay, k))
+    g = torch.Generator(device="cuda").manual_seed(n + k)
+    s = torch.randn(Hq, lay.score_stride, generator=g, device="cuda")
+    if scores == "ties":
+        s = (s * 4).round() * 0.25                                   # some thirty values, zeros of both signs among them
+    elif scores == "equal":
+        s = torch.full_like(s, -1.5)
+    elif scores == "negative":
+        s = -torch.exp(12 * s)                                       # magnitudes outside the finely divided octaves
+    s[:, n:] = float("nan")
+    idx = torch.full((Hq, k), -1, dtype=torch.int32, device="cuda")
+    ctx.fathom_topk(lay, s, k, n_sink, n_local, idx)
+    ref = O.topk(s[:, :n].double().cpu().numpy(), k, n_sink, n_local)
+    assert np.array_equal(idx.cpu().numpy(), ref)
+    assert ctx.fathom_device_status() == 0
+    ctx.close()
