@@ -23,11 +23,10 @@
 // A tile is 16 blocks (1024 tokens) of one plan (NH query heads that share the planes read).  With the planes in device
 // memory the CTAs are persistent: gridDim.x CTAs per plan walk the tiles round-robin, build the plan's row list and right
 // operand once, and fetch the next stage's plane words and scales with asynchronous copies (cp.async; a row's words are
-// one contiguous run, Sec. 3.6) into the other half of a double buffer.  A stage is a sub-tile of TB blocks and up to
-// ROWS rows: plans of up to 48 rows take whole tiles (TB = 16: 128-byte runs, a warp owns 4 blocks), up to 96 rows half
-// tiles (TB = 8), deeper plans quarter tiles (TB = 4, a warp owns one block and carries its accumulators over passes of
-// 160 rows), so that the staging buffers do not grow with the budget.  With the planes in pinned host memory the grid is
-// one CTA per tile, which keeps the requests on the host link sequential.
+// one contiguous run, Sec. 3.6) into the other half of a double buffer.  A stage is a tile and up to 96 rows (half a tile in the
+// filtering mode for plans of more than 48 rows, whose lists take the shared memory); deeper plans take half tiles in
+// passes of up to 96 rows and carry the accumulators over the passes.  The right operand of all rows stays in shared memory.
+// With the planes in pinned host memory the grid is one CTA per tile, which keeps the requests on the host link sequential.
 // Only planes p < t_j and the scales of active channels are ever read.
 #include "scan_shared.cuh"
 
@@ -40,23 +39,28 @@ namespace {
 constexpr int THREADS = 128, WARPS = 4;
 constexpr int TILE_BLOCKS = FATHOM_SCAN_TILE_BLOCKS;
 constexpr int MAX_ROWS = FATHOM_D * FATHOM_NPLANES;          // 512 (channel, plane) pairs
-constexpr int STAGE_KSTEPS = 10;                             // 16 rows per mma; a stage holds at most 160 rows
-constexpr int WORD_STAGE_BYTES = 7680;                       // staged plane words of one stage (padded rows)
-constexpr int SCALE_STAGE_BYTES = 4608;                      // staged fp16 scales of one stage (padded rows)
+constexpr int MAX_KSTEPS = MAX_ROWS / 16;                    // 16 rows per mma
+constexpr int STAGE_ROWS = 96;                               // rows per stage
 #ifndef FATHOM_SCAN_CTAS_PER_SM
 #define FATHOM_SCAN_CTAS_PER_SM 4                               // 16 warps per SM with ~115 registers each beat 24 warps with 80
 #endif
 constexpr int CTAS_PER_SM = FATHOM_SCAN_CTAS_PER_SM;
 
-// Stage geometry for sub-tiles of TB blocks.  The row pitches are padded so that the four lanes of a quad, which read
-// rows two apart, hit different banks (plane bytes: pitch / 4 = 4 mod 32 for TB = 16, ...).
+// Sub-tiles of TB blocks.  The row pitches are padded so that the four lanes of a quad, which read rows two apart, hit different
+// banks (plane bytes: pitch / 4 = 4 mod 32 for TB = 16, ...).
 template <int TB>
 struct Geo {
   static constexpr int ROW_BYTES = 8 * TB + 16;               // pitch of a staged plane-word row
-  static constexpr int SCALE_ELEMS = TB == 4 ? 12 : 24;       // pitch of a staged scale row, fp16 elements
-  static constexpr int ROWS = TB == 16 ? 48 : TB == 8 ? 96 : 160;   // rows per stage (multiples of 16)
-  static_assert(ROWS * ROW_BYTES <= WORD_STAGE_BYTES && ROWS * SCALE_ELEMS * 2 <= SCALE_STAGE_BYTES, "stage buffers too small");
+  static constexpr int SCALE_ELEMS = 24;                      // pitch of a staged scale row, fp16 elements
 };
+// plans of up to this many rows take whole tiles in the filtering mode
+constexpr int FILTER_WHOLE_ROWS = 48;
+template <int MODE>
+struct StageBytes {                                           // one buffer: MODE 2 has whole tiles of 48 rows or half tiles of 96
+  static constexpr int WORDS = MODE == 2 ? STAGE_ROWS * Geo<8>::ROW_BYTES : STAGE_ROWS * Geo<16>::ROW_BYTES;
+  static constexpr int SCALES = STAGE_ROWS * Geo<16>::SCALE_ELEMS * 2;
+};
+static_assert(FILTER_WHOLE_ROWS * Geo<16>::ROW_BYTES <= StageBytes<2>::WORDS, "stage buffer too small");
 
 // MODE 2.  A lane whose eight scores hold a candidate parks all eight in its warp's ring (three stores, no atomic, no
 // loop); when the ring may not take another round of 32, the warp sifts it with all lanes, one parked group per lane,
@@ -81,15 +85,21 @@ struct alignas(16) Smem {
   alignas(16) float4 park_hi[MODE == 2 ? WARPS * PARK_RING : 1];     //         scores 4..7
   uint32_t park_tok[MODE == 2 ? WARPS * PARK_RING : 1];       //         its first token (30 bits) and the head within the CTA (2 bits)
   uint2 clist[MODE == 2 ? 4 * CAND_LIST : 1];                 // MODE 2: (score bits, token) per head
-  alignas(16) uint2 bfr[STAGE_KSTEPS][32];                    // right operand of the rows of a pass: per 16 rows, the two B registers of every lane
-  alignas(16) unsigned char words[2][WORD_STAGE_BYTES];       // staged plane words, double buffered
-  alignas(16) unsigned char scale[2][SCALE_STAGE_BYTES];      // staged fp16 scales, double buffered
+  alignas(16) uint2 bfr[MAX_KSTEPS][32];                      // right operand of all rows: per 16 rows, the two B registers of every lane
+  alignas(16) unsigned char words[2][StageBytes<MODE>::WORDS];    // staged plane words, double buffered
+  alignas(16) unsigned char scale[2][StageBytes<MODE>::SCALES];   // staged fp16 scales, double buffered
 };
 
 // D += A B, A 16 x 16 (row), B 16 x 8 (col), fp16 operands, fp32 accumulators
 __device__ __forceinline__ void mma_16816(float (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1) {
   asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
       : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3]) : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+}
+
+// D = A B
+__device__ __forceinline__ void mma_16816_first(float (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1) {
+  asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%10,%10,%10,%10};"
+      : "=f"(c[0]), "=f"(c[1]), "=f"(c[2]), "=f"(c[3]) : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1), "f"(0.0f));
 }
 
 // the scale pair with each half's sign flipped where bit (15 - SH) resp. (31 - SH) of `bytes` is clear
@@ -109,32 +119,18 @@ __device__ __forceinline__ void store_scores8(float* row, const float (&v)[8]) {
   }
 }
 
-// One block (64 tokens: this lane's eight are byte `wp[0]` of every staged plane word) times the rows of a stage, 16 rows per
-// step: the lane's two row pairs of a step are rows 2 t4, 2 t4 + 1 and 2 t4 + 8, 2 t4 + 9 of the sixteen.  NKS > 0: that
-// many steps, unrolled (the loads of all steps are in flight at once); NKS = 0: `nks` steps in a loop.
-// Slice j of the accumulators: mma row gq = token 8 gq + 2 j, row gq + 8 = token 8 gq + 2 j + 1.
-template <int ROW_BYTES, int SCALE_ELEMS, int NKS>
-__device__ __forceinline__ void mma_rows(float (&acc)[4][4], const unsigned char* wp, const uint16_t* sp, const uint2* bfr_lane, int nks) {
-  auto step = [&](int ks) {
-    const uint2 bf = bfr_lane[ks * 32];
-    const unsigned char* w = wp + ks * (16 * ROW_BYTES);
-    const uint16_t* sc = sp + ks * (16 * SCALE_ELEMS);
-    const uint32_t x0 = __byte_perm(w[0], w[ROW_BYTES], 0x5410);
-    const uint32_t x1 = __byte_perm(w[8 * ROW_BYTES], w[9 * ROW_BYTES], 0x5410);
-    const uint32_t S0 = __byte_perm(sc[0], sc[SCALE_ELEMS], 0x5410);
-    const uint32_t S1 = __byte_perm(sc[8 * SCALE_ELEMS], sc[9 * SCALE_ELEMS], 0x5410);
-    mma_16816(acc[0], signed_pair<15>(S0, x0), signed_pair<14>(S0, x0), signed_pair<15>(S1, x1), signed_pair<14>(S1, x1), bf.x, bf.y);
-    mma_16816(acc[1], signed_pair<13>(S0, x0), signed_pair<12>(S0, x0), signed_pair<13>(S1, x1), signed_pair<12>(S1, x1), bf.x, bf.y);
-    mma_16816(acc[2], signed_pair<11>(S0, x0), signed_pair<10>(S0, x0), signed_pair<11>(S1, x1), signed_pair<10>(S1, x1), bf.x, bf.y);
-    mma_16816(acc[3], signed_pair<9>(S0, x0), signed_pair<8>(S0, x0), signed_pair<9>(S1, x1), signed_pair<8>(S1, x1), bf.x, bf.y);
+// Eight tokens of a lane (one byte of every row's plane word; x0, x1: the bytes of the lane's two row pairs of 16 rows side by
+// side, bits 0..7 and 16..23) times 16 rows.  Slice j of the accumulators: mma row gq = token 2 j, row gq + 8 = token 2 j + 1.
+template <bool FIRST>
+__device__ __forceinline__ void mma_tokens8(float (&acc)[4][4], uint32_t x0, uint32_t x1, uint32_t S0, uint32_t S1, uint2 bf) {
+  auto mma = [&](float (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3) {
+    if (FIRST) mma_16816_first(c, a0, a1, a2, a3, bf.x, bf.y);
+    else mma_16816(c, a0, a1, a2, a3, bf.x, bf.y);
   };
-  if (NKS > 0) {
-#pragma unroll
-    for (int ks = 0; ks < NKS; ++ks) step(ks);
-  } else {
-#pragma unroll 1
-    for (int ks = 0; ks < nks; ++ks) step(ks);
-  }
+  mma(acc[0], signed_pair<15>(S0, x0), signed_pair<14>(S0, x0), signed_pair<15>(S1, x1), signed_pair<14>(S1, x1));
+  mma(acc[1], signed_pair<13>(S0, x0), signed_pair<12>(S0, x0), signed_pair<13>(S1, x1), signed_pair<12>(S1, x1));
+  mma(acc[2], signed_pair<11>(S0, x0), signed_pair<10>(S0, x0), signed_pair<11>(S1, x1), signed_pair<10>(S1, x1));
+  mma(acc[3], signed_pair<9>(S0, x0), signed_pair<8>(S0, x0), signed_pair<9>(S1, x1), signed_pair<8>(S1, x1));
 }
 
 // MODE 0: scores of every token are written (fathom_scan, fathom_scan_batch).
@@ -144,17 +140,16 @@ __device__ __forceinline__ void mma_rows(float (&acc)[4][4], const unsigned char
 //         (score, token) pairs appended to the head's candidate list.
 // grid = (CTAs per plan, groups of NH query heads); MODE 1 and 2 are launched with one item.
 // IN_HBM: every store of the launch lies in device memory (its rows are staged past the L1).
-template <int NH, int MODE, bool IN_HBM>
+template <int NH, int MODE, bool IN_HBM, int CAP>
 __global__ void __launch_bounds__(THREADS, CTAS_PER_SM)
-scan_kernel(const __grid_constant__ ScanBatch B, int G, int heads_per_plan, fathom_scan_fuse fz) {
+scan_kernel(const __grid_constant__ ScanBatchOf<CAP> B, int G, int heads_per_plan, fathom_scan_fuse fz) {
   extern __shared__ __align__(16) unsigned char scan_smem[];   // sizeof(Smem<MODE>): more than the static limit in MODE 2
   Smem<MODE>& M = *reinterpret_cast<Smem<MODE>*>(scan_smem);
 
   FATHOM_PDL_WAIT();                                          // depths (and thresholds) come from the previous kernels
   if (MODE == 2 && !fathom_gate_open(fz.gate)) return;         // second attempt of the fused selection: may have nothing to do
   const int total = (int)B.tile_end[B.items - 1];              // tiles of this launch (tile and block indices fit 32 bits)
-  int g = blockIdx.x;                                          // my current tile of the launch
-  if (g >= total) return;
+  if ((int)blockIdx.x >= total) return;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   constexpr bool in_hbm = IN_HBM;
   const int gq = lane >> 2, t4 = lane & 3;                     // mma fragment coordinates: lane = (row group, column pair)
@@ -172,18 +167,17 @@ scan_kernel(const __grid_constant__ ScanBatch B, int G, int heads_per_plan, fath
   if (MODE == 2 && tid < NH)                                   // read after the barriers of the first item's row list
     M.thr[tid] = fz.state_is_score ? __uint_as_float(fz.state[(h0 + tid) * 8]) : fathom_bin_lower_edge(fz.state[(h0 + tid) * 8]);
 
-  int item = -1, nrows = 0, tb = TILE_BLOCKS, rows_stage = Geo<16>::ROWS, npass = 1, nb_item = 0;
+  int item = -1, nrows = 0, tb = TILE_BLOCKS, rows_stage = STAGE_ROWS, npass = 1, nb_item = 0;
   float hs = 1.0f, hs_tail = 0.0f;                             // E of my head and E 2^-11
 
-  // ---- right operand of the rows of pass `pass` (made visible by the barrier that precedes the pass's arithmetic): entry
-  //      (kstep, lane, i) holds rows 16 kstep + 2 (lane & 3) + 8 i and the next one of the pass, column lane >> 2 = (head, part)
-  auto fill_bfr = [&](int pass) {
-    const int s0 = pass * rows_stage, sc = min(rows_stage, nrows - s0);
-    const int entries = ((sc + 15) >> 4) * 64;
+  // ---- right operand of all rows (made visible by the barrier that precedes the first stage's arithmetic): entry
+  //      (kstep, lane, i) holds rows 16 kstep + 2 (lane & 3) + 8 i and the next one, column lane >> 2 = (head, part)
+  auto fill_bfr = [&]() {
+    const int entries = max(1, (nrows + 15) >> 4) * 64;        // (a plan without rows: 16 of weight and scale 0)
     for (int e = tid; e < entries; e += THREADS) {
       const int ks = e >> 6, ln = (e >> 1) & 31, i = e & 1;
       const int col = ln >> 2, head = col >> 1, part = col & 1;
-      const int r0 = s0 + ks * 16 + 2 * (ln & 3) + 8 * i;
+      const int r0 = ks * 16 + 2 * (ln & 3) + 8 * i;
       uint32_t packed = 0u;
       if (head < NH) {
         const float inv = M.hinv[head];
@@ -250,10 +244,9 @@ scan_kernel(const __grid_constant__ ScanBatch B, int G, int heads_per_plan, fath
     }
     __syncthreads();
     nrows = M.nrows;
-    if (nrows <= Geo<16>::ROWS) { tb = 16; rows_stage = Geo<16>::ROWS; }
-    else if (nrows <= Geo<8>::ROWS) { tb = 8; rows_stage = Geo<8>::ROWS; }
-    else { tb = 4; rows_stage = Geo<4>::ROWS; }
-    npass = nrows > rows_stage ? (nrows + rows_stage - 1) / rows_stage : 1;
+    tb = nrows <= (MODE == 2 ? FILTER_WHOLE_ROWS : STAGE_ROWS) ? 16 : 8;
+    npass = max(1, (nrows + STAGE_ROWS - 1) / STAGE_ROWS);
+    rows_stage = ((nrows + npass - 1) / npass + 15) & ~15;     // equal passes of whole ksteps, at most 96 rows
     hs = M.hscale[myh];
     hs_tail = hs * 4.8828125e-4f;                              // 2^-11
   };
@@ -274,7 +267,7 @@ scan_kernel(const __grid_constant__ ScanBatch B, int G, int heads_per_plan, fath
                              (uint64_t)(kv * FATHOM_D * FATHOM_NPLANES) * (uint64_t)(B.plane_stride[item] >> 1) + (blk0 >> 1);
     const unsigned char* scales_kv = reinterpret_cast<const unsigned char*>(B.scales[item]) +
                                      (uint64_t)(kv * FATHOM_D) * (uint64_t)B.scale_stride[item] * 2 + (uint64_t)blk0 * 2;
-    const int sh = tb == 16 ? 3 : (tb == 8 ? 2 : 1);           // 16-byte copies per row of plane words: tb / 2
+    const int sh = tb == 16 ? 3 : 2;                           // 16-byte copies per row of plane words: tb / 2
     const int row_bytes = 8 * tb + 16;
     unsigned char* wdst = M.words[buf];
     const int c = tid & ((1 << sh) - 1);                       // my 16-byte column of every row I copy
@@ -288,29 +281,19 @@ scan_kernel(const __grid_constant__ ScanBatch B, int G, int heads_per_plan, fath
       for (int r = tid >> 1; r < sc; r += THREADS >> 1)
         fathom_copy_async<16>(sdst + r * (Geo<16>::SCALE_ELEMS * 2) + cs * 16, vs ? scales_kv + (uint64_t)M.soff[s0 + r] * 16 + cs * 16 : scales_kv, vs,
                               in_hbm);
-    } else if (tb == 8) {
-      for (int r = tid; r < sc; r += THREADS)
-        fathom_copy_async<16>(sdst + r * (Geo<8>::SCALE_ELEMS * 2), scales_kv + (uint64_t)M.soff[s0 + r] * 16, true, in_hbm);
     } else {
       for (int r = tid; r < sc; r += THREADS)
-        fathom_copy_async<8>(sdst + r * (Geo<4>::SCALE_ELEMS * 2), scales_kv + (uint64_t)M.soff[s0 + r] * 16, true);
+        fathom_copy_async<16>(sdst + r * (Geo<8>::SCALE_ELEMS * 2), scales_kv + (uint64_t)M.soff[s0 + r] * 16, true, in_hbm);
     }
     // rows that pad the last 16: scale 0, so that whatever the stale plane bytes say they contribute +-0
-    const int pad = ((sc + 15) & ~15) - sc;
-    const int wpr = (tb == 4 ? Geo<4>::SCALE_ELEMS : Geo<16>::SCALE_ELEMS) / 2;   // 32-bit words per scale row
-    for (int e = tid; e < pad * wpr; e += THREADS)
-      reinterpret_cast<uint32_t*>(sdst)[(sc + e / wpr) * wpr + e % wpr] = 0u;
+    const int pad = max(16, (sc + 15) & ~15) - sc;
+    constexpr int WPR = Geo<16>::SCALE_ELEMS / 2;              // 32-bit words per scale row
+    for (int e = tid; e < pad * WPR; e += THREADS) reinterpret_cast<uint32_t*>(sdst)[(sc + e / WPR) * WPR + e % WPR] = 0u;
     fathom_copies_commit();
   };
 
-  float acc[4][4];                                             // [16-token slice of the block][c0..c3]
   uint32_t parked = 0u, stages = 0u;                           // MODE 2: groups in my warp's ring (the same in every lane); stages done
-
-  enter_item(g);
-  const float my_thr = MODE == 2 ? M.thr[myh] : 0.0f;
-  int u = 0, pass = 0, buf = 0;
-  prefetch(g, 0, 0, 0);                                        // the first stage's rows are on their way ...
-  fill_bfr(0);                                                 // ... while the right operand is made
+  float my_thr = 0.0f;
 
   // ---- MODE 2, whole warp: the parked groups, one per lane and round, into the CTA's candidate lists.  A lane marks the
   //      candidates among its group's eight scores (score reaches the head's threshold, token eligible).  Nearly always
@@ -371,173 +354,188 @@ scan_kernel(const __grid_constant__ ScanBatch B, int G, int heads_per_plan, fath
     __syncwarp();                                              // the ring may be written again
   };
 
-  while (true) {
-    // ---- the stage after this one: the next pass of the sub-tile, the next sub-tile of the tile, or my next tile
-    int g_next = g, u_next = u, pass_next = pass + 1;
-    if (pass_next == npass) {
-      pass_next = 0;
-      u_next = u + 1;
-      if (u_next * tb >= TILE_BLOCKS || first_block(g) + u_next * tb >= nb_item) { u_next = 0; g_next = g + gridDim.x; }
-    }
-    const bool more = g_next < total;
-    const bool same_item = more && g_next < B.tile_end[item];
-    fathom_copies_wait<0>();
-    __syncthreads();                                           // this stage's words and scales are in place, and every warp has
-                                                               // left the previous stage: its buffer may be refilled
-    if (same_item) prefetch(g_next, u_next, pass_next, buf ^ 1);   // lands while this stage is scanned
-
-    // ---- eight consecutive scores of head t4 (lanes with t4 < NH, tokens of an existing block): tokens tok .. tok + 7 of
-    //      the session, written at position dst of the head's row (MODE 0, 1) or tested against the head's threshold (MODE 2)
-    auto emit = [&](const float (&v)[8], uint32_t tok, uint32_t dst, uint32_t n, bool live) {
-      if (MODE != 2) {
-        if (!live) return;
-        float* row = B.scores[item] + (size_t)(h0 + t4) * (size_t)B.score_stride[item] + dst;
-        if (tok + 8 <= n) {
-          store_scores8(row, v);
-        } else {
-#pragma unroll
-          for (int x = 0; x < 8; ++x)
-            if (tok + x < n) row[x] = v[x];
-        }
+  // ---- eight consecutive scores of head t4 (lanes with t4 < NH, tokens of an existing block): tokens tok .. tok + 7 of
+  //      the session, written at position dst of the head's row (MODE 0, 1) or tested against the head's threshold (MODE 2)
+  auto emit = [&](const float (&v)[8], uint32_t tok, uint32_t dst, uint32_t n, bool live) {
+    if (MODE != 2) {
+      if (!live) return;
+      float* row = B.scores[item] + (size_t)(h0 + t4) * (size_t)B.score_stride[item] + dst;
+      if (tok + 8 <= n) {
+        store_scores8(row, v);
       } else {
-        // a lane with a candidate among its eight scores parks them (called by all lanes of the warp; `live`: the lane
-        // has scores at all).  Eligibility of the tokens is checked when the ring is sifted.
-        const float vmax = fmaxf(fmaxf(fmaxf(v[0], v[1]), fmaxf(v[2], v[3])), fmaxf(fmaxf(v[4], v[5]), fmaxf(v[6], v[7])));
-        const bool has = live && vmax >= my_thr;
-        const unsigned bal = __ballot_sync(0xffffffffu, has);
-        if (bal) {                                             // (the same for every lane)
-          if (has) {
-            const uint32_t e = warp * PARK_RING + parked + __popc(bal & ((1u << lane) - 1u));
-            M.park_lo[e] = make_float4(v[0], v[1], v[2], v[3]);
-            M.park_hi[e] = make_float4(v[4], v[5], v[6], v[7]);
-            M.park_tok[e] = tok | ((uint32_t)t4 << 30);
-          }
-          parked += __popc(bal);
-          if (parked > (uint32_t)(PARK_RING - 32)) sift();
-        }
+#pragma unroll
+        for (int x = 0; x < 8; ++x)
+          if (tok + x < n) row[x] = v[x];
       }
-    };
+    } else {
+      // a lane with a candidate among its eight scores parks them (called by all lanes of the warp; `live`: the lane
+      // has scores at all).  Eligibility of the tokens is checked when the ring is sifted.
+      const float vmax = fmaxf(fmaxf(fmaxf(v[0], v[1]), fmaxf(v[2], v[3])), fmaxf(fmaxf(v[4], v[5]), fmaxf(v[6], v[7])));
+      const bool has = live && vmax >= my_thr;
+      const unsigned bal = __ballot_sync(0xffffffffu, has);
+      if (bal) {                                             // (the same for every lane)
+        if (has) {
+          const uint32_t e = warp * PARK_RING + parked + __popc(bal & ((1u << lane) - 1u));
+          M.park_lo[e] = make_float4(v[0], v[1], v[2], v[3]);
+          M.park_hi[e] = make_float4(v[4], v[5], v[6], v[7]);
+          M.park_tok[e] = tok | ((uint32_t)t4 << 30);
+        }
+        parked += __popc(bal);
+        if (parked > (uint32_t)(PARK_RING - 32)) sift();
+      }
+    }
+  };
 
-    // ---- a whole stage of TB blocks and NKS x 16 rows, single pass: the warp's TB / 4 blocks are 16 TB tokens, and a lane
-    //      takes 2 TB consecutive ones (TB = 16: half a block, TB = 8: a quarter): ONE load of TB / 4 bytes per row gives all
-    //      their bits, and one scale pair per row pair serves them all.  They are worked eight at a time (byte k of the
-    //      loaded words): slice j of the accumulators then holds tokens 8 k + 2 j (mma row gq) and 8 k + 2 j + 1 (row gq + 8)
-    //      of the lane's tokens
-    auto owned_tokens = [&](auto tbc, auto nksc, int blk0) {
-      constexpr int TB = decltype(tbc)::value, NKS = decltype(nksc)::value;
-      constexpr int BYTES = TB / 4;                            // plane bytes per row and lane
-      using GE = Geo<TB>;
-      const int mine = warp * (TB / 4) + (gq * BYTES) / 8;     // my block of the stage
-      const int off = (gq * BYTES) % 8;                        // where my bytes start in its words
-      const unsigned char* wp = M.words[buf] + (2 * t4) * GE::ROW_BYTES + mine * 8 + off;
-      const uint16_t* sp = reinterpret_cast<const uint16_t*>(M.scale[buf]) + (2 * t4) * GE::SCALE_ELEMS + mine;
-      uint32_t w[NKS][4], S[NKS][2];
-      uint2 bf[NKS];
-      auto plane_bytes = [](const unsigned char* p) -> uint32_t {
-        return BYTES == 4 ? *reinterpret_cast<const uint32_t*>(p) : (uint32_t)*reinterpret_cast<const uint16_t*>(p);
-      };
+  // ---- eight tokens' accumulators -> scores of head t4: columns 2 t4 (head part) and 2 t4 + 1 (tail part)
+  auto finish = [&](const float (&acc)[4][4], uint32_t tok, uint32_t dst, uint32_t n) {
+    float v[8];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      v[2 * j] = fmaf(acc[j][1], hs_tail, acc[j][0] * hs);
+      v[2 * j + 1] = fmaf(acc[j][3], hs_tail, acc[j][2] * hs);
+    }
+    emit(v, tok, dst, n, t4 < NH);
+  };
+  // A warp's TB / 4 blocks of a stage are 16 TB tokens, and a lane takes 2 TB consecutive ones (TB = 16: half a block, TB = 8: a
+  // quarter): ONE load of TB / 4 bytes per row gives all their bits, and one scale pair per row pair serves them all.  They
+  // are worked eight at a time (byte k of the loaded words).  Tokens past the end of the sequence are computed from zeros or from
+  // what pads the rows and never leave.
+  struct Place { const unsigned char* wp; const uint16_t* sp; uint32_t tok0, dst0; };
+  auto place = [&](auto tbc, int g, int u, int buf) {
+    constexpr int TB = decltype(tbc)::value, BYTES = TB / 4;   // plane bytes per row and lane
+    const int mine = warp * (TB / 4) + (gq * BYTES) / 8;       // my block of the stage
+    const int off = (gq * BYTES) % 8;                          // where my bytes start in its words
+    Place p;
+    p.wp = M.words[buf] + (2 * t4) * Geo<TB>::ROW_BYTES + mine * 8 + off;
+    p.sp = reinterpret_cast<const uint16_t*>(M.scale[buf]) + (2 * t4) * Geo<TB>::SCALE_ELEMS + mine;
+    p.tok0 = (uint32_t)(first_block(g) + u * TB + mine) * FATHOM_BLOCK + off * 8;           // my first token
+    p.dst0 = MODE == 1 ? (uint32_t)g * (TILE_BLOCKS * FATHOM_BLOCK) + (uint32_t)(u * TB + mine) * FATHOM_BLOCK + off * 8 : p.tok0;
+    return p;
+  };
+  auto load_rows = [&](auto tbc, const unsigned char* wk, const uint16_t* sk, uint32_t (&w)[4], uint32_t (&S)[2]) {
+    constexpr int TB = decltype(tbc)::value, RB = Geo<TB>::ROW_BYTES, SE = Geo<TB>::SCALE_ELEMS;
+    auto plane_bytes = [](const unsigned char* p) -> uint32_t {
+      return TB == 16 ? *reinterpret_cast<const uint32_t*>(p) : (uint32_t)*reinterpret_cast<const uint16_t*>(p);
+    };
+    w[0] = plane_bytes(wk);
+    w[1] = plane_bytes(wk + RB);
+    w[2] = plane_bytes(wk + 8 * RB);
+    w[3] = plane_bytes(wk + 9 * RB);
+    S[0] = __byte_perm(sk[0], sk[SE], 0x5410);
+    S[1] = __byte_perm(sk[8 * SE], sk[9 * SE], 0x5410);
+  };
+  // single pass, NKS x 16 rows: the words and scales a lane reads are in registers before the first MMA, and so is the right
+  // operand of up to four steps (of more it would spill)
+  auto compute_single = [&](auto tbc, auto nksc, int g, int u, int buf) {
+    constexpr int TB = decltype(tbc)::value, NKS = decltype(nksc)::value;
+    constexpr bool KEEP = NKS <= 4;
+    const Place at = place(tbc, g, u, buf);
+    uint32_t w[NKS][4], S[NKS][2];
+    uint2 bf[KEEP ? NKS : 1];
+#pragma unroll
+    for (int ks = 0; ks < NKS; ++ks) {
+      if (KEEP) bf[ks] = M.bfr[ks][lane];
+      load_rows(tbc, at.wp + ks * (16 * Geo<TB>::ROW_BYTES), at.sp + ks * (16 * Geo<TB>::SCALE_ELEMS), w[ks], S[ks]);
+    }
+    const uint32_t n = (uint32_t)B.n[item];                    // n < 2^31
+#pragma unroll
+    for (int k = 0; k < TB / 4; ++k) {
+      float acc[4][4];
 #pragma unroll
       for (int ks = 0; ks < NKS; ++ks) {
-        bf[ks] = M.bfr[ks][lane];
-        const unsigned char* wk = wp + ks * (16 * GE::ROW_BYTES);
-        w[ks][0] = plane_bytes(wk);
-        w[ks][1] = plane_bytes(wk + GE::ROW_BYTES);
-        w[ks][2] = plane_bytes(wk + 8 * GE::ROW_BYTES);
-        w[ks][3] = plane_bytes(wk + 9 * GE::ROW_BYTES);
-        const uint16_t* sk = sp + ks * (16 * GE::SCALE_ELEMS);
-        S[ks][0] = __byte_perm(sk[0], sk[GE::SCALE_ELEMS], 0x5410);
-        S[ks][1] = __byte_perm(sk[8 * GE::SCALE_ELEMS], sk[9 * GE::SCALE_ELEMS], 0x5410);
+        const uint32_t x0 = __byte_perm(w[ks][0], w[ks][1], 0x0400 + 0x0101 * k);
+        const uint32_t x1 = __byte_perm(w[ks][2], w[ks][3], 0x0400 + 0x0101 * k);
+        const uint2 b = KEEP ? bf[KEEP ? ks : 0] : M.bfr[ks][lane];
+        if (ks == 0) mma_tokens8<true>(acc, x0, x1, S[ks][0], S[ks][1], b);
+        else mma_tokens8<false>(acc, x0, x1, S[ks][0], S[ks][1], b);
       }
-      const uint32_t n = (uint32_t)B.n[item];
-      const uint32_t tok0 = (uint32_t)(blk0 + mine) * FATHOM_BLOCK + off * 8;            // my first token
-      const uint32_t dst0 = MODE == 1 ? (uint32_t)g * (TILE_BLOCKS * FATHOM_BLOCK) + (uint32_t)(u * TB + mine) * FATHOM_BLOCK + off * 8 : tok0;
-#pragma unroll
-      for (int k = 0; k < BYTES; ++k) {
-#pragma unroll
-        for (int j = 0; j < 4; ++j) acc[j][0] = acc[j][1] = acc[j][2] = acc[j][3] = 0.0f;
-#pragma unroll
-        for (int ks = 0; ks < NKS; ++ks) {
-          // byte k of the two rows of a pair side by side: bits 0..7 and 16..23 (the other bytes are masked away later)
-          const uint32_t x0 = __byte_perm(w[ks][0], w[ks][1], 0x0400 + 0x0101 * k);
-          const uint32_t x1 = __byte_perm(w[ks][2], w[ks][3], 0x0400 + 0x0101 * k);
-          const uint32_t S0 = S[ks][0], S1 = S[ks][1];
-          mma_16816(acc[0], signed_pair<15>(S0, x0), signed_pair<14>(S0, x0), signed_pair<15>(S1, x1), signed_pair<14>(S1, x1), bf[ks].x, bf[ks].y);
-          mma_16816(acc[1], signed_pair<13>(S0, x0), signed_pair<12>(S0, x0), signed_pair<13>(S1, x1), signed_pair<12>(S1, x1), bf[ks].x, bf[ks].y);
-          mma_16816(acc[2], signed_pair<11>(S0, x0), signed_pair<10>(S0, x0), signed_pair<11>(S1, x1), signed_pair<10>(S1, x1), bf[ks].x, bf[ks].y);
-          mma_16816(acc[3], signed_pair<9>(S0, x0), signed_pair<8>(S0, x0), signed_pair<9>(S1, x1), signed_pair<8>(S1, x1), bf[ks].x, bf[ks].y);
-        }
-        float v[8];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          v[2 * j] = fmaf(acc[j][1], hs_tail, acc[j][0] * hs);
-          v[2 * j + 1] = fmaf(acc[j][3], hs_tail, acc[j][2] * hs);
-        }
-        emit(v, tok0 + 8 * k, dst0 + 8 * k, n, t4 < NH);
-      }
-    };
-
-    auto compute = [&](auto tbc) {
-      constexpr int TB = decltype(tbc)::value;
-      using GE = Geo<TB>;
-      constexpr int BW = TB / WARPS;                           // blocks per warp and stage
-      const int s0 = pass * GE::ROWS, sc = min(GE::ROWS, nrows - s0), nks = (sc + 15) >> 4;
-      const int blk0 = first_block(g) + u * TB;
-      const uint32_t n = (uint32_t)B.n[item];                  // n < 2^31
-      if constexpr (TB >= 8) if (npass == 1 && nks >= 1 && (uint32_t)(blk0 + TB) * FATHOM_BLOCK <= n) {
-        // ---- the common stages (plans of up to 96 rows, whole sub-tiles of a long sequence)
-        constexpr int K0 = TB == 16 ? 0 : 3;                   // TB = 8 serves 49 .. 96 rows: 4 .. 6 steps of 16
-        if (nks == K0 + 3) owned_tokens(tbc, std::integral_constant<int, K0 + 3>(), blk0);
-        else if (nks == K0 + 2) owned_tokens(tbc, std::integral_constant<int, K0 + 2>(), blk0);
-        else owned_tokens(tbc, std::integral_constant<int, K0 + 1>(), blk0);
-        return;
-      }
-#pragma unroll 1
-      for (int i = 0; i < BW; ++i) {
-        const int b = warp * BW + i;                           // my block within the sub-tile
-        if (pass == 0) {
-#pragma unroll
-          for (int j = 0; j < 4; ++j) acc[j][0] = acc[j][1] = acc[j][2] = acc[j][3] = 0.0f;
-        }
-        // my byte (tokens 8 gq .. 8 gq + 7) of the plane words and the scales of rows 2 t4, 2 t4 + 1 (+ 8, + 9) of every 16
-        const unsigned char* wp = M.words[buf] + (2 * t4) * GE::ROW_BYTES + b * 8 + gq;
-        const uint16_t* sp = reinterpret_cast<const uint16_t*>(M.scale[buf]) + (2 * t4) * GE::SCALE_ELEMS + b;
-        const uint2* bfr_lane = &M.bfr[0][lane];
-        if (nks == 3) mma_rows<GE::ROW_BYTES, GE::SCALE_ELEMS, 3>(acc, wp, sp, bfr_lane, 3);   // 33 .. 48 rows: a B = 48 plan
-        else mma_rows<GE::ROW_BYTES, GE::SCALE_ELEMS, 0>(acc, wp, sp, bfr_lane, nks);
-        if (pass != npass - 1) continue;
-
-        // ---- scores of head t4 for my eight tokens: columns 2 t4 (head part) and 2 t4 + 1 (tail part)
-        float v[8];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          v[2 * j] = fmaf(acc[j][1], hs_tail, acc[j][0] * hs);
-          v[2 * j + 1] = fmaf(acc[j][3], hs_tail, acc[j][2] * hs);
-        }
-        const bool have_block = blk0 + b < nb_item;
-        const uint32_t tok = (uint32_t)(blk0 + b) * FATHOM_BLOCK + gq * 8;                     // my first token
-        emit(v, tok, MODE == 1 ? (uint32_t)g * (TILE_BLOCKS * FATHOM_BLOCK) + (uint32_t)(u * TB + b) * FATHOM_BLOCK + gq * 8 : tok, n,
-             t4 < NH && have_block);
-      }
-    };
-    if (tb == 16) compute(std::integral_constant<int, 16>());
-    else if (tb == 8) compute(std::integral_constant<int, 8>());
-    else compute(std::integral_constant<int, 4>());
-
-    if (MODE == 2 && (++stages & 3u) == 0u) sift();            // (every warp of the CTA at the same stages)
-    if (!more) break;
-    g = g_next;
-    u = u_next;
-    pass = pass_next;
-    buf ^= 1;
-    if (!same_item) {                                          // first tile of another session: nothing was fetched ahead
-      __syncthreads();                                         // every warp is done with the previous session's row list
-      enter_item(g);
-      prefetch(g, 0, 0, buf);
-      fill_bfr(0);
-    } else if (npass > 1) {
-      __syncthreads();                                         // every warp is done with the previous pass's right operand
-      fill_bfr(pass);                                          // plans of more than 160 rows: the right operand of the next pass
+      finish(acc, at.tok0 + 8 * k, at.dst0 + 8 * k, n);
     }
+  };
+
+  auto run_single = [&](auto tbc, auto nksc, int g, int end) {
+    constexpr int TB = decltype(tbc)::value;
+    for (int u = 0, buf = 0;; buf ^= 1) {
+      int g_next = g, u_next = u + 1;                          // the stage after this one: the next sub-tile, or my next tile
+      if (u_next * TB >= TILE_BLOCKS || first_block(g) + u_next * TB >= nb_item) { u_next = 0; g_next = g + gridDim.x; }
+      const bool more = g_next < end;
+      fathom_copies_wait<0>();
+      __syncthreads();                                         // this stage's words and scales are in place, and every warp has
+                                                               // left the previous stage: its buffer may be refilled
+      if (more) prefetch(g_next, u_next, 0, buf ^ 1);          // lands while this stage is scanned
+      compute_single(tbc, nksc, g, u, buf);
+      if (MODE == 2 && (++stages & 3u) == 0u) sift();          // (every warp of the CTA at the same stages)
+      if (!more) return;
+      g = g_next;
+      u = u_next;
+    }
+  };
+  // plans of more than 96 rows: the accumulators of the lane's tokens are carried over the passes of a half tile (those of a whole
+  // tile, 64 registers, would spill)
+  auto run_passes = [&](int g, int end) {
+    constexpr std::integral_constant<int, 8> tbc{};
+    constexpr int TB = 8, BYTES = TB / 4;
+    float acc[BYTES][4][4];
+    for (int u = 0, pass = 0, buf = 0;; buf ^= 1) {
+      int g_next = g, u_next = u, pass_next = pass + 1;
+      if (pass_next == npass) {
+        pass_next = 0;
+        u_next = u + 1;
+        if (u_next * TB >= TILE_BLOCKS || first_block(g) + u_next * TB >= nb_item) { u_next = 0; g_next = g + gridDim.x; }
+      }
+      const bool more = g_next < end;
+      fathom_copies_wait<0>();
+      __syncthreads();
+      if (more) prefetch(g_next, u_next, pass_next, buf ^ 1);
+      if (pass == 0) {
+#pragma unroll
+        for (int k = 0; k < BYTES; ++k)
+#pragma unroll
+          for (int j = 0; j < 4; ++j) acc[k][j][0] = acc[k][j][1] = acc[k][j][2] = acc[k][j][3] = 0.0f;
+      }
+      const Place at = place(tbc, g, u, buf);
+      const int ks0 = pass * (rows_stage >> 4), nks = (min(rows_stage, nrows - pass * rows_stage) + 15) >> 4;
+#pragma unroll 2
+      for (int ks = 0; ks < nks; ++ks) {
+        uint32_t w[4], S[2];
+        const uint2 bf = M.bfr[ks0 + ks][lane];
+        load_rows(tbc, at.wp + ks * (16 * Geo<TB>::ROW_BYTES), at.sp + ks * (16 * Geo<TB>::SCALE_ELEMS), w, S);
+#pragma unroll
+        for (int k = 0; k < BYTES; ++k)
+          mma_tokens8<false>(acc[k], __byte_perm(w[0], w[1], 0x0400 + 0x0101 * k), __byte_perm(w[2], w[3], 0x0400 + 0x0101 * k), S[0], S[1], bf);
+      }
+      if (pass == npass - 1) {
+        const uint32_t n = (uint32_t)B.n[item];
+#pragma unroll
+        for (int k = 0; k < BYTES; ++k) finish(acc[k], at.tok0 + 8 * k, at.dst0 + 8 * k, n);
+        if (MODE == 2 && (++stages & 3u) == 0u) sift();
+      }
+      if (!more) return;
+      g = g_next;
+      u = u_next;
+      pass = pass_next;
+    }
+  };
+
+  for (int g = blockIdx.x; g < total;) {                       // session by session
+    if (item >= 0) __syncthreads();                            // every warp is done with the previous session's row list
+    enter_item(g);
+    if (MODE == 2) my_thr = M.thr[myh];
+    const int end = min(total, (int)B.tile_end[item]);
+    prefetch(g, 0, 0, 0);                                      // the first stage's rows are on their way ...
+    fill_bfr();                                                // ... while the right operand is made
+    using std::integral_constant;
+    constexpr integral_constant<int, 16> T16{};
+    constexpr integral_constant<int, MODE == 2 ? 8 : 16> TDEEP{};
+    const int nks = (nrows + 15) >> 4;
+    if (npass > 1) run_passes(g, end);
+    else if (nks <= 1) run_single(T16, integral_constant<int, 1>{}, g, end);
+    else if (nks == 2) run_single(T16, integral_constant<int, 2>{}, g, end);
+    else if (nks == 3) run_single(T16, integral_constant<int, 3>{}, g, end);
+    else if (nks == 4) run_single(TDEEP, integral_constant<int, 4>{}, g, end);
+    else if (nks == 5) run_single(TDEEP, integral_constant<int, 5>{}, g, end);
+    else run_single(TDEEP, integral_constant<int, 6>{}, g, end);
+    g += (end - g + (int)gridDim.x - 1) / (int)gridDim.x * (int)gridDim.x;      // my first tile of a later session
   }
   if (MODE == 2) {
     // ---- the CTA has scanned its last tile: what is still parked is sifted, then the four lists go to the heads' global
@@ -563,8 +561,8 @@ scan_kernel(const __grid_constant__ ScanBatch B, int G, int heads_per_plan, fath
   }
 }
 
-template <int NH, int MODE>
-int launch_scan(const ScanBatch& B, int Hkv, int Hq, int heads_per_plan, const fathom_scan_fuse& fz, bool dependent,
+template <int NH, int MODE, int CAP>
+int launch_scan(const ScanBatchOf<CAP>& B, int Hkv, int Hq, int heads_per_plan, const fathom_scan_fuse& fz, bool dependent,
                 cudaStream_t st) {
   const long long tiles = B.tile_end[B.items - 1];
   if (tiles <= 0) return FATHOM_OK;
@@ -573,7 +571,7 @@ int launch_scan(const ScanBatch& B, int Hkv, int Hq, int heads_per_plan, const f
   for (int i = 0; i < B.items; ++i) host = host || fathom_planes_in_host_memory(B.planes[i]);
   dim3 grid((unsigned)fathom_scan_grid_ctas(tiles, plans, host, CTAS_PER_SM), (unsigned)plans);
   constexpr size_t smem = sizeof(Smem<MODE>);                 // dynamic: MODE 2 needs more than the static limit
-  auto kernel = host ? scan_kernel<NH, MODE, false> : scan_kernel<NH, MODE, true>;
+  auto kernel = host ? scan_kernel<NH, MODE, false, CAP> : scan_kernel<NH, MODE, true, CAP>;
   if (smem > 48 * 1024) {
     static bool configured[64][2] = {};
     int dev = 0;
@@ -598,10 +596,19 @@ bool simt_path() {
   return v;
 }
 
-template <int MODE>
-int dispatch_scan(const ScanBatch& B, int Hkv, int Hq, int heads_per_plan, const fathom_scan_fuse& fz, bool dependent,
+template <int MODE, int CAP>
+int dispatch_scan(const ScanBatchOf<CAP>& B, int Hkv, int Hq, int heads_per_plan, const fathom_scan_fuse& fz, bool dependent,
                   cudaStream_t st) {
-  if (simt_path()) return fathom_scan_simt_dispatch(MODE, B, Hkv, Hq, heads_per_plan, fz, dependent, st);
+  if (simt_path()) {
+    ScanBatch W = {};
+    W.items = B.items;
+    for (int i = 0; i < B.items; ++i) {
+      W.planes[i] = B.planes[i]; W.scales[i] = B.scales[i]; W.q[i] = B.q[i]; W.depth[i] = B.depth[i]; W.scores[i] = B.scores[i];
+      W.n[i] = B.n[i]; W.plane_stride[i] = B.plane_stride[i]; W.scale_stride[i] = B.scale_stride[i]; W.score_stride[i] = B.score_stride[i];
+      W.tile_end[i] = B.tile_end[i];
+    }
+    return fathom_scan_simt_dispatch(MODE, W, Hkv, Hq, heads_per_plan, fz, dependent, st);
+  }
   switch (heads_per_plan) {
     case 1: return launch_scan<1, MODE>(B, Hkv, Hq, 1, fz, dependent, st);
     case 2: return launch_scan<2, MODE>(B, Hkv, Hq, 2, fz, dependent, st);
@@ -612,9 +619,9 @@ int dispatch_scan(const ScanBatch& B, int Hkv, int Hq, int heads_per_plan, const
 }
 
 // one session as a batch of one; `tile_step` > 1 lists only the sampled tiles
-ScanBatch single_item(const fathom_layout* L, const uint64_t* planes, const uint16_t* scales, const float* q, const uint8_t* depth,
-                      float* scores, long long score_stride, int tile_step) {
-  ScanBatch B = {};
+ScanBatchOf<1> single_item(const fathom_layout* L, const uint64_t* planes, const uint16_t* scales, const float* q, const uint8_t* depth,
+                           float* scores, long long score_stride, int tile_step) {
+  ScanBatchOf<1> B = {};
   B.items = 1;
   B.planes[0] = planes; B.scales[0] = scales; B.q[0] = q; B.depth[0] = depth; B.scores[0] = scores;
   B.n[0] = L->n; B.plane_stride[0] = L->plane_stride_words; B.scale_stride[0] = L->scale_stride; B.score_stride[0] = score_stride;

@@ -6,17 +6,21 @@
 constexpr int FATHOM_SCAN_TILE_BLOCKS = 16;                  // a tile = 16 blocks = 1024 tokens of one plan
 
 // ---- the sessions of one launch: their tiles are laid end to end (fathom_scan has one item)
-struct ScanBatch {
-  static constexpr int MAX_ITEMS = 32;
-  const uint64_t* planes[MAX_ITEMS];
-  const uint16_t* scales[MAX_ITEMS];
-  const float* q[MAX_ITEMS];
-  const uint8_t* depth[MAX_ITEMS];
-  float* scores[MAX_ITEMS];
-  long long n[MAX_ITEMS], plane_stride[MAX_ITEMS], scale_stride[MAX_ITEMS], score_stride[MAX_ITEMS];
-  long long tile_end[MAX_ITEMS];                              // tiles of items 0 .. i, inclusive prefix
+//      CAP: sessions it has room for.  It is a kernel parameter: one session takes 88 bytes, 32 sessions 2.6 KB, which cost
+//      every launch most of a microsecond
+template <int CAP>
+struct ScanBatchOf {
+  static constexpr int MAX_ITEMS = CAP;
+  const uint64_t* planes[CAP];
+  const uint16_t* scales[CAP];
+  const float* q[CAP];
+  const uint8_t* depth[CAP];
+  float* scores[CAP];
+  long long n[CAP], plane_stride[CAP], scale_stride[CAP], score_stride[CAP];
+  long long tile_end[CAP];                                    // tiles of items 0 .. i, inclusive prefix
   int items;
 };
+using ScanBatch = ScanBatchOf<32>;
 
 // fp32 value whose order-preserving integer image (see topk.cu) has `bin` as its 12 leading bits and zeros below:
 // the lower edge of that histogram bin
