@@ -23,9 +23,8 @@
 // A tile is 16 blocks (1024 tokens) of one plan (NH query heads that share the planes read).  With the planes in device
 // memory the CTAs are persistent: gridDim.x CTAs per plan walk the tiles round-robin, build the plan's row list and right
 // operand once, and fetch the next stage's plane words and scales with asynchronous copies (cp.async; a row's words are
-// one contiguous run, Sec. 3.6) into the other half of a double buffer.  A stage is a tile and up to 96 rows (half a tile in the
-// filtering mode for plans of more than 48 rows, whose lists take the shared memory); deeper plans take half tiles in
-// passes of up to 96 rows and carry the accumulators over the passes.  The right operand of all rows stays in shared memory.
+// one contiguous run, Sec. 3.6) into the other half of a double buffer.  A stage is a tile and up to 96 rows; deeper plans take half
+// tiles in passes of up to 96 rows and carry the accumulators over the passes.  The right operand of all rows stays in shared memory.
 // With the planes in pinned host memory the grid is one CTA per tile, which keeps the requests on the host link sequential.
 // Only planes p < t_j and the scales of active channels are ever read.
 #include "scan_shared.cuh"
@@ -53,31 +52,28 @@ struct Geo {
   static constexpr int ROW_BYTES = 8 * TB + 16;               // pitch of a staged plane-word row
   static constexpr int SCALE_ELEMS = 24;                      // pitch of a staged scale row, fp16 elements
 };
-// plans of up to this many rows take whole tiles in the filtering mode
-constexpr int FILTER_WHOLE_ROWS = 48;
-template <int MODE>
-struct StageBytes {                                           // one buffer: MODE 2 has whole tiles of 48 rows or half tiles of 96
-  static constexpr int WORDS = MODE == 2 ? STAGE_ROWS * Geo<8>::ROW_BYTES : STAGE_ROWS * Geo<16>::ROW_BYTES;
-  static constexpr int SCALES = STAGE_ROWS * Geo<16>::SCALE_ELEMS * 2;
-};
-static_assert(FILTER_WHOLE_ROWS * Geo<16>::ROW_BYTES <= StageBytes<2>::WORDS, "stage buffer too small");
+constexpr int STAGE_WORDS = STAGE_ROWS * Geo<16>::ROW_BYTES;           // one buffer of staged plane words
+constexpr int STAGE_SCALES = STAGE_ROWS * Geo<16>::SCALE_ELEMS * 2;    // one buffer of staged scales
+constexpr int STAGE_KSTEPS = STAGE_ROWS / 16;
+// deep plans stage half tiles, which leaves room for the right operand of their further rows behind the staged words
+constexpr int DEEP_WORDS = STAGE_ROWS * Geo<8>::ROW_BYTES;
+static_assert(2 * DEEP_WORDS + (MAX_KSTEPS - STAGE_KSTEPS) * 32 * 8 <= 2 * STAGE_WORDS, "room for the right operand of deep plans");
 
 // MODE 2.  A lane whose eight scores hold a candidate parks all eight in its warp's ring (three stores, no atomic, no
 // loop); when the ring may not take another round of 32, the warp sifts it with all lanes, one parked group per lane,
 // into the CTA's four candidate lists (one shared-memory atomic per head); the lists go to the heads' global lists once,
 // when the CTA has scanned its last tile (one global atomic per head and CTA).
 constexpr int PARK_RING = 64;                                // parked groups per warp
-constexpr int CAND_LIST = 256;                               // candidates per head the CTA keeps; beyond that: straight to the global list
+constexpr int CAND_LIST = 128;                               // candidates per head the CTA keeps; beyond that: straight to the global list
 
 template <int MODE>
 struct alignas(16) Smem {
   uint16_t row_id[MAX_ROWS];                                  // active row r: channel * 4 + plane
-  uint32_t woff[MAX_ROWS];                                    // where its plane words start within the KV head, in 16-byte units
-  uint32_t soff[MAX_ROWS];                                    // where its channel's scales start within the KV head, in 16-byte units
   int nrows;
   int warp_tot[WARPS];
   float wmax[WARPS][4];                                       // per warp: max_j |q_hj| of its channels
   float hscale[4], hinv[4];                                   // E_h and 1 / E_h
+  float q[4][FATHOM_D];                                       // the heads' queries
   float thr[4];                                               // MODE 2: score a token must reach, per head
   uint32_t ccount[4], cbase[4];                               // MODE 2: candidates in the CTA's lists; where they go in the global lists
   uint32_t elig[2];                                           // MODE 2: eligible tokens lo <= t < hi of the session
@@ -85,9 +81,9 @@ struct alignas(16) Smem {
   alignas(16) float4 park_hi[MODE == 2 ? WARPS * PARK_RING : 1];     //         scores 4..7
   uint32_t park_tok[MODE == 2 ? WARPS * PARK_RING : 1];       //         its first token (30 bits) and the head within the CTA (2 bits)
   uint2 clist[MODE == 2 ? 4 * CAND_LIST : 1];                 // MODE 2: (score bits, token) per head
-  alignas(16) uint2 bfr[MAX_KSTEPS][32];                      // right operand of all rows: per 16 rows, the two B registers of every lane
-  alignas(16) unsigned char words[2][StageBytes<MODE>::WORDS];    // staged plane words, double buffered
-  alignas(16) unsigned char scale[2][StageBytes<MODE>::SCALES];   // staged fp16 scales, double buffered
+  alignas(16) uint2 bfr[STAGE_KSTEPS][32];                    // right operand of the first 96 rows: per 16 rows, the two B registers of every lane
+  alignas(16) unsigned char words[2 * STAGE_WORDS];           // staged plane words, double buffered; deep plans: + the other rows' right operand
+  alignas(16) unsigned char scale[2 * STAGE_SCALES];          // staged fp16 scales, double buffered
 };
 
 // D += A B, A 16 x 16 (row), B 16 x 8 (col), fp16 operands, fp32 accumulators
@@ -102,10 +98,12 @@ __device__ __forceinline__ void mma_16816_first(float (&c)[4], uint32_t a0, uint
       : "=f"(c[0]), "=f"(c[1]), "=f"(c[2]), "=f"(c[3]) : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1), "f"(0.0f));
 }
 
-// the scale pair with each half's sign flipped where bit (15 - SH) resp. (31 - SH) of `bytes` is clear
-template <int SH>
+// byte k of two rows' plane words at the top of the two halves of a register: bits 8..15 and 24..31 (the others are masked later)
+__device__ __forceinline__ uint32_t row_bytes(uint32_t w0, uint32_t w1, int k) { return __byte_perm(w0, w1, 0x4000 + 0x1010 * k); }
+// the scale pair with each half's sign flipped where bit J of the half's byte is clear (J = 7 sits on the sign: no shift)
+template <int J>
 __device__ __forceinline__ uint32_t signed_pair(uint32_t pair, uint32_t bytes) {
-  return pair ^ (~(bytes << SH) & 0x80008000u);
+  return pair ^ (~(bytes << (7 - J)) & 0x80008000u);
 }
 
 // eight consecutive scores: one 32-byte store where the address allows it (a whole sector per lane), else two of 16 bytes
@@ -119,18 +117,17 @@ __device__ __forceinline__ void store_scores8(float* row, const float (&v)[8]) {
   }
 }
 
-// Eight tokens of a lane (one byte of every row's plane word; x0, x1: the bytes of the lane's two row pairs of 16 rows side by
-// side, bits 0..7 and 16..23) times 16 rows.  Slice j of the accumulators: mma row gq = token 2 j, row gq + 8 = token 2 j + 1.
+// Eight tokens of a lane (one byte of every row's plane word; x0, x1: row_bytes of the lane's two row pairs of 16 rows) times 16 rows.  Slice j of the accumulators: mma row gq = token 2 j, row gq + 8 = token 2 j + 1.
 template <bool FIRST>
 __device__ __forceinline__ void mma_tokens8(float (&acc)[4][4], uint32_t x0, uint32_t x1, uint32_t S0, uint32_t S1, uint2 bf) {
   auto mma = [&](float (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3) {
     if (FIRST) mma_16816_first(c, a0, a1, a2, a3, bf.x, bf.y);
     else mma_16816(c, a0, a1, a2, a3, bf.x, bf.y);
   };
-  mma(acc[0], signed_pair<15>(S0, x0), signed_pair<14>(S0, x0), signed_pair<15>(S1, x1), signed_pair<14>(S1, x1));
-  mma(acc[1], signed_pair<13>(S0, x0), signed_pair<12>(S0, x0), signed_pair<13>(S1, x1), signed_pair<12>(S1, x1));
-  mma(acc[2], signed_pair<11>(S0, x0), signed_pair<10>(S0, x0), signed_pair<11>(S1, x1), signed_pair<10>(S1, x1));
-  mma(acc[3], signed_pair<9>(S0, x0), signed_pair<8>(S0, x0), signed_pair<9>(S1, x1), signed_pair<8>(S1, x1));
+  mma(acc[0], signed_pair<0>(S0, x0), signed_pair<1>(S0, x0), signed_pair<0>(S1, x1), signed_pair<1>(S1, x1));
+  mma(acc[1], signed_pair<2>(S0, x0), signed_pair<3>(S0, x0), signed_pair<2>(S1, x1), signed_pair<3>(S1, x1));
+  mma(acc[2], signed_pair<4>(S0, x0), signed_pair<5>(S0, x0), signed_pair<4>(S1, x1), signed_pair<5>(S1, x1));
+  mma(acc[3], signed_pair<6>(S0, x0), signed_pair<7>(S0, x0), signed_pair<6>(S1, x1), signed_pair<7>(S1, x1));
 }
 
 // MODE 0: scores of every token are written (fathom_scan, fathom_scan_batch).
@@ -167,9 +164,14 @@ scan_kernel(const __grid_constant__ ScanBatchOf<CAP> B, int G, int heads_per_pla
   if (MODE == 2 && tid < NH)                                   // read after the barriers of the first item's row list
     M.thr[tid] = fz.state_is_score ? __uint_as_float(fz.state[(h0 + tid) * 8]) : fathom_bin_lower_edge(fz.state[(h0 + tid) * 8]);
 
-  int item = -1, nrows = 0, tb = TILE_BLOCKS, rows_stage = STAGE_ROWS, npass = 1, nb_item = 0;
+  int item = -1, nrows = 0, nb_item = 0;
+  uint32_t half_stride = 0, eighth_stride = 0;                 // rows of plane words and of scales in 16-byte units, and my KV head's first
+  const uint4 *planes_kv = nullptr, *scales_kv = nullptr;
   float hs = 1.0f, hs_tail = 0.0f;                             // E of my head and E 2^-11
 
+  auto bfr_of = [&](int ks) {                                  // the right operand of 16 rows, [32 lanes]
+    return ks < STAGE_KSTEPS ? M.bfr[ks] : reinterpret_cast<uint2*>(M.words + 2 * DEEP_WORDS) + (ks - STAGE_KSTEPS) * 32;
+  };
   // ---- right operand of all rows (made visible by the barrier that precedes the first stage's arithmetic): entry
   //      (kstep, lane, i) holds rows 16 kstep + 2 (lane & 3) + 8 i and the next one, column lane >> 2 = (head, part)
   auto fill_bfr = [&]() {
@@ -187,14 +189,14 @@ scan_kernel(const __grid_constant__ ScanBatchOf<CAP> B, int G, int heads_per_pla
           float v = 0.0f;
           if (r < nrows) {
             const int id = M.row_id[r];
-            v = __ldg(B.q[item] + (size_t)(h0 + head) * FATHOM_D + (id >> 2)) * inv * __int_as_float((129 - (id & 3)) << 23);
+            v = M.q[head][id >> 2] * inv * __int_as_float((129 - (id & 3)) << 23);
           }
           const __half hi = __float2half_rn(v);
           const __half out = part ? __float2half_rn((v - __half2float(hi)) * 2048.0f) : hi;
           packed |= (uint32_t)__half_as_ushort(out) << (16 * z);
         }
       }
-      reinterpret_cast<uint32_t*>(&M.bfr[ks][ln])[i] = packed;
+      reinterpret_cast<uint32_t*>(bfr_of(ks) + ln)[i] = packed;
     }
   };
 
@@ -210,7 +212,11 @@ scan_kernel(const __grid_constant__ ScanBatchOf<CAP> B, int G, int heads_per_pla
     int incl = t;                                              // inclusive prefix of depths over channels
     float qa[NH];
 #pragma unroll
-    for (int h = 0; h < NH; ++h) qa[h] = fabsf(__ldg(B.q[it] + (size_t)(h0 + h) * FATHOM_D + tid));
+    for (int h = 0; h < NH; ++h) {
+      const float x = __ldg(B.q[it] + (size_t)(h0 + h) * FATHOM_D + tid);
+      M.q[h][tid] = x;
+      qa[h] = fabsf(x);
+    }
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
       const int y = __shfl_up_sync(0xffffffffu, incl, o);
@@ -226,12 +232,7 @@ scan_kernel(const __grid_constant__ ScanBatchOf<CAP> B, int G, int heads_per_pla
     int before = 0;
     for (int w = 0; w < warp; ++w) before += M.warp_tot[w];
     const int start = before + incl - t;
-    const uint32_t half_stride = (uint32_t)(B.plane_stride[it] >> 1), eighth_stride = (uint32_t)(B.scale_stride[it] >> 3);
-    for (int p = 0; p < t; ++p) {                              // (511 * half_stride < 2^32: fathom_check_layout)
-      M.row_id[start + p] = (uint16_t)(tid * FATHOM_NPLANES + p);
-      M.woff[start + p] = (uint32_t)(tid * FATHOM_NPLANES + p) * half_stride;
-      M.soff[start + p] = (uint32_t)tid * eighth_stride;
-    }
+    for (int p = 0; p < t; ++p) M.row_id[start + p] = (uint16_t)(tid * FATHOM_NPLANES + p);
     if (tid == FATHOM_D - 1) M.nrows = before + incl;
     if (tid < NH) {                                            // E = 2^floor(log2 max|q|), kept inside the normal range
       float m = 0.0f;
@@ -244,9 +245,10 @@ scan_kernel(const __grid_constant__ ScanBatchOf<CAP> B, int G, int heads_per_pla
     }
     __syncthreads();
     nrows = M.nrows;
-    tb = nrows <= (MODE == 2 ? FILTER_WHOLE_ROWS : STAGE_ROWS) ? 16 : 8;
-    npass = max(1, (nrows + STAGE_ROWS - 1) / STAGE_ROWS);
-    rows_stage = ((nrows + npass - 1) / npass + 15) & ~15;     // equal passes of whole ksteps, at most 96 rows
+    half_stride = (uint32_t)(B.plane_stride[it] >> 1);          // (511 * half_stride < 2^32: fathom_check_layout)
+    eighth_stride = (uint32_t)(B.scale_stride[it] >> 3);
+    planes_kv = reinterpret_cast<const uint4*>(B.planes[it]) + (uint64_t)(kv * FATHOM_D * FATHOM_NPLANES) * (uint64_t)half_stride;
+    scales_kv = reinterpret_cast<const uint4*>(B.scales[it]) + (uint64_t)(kv * FATHOM_D) * (uint64_t)eighth_stride;
     hs = M.hscale[myh];
     hs_tail = hs * 4.8828125e-4f;                              // 2^-11
   };
@@ -257,39 +259,12 @@ scan_kernel(const __grid_constant__ ScanBatchOf<CAP> B, int G, int heads_per_pla
     return tl * (MODE == 1 ? fz.tile_step : 1) * TILE_BLOCKS;
   };
 
-  // ---- asynchronous copies of the plane words and scales of one stage: sub-tile u of `tile`, rows of `pass`
-  auto prefetch = [&](int tile, int u, int pass, int buf) {
-    const int blk0 = first_block(tile) + u * tb;
-    const int nblk = min(tb, nb_item - blk0);                  // >= 1: stages past the last block are never entered
-    const int s0 = pass * rows_stage, sc = min(rows_stage, nrows - s0);
-    // 16-byte units throughout: plane_stride is even, scale_stride a multiple of 8, blk0 a multiple of tb
-    const uint4* planes_kv = reinterpret_cast<const uint4*>(B.planes[item]) +
-                             (uint64_t)(kv * FATHOM_D * FATHOM_NPLANES) * (uint64_t)(B.plane_stride[item] >> 1) + (blk0 >> 1);
-    const unsigned char* scales_kv = reinterpret_cast<const unsigned char*>(B.scales[item]) +
-                                     (uint64_t)(kv * FATHOM_D) * (uint64_t)B.scale_stride[item] * 2 + (uint64_t)blk0 * 2;
-    const int sh = tb == 16 ? 3 : 2;                           // 16-byte copies per row of plane words: tb / 2
-    const int row_bytes = 8 * tb + 16;
-    unsigned char* wdst = M.words[buf];
-    const int c = tid & ((1 << sh) - 1);                       // my 16-byte column of every row I copy
-    const bool valid = 2 * c < nblk;
-    for (int r = tid >> sh; r < sc; r += THREADS >> sh)
-      fathom_copy_async<16>(wdst + r * row_bytes + c * 16, valid ? planes_kv + M.woff[s0 + r] + c : planes_kv, valid, in_hbm);
-    unsigned char* sdst = M.scale[buf];
-    if (tb == 16) {
-      const int cs = tid & 1;
-      const bool vs = 8 * cs < nblk;
-      for (int r = tid >> 1; r < sc; r += THREADS >> 1)
-        fathom_copy_async<16>(sdst + r * (Geo<16>::SCALE_ELEMS * 2) + cs * 16, vs ? scales_kv + (uint64_t)M.soff[s0 + r] * 16 + cs * 16 : scales_kv, vs,
-                              in_hbm);
-    } else {
-      for (int r = tid; r < sc; r += THREADS)
-        fathom_copy_async<16>(sdst + r * (Geo<8>::SCALE_ELEMS * 2), scales_kv + (uint64_t)M.soff[s0 + r] * 16, true, in_hbm);
-    }
-    // rows that pad the last 16: scale 0, so that whatever the stale plane bytes say they contribute +-0
-    const int pad = max(16, (sc + 15) & ~15) - sc;
+  // a buffer's scale rows from `first` up to the next multiple of 16 (at least 16) hold 0, so that whatever the stale plane bytes of
+  // those rows say they contribute +-0
+  auto clear_pad = [&](int first, int buf) {
+    const int pad = max(16, (first + 15) & ~15) - first;
     constexpr int WPR = Geo<16>::SCALE_ELEMS / 2;              // 32-bit words per scale row
-    for (int e = tid; e < pad * WPR; e += THREADS) reinterpret_cast<uint32_t*>(sdst)[(sc + e / WPR) * WPR + e % WPR] = 0u;
-    fathom_copies_commit();
+    for (int e = tid; e < pad * WPR; e += THREADS) reinterpret_cast<uint32_t*>(M.scale + buf * STAGE_SCALES)[first * WPR + e] = 0u;
   };
 
   uint32_t parked = 0u, stages = 0u;                           // MODE 2: groups in my warp's ring (the same in every lane); stages done
@@ -406,8 +381,8 @@ scan_kernel(const __grid_constant__ ScanBatchOf<CAP> B, int G, int heads_per_pla
     const int mine = warp * (TB / 4) + (gq * BYTES) / 8;       // my block of the stage
     const int off = (gq * BYTES) % 8;                          // where my bytes start in its words
     Place p;
-    p.wp = M.words[buf] + (2 * t4) * Geo<TB>::ROW_BYTES + mine * 8 + off;
-    p.sp = reinterpret_cast<const uint16_t*>(M.scale[buf]) + (2 * t4) * Geo<TB>::SCALE_ELEMS + mine;
+    p.wp = M.words + buf * (TB == 16 ? STAGE_WORDS : DEEP_WORDS) + (2 * t4) * Geo<TB>::ROW_BYTES + mine * 8 + off;
+    p.sp = reinterpret_cast<const uint16_t*>(M.scale + buf * STAGE_SCALES) + (2 * t4) * Geo<TB>::SCALE_ELEMS + mine;
     p.tok0 = (uint32_t)(first_block(g) + u * TB + mine) * FATHOM_BLOCK + off * 8;           // my first token
     p.dst0 = MODE == 1 ? (uint32_t)g * (TILE_BLOCKS * FATHOM_BLOCK) + (uint32_t)(u * TB + mine) * FATHOM_BLOCK + off * 8 : p.tok0;
     return p;
@@ -424,50 +399,72 @@ scan_kernel(const __grid_constant__ ScanBatchOf<CAP> B, int G, int heads_per_pla
     S[0] = __byte_perm(sk[0], sk[SE], 0x5410);
     S[1] = __byte_perm(sk[8 * SE], sk[9 * SE], 0x5410);
   };
-  // single pass, NKS x 16 rows: the words and scales a lane reads are in registers before the first MMA, and so is the right
-  // operand of up to four steps (of more it would spill)
-  auto compute_single = [&](auto tbc, auto nksc, int g, int u, int buf) {
-    constexpr int TB = decltype(tbc)::value, NKS = decltype(nksc)::value;
+  // plans of up to 96 rows, NKS x 16 of them (the last 16 may be padded): a stage is a tile.  A thread copies the same 16-byte
+  // column of the same rows in every stage, so where they start is kept in registers.  The words and scales a lane reads are in
+  // registers before the first MMA, and so is the right operand of up to four steps (of more it would spill)
+  auto run_single = [&](auto nksc, int g, int end) {
+    constexpr int NKS = decltype(nksc)::value;
     constexpr bool KEEP = NKS <= 4;
-    const Place at = place(tbc, g, u, buf);
-    uint32_t w[NKS][4], S[NKS][2];
-    uint2 bf[KEEP ? NKS : 1];
+    constexpr std::integral_constant<int, 16> T16{};
+    constexpr int SC = (16 * NKS + 63) / 64;                   // sweeps of 64 rows over the scales
+    static_assert(THREADS == 128, "16 rows of plane words and 64 of scales per sweep of the CTA");
+    const int c = tid & 7, cs = tid & 1;
+    uint32_t wo[NKS], so[SC];
 #pragma unroll
-    for (int ks = 0; ks < NKS; ++ks) {
-      if (KEEP) bf[ks] = M.bfr[ks][lane];
-      load_rows(tbc, at.wp + ks * (16 * Geo<TB>::ROW_BYTES), at.sp + ks * (16 * Geo<TB>::SCALE_ELEMS), w[ks], S[ks]);
-    }
+    for (int i = 0; i < NKS; ++i) wo[i] = (uint32_t)M.row_id[min((tid >> 3) + 16 * i, MAX_ROWS - 1)] * half_stride;
+#pragma unroll
+    for (int i = 0; i < SC; ++i) so[i] = (uint32_t)(M.row_id[min((tid >> 1) + 64 * i, MAX_ROWS - 1)] >> 2) * eighth_stride;
+    const bool last_row = (tid >> 3) + 16 * (NKS - 1) < nrows;
+    auto prefetch = [&](int blk0, int buf) {
+      const int nblk = nb_item - blk0;                         // >= 1
+      const bool vw = 2 * c < nblk, vs = 8 * cs < nblk;
+      const uint4* words_src = planes_kv + (vw ? (blk0 >> 1) + c : 0);       // (nothing is read where there is no block)
+      const uint4* scales_src = scales_kv + (vs ? (blk0 >> 3) + cs : 0);
+      unsigned char* wd = M.words + buf * STAGE_WORDS + (tid >> 3) * Geo<16>::ROW_BYTES + c * 16;
+      unsigned char* sd = M.scale + buf * STAGE_SCALES + (tid >> 1) * (Geo<16>::SCALE_ELEMS * 2) + cs * 16;
+#pragma unroll
+      for (int i = 0; i < NKS; ++i)
+        if (i < NKS - 1 || last_row) fathom_copy_async<16>(wd + i * (16 * Geo<16>::ROW_BYTES), words_src + wo[i], vw, in_hbm);
+#pragma unroll
+      for (int i = 0; i < SC; ++i)
+        if ((tid >> 1) + 64 * i < nrows) fathom_copy_async<16>(sd + i * (64 * Geo<16>::SCALE_ELEMS * 2), scales_src + so[i], vs, in_hbm);
+      fathom_copies_commit();
+    };
+    prefetch(first_block(g), 0);                               // the first stage's rows are on their way ...
+    clear_pad(nrows, 0);
+    clear_pad(nrows, 1);
+    fill_bfr();                                                // ... while the right operand is made
     const uint32_t n = (uint32_t)B.n[item];                    // n < 2^31
-#pragma unroll
-    for (int k = 0; k < TB / 4; ++k) {
-      float acc[4][4];
-#pragma unroll
-      for (int ks = 0; ks < NKS; ++ks) {
-        const uint32_t x0 = __byte_perm(w[ks][0], w[ks][1], 0x0400 + 0x0101 * k);
-        const uint32_t x1 = __byte_perm(w[ks][2], w[ks][3], 0x0400 + 0x0101 * k);
-        const uint2 b = KEEP ? bf[KEEP ? ks : 0] : M.bfr[ks][lane];
-        if (ks == 0) mma_tokens8<true>(acc, x0, x1, S[ks][0], S[ks][1], b);
-        else mma_tokens8<false>(acc, x0, x1, S[ks][0], S[ks][1], b);
-      }
-      finish(acc, at.tok0 + 8 * k, at.dst0 + 8 * k, n);
-    }
-  };
-
-  auto run_single = [&](auto tbc, auto nksc, int g, int end) {
-    constexpr int TB = decltype(tbc)::value;
-    for (int u = 0, buf = 0;; buf ^= 1) {
-      int g_next = g, u_next = u + 1;                          // the stage after this one: the next sub-tile, or my next tile
-      if (u_next * TB >= TILE_BLOCKS || first_block(g) + u_next * TB >= nb_item) { u_next = 0; g_next = g + gridDim.x; }
+    uint2 bf[KEEP ? NKS : 1];
+    for (int buf = 0;; buf ^= 1) {
+      const int g_next = g + gridDim.x;
       const bool more = g_next < end;
       fathom_copies_wait<0>();
       __syncthreads();                                         // this stage's words and scales are in place, and every warp has
                                                                // left the previous stage: its buffer may be refilled
-      if (more) prefetch(g_next, u_next, 0, buf ^ 1);          // lands while this stage is scanned
-      compute_single(tbc, nksc, g, u, buf);
+      if (more) prefetch(first_block(g_next), buf ^ 1);        // lands while this stage is scanned
+      const Place at = place(T16, g, 0, buf);
+      uint32_t w[NKS][4], S[NKS][2];
+#pragma unroll
+      for (int ks = 0; ks < NKS; ++ks) {
+        if (KEEP) bf[ks] = M.bfr[ks][lane];
+        load_rows(T16, at.wp + ks * (16 * Geo<16>::ROW_BYTES), at.sp + ks * (16 * Geo<16>::SCALE_ELEMS), w[ks], S[ks]);
+      }
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        float acc[4][4];
+#pragma unroll
+        for (int ks = 0; ks < NKS; ++ks) {
+          const uint32_t x0 = row_bytes(w[ks][0], w[ks][1], k), x1 = row_bytes(w[ks][2], w[ks][3], k);
+          const uint2 b = KEEP ? bf[KEEP ? ks : 0] : M.bfr[ks][lane];
+          if (ks == 0) mma_tokens8<true>(acc, x0, x1, S[ks][0], S[ks][1], b);
+          else mma_tokens8<false>(acc, x0, x1, S[ks][0], S[ks][1], b);
+        }
+        finish(acc, at.tok0 + 8 * k, at.dst0 + 8 * k, n);
+      }
       if (MODE == 2 && (++stages & 3u) == 0u) sift();          // (every warp of the CTA at the same stages)
       if (!more) return;
       g = g_next;
-      u = u_next;
     }
   };
   // plans of more than 96 rows: the accumulators of the lane's tokens are carried over the passes of a half tile (those of a whole
@@ -475,6 +472,27 @@ scan_kernel(const __grid_constant__ ScanBatchOf<CAP> B, int G, int heads_per_pla
   auto run_passes = [&](int g, int end) {
     constexpr std::integral_constant<int, 8> tbc{};
     constexpr int TB = 8, BYTES = TB / 4;
+    const int npass = (nrows + STAGE_ROWS - 1) / STAGE_ROWS;
+    const int rows_stage = ((nrows + npass - 1) / npass + 15) & ~15;          // equal passes of whole ksteps, at most 96 rows
+    // plane words and scales of one stage: half tile u of tile g, rows of `pass`
+    auto prefetch = [&](int g, int u, int pass, int buf) {
+      const int blk0 = first_block(g) + u * TB;
+      const int nblk = nb_item - blk0;                         // >= 1: stages past the last block are never entered
+      const int s0 = pass * rows_stage, sc = min(rows_stage, nrows - s0);
+      const int c = tid & 3;                                   // my 16-byte column of every row I copy
+      const bool valid = 2 * c < nblk;
+      const uint4* words_src = planes_kv + (valid ? (blk0 >> 1) + c : 0);
+      unsigned char* wd = M.words + buf * DEEP_WORDS + c * 16;
+      for (int r = tid >> 2; r < sc; r += THREADS >> 2)
+        fathom_copy_async<16>(wd + r * Geo<TB>::ROW_BYTES, words_src + (uint32_t)M.row_id[s0 + r] * half_stride, valid, in_hbm);
+      unsigned char* sd = M.scale + buf * STAGE_SCALES;
+      for (int r = tid; r < sc; r += THREADS)
+        fathom_copy_async<16>(sd + r * (Geo<TB>::SCALE_ELEMS * 2), scales_kv + (blk0 >> 3) + (uint32_t)(M.row_id[s0 + r] >> 2) * eighth_stride, true, in_hbm);
+      clear_pad(sc, buf);
+      fathom_copies_commit();
+    };
+    prefetch(g, 0, 0, 0);
+    fill_bfr();
     float acc[BYTES][4][4];
     for (int u = 0, pass = 0, buf = 0;; buf ^= 1) {
       int g_next = g, u_next = u, pass_next = pass + 1;
@@ -498,11 +516,11 @@ scan_kernel(const __grid_constant__ ScanBatchOf<CAP> B, int G, int heads_per_pla
 #pragma unroll 2
       for (int ks = 0; ks < nks; ++ks) {
         uint32_t w[4], S[2];
-        const uint2 bf = M.bfr[ks0 + ks][lane];
+        const uint2 bf = bfr_of(ks0 + ks)[lane];
         load_rows(tbc, at.wp + ks * (16 * Geo<TB>::ROW_BYTES), at.sp + ks * (16 * Geo<TB>::SCALE_ELEMS), w, S);
 #pragma unroll
         for (int k = 0; k < BYTES; ++k)
-          mma_tokens8<false>(acc[k], __byte_perm(w[0], w[1], 0x0400 + 0x0101 * k), __byte_perm(w[2], w[3], 0x0400 + 0x0101 * k), S[0], S[1], bf);
+          mma_tokens8<false>(acc[k], row_bytes(w[0], w[1], k), row_bytes(w[2], w[3], k), S[0], S[1], bf);
       }
       if (pass == npass - 1) {
         const uint32_t n = (uint32_t)B.n[item];
@@ -522,19 +540,14 @@ scan_kernel(const __grid_constant__ ScanBatchOf<CAP> B, int G, int heads_per_pla
     enter_item(g);
     if (MODE == 2) my_thr = M.thr[myh];
     const int end = min(total, (int)B.tile_end[item]);
-    prefetch(g, 0, 0, 0);                                      // the first stage's rows are on their way ...
-    fill_bfr();                                                // ... while the right operand is made
-    using std::integral_constant;
-    constexpr integral_constant<int, 16> T16{};
-    constexpr integral_constant<int, MODE == 2 ? 8 : 16> TDEEP{};
     const int nks = (nrows + 15) >> 4;
-    if (npass > 1) run_passes(g, end);
-    else if (nks <= 1) run_single(T16, integral_constant<int, 1>{}, g, end);
-    else if (nks == 2) run_single(T16, integral_constant<int, 2>{}, g, end);
-    else if (nks == 3) run_single(T16, integral_constant<int, 3>{}, g, end);
-    else if (nks == 4) run_single(TDEEP, integral_constant<int, 4>{}, g, end);
-    else if (nks == 5) run_single(TDEEP, integral_constant<int, 5>{}, g, end);
-    else run_single(TDEEP, integral_constant<int, 6>{}, g, end);
+    if (nks > STAGE_KSTEPS) run_passes(g, end);
+    else if (nks <= 1) run_single(std::integral_constant<int, 1>{}, g, end);
+    else if (nks == 2) run_single(std::integral_constant<int, 2>{}, g, end);
+    else if (nks == 3) run_single(std::integral_constant<int, 3>{}, g, end);
+    else if (nks == 4) run_single(std::integral_constant<int, 4>{}, g, end);
+    else if (nks == 5) run_single(std::integral_constant<int, 5>{}, g, end);
+    else run_single(std::integral_constant<int, 6>{}, g, end);
     g += (end - g + (int)gridDim.x - 1) / (int)gridDim.x * (int)gridDim.x;      // my first tile of a later session
   }
   if (MODE == 2) {
