@@ -2,20 +2,20 @@
 //
 // Eq. 4 at the smallest water line that fits the budget grants exactly the min(B, 4d) candidate planes
 // (channel j, plane m = 1..4) with the largest priority g_j 4^-m, so a candidate is granted when fewer than
-// B others rank before it (ties: lower channel, then lower plane).  Four CTAs of 512 threads serve a plan:
+// B others rank before it (ties: lower channel, then lower plane).  Eight CTAs of 512 threads serve a plan:
 // every CTA computes all 128 importances (thread = channel; fp64 with explicit round-to-nearest intrinsics,
 // no fused multiply-add, so the ranking is identical on every machine; no logarithm is evaluated) and ranks
-// the 128 candidates of its own 32 channels against all 512, four threads per candidate (each counts over a
-// quarter of the others: the kernel is a latency chain, and the counting loop is its longest link).
+// the 64 candidates of its own 16 channels against all 512, eight threads per candidate (each counts over an
+// eighth of the others: the kernel is a latency chain, and the counting loop is its longest link).
 // Non-negative doubles order like their bit patterns, so the comparisons run on 64-bit integers.
 #include "fathom_common.cuh"
 
 namespace {
 
 constexpr int NCAND = FATHOM_D * FATHOM_NPLANES;   // 512
-constexpr int CTAS_PER_PLAN = 4;
-constexpr int AD_CAND = NCAND / CTAS_PER_PLAN;     // 128 candidates ranked per CTA
-constexpr int AD_SPLIT = 4;                        // threads per candidate
+constexpr int CTAS_PER_PLAN = 8;
+constexpr int AD_CAND = NCAND / CTAS_PER_PLAN;     // 64 candidates ranked per CTA
+constexpr int AD_SPLIT = 8;                        // threads per candidate
 constexpr int AD_THREADS = AD_CAND * AD_SPLIT;     // 512
 
 __global__ void __launch_bounds__(AD_THREADS)
@@ -67,11 +67,11 @@ alloc_depth_kernel(const float* __restrict__ q, const float* __restrict__ var, i
   }
   __syncthreads();
 
-  const int cand = tid & (AD_CAND - 1), quarter = tid / AD_CAND;
+  const int cand = tid & (AD_CAND - 1), share = tid / AD_CAND;
   const int id = part * AD_CAND + cand;                       // my candidate: channel id / 4, plane id % 4 + 1
   const unsigned long long key = pri[id];
   int rank = 0;
-  const int o0 = quarter * (NCAND / AD_SPLIT), o1 = o0 + NCAND / AD_SPLIT;
+  const int o0 = share * (NCAND / AD_SPLIT), o1 = o0 + NCAND / AD_SPLIT;
   if (mode == FATHOM_DEPTH_WATERFILL) {
 #pragma unroll 8
     for (int o = o0; o < o1; o += 2) {
@@ -86,10 +86,12 @@ alloc_depth_kernel(const float* __restrict__ q, const float* __restrict__ var, i
       rank += (p > key) || (p == key && o < (id & ~3));
     }
   }
-  partial[quarter][cand] = rank;
+  partial[share][cand] = rank;
   __syncthreads();
-  if (quarter == 0) {                                         // the first four warps: one thread per candidate
-    rank = partial[0][cand] + partial[1][cand] + partial[2][cand] + partial[3][cand];
+  if (share == 0) {                                           // the first two warps: one thread per candidate
+    rank = 0;
+#pragma unroll
+    for (int s = 0; s < AD_SPLIT; ++s) rank += partial[s][cand];
     const bool granted = rank < budget;                       // fixed mode: all four planes of a chosen channel
     const unsigned ball = __ballot_sync(0xffffffffu, granted);
     if ((id & 3) == 0) out[id >> 2] = (uint8_t)__popc((ball >> (tid & 31)) & 0xFu);

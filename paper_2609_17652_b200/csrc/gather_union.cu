@@ -2,19 +2,86 @@
 // (Sec. 1: the heads of a group mostly pick the same tokens, so a KV head's distinct rows - at most G k - cross the link
 // once; Sec. 4 "Offload harness": the row fetch of a decode step is that union).
 //
-// Three kernels on the caller's stream, no host round trip:
-//   mark    every selected token sets its bit in a per-KV-head bitmap (atomic OR: idempotent, so order-free);
-//   rank    one CTA per KV head: popcount prefix over the bitmap words gives every word its rank base, the
-//           ascending list of distinct tokens and their number;
-//   fetch   one warp per staged row copies the K and the V row (16-byte loads; rows may live in pinned host
-//           memory and are then read over the host link exactly once), and every (head, i) learns the position
-//           of its token among the staged rows: rank base of its word + popcount of the lower bits.
+// Two kernels on the caller's stream, no host round trip:
+//   list    one CTA per KV head: every selected token sets its bit in a bitmap in shared memory (atomic OR: idempotent, so
+//           order-free), a popcount prefix over the bitmap gives the ascending list of distinct tokens, their number and,
+//           for every (head, i), the position of its token among the staged rows;
+//   fetch   one warp per staged row copies the K and the V row (16-byte loads; rows may live in pinned host memory and are
+//           then read over the host link exactly once).
+// The fetch of an offloaded step is bound by the link; what was left to save is the time in which the link is idle: clearing,
+// marking and ranking a bitmap in global memory were three launches in front of it (12 us a session, now 5).  A sequence whose
+// bitmap does not fit in shared memory (more than 1.7 M tokens) still takes those.
 #include "fathom_common.cuh"
 
 namespace {
 
 constexpr int GU_THREADS = 256;
 constexpr int RANK_THREADS = 1024;
+
+constexpr long long LIST_MAX_WORDS = 52 * 1024;              // bitmap words (32 tokens each) kept in shared memory: 208 KB
+constexpr int LIST_THREADS = 1024;
+
+// Thread t owns `per` consecutive words (an odd multiple of four: 16-byte reads without bank conflicts), so that one block prefix
+// ranks the whole bitmap.
+__global__ void __launch_bounds__(LIST_THREADS)
+union_list_kernel(const int32_t* __restrict__ idx, int k, long long n, int G, int per, int32_t* __restrict__ ulist, int capacity,
+                  int32_t* __restrict__ union_count, int32_t* __restrict__ idx_local) {
+  extern __shared__ __align__(16) uint32_t s_bitmap[];        // [LIST_THREADS * per]
+  __shared__ uint32_t s_warp[LIST_THREADS / 32];
+  __shared__ uint32_t s_base[LIST_THREADS];                   // distinct tokens before a thread's words
+  const int kv = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  uint4* mine = reinterpret_cast<uint4*>(s_bitmap + tid * per);
+  for (int w = tid; w < LIST_THREADS * per / 4; w += LIST_THREADS) reinterpret_cast<uint4*>(s_bitmap)[w] = make_uint4(0u, 0u, 0u, 0u);
+  __syncthreads();
+  FATHOM_PDL_WAIT();                                          // the picks come from the previous kernel
+  FATHOM_PDL_RELEASE();                                       // the fetch may become resident now
+  const int picks = G * k;                                    // heads kv*G .. kv*G+G-1 are contiguous in idx
+  const int32_t* my_idx = idx + (size_t)kv * picks;
+  int32_t* my_local = idx_local + (size_t)kv * picks;
+  auto clamped = [&](int32_t t) { return t < 0 ? 0 : ((long long)t >= n ? (int32_t)(n - 1) : t); };   // like in attention
+#pragma unroll 8
+  for (int e = tid; e < picks; e += LIST_THREADS) {
+    const int32_t t = clamped(__ldg(my_idx + e));
+    atomicOr(&s_bitmap[t >> 5], 1u << (t & 31));
+  }
+  __syncthreads();
+  uint32_t own = 0u;
+  for (int w = 0; w < per / 4; ++w) {
+    const uint4 x = mine[w];
+    own += __popc(x.x) + __popc(x.y) + __popc(x.z) + __popc(x.w);
+  }
+  uint32_t incl = own;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+    if (lane >= o) incl += y;
+  }
+  if (lane == 31) s_warp[warp] = incl;
+  __syncthreads();
+  uint32_t ahead = lane < warp ? s_warp[lane] : 0u;           // (32 warps)
+  ahead = __reduce_add_sync(0xffffffffu, ahead);
+  uint32_t pos = ahead + incl - own;
+  s_base[tid] = pos;
+  if (tid == LIST_THREADS - 1) union_count[kv] = (int32_t)(pos + own);
+  int32_t* ul = ulist + (size_t)kv * capacity;
+  for (int w = 0; own && w < per; ++w) {
+    uint32_t b = s_bitmap[tid * per + w];
+    while (b) {
+      const int l = __ffs(b) - 1;
+      b &= b - 1;
+      if (pos < (uint32_t)capacity) ul[pos] = (tid * per + w) * 32 + l;
+      ++pos;
+    }
+  }
+  __syncthreads();
+  for (int e = tid; e < picks; e += LIST_THREADS) {
+    const int32_t t = clamped(__ldg(my_idx + e));
+    const int word = t >> 5, owner = word / per;
+    uint32_t r = s_base[owner] + __popc(s_bitmap[word] & ((1u << (t & 31)) - 1u));
+    for (int w = owner * per; w < word; ++w) r += __popc(s_bitmap[w]);
+    my_local[e] = (int32_t)r;
+  }
+}
 
 __global__ void __launch_bounds__(GU_THREADS)
 union_mark_kernel(const int32_t* __restrict__ idx, int k, long long n, int G, long long total, uint32_t* __restrict__ bitmap,
@@ -81,6 +148,8 @@ union_fetch_kernel(const T* __restrict__ Krows, const T* __restrict__ Vrows, lon
                    const int32_t* __restrict__ union_count, int capacity, T* __restrict__ K_stage, T* __restrict__ V_stage,
                    const int32_t* __restrict__ idx, int k, int G, int Hq, const uint32_t* __restrict__ bitmap,
                    const uint32_t* __restrict__ word_rank, long long words, int32_t* __restrict__ idx_local) {
+  FATHOM_PDL_WAIT();                                          // the list comes from the previous kernel
+  FATHOM_PDL_RELEASE();                                       // the attention may become resident where this kernel has finished
   constexpr int ROW_U4 = FATHOM_D * sizeof(T) / 16;           // 16-byte pieces per row: 16 (bf16) or 32 (fp32)
   constexpr int ROWS_PER_WARP_STEP = 32 / ROW_U4 > 0 ? 32 / ROW_U4 : 1;
   const int kv = blockIdx.y, lane = threadIdx.x & 31;
@@ -102,7 +171,8 @@ union_fetch_kernel(const T* __restrict__ Krows, const T* __restrict__ Vrows, lon
       reinterpret_cast<uint4*>(Vs + (size_t)r * FATHOM_D)[piece] = b;
     }
   }
-  // ---- positions of the G heads' picks among the staged rows
+  // ---- positions of the G heads' picks among the staged rows (bitmap null: the list kernel wrote them)
+  if (bitmap == nullptr) return;
   const uint32_t* bm = bitmap + (size_t)kv * words;
   const uint32_t* wr = word_rank + (size_t)kv * words;
   const long long picks = (long long)G * k;
@@ -144,22 +214,35 @@ extern "C" int fathom_gather_union(fathom_ctx* ctx, const fathom_layout* L, cons
   uint32_t* word_rank = reinterpret_cast<uint32_t*>(base + bm_bytes);
   int32_t* ulist = reinterpret_cast<int32_t*>(base + 2 * bm_bytes);
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  FATHOM_CUDA_TRY(ctx, cudaMemsetAsync(bitmap, 0, bm_bytes, st));
-  const long long total = (long long)Hq * k;
-  union_mark_kernel<<<(unsigned)((total + GU_THREADS - 1) / GU_THREADS), GU_THREADS, 0, st>>>(idx, k, L->n, G, total, bitmap, words);
-  union_rank_kernel<<<Hkv, RANK_THREADS, 0, st>>>(bitmap, words, word_rank, ulist, capacity, union_count);
+  if (words <= LIST_MAX_WORDS) {
+    const int per = (int)(((words + LIST_THREADS * 4 - 1) / (LIST_THREADS * 4)) | 1) * 4;
+    static bool configured[64] = {};
+    if (ctx->device < 0 || ctx->device >= 64 || !configured[ctx->device]) {
+      FATHOM_CUDA_TRY(ctx, cudaFuncSetAttribute(union_list_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)LIST_MAX_WORDS * 4));
+      if (ctx->device >= 0 && ctx->device < 64) configured[ctx->device] = true;
+    }
+    FATHOM_CUDA_TRY(ctx, fathom_launch_dependent(union_list_kernel, dim3(Hkv), dim3(LIST_THREADS), (size_t)LIST_THREADS * per * 4, st, idx, k,
+                                                 (long long)L->n, G, per, ulist, capacity, union_count, idx_local));
+    bitmap = nullptr;
+  } else {
+    FATHOM_CUDA_TRY(ctx, cudaMemsetAsync(bitmap, 0, bm_bytes, st));
+    const long long total = (long long)Hq * k;
+    union_mark_kernel<<<(unsigned)((total + GU_THREADS - 1) / GU_THREADS), GU_THREADS, 0, st>>>(idx, k, L->n, G, total, bitmap, words);
+    union_rank_kernel<<<Hkv, RANK_THREADS, 0, st>>>(bitmap, words, word_rank, ulist, capacity, union_count);
+  }
   // enough warps to keep a slow link busy: 16 CTAs of 8 warps per KV head, each warp 2 x 256-byte rows in flight per step
   dim3 grid((unsigned)max(1, min(64, (capacity + 63) / 64)), (unsigned)Hkv);
   if (row_dtype == FATHOM_BF16)
-    union_fetch_kernel<__nv_bfloat16><<<grid, GU_THREADS, 0, st>>>(
-        static_cast<const __nv_bfloat16*>(Krows), static_cast<const __nv_bfloat16*>(Vrows), L->n, ulist, union_count, capacity,
-        static_cast<__nv_bfloat16*>(K_stage), static_cast<__nv_bfloat16*>(V_stage), idx, k, G, Hq, bitmap, word_rank, words,
-        idx_local);
+    FATHOM_CUDA_TRY(ctx, fathom_launch_dependent(
+        union_fetch_kernel<__nv_bfloat16>, grid, dim3(GU_THREADS), 0, st, static_cast<const __nv_bfloat16*>(Krows),
+        static_cast<const __nv_bfloat16*>(Vrows), (long long)L->n, (const int32_t*)ulist, (const int32_t*)union_count, capacity,
+        static_cast<__nv_bfloat16*>(K_stage), static_cast<__nv_bfloat16*>(V_stage), idx, k, G, Hq, (const uint32_t*)bitmap,
+        (const uint32_t*)word_rank, words, idx_local));
   else
-    union_fetch_kernel<float><<<grid, GU_THREADS, 0, st>>>(static_cast<const float*>(Krows), static_cast<const float*>(Vrows),
-                                                           L->n, ulist, union_count, capacity, static_cast<float*>(K_stage),
-                                                           static_cast<float*>(V_stage), idx, k, G, Hq, bitmap, word_rank,
-                                                           words, idx_local);
+    FATHOM_CUDA_TRY(ctx, fathom_launch_dependent(
+        union_fetch_kernel<float>, grid, dim3(GU_THREADS), 0, st, static_cast<const float*>(Krows), static_cast<const float*>(Vrows),
+        (long long)L->n, (const int32_t*)ulist, (const int32_t*)union_count, capacity, static_cast<float*>(K_stage),
+        static_cast<float*>(V_stage), idx, k, G, Hq, (const uint32_t*)bitmap, (const uint32_t*)word_rank, words, idx_local));
   FATHOM_CUDA_TRY(ctx, cudaGetLastError());
   return FATHOM_OK;
 }

@@ -34,3 +34,26 @@ def test_topk_of_rows_held_in_registers(n, k, n_sink, n_local, scores):
     assert np.array_equal(idx.cpu().numpy(), ref)
     assert ctx.fathom_device_status() == 0
     ctx.close()
+
+
+# the longest sequence whose bitmap fits in shared memory and one token more; an odd length with picks in its first and last word
+@pytest.mark.parametrize("n,k", [(33, 33), (70001, 700), (52 * 1024 * 32, 2048), (52 * 1024 * 32 + 1, 2048)])
+def test_union_of_picks_on_both_sides_of_the_bitmap_limit(n, k):
+    from paper_2609_17652_b200 import binding as fb
+    Hkv, G = 2, 4
+    r = np.random.default_rng(n)
+    idx = np.stack([np.sort(np.concatenate([[0, n - 1], 1 + r.choice(n - 2, k - 2, replace=False)])) for _ in range(Hkv * G)]).astype(np.int32)
+    lay = fb.make_layout(Hkv, Hkv * G, n)
+    ctx = fb.Context(0, fb.fathom_scratch_bytes(lay, k))
+    K = torch.randn(Hkv, n, 128, device="cuda").to(torch.bfloat16)
+    Ks, Vs = (torch.zeros(Hkv, G * k, 128, dtype=torch.bfloat16, device="cuda") for _ in range(2))
+    local = torch.full((Hkv * G, k), -1, dtype=torch.int32, device="cuda")
+    count = torch.zeros(Hkv, dtype=torch.int32, device="cuda")
+    ctx.fathom_gather_union(lay, torch.from_numpy(idx).cuda(), k, K, K, Ks, Vs, local, count)
+    for h in range(Hkv):
+        tokens = np.unique(idx[h * G:(h + 1) * G])
+        assert int(count[h]) == len(tokens)
+        assert np.array_equal(tokens[local[h * G:(h + 1) * G].cpu().numpy()], idx[h * G:(h + 1) * G])
+        rows = K[h][torch.from_numpy(tokens.astype(np.int64)).cuda()]
+        assert torch.equal(Ks[h, :len(tokens)], rows) and torch.equal(Vs[h, :len(tokens)], rows)
+    ctx.close()
