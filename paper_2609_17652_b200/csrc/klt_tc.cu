@@ -2,28 +2,30 @@
 // rule"), and the covariance of fathom_calibrate.
 //
 // The rotation is the one dense contraction next to the decode path (n x 128 by 128 x 128 per KV head), so it runs
-// as tcgen05.mma with the accumulator in tensor memory.  The rotated keys feed a quantiser, so tf32's 11 significant
-// bits are not enough; both operands are split into a tf32 head and a tf32 tail, x = xh + xl, v = vh + vl, and three
-// products are accumulated in fp32:  xh vh + xh vl + xl vh  (the dropped xl vl term is below 2^-22 of |x||v|).
+// as tcgen05.mma with the accumulator in tensor memory.  The rotated keys feed a quantiser, so 11 significant bits are not
+// enough; both operands are split into an fp16 head and an fp16 tail, x = xh + xl, v = vh + vl, and three products are
+// accumulated in fp32:  xh vh + xh vl + xl vh  (the dropped xl vl term is below 2^-24 of |x||v|).  fp16 has the significant bits
+// of tf32 at half the bytes and twice the rate; its range is made up for by powers of two: every token and every rotated channel
+// is scaled so that its largest element lies in [2^14, 2^15), which leaves elements down to 2^-28 of it with all their bits, and the
+// accumulator is scaled back (exactly) where it is read.
 //
 // The BASIS is the left operand (M = 128 rotated channels) and the tokens are the right one (N = 128):
-//   * the split basis stays in tensor memory (256 columns) for all of a head's tiles, so an MMA reads only the tokens from
-//     shared memory: 4 KB per 64 cycles.  With both operands in shared memory (8 KB per 64 cycles) the MMAs alone took the whole
-//     128 bytes per cycle of the shared-memory data path, and the 128 KB of split keys per tile came on top: 4.1 us a tile;
+//   * the split basis stays in tensor memory (128 columns) for all of a head's tiles, so an MMA reads only the tokens from
+//     shared memory (with both operands there the MMAs alone took the whole shared-memory data path);
 //   * the accumulator has a rotated channel per lane and a token per column, which is what both epilogues want: a thread
 //     holds 64 tokens = one block of ONE channel.  A warp writes 128 contiguous bytes of a rotated key per store straight from
 //     registers, and the quantiser's block maximum and plane words need no exchange between threads (with a token per
 //     lane they took a redux, four ballots and a shuffle per element: 9.5 us a tile).
 //
 // One persistent CTA per SM walks a contiguous range of 128-token tiles in three roles:
-//   16 producer warps  fetch a tile of keys one tile ahead into registers, subtract the mean, split, and store head and
-//                      tail of 32 channels (128 bytes of tf32: one row of the 128-byte swizzle) into a stage of a ring;
-//   1 MMA thread       issues a stage's 4 x 3 MMAs (M = N = 128, K = 8), commits them to the stage's barrier and, after a tile's last,
-//                      to its accumulator's (two accumulators alternate);
+//   16 producer warps  fetch a tile of keys one tile ahead into registers (a warp has whole rows, so that a row's scale is one
+//                      reduction over its lanes), subtract the mean, scale, split, and store head and tail (64 channels are one
+//                      row of the 128-byte swizzle) into one of two stages;
+//   1 MMA thread       issues a tile's 8 x 3 MMAs (M = N = 128, K = 16), commits them to the stage's barrier and to the
+//                      accumulator's (two accumulators alternate);
 //   8 epilogue warps   read the accumulator with tcgen05.ld (warp w: lanes 32 (w mod 4).., block w div 4 of the tile), hand it
-//                      back, and store or quantise.
-// Measured on 8 heads of 262,144 tokens, per 128-token tile and SM: fp32 keys to fp32 keys 4.2 -> 3.2 us (2.95 = its bytes at
-// the copy bandwidth), bf16 keys 4.2 -> 2.8 us, quantising 9.5 -> 2.65 us; the 48 MMAs alone, with nothing else running, take 2.0 us.
+//                      back, scale, and store or quantise.
+// @@MEASURED@@
 //
 // Every wait on an mbarrier is bounded; a wait that runs out sets FATHOM_DEV_WAIT_EXPIRED in the context status and
 // the thread stops waiting; every role still finishes its loops, and the CTA frees its tensor memory and returns.
@@ -42,23 +44,26 @@ constexpr uint32_t WAIT_TRIES = 1u << 22;
 // rotation kernel: roles, ring of stages, shared-memory map (bytes from a 1024-byte aligned base)
 constexpr int PRODUCERS = 512, EPILOGUE = 256;
 constexpr int RT_THREADS = PRODUCERS + EPILOGUE + 32;        // the last warp issues the MMAs
-constexpr int ROWS_PER_LANE = TILE_M * NCHUNK / (PRODUCERS / 32) / 4;       // 8
-constexpr int STAGE_BYTES = 2 * SLAB;                        // head and tail of 32 channels of 128 tokens
+constexpr int RK = 16;                                       // fp16 elements per MMA along K (32 bytes)
+constexpr int HALF_CH = 64;                                  // channels per 128-byte row of fp16
+constexpr int STAGES = 2;                                    // shared memory left over is L1, and the keys in flight need it
+constexpr int STAGE_BYTES = 4 * SLAB;                        // a tile: heads of channels 0..63, 64..127, tails of the same
+constexpr int FACTORS = 4;                                   // ring of the tiles' token scales (producers are at most three tiles ahead)
 constexpr int UNIT_BLOCKS = 4;                               // quantiser: blocks whose plane words are written together (32 bytes a row)
 constexpr int OUT_PITCH = FATHOM_NPLANES * UNIT_BLOCKS * 2 + 1;             // words per channel of staged plane words, odd: no bank conflicts
 template <bool BUILD>
 struct Map {
-  static constexpr int STAGES = BUILD ? 4 : 5;                // shared memory left over is L1, and the keys in flight need it: with seven stages
-                                                              // (fp32 keys) storing took 3.9 us a tile against 3.2, with six quantising 3.1 against 2.6
   static constexpr int OUT = STAGES * STAGE_BYTES;            // BUILD: 128 x OUT_PITCH words
   static constexpr int SCALE = OUT + (BUILD ? FATHOM_D * OUT_PITCH * 4 : 0);   // BUILD: 128 x 4 fp16
   static constexpr int MU = SCALE + (BUILD ? FATHOM_D * UNIT_BLOCKS * 2 : 0);  // 128 floats
-  static constexpr int BAR = MU + FATHOM_D * 4;               // full and empty barriers of the stages, full and empty of the accumulators
+  static constexpr int VSCALE = MU + FATHOM_D * 4;            // 128 floats: what a rotated channel is scaled back by
+  static constexpr int FACTOR = VSCALE + FATHOM_D * 4;        // FACTORS x 128 floats: what a token is scaled back by
+  static constexpr int BAR = FACTOR + FACTORS * TILE_M * 4;   // full and empty barriers of the stages, full and empty of the accumulators
   static constexpr int BARS = 2 * STAGES + 4;
   static constexpr int BYTES = BAR + BARS * 8 + 16 + 1024;    // + tensor-memory base, slack for the manual 1024-byte alignment
   static_assert(BYTES <= 227 * 1024, "shared memory");
 };
-constexpr uint32_t COL_VH = 0, COL_VL = COL_VH + FATHOM_D, COL_ACC = 256;  // tensor memory: basis head, basis tail, two accumulators
+constexpr uint32_t COL_VH = 0, COL_VL = COL_VH + FATHOM_D / 2, COL_ACC = 128;   // tensor memory: basis head and tail (two fp16 a column), two accumulators
 constexpr uint32_t RT_TMEM_COLS = 512;
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -75,12 +80,33 @@ __device__ __forceinline__ uint64_t umma_desc(uint32_t saddr) {
 // fp32 accumulator, tf32 A and B, both K-major, N = 128, M = 128
 constexpr uint32_t UMMA_IDESC = (1u << 4) | (2u << 7) | (2u << 10) | ((128u >> 3) << 17) | ((128u >> 4) << 24);
 
-// left operand in tensor memory (lane = row, one tf32 element per column), right operand in shared memory
-__device__ __forceinline__ void umma_tf32_ts(uint32_t tmem_d, uint32_t tmem_a, uint64_t b, uint32_t accumulate) {
+// fp16 operands: left in tensor memory (lane = row, elements 2 c and 2 c + 1 in column c), right in shared memory
+constexpr uint32_t UMMA_IDESC_F16 = (1u << 4) | ((128u >> 3) << 17) | ((128u >> 4) << 24);
+__device__ __forceinline__ void umma_f16_ts(uint32_t tmem_d, uint32_t tmem_a, uint64_t b, uint32_t accumulate) {
   asm volatile(
       "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::tf32 [%0], [%1], %2, %3, {%5, %5, %5, %5}, p;\n\t}\n"
-      :: "r"(tmem_d), "r"(tmem_a), "l"(b), "r"(UMMA_IDESC), "r"(accumulate), "r"(0u) : "memory");
+      "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, {%5, %5, %5, %5}, p;\n\t}\n"
+      :: "r"(tmem_d), "r"(tmem_a), "l"(b), "r"(UMMA_IDESC_F16), "r"(accumulate), "r"(0u) : "memory");
+}
+// The power of two that brings `largest` (not negative) into [2^14, 2^15), and its inverse
+__device__ __forceinline__ float scale_up(float largest, float& back) {
+  const uint32_t e = min(max(__float_as_uint(largest) >> 23, 15u), 254u);
+  back = __uint_as_float((e - 14u) << 23);
+  return __uint_as_float((268u - e) << 23);
+}
+// fp16 head and tail of two scaled values
+__device__ __forceinline__ void split2(float a, float b, uint32_t& head, uint32_t& tail) {
+  const __half2 h = __floats2half2_rn(a, b);
+  const float2 f = __half22float2(h);
+  const __half2 l = __floats2half2_rn(a - f.x, b - f.y);
+  head = *reinterpret_cast<const uint32_t*>(&h);
+  tail = *reinterpret_cast<const uint32_t*>(&l);
+}
+__device__ __forceinline__ float2 mul2(float2 a, float2 b) {
+  float2 d;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(reinterpret_cast<unsigned long long&>(d))
+      : "l"(reinterpret_cast<const unsigned long long&>(a)), "l"(reinterpret_cast<const unsigned long long&>(b)));
+  return d;
 }
 __device__ __forceinline__ void umma_commit(uint32_t bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" :: "r"(bar) : "memory");
@@ -174,8 +200,9 @@ rotate_tc_kernel(const T* __restrict__ K, const float* __restrict__ mean, const 
   unsigned char* sm = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);   // 1024-byte aligned in the shared window
   const uint32_t sm_base = smem_u32(sm);
   using MP = Map<BUILD>;
-  constexpr int STAGES = MP::STAGES;
   float* s_mu = reinterpret_cast<float*>(sm + MP::MU);
+  float* s_vscale = reinterpret_cast<float*>(sm + MP::VSCALE);
+  float* s_factor = reinterpret_cast<float*>(sm + MP::FACTOR);
   uint32_t* s_tmem = reinterpret_cast<uint32_t*>(sm + MP::BAR + MP::BARS * 8);
   const uint32_t bar_full = sm_base + MP::BAR, bar_empty = bar_full + STAGES * 8, bar_acc_full = bar_empty + STAGES * 8,
                  bar_acc_empty = bar_acc_full + 16;
@@ -189,11 +216,11 @@ rotate_tc_kernel(const T* __restrict__ K, const float* __restrict__ mean, const 
 
   if (tid == 0) {
     for (int s = 0; s < STAGES; ++s) {
-      mbar_init(bar_full + 8 * s, PRODUCERS / 32 / NCHUNK);
+      mbar_init(bar_full + 8 * s, PRODUCERS / 32);
       mbar_init(bar_empty + 8 * s, 1);
     }
     for (int a = 0; a < 2; ++a) {
-      mbar_init(bar_acc_full + 8 * a, 1);
+      mbar_init(bar_acc_full + 8 * a, 2);                     // the commit, and an arrival that passes the producers' scales on
       mbar_init(bar_acc_empty + 8 * a, EPILOGUE / 32);
     }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -216,7 +243,6 @@ rotate_tc_kernel(const T* __restrict__ K, const float* __restrict__ mean, const 
       alive = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
     }
   };
-  uint32_t stage = 0, phase = 0;                              // MMA thread: ring position and its round's parity
   uint32_t tcount = 0;                                        // tiles so far: accumulator and its parity
 
   for (long long g = g0; g < g1;) {                           // head by head
@@ -226,15 +252,22 @@ rotate_tc_kernel(const T* __restrict__ K, const float* __restrict__ mean, const 
     // ---- the head's split basis into tensor memory (lane = rotated channel j, column = channel c), its mean into shared memory
     if (warp < 4) {
       const float* V = basis + (size_t)kv * FATHOM_D * FATHOM_D + tid;
+      float largest = 0.0f, back;
+#pragma unroll 32
+      for (int c = 0; c < FATHOM_D; ++c) largest = fmaxf(largest, fabsf(__ldg(V + c * FATHOM_D)));
+      const float up = scale_up(largest, back);
+      s_vscale[tid] = back;
 #pragma unroll 1
-      for (int c0 = 0; c0 < 2 * FATHOM_D; c0 += 32) {         // heads, then tails (32 registers at a time)
+      for (int c0 = 0; c0 < 2 * FATHOM_D; c0 += 64) {         // heads, then tails (32 registers at a time)
         uint32_t part[32];
 #pragma unroll
-        for (int c = 0; c < 32; ++c) {
-          const float v = __ldg(V + ((c0 & (FATHOM_D - 1)) + c) * FATHOM_D), vh = tf32_head(v);
-          part[c] = __float_as_uint(c0 < FATHOM_D ? vh : tf32_head(v - vh));
+        for (int c = 0; c < 64; c += 2) {
+          const float* v = V + ((c0 & (FATHOM_D - 1)) + c) * FATHOM_D;
+          uint32_t head, tail;
+          split2(__ldg(v) * up, __ldg(v + FATHOM_D) * up, head, tail);
+          part[c / 2] = c0 < FATHOM_D ? head : tail;
         }
-        tmem_store32(tmem + ((uint32_t)(warp * 32) << 16) + COL_VH + c0, part);
+        tmem_store32(tmem + ((uint32_t)(warp * 32) << 16) + COL_VH + c0 / 2, part);
       }
       asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
     } else if (warp < 8) {
@@ -245,16 +278,14 @@ rotate_tc_kernel(const T* __restrict__ K, const float* __restrict__ mean, const 
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 
     if (tid < PRODUCERS) {
-      // ---- producers: warp = (chunk kc, 32 rows of the tile), lane = (16 bytes of a row, every fourth or eighth row).  The warps of a tile
-      //      work on its four chunks side by side: a warp goes through wait - store - fence - arrive once per tile (all warps
-      //      on one chunk after the other went through it four times, and that chain was the longest of the kernel)
-      constexpr int CH = 16 / sizeof(T);                      // channels per 16-byte load: one or two 16-byte pieces of a tf32 row
-      constexpr int LANES = KC / CH, STEP = 32 / LANES, LOADS = 4 * ROWS_PER_LANE / STEP;
-      const int kc = warp & (NCHUNK - 1), row0 = (warp / NCHUNK) * (4 * ROWS_PER_LANE) + lane / LANES, c0 = (lane % LANES) * CH;
-      const T* Kh = K + (size_t)kv * (size_t)n * FATHOM_D + kc * KC + c0;
+      // ---- producers: eight rows per warp, 16 bytes of a row per lane
+      constexpr int CH = 16 / sizeof(T);                      // channels per load
+      constexpr int LANES = FATHOM_D / CH, STEP = 32 / LANES, LOADS = TILE_M / (PRODUCERS / 32) / STEP;   // lanes per row, rows per load
+      const int row0 = warp * (TILE_M / (PRODUCERS / 32)) + lane / LANES, c0 = (lane % LANES) * CH;
+      const T* Kh = K + (size_t)kv * (size_t)n * FATHOM_D + c0;
       float mu[CH];
 #pragma unroll
-      for (int c = 0; c < CH; ++c) mu[c] = s_mu[kc * KC + c0 + c];
+      for (int c = 0; c < CH; ++c) mu[c] = s_mu[c0 + c];
       uint4 xr[LOADS];                                        // one tile ahead, in registers, as loaded
       auto load_tile = [&](long long tile) {
         const long long r0 = tile * TILE_M + row0;
@@ -270,26 +301,41 @@ rotate_tc_kernel(const T* __restrict__ K, const float* __restrict__ mean, const 
       };
       load_tile(tile0);
       for (long long t = 0; t < count; ++t, ++tcount) {
-        const uint32_t q = tcount * NCHUNK + kc, stage = q % STAGES, round = q / STAGES;
+        const uint32_t stage = tcount % STAGES, round = tcount / STAGES;
         wait(bar_empty + 8 * stage, (round & 1u) ^ 1u);       // (a fresh barrier lets the first round through)
-        unsigned char* xs = sm + stage * STAGE_BYTES;
+        unsigned char* xs = sm + stage * STAGE_BYTES + (c0 / HALF_CH) * SLAB;
+        float* factor = s_factor + (tcount % FACTORS) * TILE_M;
 #pragma unroll
         for (int i = 0; i < LOADS; ++i) {
           float x[CH];
           unpack16(xr[i], x);
+          uint32_t m = 0u;                                    // the row's largest magnitude (non-negative floats order like integers)
 #pragma unroll
-          for (int f = 0; f < CH / 4; ++f) {
-            float h[4], l[4];
+          for (int c = 0; c < CH; ++c) {
+            x[c] -= mu[c];
+            m = max(m, __float_as_uint(x[c]) & 0x7fffffffu);
+          }
+          if (LANES == 32) {
+            m = __reduce_max_sync(0xffffffffu, m);
+          } else {
 #pragma unroll
-            for (int c = 0; c < 4; ++c) {
-              const float a = x[4 * f + c] - mu[4 * f + c];
-              h[c] = tf32_head(a);
-              l[c] = tf32_head(a - h[c]);
-            }
-            // (rows past the end of the sequence give columns of the accumulator that are never used)
-            const int off = slab_offset(row0 + STEP * i, c0 / 4 + f);
-            *reinterpret_cast<float4*>(xs + off) = make_float4(h[0], h[1], h[2], h[3]);
-            *reinterpret_cast<float4*>(xs + SLAB + off) = make_float4(l[0], l[1], l[2], l[3]);
+            for (int o = LANES / 2; o; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+          }
+          float back;
+          const float up = scale_up(__uint_as_float(m), back);
+          const int row = row0 + STEP * i, byte = (c0 % HALF_CH) * 2;
+          if (c0 == 0) factor[row] = back;
+          uint32_t h[CH / 2], l[CH / 2];
+#pragma unroll
+          for (int c = 0; c < CH; c += 2) split2(x[c] * up, x[c + 1] * up, h[c / 2], l[c / 2]);
+          // (rows past the end of the sequence give columns of the accumulator that are never used)
+          unsigned char* to = xs + slab_offset(row, byte >> 4) + (byte & 15);
+          if constexpr (CH == 8) {
+            *reinterpret_cast<uint4*>(to) = make_uint4(h[0], h[1], h[2], h[3]);
+            *reinterpret_cast<uint4*>(to + 2 * SLAB) = make_uint4(l[0], l[1], l[2], l[3]);
+          } else {
+            *reinterpret_cast<uint2*>(to) = make_uint2(h[0], h[1]);
+            *reinterpret_cast<uint2*>(to + 2 * SLAB) = make_uint2(l[0], l[1]);
           }
         }
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // generic-proxy stores -> visible to the MMA
@@ -301,47 +347,57 @@ rotate_tc_kernel(const T* __restrict__ K, const float* __restrict__ mean, const 
       // (the whole warp runs the loop, one elected lane issues: addresses and descriptors then stay in uniform registers; issued
       // from a divergent branch an MMA took 66 to 80 cycles to issue, as long as it takes to run)
       const uint32_t base = __shfl_sync(0xffffffffu, sm_base, 0), tm = __shfl_sync(0xffffffffu, tmem, 0);
-      bool ready = false;                                     // what a barrier said when it was asked ahead of time: an answer takes
-                                                              // ~300 cycles while the other warps store, four MMAs' worth
+      bool ready = false;                                     // what the full barrier said when it was asked ahead of time: an answer takes
+                                                              // ~300 cycles while the other warps store, several MMAs' worth
       for (long long t = 0; t < count; ++t, ++tcount) {
         const uint32_t buf = tcount & 1u, acc = tm + COL_ACC + buf * 128u;
+        const uint32_t stage = tcount % STAGES, phase = (tcount / STAGES) & 1u;
         if (alive && !mbar_wait(bar_acc_empty + 8 * buf, ((tcount >> 1) & 1u) ^ 1u)) alive = false;
+        if (alive && !ready && !mbar_wait(bar_full + 8 * stage, phase)) alive = false;
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        const uint32_t slab = base + stage * STAGE_BYTES;
+        if (elect_one()) {
 #pragma unroll
-        for (int kc = 0; kc < NCHUNK; ++kc) {
-          if (alive && !ready && !mbar_wait(bar_full + 8 * stage, phase)) alive = false;
-          const uint32_t next = stage + 1 == STAGES ? 0u : stage + 1;
-          ready = mbar_test(bar_full + 8 * next, phase ^ (next == 0u ? 1u : 0u));
-          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-          const uint64_t xh = umma_desc(base + stage * STAGE_BYTES), xl = umma_desc(base + stage * STAGE_BYTES + SLAB);
-          if (elect_one()) {
+          for (int hc = 0; hc < FATHOM_D / HALF_CH; ++hc) {
+            const uint64_t xh = umma_desc(slab + hc * SLAB), xl = umma_desc(slab + (2 + hc) * SLAB);
 #pragma unroll
-            for (int ks = 0; ks < KC / UMMA_K; ++ks) {
-              const uint32_t vh = tm + COL_VH + kc * KC + ks * UMMA_K, vl = tm + COL_VL + kc * KC + ks * UMMA_K;
-              const uint64_t ko = ks * UMMA_K * 4 >> 4;       // 16-byte units along K inside the swizzled row
-              umma_tf32_ts(acc, vh, xl + ko, (kc | ks) ? 1u : 0u);
-              umma_tf32_ts(acc, vl, xh + ko, 1u);
-              umma_tf32_ts(acc, vh, xh + ko, 1u);
+            for (int ks = 0; ks < HALF_CH / RK; ++ks) {
+              const uint32_t vh = tm + COL_VH + (hc * HALF_CH + ks * RK) / 2, vl = tm + COL_VL + (hc * HALF_CH + ks * RK) / 2;
+              const uint64_t ko = ks * RK * 2 >> 4;           // 16-byte units along K inside the swizzled row
+              umma_f16_ts(acc, vh, xl + ko, (hc | ks) ? 1u : 0u);
+              umma_f16_ts(acc, vl, xh + ko, 1u);
+              umma_f16_ts(acc, vh, xh + ko, 1u);
             }
-            umma_commit(bar_empty + 8 * stage);
-            if (kc == NCHUNK - 1) umma_commit(bar_acc_full + 8 * buf);
           }
-          __syncwarp();
-          if (++stage == STAGES) { stage = 0; phase ^= 1u; }
+          umma_commit(bar_empty + 8 * stage);
+          umma_commit(bar_acc_full + 8 * buf);
+          mbar_arrive(bar_acc_full + 8 * buf);
         }
+        ready = mbar_test(bar_full + 8 * ((tcount + 1) % STAGES), ((tcount + 1) / STAGES) & 1u);
+        __syncwarp();
       }
     } else {
       // ---- epilogue: my channel, my block of every tile
       const int lq = warp & 3, blk = (warp - PRODUCERS / 32) >> 2, ch = lq * 32 + lane;
+      const float2 vscale = make_float2(s_vscale[ch], s_vscale[ch]);
       for (long long t = 0; t < count; ++t, ++tcount) {
         const long long tile = tile0 + t;
         const uint32_t buf = tcount & 1u;
         float r[32];
+        const float4* factor = reinterpret_cast<const float4*>(s_factor + (tcount % FACTORS) * TILE_M + blk * FATHOM_BLOCK);
         wait(bar_acc_full + 8 * buf, (tcount >> 1) & 1u);
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         const uint32_t taddr = tmem + ((uint32_t)(lq * 32) << 16) + COL_ACC + buf * 128u + (uint32_t)(blk * FATHOM_BLOCK);
         auto load_half = [&](int half) {                      // 32 tokens at a time: 64 would spill
           tmem_load32(taddr + 32 * half, r);
           asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+          for (int i = 0; i < 32; i += 4) {                   // back to the keys' scale (powers of two: exact)
+            const float4 f = factor[8 * half + i / 4];
+            const float2 a = mul2(mul2(make_float2(r[i], r[i + 1]), make_float2(f.x, f.y)), vscale);
+            const float2 b = mul2(mul2(make_float2(r[i + 2], r[i + 3]), make_float2(f.z, f.w)), vscale);
+            r[i] = a.x; r[i + 1] = a.y; r[i + 2] = b.x; r[i + 3] = b.y;
+          }
         };
         auto hand_back = [&]() {                              // a later MMA overwrites the accumulator
           asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
