@@ -51,11 +51,12 @@ constexpr int STAGE_BYTES = 4 * SLAB;                        // a tile: heads of
 constexpr int FACTORS = 4;                                   // ring of the tiles' token scales (producers are at most three tiles ahead)
 constexpr int UNIT_BLOCKS = 4;                               // quantiser: blocks whose plane words are written together (32 bytes a row)
 constexpr int OUT_PITCH = FATHOM_NPLANES * UNIT_BLOCKS * 2 + 1;             // words per channel of staged plane words, odd: no bank conflicts
+constexpr int OUT_BYTES = FATHOM_D * OUT_PITCH * 4;
 template <bool BUILD>
 struct Map {
-  static constexpr int OUT = STAGES * STAGE_BYTES;            // BUILD: 128 x OUT_PITCH words
-  static constexpr int SCALE = OUT + (BUILD ? FATHOM_D * OUT_PITCH * 4 : 0);   // BUILD: 128 x 4 fp16
-  static constexpr int MU = SCALE + (BUILD ? FATHOM_D * UNIT_BLOCKS * 2 : 0);  // 128 floats
+  static constexpr int OUT = STAGES * STAGE_BYTES;            // BUILD: 2 x 128 x OUT_PITCH words (double buffer)
+  static constexpr int SCALE = OUT + (BUILD ? 2 * OUT_BYTES : 0);              // BUILD: 2 x 128 x 4 fp16
+  static constexpr int MU = SCALE + (BUILD ? 2 * FATHOM_D * UNIT_BLOCKS * 2 : 0);   // 128 floats
   static constexpr int VSCALE = MU + FATHOM_D * 4;            // 128 floats: what a rotated channel is scaled back by
   static constexpr int FACTOR = VSCALE + FATHOM_D * 4;        // FACTORS x 128 floats: what a token is scaled back by
   static constexpr int BAR = FACTOR + FACTORS * TILE_M * 4;   // full and empty barriers of the stages, full and empty of the accumulators
@@ -379,7 +380,7 @@ rotate_tc_kernel(const T* __restrict__ K, const float* __restrict__ mean, const 
     } else {
       // ---- epilogue: my channel, my block of every tile
       const int lq = warp & 3, blk = (warp - PRODUCERS / 32) >> 2, ch = lq * 32 + lane;
-      const float2 vscale = make_float2(s_vscale[ch], s_vscale[ch]);
+      const float vscale = s_vscale[ch];
       for (long long t = 0; t < count; ++t, ++tcount) {
         const long long tile = tile0 + t;
         const uint32_t buf = tcount & 1u;
@@ -392,10 +393,10 @@ rotate_tc_kernel(const T* __restrict__ K, const float* __restrict__ mean, const 
           tmem_load32(taddr + 32 * half, r);
           asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
-          for (int i = 0; i < 32; i += 4) {                   // back to the keys' scale (powers of two: exact)
+          for (int i = 0; i < 32; i += 4) {                   // the token's scale taken back (powers of two: exact); the channel's is left
             const float4 f = factor[8 * half + i / 4];
-            const float2 a = mul2(mul2(make_float2(r[i], r[i + 1]), make_float2(f.x, f.y)), vscale);
-            const float2 b = mul2(mul2(make_float2(r[i + 2], r[i + 3]), make_float2(f.z, f.w)), vscale);
+            const float2 a = mul2(make_float2(r[i], r[i + 1]), make_float2(f.x, f.y));
+            const float2 b = mul2(make_float2(r[i + 2], r[i + 3]), make_float2(f.z, f.w));
             r[i] = a.x; r[i + 1] = a.y; r[i + 2] = b.x; r[i + 3] = b.y;
           }
         };
@@ -414,11 +415,11 @@ rotate_tc_kernel(const T* __restrict__ K, const float* __restrict__ mean, const 
             if (half == 1) hand_back();
             if (valid == FATHOM_BLOCK) {
 #pragma unroll
-              for (int i = 0; i < 32; ++i) out[(32 * half + i) * FATHOM_D] = r[i];
+              for (int i = 0; i < 32; ++i) out[(32 * half + i) * FATHOM_D] = r[i] * vscale;
             } else {
 #pragma unroll
               for (int i = 0; i < 32; ++i)
-                if (32 * half + i < valid) out[(32 * half + i) * FATHOM_D] = r[i];
+                if (32 * half + i < valid) out[(32 * half + i) * FATHOM_D] = r[i] * vscale;
             }
           }
         } else {
@@ -437,10 +438,11 @@ rotate_tc_kernel(const T* __restrict__ K, const float* __restrict__ mean, const 
           largest(1);
           load_half(0);
           largest(0);
-          const __half sh = __float2half_rn(a * 0.125f);      // a/8 is exact; one rounding to fp16
-          const float sc = __half2float(sh), inv = 1.0f / sc;
-          const int bu = (int)(tile % UNIT) * (TILE_M / FATHOM_BLOCK) + blk;
-          uint32_t* o = reinterpret_cast<uint32_t*>(sm + MP::OUT) + ch * OUT_PITCH + bu * 2;
+          const __half sh = __float2half_rn(a * vscale * 0.125f);   // (exact but for the one rounding to fp16)
+          // the quantiser compares multiples of the stored scale with the values, so it may have both without the channel's scale
+          const float sc = __half2float(sh) / vscale, inv = 1.0f / sc;
+          const int ubuf = (int)((tcount / UNIT) & 1u), bu = (int)(tile % UNIT) * (TILE_M / FATHOM_BLOCK) + blk;
+          uint32_t* o = reinterpret_cast<uint32_t*>(sm + MP::OUT + ubuf * OUT_BYTES) + ch * OUT_PITCH + bu * 2;
 #pragma unroll
           for (int half = 0; half < 2; ++half) {
             if (half == 1) {
@@ -455,17 +457,23 @@ rotate_tc_kernel(const T* __restrict__ K, const float* __restrict__ mean, const 
 #pragma unroll
             for (int p = 0; p < FATHOM_NPLANES; ++p) o[p * UNIT_BLOCKS * 2 + half] = w[p] & keep;
           }
-          reinterpret_cast<uint16_t*>(sm + MP::SCALE)[ch * UNIT_BLOCKS + bu] = __half_as_ushort(sh);
+          reinterpret_cast<uint16_t*>(sm + MP::SCALE)[(ubuf * FATHOM_D + ch) * UNIT_BLOCKS + bu] = __half_as_ushort(sh);
           if ((tile + 1) % UNIT == 0) {
-            // ---- flush: the unit's four blocks of every (channel, plane) row are 32 contiguous bytes
+            // ---- flush: the unit's four blocks of every (channel, plane) row are 32 contiguous bytes.  (The other buffer
+            //      takes the next unit; a warp that is a unit ahead waits here before it can come back to this one)
             epilogue_barrier();
             const int et = tid - PRODUCERS;
             const long long nb = (n + FATHOM_BLOCK - 1) / FATHOM_BLOCK, b0 = tile / UNIT * UNIT_BLOCKS;
             const int nblk = (int)min((long long)UNIT_BLOCKS, nb - b0);
-            const uint32_t* staged = reinterpret_cast<const uint32_t*>(sm + MP::OUT);
+            const uint32_t* staged = reinterpret_cast<const uint32_t*>(sm + MP::OUT + ubuf * OUT_BYTES);
             for (int e = et; e < FATHOM_D * FATHOM_NPLANES; e += EPILOGUE) {
               const uint32_t* src = staged + (e >> 2) * OUT_PITCH + (e & 3) * UNIT_BLOCKS * 2;
               uint64_t* dst = planes + ((size_t)kv * FATHOM_D * FATHOM_NPLANES + e) * (size_t)plane_stride + b0;
+              if (nblk == UNIT_BLOCKS && (reinterpret_cast<uintptr_t>(dst) & 31u) == 0) {   // a whole sector
+                asm volatile("st.global.v8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"l"(dst), "r"(src[0]), "r"(src[1]), "r"(src[2]), "r"(src[3]),
+                             "r"(src[4]), "r"(src[5]), "r"(src[6]), "r"(src[7]) : "memory");
+                continue;
+              }
 #pragma unroll
               for (int pair = 0; pair < UNIT_BLOCKS / 2; ++pair) {
                 if (2 * pair + 1 < nblk) {
@@ -476,7 +484,7 @@ rotate_tc_kernel(const T* __restrict__ K, const float* __restrict__ mean, const 
               }
             }
             if (et < FATHOM_D) {
-              const uint16_t* src = reinterpret_cast<const uint16_t*>(sm + MP::SCALE) + et * UNIT_BLOCKS;
+              const uint16_t* src = reinterpret_cast<const uint16_t*>(sm + MP::SCALE) + (ubuf * FATHOM_D + et) * UNIT_BLOCKS;
               uint16_t* dst = scales + ((size_t)kv * FATHOM_D + et) * (size_t)scale_stride + b0;
               if (nblk == UNIT_BLOCKS) {
                 *reinterpret_cast<uint2*>(dst) = *reinterpret_cast<const uint2*>(src);
@@ -484,7 +492,6 @@ rotate_tc_kernel(const T* __restrict__ K, const float* __restrict__ mean, const 
                 for (int x = 0; x < nblk; ++x) dst[x] = src[x];
               }
             }
-            epilogue_barrier();                               // the staging is rewritten by the next unit
           }
         }
       }
