@@ -6,9 +6,17 @@
 // publishes its (max, denominator, weighted sum) triple and takes a ticket; the CTA that draws the last
 // ticket of a head merges all triples in split order, so the output is bit-reproducible whichever CTA
 // that is, and no second launch is needed.
+//
+// Few rows (k <= 1024) are a chain of latencies, not bytes, and take a kernel of their own: a cluster of up to eight CTAs per head,
+// each lane requests its share of 4 or 8 K rows AND of their V rows as soon as the indices are here, and the CTAs' triples meet
+// in the first one's shared memory instead of in global memory behind a fence, a ticket and a second fence.
+// Decode steps with it: 4096 tokens, k = 64, one head 19.3 -> 15.9 us; 33,001 tokens, k = 512, 32 heads 32.3 -> 28.5 us.
 #include "fathom_common.cuh"
 
+#include <cooperative_groups.h>
 #include <mutex>
+
+namespace cg = cooperative_groups;
 
 namespace {
 
@@ -151,6 +159,145 @@ attend_partial_kernel(const float* __restrict__ q, const T* __restrict__ Krows, 
   result[(size_t)head * FATHOM_D + tid] = num / den;
 }
 
+// ---- few rows: one cluster per head, gridDim.x CTAs of 16 half-warps x ROWS rows
+constexpr int FEW_THREADS = 256, FEW_HW = FEW_THREADS / 16, FEW_CLUSTER = 8;
+template <typename T, int ROWS>
+__global__ void __launch_bounds__(FEW_THREADS)
+attend_few_kernel(const float* __restrict__ q, const T* __restrict__ Krows, const T* __restrict__ Vrows, const int32_t* __restrict__ idx, int k,
+                  long long n, int G, float softmax_scale, float* __restrict__ result) {
+  __shared__ float s_max[FEW_HW], s_sum[FEW_HW];
+  __shared__ __align__(16) float s_acc[FEW_HW][FATHOM_D];     // one partial sum per half-warp
+  __shared__ float s_num[FEW_CLUSTER][FATHOM_D], s_m[FEW_CLUSTER], s_den[FEW_CLUSTER];   // first CTA: the cluster's triples
+  cg::cluster_group cluster = cg::this_cluster();
+  const int rank = blockIdx.x, ctas = gridDim.x, head = blockIdx.y, tid = threadIdx.x, hw = tid >> 4, l16 = tid & 15;
+  auto started = cluster.barrier_arrive();                    // (its shared memory may be written once everyone has started)
+  FATHOM_PDL_WAIT();                                          // the indices come from the previous kernel
+  FATHOM_PDL_RELEASE();
+  const size_t rows0 = (size_t)(head / G) * (size_t)n;
+  const int pos = (rank * FEW_HW + hw) * ROWS;                // first of the half-warp's positions
+  int32_t mine = 0;
+  if (l16 < ROWS && pos + l16 < k) {
+    mine = __ldg(idx + (size_t)head * k + pos + l16);
+    mine = (mine < 0) ? 0 : ((long long)mine >= n ? (int32_t)(n - 1) : mine);   // out-of-range indices are clamped, never dereferenced
+  }
+  const float4* qp = reinterpret_cast<const float4*>(q + (size_t)head * FATHOM_D + l16 * 8);
+  float qv[8];
+  if ((reinterpret_cast<uintptr_t>(q) & 15u) == 0) {
+    const float4 a = __ldg(qp), b = __ldg(qp + 1);
+    qv[0] = a.x; qv[1] = a.y; qv[2] = a.z; qv[3] = a.w; qv[4] = b.x; qv[5] = b.y; qv[6] = b.z; qv[7] = b.w;
+  } else {
+#pragma unroll
+    for (int c = 0; c < 8; ++c) qv[c] = __ldg(q + (size_t)head * FATHOM_D + l16 * 8 + c);
+  }
+  using Raw = typename RawOf<T>::type;
+  Raw kr[ROWS], vr[ROWS];
+  size_t at[ROWS];
+#pragma unroll
+  for (int u = 0; u < ROWS; ++u) at[u] = (rows0 + (size_t)__shfl_sync(0xffffffffu, mine, u, 16)) * FATHOM_D + l16 * 8;
+#pragma unroll
+  for (int u = 0; u < ROWS; ++u) {                            // (positions past k: nothing is loaded)
+    kr[u] = Raw{};
+    if (pos + u < k) kr[u] = load_raw(Krows + at[u]);
+  }
+#pragma unroll
+  for (int u = 0; u < ROWS; ++u) {
+    vr[u] = Raw{};
+    if (pos + u < k) vr[u] = load_raw(Vrows + at[u]);
+  }
+  float e[ROWS], m = -INFINITY;
+#pragma unroll
+  for (int u = 0; u < ROWS; ++u) {
+    float x[8], part = 0.0f;
+    unpack(kr[u], x);
+#pragma unroll
+    for (int c = 0; c < 8; ++c) part = fmaf(x[c], qv[c], part);
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);   // every lane has the sum
+    e[u] = pos + u < k ? part * softmax_scale : -INFINITY;
+    m = fmaxf(m, e[u]);
+  }
+  if (l16 == 0) s_max[hw] = m;
+  __syncthreads();
+  m = -INFINITY;
+#pragma unroll
+  for (int h = 0; h < FEW_HW; ++h) m = fmaxf(m, s_max[h]);    // of the CTA (it has at least one row)
+  float l = 0.0f, acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+  for (int u = 0; u < ROWS; ++u) {
+    const float p = pos + u < k ? expf(e[u] - m) : 0.0f;
+    float x[8];
+    unpack(vr[u], x);
+    l += p;
+#pragma unroll
+    for (int c = 0; c < 8; ++c) acc[c] = fmaf(p, x[c], acc[c]);
+  }
+  float4* to = reinterpret_cast<float4*>(&s_acc[hw][l16 * 8]);
+  to[0] = make_float4(acc[0], acc[1], acc[2], acc[3]);
+  to[1] = make_float4(acc[4], acc[5], acc[6], acc[7]);
+  if (l16 == 0) s_sum[hw] = l;
+  __syncthreads();
+  float num = 0.0f, den = 0.0f;
+  if (tid < FATHOM_D) {
+#pragma unroll
+    for (int h = 0; h < FEW_HW; ++h) { num += s_acc[h][tid]; den += s_sum[h]; }
+  }
+  cluster.barrier_wait(std::move(started));
+  if (ctas == 1) {
+    if (tid < FATHOM_D) result[(size_t)head * FATHOM_D + tid] = num / den;
+    return;
+  }
+  if (tid < FATHOM_D) {
+    cluster.map_shared_rank(&s_num[0][0], 0)[rank * FATHOM_D + tid] = num;
+    if (tid == 0) {
+      cluster.map_shared_rank(s_m, 0)[rank] = m;
+      cluster.map_shared_rank(s_den, 0)[rank] = den;
+    }
+  }
+  cluster.sync();
+  if (rank != 0 || tid >= FATHOM_D) return;
+  m = s_m[0];
+  for (int c = 1; c < ctas; ++c) m = fmaxf(m, s_m[c]);
+  num = den = 0.0f;
+  for (int c = 0; c < ctas; ++c) {                            // in rank order
+    const float w = expf(s_m[c] - m);
+    den = fmaf(w, s_den[c], den);
+    num = fmaf(w, s_num[c][tid], num);
+  }
+  result[(size_t)head * FATHOM_D + tid] = num / den;
+}
+
+template <typename T, int ROWS>
+cudaError_t launch_few(const float* q, const void* K, const void* V, const int32_t* idx, int k, long long n, int Hq, int G, float scale, float* out,
+                       cudaStream_t st) {
+  cudaLaunchConfig_t cfg = {};
+  const unsigned ctas = (unsigned)((k + FEW_HW * ROWS - 1) / (FEW_HW * ROWS));
+  cfg.gridDim = dim3(ctas, (unsigned)Hq);
+  cfg.blockDim = dim3(FEW_THREADS);
+  cfg.stream = st;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = ctas;
+  attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 2;
+  return cudaLaunchKernelEx(&cfg, attend_few_kernel<T, ROWS>, q, static_cast<const T*>(K), static_cast<const T*>(V), idx, k, n, G, scale, out);
+}
+
+// The kernel for k rows, the same for both entry points.  Beyond 1024 rows the gather is bound by memory, which the CTAs of 128 rows
+// fill better than clusters do.
+constexpr int FEW_ROWS = FEW_CLUSTER * FEW_HW * 8;
+template <typename T>
+cudaError_t launch_attend(const float* q, const void* K, const void* V, const int32_t* idx, int k, long long n, int Hq, int G, float scale,
+                          float* partial, int splits, unsigned int* tickets, float* out, cudaStream_t st) {
+  if (k <= FEW_ROWS / 2) return launch_few<T, 4>(q, K, V, idx, k, n, Hq, G, scale, out, st);
+  if (k <= FEW_ROWS) return launch_few<T, 8>(q, K, V, idx, k, n, Hq, G, scale, out, st);
+  // (launched so that its CTAs may become resident while the selection kernel still runs)
+  return fathom_launch_dependent(attend_partial_kernel<T>, dim3((unsigned)splits, (unsigned)Hq), dim3(AT_THREADS), 0, st, q, static_cast<const T*>(K),
+                                 static_cast<const T*>(V), idx, k, n, G, scale, partial, splits, tickets, out);
+}
+
 }  // namespace
 
 extern "C" int fathom_sparse_attend(fathom_ctx* ctx, const fathom_layout* L, const float* q, const void* Krows,
@@ -168,17 +315,8 @@ extern "C" int fathom_sparse_attend(fathom_ctx* ctx, const fathom_layout* L, con
   if (S.bytes > ctx->scratch_bytes) return FATHOM_ERR_SCRATCH_TOO_SMALL;
   unsigned int* tickets = ctx->dev_status + FATHOM_CTL_TICKETS;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  dim3 grid((unsigned)S.splits, (unsigned)Hq);
-  // launched so that its CTAs may become resident while the selection kernel (one CTA per head) still runs
-  if (row_dtype == FATHOM_BF16)
-    FATHOM_CUDA_TRY(ctx, fathom_launch_dependent(attend_partial_kernel<__nv_bfloat16>, grid, dim3(AT_THREADS), 0, st, q,
-                                                 static_cast<const __nv_bfloat16*>(Krows), static_cast<const __nv_bfloat16*>(Vrows), idx, k,
-                                                 (long long)L->n, G, softmax_scale, S.partial, S.splits, tickets, out));
-  else
-    FATHOM_CUDA_TRY(ctx, fathom_launch_dependent(attend_partial_kernel<float>, grid, dim3(AT_THREADS), 0, st, q,
-                                                 static_cast<const float*>(Krows), static_cast<const float*>(Vrows), idx, k,
-                                                 (long long)L->n, G, softmax_scale, S.partial, S.splits, tickets, out));
-  FATHOM_CUDA_TRY(ctx, cudaGetLastError());
+  FATHOM_CUDA_TRY(ctx, (row_dtype == FATHOM_BF16 ? launch_attend<__nv_bfloat16> : launch_attend<float>)(
+      q, Krows, Vrows, idx, k, (long long)L->n, Hq, G, softmax_scale, S.partial, S.splits, tickets, out, st));
   return FATHOM_OK;
 }
 
@@ -232,15 +370,8 @@ extern "C" int fathom_sparse_attend_static(const fathom_layout* L, const float* 
   }
 
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  dim3 grid((unsigned)splits, (unsigned)Hq);
-  if (row_dtype == FATHOM_BF16)
-    attend_partial_kernel<__nv_bfloat16><<<grid, AT_THREADS, 0, st>>>(
-        q, static_cast<const __nv_bfloat16*>(Krows), static_cast<const __nv_bfloat16*>(Vrows), idx, k, L->n, G,
-        softmax_scale, partial, splits, tickets, out);
-  else
-    attend_partial_kernel<float><<<grid, AT_THREADS, 0, st>>>(q, static_cast<const float*>(Krows),
-                                                              static_cast<const float*>(Vrows), idx, k, L->n, G,
-                                                              softmax_scale, partial, splits, tickets, out);
-  if (cudaGetLastError() != cudaSuccess) return FATHOM_ERR_CUDA;
+  if ((row_dtype == FATHOM_BF16 ? launch_attend<__nv_bfloat16> : launch_attend<float>)(
+          q, Krows, Vrows, idx, k, (long long)L->n, Hq, G, softmax_scale, partial, splits, tickets, out, st) != cudaSuccess)
+    return FATHOM_ERR_CUDA;
   return FATHOM_OK;
 }

@@ -57,3 +57,23 @@ def test_union_of_picks_on_both_sides_of_the_bitmap_limit(n, k):
         rows = K[h][torch.from_numpy(tokens.astype(np.int64)).cuda()]
         assert torch.equal(Ks[h, :len(tokens)], rows) and torch.equal(Vs[h, :len(tokens)], rows)
     ctx.close()
+
+
+# one CTA and clusters of 2 and 8; 4 and 8 rows per half-warp; full and ragged last CTAs; the last k of the small kernel and one more
+@pytest.mark.parametrize("k", [1, 3, 64, 65, 511, 512, 513, 1023, 1024, 1025])
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+def test_attention_over_few_rows(k, dtype):
+    from paper_2609_17652_b200 import binding as fb
+    n, Hkv, Hq = 3001, 2, 6
+    lay = fb.make_layout(Hkv, Hq, n)
+    ctx = fb.Context(0, fb.fathom_scratch_bytes(lay, k))
+    g = torch.Generator(device="cuda").manual_seed(k)
+    q = 2.0 * torch.randn(Hq, 128, generator=g, device="cuda")
+    K, V = (torch.randn(Hkv, n, 128, generator=g, device="cuda").to(dtype) for _ in range(2))
+    idx = torch.stack([torch.randperm(n, generator=g, device="cuda")[:k].sort().values for _ in range(Hq)]).to(torch.int32)
+    out = torch.full((Hq, 128), float("nan"), device="cuda")
+    ctx.fathom_sparse_attend(lay, q, K, V, idx, k, 1.0 / np.sqrt(128), out)
+    ref = O.sparse_attend(q.cpu().numpy(), K.float().cpu().numpy(), V.float().cpu().numpy(), idx.cpu().numpy(), 1.0 / np.sqrt(128))
+    # logits below 12 in magnitude, each an fp32 sum of 128 products: their rounding, exponentiated, stays below 1e-5
+    assert np.all(np.linalg.norm(out.cpu().numpy() - ref, axis=1) <= 2e-5 * np.linalg.norm(ref, axis=1))
+    ctx.close()
