@@ -18,14 +18,20 @@
 //     lane they took a redux, four ballots and a shuffle per element: 9.5 us a tile).
 //
 // One persistent CTA per SM walks a contiguous range of 128-token tiles in three roles:
-//   16 producer warps  fetch a tile of keys one tile ahead into registers (a warp has whole rows, so that a row's scale is one
-//                      reduction over its lanes), subtract the mean, scale, split, and store head and tail (64 channels are one
-//                      row of the 128-byte swizzle) into one of two stages;
+//   16 producer warps  own eight rows of every tile each: one bulk copy brings them into the stage two tiles ahead, and where
+//                      they lie the warp subtracts the mean, scales (a row's scale is one reduction over its lanes), splits and
+//                      writes head and tail back (64 channels are one row of the 128-byte swizzle): fp32 keys take exactly
+//                      the bytes of their head and tail, so a stage is one buffer for both, and three stages fit.  With the keys
+//                      in flight in registers a warp either waited for memory or converted: 3.6 us a tile, the sum of the two;
 //   1 MMA thread       issues a tile's 8 x 3 MMAs (M = N = 128, K = 16), commits them to the stage's barrier and to the
 //                      accumulator's (two accumulators alternate);
 //   8 epilogue warps   read the accumulator with tcgen05.ld (warp w: lanes 32 (w mod 4).., block w div 4 of the tile), hand it
 //                      back, scale, and store or quantise.
-// @@MEASURED@@
+// Measured: 262,144 fp32 tokens x 8 heads to planes 1057 us (both operands in shared memory, tf32) -> 386 us = 2.8 TB/s; 200,001 bf16
+// tokens to rotated keys 290 us = 4.2 TB/s.  Stamps inside the kernel (fp32 to planes, ~5000 cycles a tile): a tile's MMAs take 2300
+// cycles, its conversion 2100 while the epilogue rests and up to 4000 beside it, its epilogue 4900 (2500 of them the
+// quantiser): the roles share the ALU's issue slots, and eight epilogue warps set the pace.  Tried: 8 producer and 16 epilogue warps, a block on
+// two threads, the accumulator handed back before the quantiser runs: the producers set the pace instead (411 us).
 //
 // Every wait on an mbarrier is bounded; a wait that runs out sets FATHOM_DEV_WAIT_EXPIRED in the context status and
 // the thread stops waiting; every role still finishes its loops, and the CTA frees its tensor memory and returns.
@@ -46,21 +52,24 @@ constexpr int PRODUCERS = 512, EPILOGUE = 256;
 constexpr int RT_THREADS = PRODUCERS + EPILOGUE + 32;        // the last warp issues the MMAs
 constexpr int RK = 16;                                       // fp16 elements per MMA along K (32 bytes)
 constexpr int HALF_CH = 64;                                  // channels per 128-byte row of fp16
-constexpr int STAGES = 2;                                    // shared memory left over is L1, and the keys in flight need it
-constexpr int STAGE_BYTES = 4 * SLAB;                        // a tile: heads of channels 0..63, 64..127, tails of the same
-constexpr int FACTORS = 4;                                   // ring of the tiles' token scales (producers are at most three tiles ahead)
+constexpr int STAGES = 3;                                    // one arrives, one is converted, one is multiplied
+constexpr int STAGE_BYTES = 4 * SLAB;                        // a tile: per group of eight rows, heads of channels 0..63, 64..127, tails of the same
+constexpr int GROUP = 8, GROUPS = TILE_M / GROUP;            // rows that a producer warp owns; 1 KB per group and quarter
+constexpr int GROUP_BYTES = 4 * 1024;
+static_assert(GROUPS == PRODUCERS / 32 && GROUPS * GROUP_BYTES == STAGE_BYTES, "a producer warp per group");
+constexpr int FACTORS = 8;                                   // ring of the tiles' token scales (producers are at most four tiles ahead)
 constexpr int UNIT_BLOCKS = 4;                               // quantiser: blocks whose plane words are written together (32 bytes a row)
 constexpr int OUT_PITCH = FATHOM_NPLANES * UNIT_BLOCKS * 2 + 1;             // words per channel of staged plane words, odd: no bank conflicts
 constexpr int OUT_BYTES = FATHOM_D * OUT_PITCH * 4;
 template <bool BUILD>
 struct Map {
-  static constexpr int OUT = STAGES * STAGE_BYTES;            // BUILD: 2 x 128 x OUT_PITCH words (double buffer)
-  static constexpr int SCALE = OUT + (BUILD ? 2 * OUT_BYTES : 0);              // BUILD: 2 x 128 x 4 fp16
-  static constexpr int MU = SCALE + (BUILD ? 2 * FATHOM_D * UNIT_BLOCKS * 2 : 0);   // 128 floats
+  static constexpr int OUT = STAGES * STAGE_BYTES;            // BUILD: 128 x OUT_PITCH words
+  static constexpr int SCALE = OUT + (BUILD ? OUT_BYTES : 0); // BUILD: 128 x 4 fp16
+  static constexpr int MU = SCALE + (BUILD ? FATHOM_D * UNIT_BLOCKS * 2 : 0);   // 128 floats
   static constexpr int VSCALE = MU + FATHOM_D * 4;            // 128 floats: what a rotated channel is scaled back by
   static constexpr int FACTOR = VSCALE + FATHOM_D * 4;        // FACTORS x 128 floats: what a token is scaled back by
-  static constexpr int BAR = FACTOR + FACTORS * TILE_M * 4;   // full and empty barriers of the stages, full and empty of the accumulators
-  static constexpr int BARS = 2 * STAGES + 4;
+  static constexpr int BAR = FACTOR + FACTORS * TILE_M * 4;   // full and empty barriers of the stages, full and empty of the accumulators,
+  static constexpr int BARS = 2 * STAGES + 4 + STAGES * GROUPS;   // arrival of every group's keys
   static constexpr int BYTES = BAR + BARS * 8 + 16 + 1024;    // + tensor-memory base, slack for the manual 1024-byte alignment
   static_assert(BYTES <= 227 * 1024, "shared memory");
 };
@@ -70,13 +79,13 @@ constexpr uint32_t RT_TMEM_COLS = 512;
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 __device__ __forceinline__ float tf32_head(float x) { return __uint_as_float(__float_as_uint(x) & 0xffffe000u); }
 
-// byte offset inside a slab of the 16-byte piece `c4` (0..7) of row `row`: rows are 128 bytes, eight rows form a
-// 1024-byte group, and inside a group piece c4 of row r sits at position c4 ^ r (the 128-byte swizzle)
-__device__ __forceinline__ int slab_offset(int row, int c4) { return (row >> 3) * 1024 + (row & 7) * 128 + ((c4 ^ (row & 7)) << 4); }
+// byte offset inside a group's quarter of the 16-byte piece `c4` (0..7) of row `row`: rows are 128 bytes and piece c4 of row r sits
+// at position c4 ^ r (the 128-byte swizzle)
+__device__ __forceinline__ int swizzled(int row, int c4) { return row * 128 + ((c4 ^ row) << 4); }
 
-// K-major, 128-byte swizzle: start address, leading offset 1 (unused), 1024 bytes between 8-row groups, version 1
+// K-major, 128-byte swizzle: start address, leading offset 1 (unused), GROUP_BYTES between 8-row groups, version 1
 __device__ __forceinline__ uint64_t umma_desc(uint32_t saddr) {
-  return (uint64_t)((saddr & 0x3ffffu) >> 4) | (1ull << 16) | ((uint64_t)(1024 >> 4) << 32) | (1ull << 46) | (2ull << 61);
+  return (uint64_t)((saddr & 0x3ffffu) >> 4) | (1ull << 16) | ((uint64_t)(GROUP_BYTES >> 4) << 32) | (1ull << 46) | (2ull << 61);
 }
 // fp32 accumulator, tf32 A and B, both K-major, N = 128, M = 128
 constexpr uint32_t UMMA_IDESC = (1u << 4) | (2u << 7) | (2u << 10) | ((128u >> 3) << 17) | ((128u >> 4) << 24);
@@ -96,10 +105,9 @@ __device__ __forceinline__ float scale_up(float largest, float& back) {
   return __uint_as_float((268u - e) << 23);
 }
 // fp16 head and tail of two scaled values
-__device__ __forceinline__ void split2(float a, float b, uint32_t& head, uint32_t& tail) {
-  const __half2 h = __floats2half2_rn(a, b);
-  const float2 f = __half22float2(h);
-  const __half2 l = __floats2half2_rn(a - f.x, b - f.y);
+__device__ __forceinline__ void split2(float2 v, uint32_t& head, uint32_t& tail) {
+  const __half2 h = __float22half2_rn(v);
+  const __half2 l = __float22half2_rn(fathom_fma2(__half22float2(h), make_float2(-1.0f, -1.0f), v));
   head = *reinterpret_cast<const uint32_t*>(&h);
   tail = *reinterpret_cast<const uint32_t*>(&l);
 }
@@ -170,7 +178,14 @@ __device__ __forceinline__ void tmem_store32(uint32_t taddr, const uint32_t (&r)
          "r"(r[20]), "r"(r[21]), "r"(r[22]), "r"(r[23]), "r"(r[24]), "r"(r[25]), "r"(r[26]), "r"(r[27]), "r"(r[28]), "r"(r[29]),
          "r"(r[30]), "r"(r[31]) : "memory");
 }
-__device__ __forceinline__ void epilogue_barrier() { asm volatile("bar.sync 1, %0;" :: "n"(EPILOGUE) : "memory"); }
+// the two epilogue warps that share 32 channels
+__device__ __forceinline__ void pair_barrier(int pair) { asm volatile("bar.sync %0, 64;" :: "r"(1 + pair) : "memory"); }
+__device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {   // one arrival; bytes may be 0
+  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" :: "r"(bar), "r"(bytes) : "memory");
+  if (bytes)
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                 :: "r"(dst), "l"(src), "r"(bytes), "r"(bar) : "memory");
+}
 
 // 16 bytes of a key row: four fp32 or eight bf16 channels
 __device__ __forceinline__ void unpack16(const uint4& u, float (&x)[4]) {
@@ -206,7 +221,7 @@ rotate_tc_kernel(const T* __restrict__ K, const float* __restrict__ mean, const 
   float* s_factor = reinterpret_cast<float*>(sm + MP::FACTOR);
   uint32_t* s_tmem = reinterpret_cast<uint32_t*>(sm + MP::BAR + MP::BARS * 8);
   const uint32_t bar_full = sm_base + MP::BAR, bar_empty = bar_full + STAGES * 8, bar_acc_full = bar_empty + STAGES * 8,
-                 bar_acc_empty = bar_acc_full + 16;
+                 bar_acc_empty = bar_acc_full + 16, bar_raw = bar_acc_empty + 16;
   const int tid = threadIdx.x, lane = tid & 31, warp = __shfl_sync(0xffffffffu, tid >> 5, 0);   // (uniform)
   constexpr int MMA_WARP = (PRODUCERS + EPILOGUE) / 32;
 
@@ -219,6 +234,7 @@ rotate_tc_kernel(const T* __restrict__ K, const float* __restrict__ mean, const 
     for (int s = 0; s < STAGES; ++s) {
       mbar_init(bar_full + 8 * s, PRODUCERS / 32);
       mbar_init(bar_empty + 8 * s, 1);
+      for (int w = 0; w < GROUPS; ++w) mbar_init(bar_raw + 8 * (s * GROUPS + w), 1);
     }
     for (int a = 0; a < 2; ++a) {
       mbar_init(bar_acc_full + 8 * a, 2);                     // the commit, and an arrival that passes the producers' scales on
@@ -245,11 +261,31 @@ rotate_tc_kernel(const T* __restrict__ K, const float* __restrict__ mean, const 
     }
   };
   uint32_t tcount = 0;                                        // tiles so far: accumulator and its parity
+  uint32_t requested = 0;                                     // producers: tiles whose keys are on their way or here (each is waited for)
 
   for (long long g = g0; g < g1;) {                           // head by head
     const long long kv = g / tiles_per_head, tile0 = g - kv * tiles_per_head;
     const long long count = min(g1, (kv + 1) * tiles_per_head) - g;
     g += count;
+    // keys of this warp's rows of the head's tile t into their stage (bytes past the end of the sequence are left as they are: they become
+    // columns of the accumulator that are never used); c: its number among all tiles of this CTA
+    constexpr int ROW = FATHOM_D * sizeof(T);
+    auto request = [&](long long t, uint32_t c) {
+      if (t >= count) return;
+      const uint32_t stage = c % STAGES;
+      wait(bar_empty + 8 * stage, ((c / STAGES) & 1u) ^ 1u);  // (a fresh barrier lets the first round through)
+      if (!alive) return;
+      requested = c + 1;
+      if (lane != 0) return;
+      const long long r0 = (tile0 + t) * TILE_M + warp * GROUP;
+      const int rows = (int)max(0ll, min((long long)GROUP, n - r0));
+      bulk_load(sm_base + stage * STAGE_BYTES + warp * GROUP_BYTES, reinterpret_cast<const unsigned char*>(K) + ((size_t)kv * (size_t)n + (size_t)r0) * ROW,
+                (uint32_t)(rows * ROW), bar_raw + 8 * (stage * GROUPS + warp));
+    };
+    if (warp < GROUPS) {
+      request(0, tcount);
+      request(1, tcount + 1);
+    }
     // ---- the head's split basis into tensor memory (lane = rotated channel j, column = channel c), its mean into shared memory
     if (warp < 4) {
       const float* V = basis + (size_t)kv * FATHOM_D * FATHOM_D + tid;
@@ -265,7 +301,7 @@ rotate_tc_kernel(const T* __restrict__ K, const float* __restrict__ mean, const 
         for (int c = 0; c < 64; c += 2) {
           const float* v = V + ((c0 & (FATHOM_D - 1)) + c) * FATHOM_D;
           uint32_t head, tail;
-          split2(__ldg(v) * up, __ldg(v + FATHOM_D) * up, head, tail);
+          split2(make_float2(__ldg(v) * up, __ldg(v + FATHOM_D) * up), head, tail);
           part[c / 2] = c0 < FATHOM_D ? head : tail;
         }
         tmem_store32(tmem + ((uint32_t)(warp * 32) << 16) + COL_VH + c0 / 2, part);
@@ -279,43 +315,36 @@ rotate_tc_kernel(const T* __restrict__ K, const float* __restrict__ mean, const 
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 
     if (tid < PRODUCERS) {
-      // ---- producers: eight rows per warp, 16 bytes of a row per lane
+      // ---- producers: 16 bytes of a row per lane
       constexpr int CH = 16 / sizeof(T);                      // channels per load
-      constexpr int LANES = FATHOM_D / CH, STEP = 32 / LANES, LOADS = TILE_M / (PRODUCERS / 32) / STEP;   // lanes per row, rows per load
-      const int row0 = warp * (TILE_M / (PRODUCERS / 32)) + lane / LANES, c0 = (lane % LANES) * CH;
-      const T* Kh = K + (size_t)kv * (size_t)n * FATHOM_D + c0;
-      float mu[CH];
+      constexpr int LANES = FATHOM_D / CH, STEP = 32 / LANES, LOADS = GROUP / STEP;   // lanes per row, rows per load
+      const int row0 = lane / LANES, c0 = (lane % LANES) * CH, byte = (c0 % HALF_CH) * 2;
+      float2 mu[CH / 2];                                      // negated
 #pragma unroll
-      for (int c = 0; c < CH; ++c) mu[c] = s_mu[c0 + c];
-      uint4 xr[LOADS];                                        // one tile ahead, in registers, as loaded
-      auto load_tile = [&](long long tile) {
-        const long long r0 = tile * TILE_M + row0;
-        const uint4* p = reinterpret_cast<const uint4*>(Kh + (size_t)r0 * FATHOM_D);
-        constexpr int PITCH = STEP * FATHOM_D / CH;
-        if (r0 + STEP * (LOADS - 1) < n) {
-#pragma unroll
-          for (int i = 0; i < LOADS; ++i) xr[i] = __ldg(p + i * PITCH);
-        } else {
-#pragma unroll
-          for (int i = 0; i < LOADS; ++i) xr[i] = r0 + STEP * i < n ? __ldg(p + i * PITCH) : make_uint4(0u, 0u, 0u, 0u);
-        }
-      };
-      load_tile(tile0);
+      for (int c = 0; c < CH / 2; ++c) mu[c] = make_float2(-s_mu[c0 + 2 * c], -s_mu[c0 + 2 * c + 1]);
+      const float2 one = make_float2(1.0f, 1.0f);
       for (long long t = 0; t < count; ++t, ++tcount) {
-        const uint32_t stage = tcount % STAGES, round = tcount / STAGES;
-        wait(bar_empty + 8 * stage, (round & 1u) ^ 1u);       // (a fresh barrier lets the first round through)
-        unsigned char* xs = sm + stage * STAGE_BYTES + (c0 / HALF_CH) * SLAB;
-        float* factor = s_factor + (tcount % FACTORS) * TILE_M;
+        const uint32_t stage = tcount % STAGES;
+        unsigned char* group = sm + stage * STAGE_BYTES + warp * GROUP_BYTES;
+        unsigned char* to = group + (c0 / HALF_CH) * 1024;
+        float* factor = s_factor + (tcount % FACTORS) * TILE_M + warp * GROUP;
+        if (tcount < requested && !mbar_wait(bar_raw + 8 * (stage * GROUPS + warp), (tcount / STAGES) & 1u)) alive = false;
+        uint4 xr[LOADS];
+#pragma unroll
+        for (int i = 0; i < LOADS; ++i) xr[i] = reinterpret_cast<const uint4*>(group)[i * 32 + lane];
+        __syncwarp();                                         // (what is read here is written below)
 #pragma unroll
         for (int i = 0; i < LOADS; ++i) {
           float x[CH];
+          float2 d[CH / 2];
           unpack16(xr[i], x);
-          uint32_t m = 0u;                                    // the row's largest magnitude (non-negative floats order like integers)
+          float largest = 0.0f;                               // the row's largest magnitude (non-negative floats order like integers)
 #pragma unroll
-          for (int c = 0; c < CH; ++c) {
-            x[c] -= mu[c];
-            m = max(m, __float_as_uint(x[c]) & 0x7fffffffu);
+          for (int c = 0; c < CH / 2; ++c) {
+            d[c] = fathom_fma2(make_float2(x[2 * c], x[2 * c + 1]), one, mu[c]);
+            largest = fmaxf(largest, fmaxf(fabsf(d[c].x), fabsf(d[c].y)));
           }
+          uint32_t m = __float_as_uint(largest);
           if (LANES == 32) {
             m = __reduce_max_sync(0xffffffffu, m);
           } else {
@@ -324,25 +353,24 @@ rotate_tc_kernel(const T* __restrict__ K, const float* __restrict__ mean, const 
           }
           float back;
           const float up = scale_up(__uint_as_float(m), back);
-          const int row = row0 + STEP * i, byte = (c0 % HALF_CH) * 2;
+          const int row = row0 + STEP * i;
           if (c0 == 0) factor[row] = back;
           uint32_t h[CH / 2], l[CH / 2];
 #pragma unroll
-          for (int c = 0; c < CH; c += 2) split2(x[c] * up, x[c + 1] * up, h[c / 2], l[c / 2]);
-          // (rows past the end of the sequence give columns of the accumulator that are never used)
-          unsigned char* to = xs + slab_offset(row, byte >> 4) + (byte & 15);
+          for (int c = 0; c < CH / 2; ++c) split2(mul2(d[c], make_float2(up, up)), h[c], l[c]);
+          unsigned char* p = to + swizzled(row, byte >> 4) + (byte & 15);
           if constexpr (CH == 8) {
-            *reinterpret_cast<uint4*>(to) = make_uint4(h[0], h[1], h[2], h[3]);
-            *reinterpret_cast<uint4*>(to + 2 * SLAB) = make_uint4(l[0], l[1], l[2], l[3]);
+            *reinterpret_cast<uint4*>(p) = make_uint4(h[0], h[1], h[2], h[3]);
+            *reinterpret_cast<uint4*>(p + 2048) = make_uint4(l[0], l[1], l[2], l[3]);
           } else {
-            *reinterpret_cast<uint2*>(to) = make_uint2(h[0], h[1]);
-            *reinterpret_cast<uint2*>(to + 2 * SLAB) = make_uint2(l[0], l[1]);
+            *reinterpret_cast<uint2*>(p) = make_uint2(h[0], h[1]);
+            *reinterpret_cast<uint2*>(p + 2048) = make_uint2(l[0], l[1]);
           }
         }
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // generic-proxy stores -> visible to the MMA
         __syncwarp();
         if (lane == 0) mbar_arrive(bar_full + 8 * stage);
-        if (t + 1 < count) load_tile(tile0 + t + 1);          // (not before the fence, which would wait for the loads' issue)
+        request(t + 2, tcount + 2);
       }
     } else if (warp == MMA_WARP) {
       // (the whole warp runs the loop, one elected lane issues: addresses and descriptors then stay in uniform registers; issued
@@ -360,7 +388,7 @@ rotate_tc_kernel(const T* __restrict__ K, const float* __restrict__ mean, const 
         if (elect_one()) {
 #pragma unroll
           for (int hc = 0; hc < FATHOM_D / HALF_CH; ++hc) {
-            const uint64_t xh = umma_desc(slab + hc * SLAB), xl = umma_desc(slab + (2 + hc) * SLAB);
+            const uint64_t xh = umma_desc(slab + hc * 1024), xl = umma_desc(slab + (2 + hc) * 1024);
 #pragma unroll
             for (int ks = 0; ks < HALF_CH / RK; ++ks) {
               const uint32_t vh = tm + COL_VH + (hc * HALF_CH + ks * RK) / 2, vl = tm + COL_VL + (hc * HALF_CH + ks * RK) / 2;
@@ -441,8 +469,9 @@ rotate_tc_kernel(const T* __restrict__ K, const float* __restrict__ mean, const 
           const __half sh = __float2half_rn(a * vscale * 0.125f);   // (exact but for the one rounding to fp16)
           // the quantiser compares multiples of the stored scale with the values, so it may have both without the channel's scale
           const float sc = __half2float(sh) / vscale, inv = 1.0f / sc;
-          const int ubuf = (int)((tcount / UNIT) & 1u), bu = (int)(tile % UNIT) * (TILE_M / FATHOM_BLOCK) + blk;
-          uint32_t* o = reinterpret_cast<uint32_t*>(sm + MP::OUT + ubuf * OUT_BYTES) + ch * OUT_PITCH + bu * 2;
+          const int bu = (int)(tile % UNIT) * (TILE_M / FATHOM_BLOCK) + blk;
+          uint32_t* o = reinterpret_cast<uint32_t*>(sm + MP::OUT) + ch * OUT_PITCH + bu * 2;
+          if (tile % UNIT == 0) pair_barrier(lq);             // the last unit's flush has read them
 #pragma unroll
           for (int half = 0; half < 2; ++half) {
             if (half == 1) {
@@ -457,16 +486,15 @@ rotate_tc_kernel(const T* __restrict__ K, const float* __restrict__ mean, const 
 #pragma unroll
             for (int p = 0; p < FATHOM_NPLANES; ++p) o[p * UNIT_BLOCKS * 2 + half] = w[p] & keep;
           }
-          reinterpret_cast<uint16_t*>(sm + MP::SCALE)[(ubuf * FATHOM_D + ch) * UNIT_BLOCKS + bu] = __half_as_ushort(sh);
+          reinterpret_cast<uint16_t*>(sm + MP::SCALE)[ch * UNIT_BLOCKS + bu] = __half_as_ushort(sh);
           if ((tile + 1) % UNIT == 0) {
-            // ---- flush: the unit's four blocks of every (channel, plane) row are 32 contiguous bytes.  (The other buffer
-            //      takes the next unit; a warp that is a unit ahead waits here before it can come back to this one)
-            epilogue_barrier();
-            const int et = tid - PRODUCERS;
+            // ---- flush: the unit's four blocks of every (channel, plane) row are 32 contiguous bytes
+            pair_barrier(lq);
+            const int et = blk * 32 + lane;                   // of the 64 threads that have these 32 channels
             const long long nb = (n + FATHOM_BLOCK - 1) / FATHOM_BLOCK, b0 = tile / UNIT * UNIT_BLOCKS;
             const int nblk = (int)min((long long)UNIT_BLOCKS, nb - b0);
-            const uint32_t* staged = reinterpret_cast<const uint32_t*>(sm + MP::OUT + ubuf * OUT_BYTES);
-            for (int e = et; e < FATHOM_D * FATHOM_NPLANES; e += EPILOGUE) {
+            const uint32_t* staged = reinterpret_cast<const uint32_t*>(sm + MP::OUT);
+            for (int e = lq * 32 * FATHOM_NPLANES + et; e < (lq + 1) * 32 * FATHOM_NPLANES; e += 64) {
               const uint32_t* src = staged + (e >> 2) * OUT_PITCH + (e & 3) * UNIT_BLOCKS * 2;
               uint64_t* dst = planes + ((size_t)kv * FATHOM_D * FATHOM_NPLANES + e) * (size_t)plane_stride + b0;
               if (nblk == UNIT_BLOCKS && (reinterpret_cast<uintptr_t>(dst) & 31u) == 0) {   // a whole sector
@@ -483,9 +511,9 @@ rotate_tc_kernel(const T* __restrict__ K, const float* __restrict__ mean, const 
                 }
               }
             }
-            if (et < FATHOM_D) {
-              const uint16_t* src = reinterpret_cast<const uint16_t*>(sm + MP::SCALE) + (ubuf * FATHOM_D + et) * UNIT_BLOCKS;
-              uint16_t* dst = scales + ((size_t)kv * FATHOM_D + et) * (size_t)scale_stride + b0;
+            if (blk == 0) {
+              const uint16_t* src = reinterpret_cast<const uint16_t*>(sm + MP::SCALE) + ch * UNIT_BLOCKS;
+              uint16_t* dst = scales + ((size_t)kv * FATHOM_D + ch) * (size_t)scale_stride + b0;
               if (nblk == UNIT_BLOCKS) {
                 *reinterpret_cast<uint2*>(dst) = *reinterpret_cast<const uint2*>(src);
               } else {
