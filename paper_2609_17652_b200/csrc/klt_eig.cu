@@ -13,9 +13,10 @@
 //     the index arithmetic: 1.8 us a step) and a warp's accesses are runs of consecutive doubles;
 //   * the rotations of the next step are computed in the same phase by the 64 threads that update the elements (p', q') they
 //     need: one barrier per step, and the chain of a rotation (two reciprocal square roots) runs beside the other warps' updates;
-//   * CTA 0 logs a sweep's rotations (fp32 c, s); the seven other CTAs fetch the log through distributed shared memory and apply
-//     it to their rows of the accumulated basis (fp32) while CTA 0 runs the next sweep.  A row is owned by one warp, so
-//     nothing but __syncwarp separates the steps.
+//   * CTA 0 logs the rotations (fp32 c, s); the seven other CTAs fetch the log through distributed shared memory, 32 steps at a
+//     time, and apply them to their rows of the accumulated basis (fp32) while CTA 0 goes on.  A row is owned by one warp, so
+//     nothing but __syncwarp separates the steps.  (A sweep at a time, CTA 0 stood still for 20 K cycles while its log was copied,
+//     and 38 K at the end while the last sweep was applied: a step takes 1.2 K.)
 // A step in fp64 is bound by the shared-memory data path all the same (128 KB read and written), so the sweeps that only have to
 // come close run in fp32 (half the bytes, a shorter chain), and fp64 finishes, the columns dealt out over the eight CTAs: the
 // accumulated basis is made orthonormal by one Newton-Schulz step W = V (3 I - V^T V) / 2, B = W^T C W is formed from the
@@ -31,7 +32,9 @@
 // choice.  Eigenvalues are clamped at zero.
 #include "fathom_common.cuh"
 
+#include <climits>
 #include <cooperative_groups.h>
+#include <utility>
 
 namespace cg = cooperative_groups;
 
@@ -51,7 +54,11 @@ constexpr int TYPE = DIST * PAIRS;                            // blocks; element
 constexpr int BUF = 4 * TYPE;                                 // 8192 doubles: one triangle by slots
 constexpr int TRIANGLES = 10;
 constexpr int EIG_THREADS = PAIRS * (TRIANGLES + 1) + 32;     // 736: the pivots' blocks, the triangles, d = 32
+constexpr int SEG = 32, SEGS = (STEPS + SEG - 1) / SEG;        // steps that are handed over together; a sweep's (the log is a ring of these)
 constexpr int COLS = N / EIG_CLUSTER;                         // columns of the finish per CTA: 16
+constexpr int LDC = COLS + 1;                                 // their pitch: lanes walk rows and columns
+constexpr int KPARTS = 4;                                     // a product's sum is split over this many groups of 128 threads
+static_assert(KPARTS * 128 <= EIG_THREADS, "threads of a product");
 static_assert(EIG_THREADS / 32 >= V_ROWS && EIG_THREADS / 32 <= 32, "a warp per basis row; one warp sums the warps' partial sums");
 // Distances 1, 3 .. 31 in triples a, b, c with c = a + b or a + b + c = 64: the pairs k, k + a, k + a + b are the corners of three
 // blocks, so a thread reads three rotations for three blocks (two blocks of one pair took three as well: 128 of 1600 wavefronts)
@@ -63,10 +70,11 @@ struct EigSmem {
                                                               // 64 of a buffer take the stores of elements that became a pivot.
                                                               // Other CTAs: rows of the basis.  Finish: a full matrix in fp64
   union {
-    float2 log[STEPS][PAIRS];                                 // (c, s) of a sweep: written by CTA 0, copied by the others
+    float2 log[STEPS][PAIRS];                                 // (c, s) of the last SEGS segments: written by CTA 0, copied by the others
     struct {                                                  // finish: [row][my columns]
-      double G[N][COLS];                                      // V^T V, later B
-      double W[N][COLS], T[N][COLS];                          // W; C W, later the angles
+      double G[N][LDC];                                       // V^T V, later B
+      double W[N][LDC], T[N][LDC];                            // W; C W, later the angles
+      double P[KPARTS - 2][N][LDC];                           // partial sums of a product
     };
   };
   double2 cs[2][PAIRS];                                       // rotations of this step and of the next
@@ -77,7 +85,7 @@ struct EigSmem {
   double cta_red[EIG_CLUSTER];
   int rank[N];
   float big[N];                                               // basis CTAs: the largest component of every column over my rows
-  int done;
+  int segments;                                               // CTA 0: how many there are in all, once that is known
 };
 
 // the pair k of a step: p = step + k, q = step - k (mod 127), q = 127 for k = 0
@@ -141,24 +149,23 @@ __device__ __forceinline__ Unit unit_of(int i, int d, int trash) {
   }
   return u;
 }
+// A thread reads all its blocks before it writes the first (the compiler cannot: the two buffers might be one, for all it knows)
+template <typename Real>
+__device__ __forceinline__ void load_block(const Real* from, const Unit& u, Real (&x)[4]) {
+#pragma unroll
+  for (int e = 0; e < 4; ++e) x[e] = from[u.load + e * TYPE];
+}
 // the 2 x 2 block, rotated from both sides: rows (pair i) by ri, columns (pair j) by rj
 template <typename Real, typename R2>
-__device__ __forceinline__ void rotate_block(const Real* __restrict__ from, Real* __restrict__ to, const Unit& u, R2 ri, R2 rj, Real (&z)[4]) {
-  const Real x0 = from[u.load], x1 = from[u.load + TYPE], x2 = from[u.load + 2 * TYPE], x3 = from[u.load + 3 * TYPE];
-  const Real y0 = ri.x * x0 - ri.y * x2, y1 = ri.x * x1 - ri.y * x3;
-  const Real y2 = ri.y * x0 + ri.x * x2, y3 = ri.y * x1 + ri.x * x3;
+__device__ __forceinline__ void rotate_block(Real* to, const Unit& u, R2 ri, R2 rj, const Real (&x)[4], Real (&z)[4]) {
+  const Real y0 = ri.x * x[0] - ri.y * x[2], y1 = ri.x * x[1] - ri.y * x[3];
+  const Real y2 = ri.y * x[0] + ri.x * x[2], y3 = ri.y * x[1] + ri.x * x[3];
   z[0] = rj.x * y0 - rj.y * y1;
   z[1] = rj.y * y0 + rj.x * y1;
   z[2] = rj.x * y2 - rj.y * y3;
   z[3] = rj.y * y2 + rj.x * y3;
 #pragma unroll
   for (int e = 0; e < 4; ++e) to[u.to[e]] = z[e];
-}
-
-template <typename Cluster>
-__device__ __forceinline__ void stop_or_go(EigSmem& M, Cluster& cluster, int sweep, bool done) {
-  if (sweep > 0) cluster.sync();                              // the others have copied the previous sweep's log
-  if (threadIdx.x == 0) M.done = done;
 }
 
 // CTA 0: sweeps over the symmetric matrix whose elements (i <= j) `get` returns, until off-diagonal mass <= tol * diagonal mass or
@@ -203,10 +210,20 @@ __device__ __forceinline__ int sweeps(EigSmem& M, Cluster& cluster, int max_swee
 
   for (int e = tid; e < 2 * LDB; e += EIG_THREADS) A[e] = Real(0);             // (the unused half of d = 32 stays zero)
   __syncthreads();
-  for (int e = tid; e < N * N; e += EIG_THREADS) {
-    const int i = e >> 7, j = e & (N - 1);
-    if (i <= j) {
-      const Real a = get(i, j);
+  if (tid == 0) M.segments = INT_MAX;
+  constexpr int BATCH = 8;                                    // elements a thread fetches together
+  for (int e0 = tid; e0 < N * N; e0 += BATCH * EIG_THREADS) {
+   Real fetched[BATCH];
+#pragma unroll
+   for (int u = 0; u < BATCH; ++u) {
+    const int e = e0 + u * EIG_THREADS, i = e >> 7, j = e & (N - 1);
+    fetched[u] = e < N * N && i <= j ? get(i, j) : Real(0);
+   }
+#pragma unroll
+   for (int u = 0; u < BATCH; ++u) {
+    const int e = e0 + u * EIG_THREADS, i = e >> 7, j = e & (N - 1);
+    if (e < N * N && i <= j) {
+      const Real a = fetched[u];
       const Slot si = slot_of_player(i, 0), sj = slot_of_player(j, 0);
       if (i == j) {                                           // "after step -1", in the slots of step -1 = 126 (mod 127)
         const Slot s = slot_of_player(i, STEPS - 1);
@@ -215,6 +232,7 @@ __device__ __forceinline__ int sweeps(EigSmem& M, Cluster& cluster, int max_swee
       } else if (si.pair == sj.pair) pivot[si.pair] = a;
       else A[element(si, sj)] = a;
     }
+   }
   }
   __syncthreads();
   if (ahead) {
@@ -222,6 +240,14 @@ __device__ __forceinline__ int sweeps(EigSmem& M, Cluster& cluster, int max_swee
     rot[k] = rotation<Real>(app, aqq, pivot[k], diag[k], diag[PAIRS + k]);
   }
   int g = 0;                                                  // steps so far (parity of the double buffers)
+  int handed = 0;                                             // segments so far: one phase of the cluster barrier each, arrived at when the segment is
+                                                              // complete and waited for one segment later.  The others arrive at a phase when they
+                                                              // have copied the segments before it, so a ring of SEGS is never overrun
+  typename Cluster::arrival_token phase;
+  auto hand_over = [&]() {
+    if (handed++ > 0) cluster.barrier_wait(std::move(phase));
+    phase = cluster.barrier_arrive();
+  };
   for (int sweep = 0;; ++sweep) {
     // ---- how far from diagonal?  (fixed-order reduction: per thread, per warp, then over the warps)
     double off = 0.0, dg = 0.0;
@@ -246,18 +272,18 @@ __device__ __forceinline__ int sweeps(EigSmem& M, Cluster& cluster, int max_swee
       dg += __shfl_xor_sync(0xffffffffu, dg, o);
     }
     const bool done = sweep == max_sweeps || off <= tol * dg;  // the same for every thread
-    stop_or_go(M, cluster, sweep, done);
     if (!done) {
       for (int step = 0; step < STEPS; ++step, ++g) {
         const int par = g & 1;
         const Real* from = A + par * LDB;
         Real* to = A + (par ^ 1) * LDB;
         const R2* cs = rot + par * PAIRS;
-        Real z[4];
+        Real x0[4], x1[4], x2[4], z[4];
+        load_block(from, u0, x0);
         if (ahead) {
           const R2 mine = cs[k];
           const Real app = diag[par * N + src_p], aqq = diag[par * N + src_q];
-          rotate_block<Real, R2>(from, to, u0, cs[u0.i], cs[u0.j], z);
+          rotate_block<Real, R2>(to, u0, cs[u0.i], cs[u0.j], x0, z);
           const Real apq = pivot_element == 0 ? z[0] : (pivot_element == 2 ? z[2] : z[3]);
           Real* after = diag + (par ^ 1) * N;
           rot[(par ^ 1) * PAIRS + k] = rotation<Real>(app, aqq, apq, after[k], after[PAIRS + k]);
@@ -266,18 +292,26 @@ __device__ __forceinline__ int sweeps(EigSmem& M, Cluster& cluster, int max_swee
           if (step == STEPS - 1) pivot[k] = apq;
         } else {
           const R2 ri = cs[u0.i], rj = cs[u0.j];
-          rotate_block<Real, R2>(from, to, u0, ri, rj, z);
-          if (!opposite) {
+          if (opposite) {
+            rotate_block<Real, R2>(to, u0, ri, rj, x0, z);
+          } else {
             const R2 r0 = group == 0 ? cs[k] : ri, r1 = group == 0 ? cs[u1.i] : rj, r2 = cs[corner];
-            rotate_block<Real, R2>(from, to, u1, r1, r2, z);
-            rotate_block<Real, R2>(from, to, u2, closed ? r0 : r2, closed ? r2 : r0, z);
+            load_block(from, u1, x1);
+            load_block(from, u2, x2);
+            rotate_block<Real, R2>(to, u0, ri, rj, x0, z);
+            rotate_block<Real, R2>(to, u1, r1, r2, x1, z);
+            rotate_block<Real, R2>(to, u2, closed ? r0 : r2, closed ? r2 : r0, x2, z);
           }
         }
         __syncthreads();
+        if (step % SEG == SEG - 1 || step == STEPS - 1) hand_over();
       }
+    } else {
+      if (tid == 0) M.segments = handed;
+      hand_over();                                            // the last phase, without a segment
+      cluster.barrier_wait(std::move(phase));                 // everything is applied
+      return g;
     }
-    cluster.sync();                                           // log and flag are complete
-    if (done) return g;
   }
 }
 
@@ -285,15 +319,16 @@ __device__ __forceinline__ int sweeps(EigSmem& M, Cluster& cluster, int max_swee
 template <typename Cluster>
 __device__ __forceinline__ void apply_sweeps(EigSmem& M, EigSmem& M0, Cluster& cluster, float* V, int rows) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  while (true) {
-    cluster.sync();                                           // a sweep's log is complete
-    if (M0.done) return;                                      // (the same for every thread)
-    for (int e = tid; e < STEPS * PAIRS / 2; e += EIG_THREADS)
+  for (int segment = 0;; ++segment) {
+    cluster.sync();                                           // the segment's log is complete
+    if (segment >= M0.segments) return;                       // (the same for every thread)
+    const int first = segment % SEGS * SEG, last = min(first + SEG, STEPS);
+    for (int e = first * PAIRS / 2 + tid; e < last * PAIRS / 2; e += EIG_THREADS)
       reinterpret_cast<float4*>(M.log)[e] = reinterpret_cast<const float4*>(M0.log)[e];
-    cluster.sync();                                           // CTA 0 may write the next sweep's (also: my copy is complete)
+    __syncthreads();                                          // (a warp that is still in the segment before has that in another part of the ring)
     if (warp < rows) {
       float* row = V + warp * N;
-      for (int step = 0; step < STEPS; ++step) {
+      for (int step = first; step < last; ++step) {
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
           const int k = lane + 32 * h, p = player_p(step, k), q = player_q(step, k);
@@ -305,7 +340,6 @@ __device__ __forceinline__ void apply_sweeps(EigSmem& M, EigSmem& M0, Cluster& c
         __syncwarp();
       }
     }
-    __syncthreads();                                          // the log may be overwritten
   }
 }
 
@@ -344,19 +378,20 @@ klt_eig_kernel(const float* __restrict__ cov, float* __restrict__ basis_out, flo
   constexpr int LDX = N + 1;
   static_assert(N * LDX <= 2 * (BUF + PAIRS), "a full fp64 matrix lies where the sweeps keep theirs");
   const int J0 = part * COLS;
-  // Products of 128 x 128 by 128 x 16: a thread has four rows (row, + 32, ..) by four columns and half of the sum, so that ten 128-byte
-  // reads of shared memory serve 512 multiply-adds (a row by four columns took three times as many); 256 threads
-  const int row = tid & 31, pj = ((tid >> 5) & 3) * 4, half = tid >> 7;
-  // out[i][j] = finish(i, j, sum over k of (by_column ? X[k][i] : X[i][k]) * R[k][j]); R and out are different arrays of [N][COLS]
-  auto product = [&](bool by_column, const double* right, int ld_right, double (*out)[COLS], auto finish) {
+  // Products of 128 x 128 by 128 x 16: a thread has four rows (row, + 32, ..) by four columns and a quarter of the sum, so that ten 128-byte
+  // reads of shared memory serve 512 multiply-adds (a row by four columns took three times as many); 512 threads (half as many, and
+  // results at a pitch of 16, where 32 rows share a bank: 13.5 K cycles a product)
+  const int row = tid & 31, pj = ((tid >> 5) & 3) * 4, kpart = tid >> 7;
+  // out[i][j] = finish(i, j, sum over k of (by_column ? X[k][i] : X[i][k]) * R[k][j]); R and out are different arrays
+  auto product = [&](bool by_column, const double* right, int ld_right, double (*out)[LDC], auto finish) {
     double s[4][4];
 #pragma unroll
     for (int r = 0; r < 4; ++r) s[r][0] = s[r][1] = s[r][2] = s[r][3] = 0.0;
-    if (half < 2) {
+    if (kpart < KPARTS) {
       const double* x = by_column ? X + row : X + row * LDX;
       const int step = by_column ? LDX : 1, rows32 = by_column ? 32 : 32 * LDX;
 #pragma unroll 2
-      for (int k = half * (N / 2); k < (half + 1) * (N / 2); ++k) {
+      for (int k = kpart * (N / KPARTS); k < (kpart + 1) * (N / KPARTS); ++k) {
         double a[4], b[4];
 #pragma unroll
         for (int r = 0; r < 4; ++r) a[r] = x[k * step + r * rows32];
@@ -368,20 +403,24 @@ klt_eig_kernel(const float* __restrict__ cov, float* __restrict__ basis_out, flo
           for (int c = 0; c < 4; ++c) s[r][c] = fma(a[r], b[c], s[r][c]);
       }
     }
-    if (half == 1) {
+    if (kpart > 0 && kpart < KPARTS) {
+      double (*part)[LDC] = kpart == 1 ? out : M.P[kpart - 2];
 #pragma unroll
       for (int r = 0; r < 4; ++r)
 #pragma unroll
-        for (int c = 0; c < 4; ++c) out[row + 32 * r][pj + c] = s[r][c];
+        for (int c = 0; c < 4; ++c) part[row + 32 * r][pj + c] = s[r][c];
     }
     __syncthreads();
-    if (half == 0) {
+    if (kpart == 0) {
 #pragma unroll
       for (int r = 0; r < 4; ++r)
 #pragma unroll
         for (int c = 0; c < 4; ++c) {
           const int i = row + 32 * r, j = pj + c;
-          out[i][j] = finish(i, j, s[r][c] + out[i][j]);
+          double sum = s[r][c] + out[i][j];
+#pragma unroll
+          for (int h = 0; h < KPARTS - 2; ++h) sum += M.P[h][i][j];
+          out[i][j] = finish(i, j, sum);
         }
     }
     __syncthreads();
@@ -411,7 +450,7 @@ klt_eig_kernel(const float* __restrict__ cov, float* __restrict__ basis_out, flo
       for (int c = 0; c < 4; ++c)
 #pragma unroll
         for (int u = 0; u < PER; ++u)
-          if (tid + u * EIG_THREADS < N * COLS) v[c][u] = (&cluster.map_shared_rank(&M, c0 + c)->W[0][0])[tid + u * EIG_THREADS];
+          if (tid + u * EIG_THREADS < N * COLS) v[c][u] = cluster.map_shared_rank(&M, c0 + c)->W[(tid + u * EIG_THREADS) / COLS][(tid + u * EIG_THREADS) % COLS];
 #pragma unroll
       for (int c = 0; c < 4; ++c)
 #pragma unroll
@@ -429,7 +468,7 @@ klt_eig_kernel(const float* __restrict__ cov, float* __restrict__ basis_out, flo
     // one step squares the distance from orthonormal, 1e-6 after the fp32 sweeps; after a round it is the worst product
     for (bool last = round == 0 || worst <= 1e-4;; last = true) {
       product(true, X + J0, LDX, M.G, as_is);                                                                // V^T V
-      product(false, &M.G[0][0], COLS, M.W, [&](int i, int j, double v) { return 1.5 * X[i * LDX + J0 + j] - 0.5 * v; });   // V (3 I - V^T V) / 2
+      product(false, &M.G[0][0], LDC, M.W, [&](int i, int j, double v) { return 1.5 * X[i * LDX + J0 + j] - 0.5 * v; });   // V (3 I - V^T V) / 2
       if (last) break;
       cluster.sync();
       gather();
@@ -442,10 +481,10 @@ klt_eig_kernel(const float* __restrict__ cov, float* __restrict__ basis_out, flo
       if (i < j) X[i * LDX + j] = X[j * LDX + i] = 0.5 * (X[i * LDX + j] + X[j * LDX + i]);
     }
     __syncthreads();
-    product(true, &M.W[0][0], COLS, M.T, as_is);                                                             // C W
+    product(true, &M.W[0][0], LDC, M.T, as_is);                                                             // C W
     cluster.sync();                                           // every CTA's columns of W
     gather();
-    product(true, &M.T[0][0], COLS, M.G, as_is);                                                             // B = W^T C W
+    product(true, &M.T[0][0], LDC, M.G, as_is);                                                             // B = W^T C W
     if (tid < COLS * EIG_CLUSTER) cluster.map_shared_rank(&M, tid / COLS)->lambda[J0 + tid % COLS] = M.G[J0 + tid % COLS][tid % COLS];
     cluster.sync();                                           // B, and its diagonal everywhere
 
@@ -485,7 +524,7 @@ klt_eig_kernel(const float* __restrict__ cov, float* __restrict__ basis_out, flo
     cluster.sync();
     for (int r = 0; r < EIG_CLUSTER; ++r) worst = fmax(worst, M.cta_red[r]);
     if (worst > (round == MAX_FINISHES - 1 ? MAX_PRODUCT : AGAIN_PRODUCT)) break;   // (the same for the whole cluster)
-    product(false, &M.T[0][0], COLS, M.W, [&](int i, int j, double v) { return X[i * LDX + J0 + j] + v; });  // W + W K
+    product(false, &M.T[0][0], LDC, M.W, [&](int i, int j, double v) { return X[i * LDX + J0 + j] + v; });  // W + W K
     if (warp < COLS) {                                        // a warp per column: its length
       double len = 0.0;
       for (int i = lane; i < N; i += 32) len = fma(M.W[i][warp], M.W[i][warp], len);
