@@ -214,7 +214,7 @@ var_partial_kernel(const T* __restrict__ K, long long n, float* __restrict__ par
 // A CTA per (16 channels, KV head): thread (channel, lane) merges tiles lane, lane + 64, ... and the 64 lanes are then
 // combined in lane order, so the result does not depend on scheduling.  (One CTA per KV head with 8 lanes per channel was a chain of
 // 2 x 128 dependent loads at n = 1M: 116 us, against 600 us for the pass over the keys; now 19 us.)
-constexpr int VF_CHANNELS = 16, VF_LANES = 64;
+constexpr int VF_CHANNELS = 8, VF_LANES = 128;
 __global__ void __launch_bounds__(VF_CHANNELS * VF_LANES)
 var_final_kernel(const float* __restrict__ partial, int tiles, long long n, float* __restrict__ mean, float* __restrict__ var) {
   __shared__ double s_acc[VF_LANES][VF_CHANNELS];
@@ -222,19 +222,27 @@ var_final_kernel(const float* __restrict__ partial, int tiles, long long n, floa
   const int kv = blockIdx.y, cl = threadIdx.x % VF_CHANNELS, tl = threadIdx.x / VF_CHANNELS, c = blockIdx.x * VF_CHANNELS + cl;
   FATHOM_PDL_WAIT();
   const float* P = partial + (size_t)kv * tiles * 3 * FATHOM_D + c;
-  auto sum_lanes = [&]() {                                    // fixed order: four sums of sixteen lanes, then their sum
+  auto sum_lanes = [&]() {                                    // fixed order: sixteen sums of eight lanes, then their sum
+    constexpr int EACH = VF_LANES / 16;
     __syncthreads();
-    if (tl < 4) {
+    if (tl < 16) {
       double s = 0.0;
 #pragma unroll
-      for (int w = 0; w < VF_LANES / 4; ++w) s += s_acc[tl * (VF_LANES / 4) + w][cl];
-      s_acc[tl * (VF_LANES / 4)][cl] = s;
+      for (int w = 0; w < EACH; ++w) s += s_acc[tl * EACH + w][cl];
+      s_acc[tl * EACH][cl] = s;
     }
     __syncthreads();
-    return (s_acc[0][cl] + s_acc[VF_LANES / 4][cl]) + (s_acc[VF_LANES / 2][cl] + s_acc[3 * (VF_LANES / 4)][cl]);
+    double s[16];
+#pragma unroll
+    for (int w = 0; w < 16; ++w) s[w] = s_acc[w * EACH][cl];
+#pragma unroll
+    for (int h = 8; h; h >>= 1)
+#pragma unroll
+      for (int w = 0; w < h; ++w) s[w] += s[w + h];
+    return s[0];
   };
   double total = 0.0;
-#pragma unroll 4
+#pragma unroll 8
   for (int t = tl; t < tiles; t += VF_LANES) {
     const double nt = (double)min((long long)MEAN_ROWS, n - (long long)t * MEAN_ROWS);
     total += nt * (double)P[(size_t)t * 3 * FATHOM_D] + (double)P[(size_t)t * 3 * FATHOM_D + FATHOM_D];
@@ -245,12 +253,13 @@ var_final_kernel(const float* __restrict__ partial, int tiles, long long n, floa
   __syncthreads();
   const double mu = s_mu[cl];
   double m2 = 0.0;
-#pragma unroll 4
+#pragma unroll 8
   for (int t = tl; t < tiles; t += VF_LANES) {
     const double nt = (double)min((long long)MEAN_ROWS, n - (long long)t * MEAN_ROWS);
     const double s1 = (double)P[(size_t)t * 3 * FATHOM_D + FATHOM_D], s2 = (double)P[(size_t)t * 3 * FATHOM_D + 2 * FATHOM_D];
-    const double dm = (double)P[(size_t)t * 3 * FATHOM_D] + s1 / nt - mu;
-    m2 += (s2 - s1 * s1 / nt) + nt * dm * dm;
+    const double avg = t == tiles - 1 ? s1 / nt : s1 * (1.0 / MEAN_ROWS);      // (exact: a power of two; a division per tile took half the time)
+    const double dm = (double)P[(size_t)t * 3 * FATHOM_D] + avg - mu;
+    m2 += (s2 - s1 * avg) + nt * dm * dm;
   }
   s_acc[tl][cl] = m2;
   const double squares = sum_lanes();
@@ -262,28 +271,42 @@ var_final_kernel(const float* __restrict__ partial, int tiles, long long n, floa
 
 // reduction of the tensor-core partials (fp64, slot order): S = sum_t sums[kv][t], mean = shift + S / n,
 // cov = (sum_t (P1 + P2 + P2^T) - S S^T / n) / (n - 1)  with the partials [kv][t][2][d][d] of the shifted keys
-__global__ void __launch_bounds__(FATHOM_D)
+// A CTA per 32 x 32 tile of the result, a thread per element; the transposed tile of P2 is summed where it lies and turned round once
+// at the end (read element by element along its columns it was a sector per element: 15 -> 6 us for 8 heads of 18 partials).
+constexpr int CF_TILE = 32;
+__global__ void __launch_bounds__(CF_TILE * CF_TILE)
 cov_final_tc_kernel(const float* __restrict__ partial, const float* __restrict__ partial_sum, const float* __restrict__ shift,
                     int slots, long long n, float* __restrict__ mean, float* __restrict__ cov) {
-  __shared__ double s_S[FATHOM_D];
-  const int kv = blockIdx.y, i = blockIdx.x, j = threadIdx.x;
-  {
+  __shared__ double s_S[2][CF_TILE];                          // of the tile's rows, of its columns
+  __shared__ double s_t[CF_TILE][CF_TILE + 1];
+  constexpr int TILES = FATHOM_D / CF_TILE;
+  FATHOM_PDL_WAIT();
+  FATHOM_PDL_RELEASE();
+  const int kv = blockIdx.y, i0 = blockIdx.x / TILES * CF_TILE, j0 = blockIdx.x % TILES * CF_TILE;
+  const int x = threadIdx.x % CF_TILE, y = threadIdx.x / CF_TILE;
+  if (y < 2) {
+    const int c = (y ? j0 : i0) + x;
     double t = 0.0;
-    for (int u = 0; u < slots; ++u) t += (double)partial_sum[((size_t)kv * slots + u) * FATHOM_D + j];
-    s_S[j] = t;
-    if (i == 0) mean[(size_t)kv * FATHOM_D + j] = (float)((double)shift[(size_t)kv * FATHOM_D + j] + t / (double)n);
+#pragma unroll 8
+    for (int u = 0; u < slots; ++u) t += (double)partial_sum[((size_t)kv * slots + u) * FATHOM_D + c];
+    s_S[y][x] = t;
+    if (y == 0 && j0 == 0) mean[(size_t)kv * FATHOM_D + c] = (float)((double)shift[(size_t)kv * FATHOM_D + c] + t / (double)n);
   }
-  __syncthreads();
   const float* P = partial + (size_t)kv * slots * 2 * FATHOM_D * FATHOM_D;
-  double s = 0.0;
-#pragma unroll 4
+  const int here = (i0 + y) * FATHOM_D + j0 + x, there = (j0 + y) * FATHOM_D + i0 + x;
+  double s = 0.0, turned = 0.0;
+#pragma unroll 6
   for (int t = 0; t < slots; ++t) {
     const float* p1 = P + (size_t)t * 2 * FATHOM_D * FATHOM_D;
     const float* p2 = p1 + FATHOM_D * FATHOM_D;
-    s += (double)p1[i * FATHOM_D + j] + ((double)p2[i * FATHOM_D + j] + (double)p2[j * FATHOM_D + i]);
+    s += (double)p1[here] + (double)p2[here];
+    turned += (double)p2[there];
   }
-  s -= s_S[i] * s_S[j] / (double)n;
-  cov[((size_t)kv * FATHOM_D + i) * FATHOM_D + j] = (float)(s / (double)(n > 1 ? n - 1 : 1));
+  s_t[y][x] = turned;
+  __syncthreads();
+  s += s_t[x][y];
+  s -= s_S[0][y] * s_S[1][x] / (double)n;
+  cov[(size_t)kv * FATHOM_D * FATHOM_D + here] = (float)(s / (double)(n > 1 ? n - 1 : 1));
 }
 
 }  // namespace
@@ -354,8 +377,9 @@ extern "C" int fathom_calibrate(fathom_ctx* ctx, const fathom_layout* L, const v
     float* psum = reinterpret_cast<float*>(base + stats_partial_bytes(Hkv, n) + cov_bytes + fathom_round_up((size_t)Hkv * FATHOM_D * 4, 256));   // [Hkv][slots][d]
     rc = fathom_launch_cov_tc(ctx, L, K, k_dtype, var_tmp, pcov, psum, slots, st);
     if (rc != FATHOM_OK) return rc;
-    cov_final_tc_kernel<<<dim3(FATHOM_D, Hkv), FATHOM_D, 0, st>>>(pcov, psum, var_tmp, slots, n, mean, cov);
-    FATHOM_CUDA_TRY(ctx, cudaGetLastError());
+    constexpr int TILES = FATHOM_D / CF_TILE;
+    FATHOM_CUDA_TRY(ctx, fathom_launch_dependent(cov_final_tc_kernel, dim3(TILES * TILES, Hkv), dim3(CF_TILE * CF_TILE), 0, st, pcov, psum, var_tmp, slots, n,
+                                                 mean, cov));
     return FATHOM_OK;
   }
   // plain fp32 kernels: (1) mean

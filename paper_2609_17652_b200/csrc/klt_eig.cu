@@ -356,6 +356,8 @@ klt_eig_kernel(const float* __restrict__ cov, float* __restrict__ basis_out, flo
   float* V = reinterpret_cast<float*>(M.A);                   // CTAs 1..7: [V_ROWS][N]
   const int first_row = (part - 1) * V_ROWS, rows = min(V_ROWS, N - first_row);
 
+  FATHOM_PDL_WAIT();                                          // the covariance comes from the previous kernel
+  FATHOM_PDL_RELEASE();
   // ---- 1. fp32 sweeps; the accumulated basis goes through the output buffer to every CTA
   if (part == 0) {
     float m = 0.0f;                                           // scaled by a power of two so that the largest diagonal element is near one
@@ -646,7 +648,7 @@ extern "C" int fathom_klt_basis(fathom_ctx* ctx, const fathom_layout* L, const f
     FATHOM_CUDA_TRY(ctx, cudaFuncSetAttribute(klt_eig_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(EigSmem)));
     configured[dev] = true;
   }
-  klt_eig_kernel<<<L->n_kv_heads * EIG_CLUSTER, EIG_THREADS, sizeof(EigSmem), static_cast<cudaStream_t>(stream)>>>(cov, basis, eigenvalues);
-  FATHOM_CUDA_TRY(ctx, cudaGetLastError());
+  FATHOM_CUDA_TRY(ctx, fathom_launch_dependent(klt_eig_kernel, dim3(L->n_kv_heads * EIG_CLUSTER), dim3(EIG_THREADS), sizeof(EigSmem),
+                                               static_cast<cudaStream_t>(stream), cov, basis, eigenvalues));
   return FATHOM_OK;
 }

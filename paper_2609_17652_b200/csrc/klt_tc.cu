@@ -568,19 +568,27 @@ __device__ __forceinline__ void umma_tf32_mn(uint32_t tmem_d, uint64_t a, uint64
 // shift[kv][c] = mean of channel c over 64 keys spread evenly over the head's sequence (any value near the data would
 // do; it only has to keep S S^T / n small against the sum of squares - keys from one place, e.g. the first tokens of a
 // prompt, may sit far from the rest)
+// (sixteen keys per thread, requested together: eight at a time per channel took 11 us)
+constexpr int SHIFT_KEYS = 64, SHIFT_GROUPS = 4;
 template <typename T>
-__global__ void __launch_bounds__(FATHOM_D)
+__global__ void __launch_bounds__(FATHOM_D * SHIFT_GROUPS)
 cov_shift_kernel(const T* __restrict__ K, long long n, float* __restrict__ shift) {
-  const int kv = blockIdx.x, c = threadIdx.x;
+  constexpr int EACH = SHIFT_KEYS / SHIFT_GROUPS;
+  __shared__ float s_sum[SHIFT_GROUPS][FATHOM_D];
+  FATHOM_PDL_WAIT();
+  FATHOM_PDL_RELEASE();
+  const int kv = blockIdx.x, c = threadIdx.x % FATHOM_D, g = threadIdx.x / FATHOM_D;
   const T* Kh = K + (size_t)kv * (size_t)n * FATHOM_D;
-  const int rows = (int)min((long long)64, n);
+  const int rows = (int)min((long long)SHIFT_KEYS, n);
   const long long step = n / rows;                            // >= 1
-  float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-  for (int r = 0; r < rows; r += 8)
+  float v[EACH], sum = 0.0f;
 #pragma unroll
-    for (int u = 0; u < 8; ++u)
-      if (r + u < rows) acc[u] += (float)Kh[(size_t)((r + u) * step) * FATHOM_D + c];
-  shift[(size_t)kv * FATHOM_D + c] = (((acc[0] + acc[1]) + (acc[2] + acc[3])) + ((acc[4] + acc[5]) + (acc[6] + acc[7]))) / (float)rows;
+  for (int u = 0; u < EACH; ++u) v[u] = g * EACH + u < rows ? (float)Kh[(size_t)((g * EACH + u) * step) * FATHOM_D + c] : 0.0f;
+#pragma unroll
+  for (int u = 0; u < EACH; ++u) sum += v[u];
+  s_sum[g][c] = sum;
+  __syncthreads();
+  if (g == 0) shift[(size_t)kv * FATHOM_D + c] = ((s_sum[0][c] + s_sum[1][c]) + (s_sum[2][c] + s_sum[3][c])) / (float)rows;
 }
 
 template <typename T>
@@ -610,6 +618,8 @@ cov_partial_tc_kernel(const T* __restrict__ K, const float* __restrict__ shift, 
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" :: "r"(smem_u32(s_tmem)), "r"(256u) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
+  FATHOM_PDL_WAIT();                                          // the shift comes from the previous kernel
+  FATHOM_PDL_RELEASE();
   if (tid < FATHOM_D) s_mu[tid] = shift[(size_t)kv * FATHOM_D + tid];
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
@@ -773,24 +783,25 @@ int fathom_cov_tc_ctas_per_head(int Hkv) {
   return c < 1 ? 1 : c;
 }
 
+namespace {
+template <typename T>
+int launch_cov(fathom_ctx* ctx, const fathom_layout* L, const void* K, float* shift, float* partial, float* partial_sum, dim3 grid, cudaStream_t st) {
+  FATHOM_CUDA_TRY(ctx, cudaFuncSetAttribute(cov_partial_tc_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, CV_SMEM));
+  FATHOM_CUDA_TRY(ctx, fathom_launch_dependent(cov_shift_kernel<T>, dim3(L->n_kv_heads), dim3(FATHOM_D * SHIFT_GROUPS), 0, st, static_cast<const T*>(K),
+                                               (long long)L->n, shift));
+  FATHOM_CUDA_TRY(ctx, fathom_launch_dependent(cov_partial_tc_kernel<T>, grid, dim3(TC_THREADS), CV_SMEM, st, static_cast<const T*>(K), shift, partial,
+                                               partial_sum, (long long)L->n, ctx->dev_status));
+  return FATHOM_OK;
+}
+}  // namespace
+
 // Enqueues the shift, the covariance partials [Hkv][ctas][2][128][128] (sum xh xh^T and sum xh xl^T of the shifted
 // keys, per CTA) and the per-channel sums [Hkv][ctas][128].
 int fathom_launch_cov_tc(fathom_ctx* ctx, const fathom_layout* L, const void* K, int k_dtype, float* shift, float* partial,
                          float* partial_sum, int ctas_per_head, cudaStream_t st) {
   dim3 grid((unsigned)ctas_per_head, (unsigned)L->n_kv_heads);
-  if (k_dtype == FATHOM_F32) {
-    FATHOM_CUDA_TRY(ctx, cudaFuncSetAttribute(cov_partial_tc_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, CV_SMEM));
-    cov_shift_kernel<float><<<L->n_kv_heads, FATHOM_D, 0, st>>>(static_cast<const float*>(K), L->n, shift);
-    cov_partial_tc_kernel<float><<<grid, TC_THREADS, CV_SMEM, st>>>(static_cast<const float*>(K), shift, partial, partial_sum, L->n,
-                                                                     ctx->dev_status);
-  } else {
-    FATHOM_CUDA_TRY(ctx, cudaFuncSetAttribute(cov_partial_tc_kernel<__nv_bfloat16>, cudaFuncAttributeMaxDynamicSharedMemorySize, CV_SMEM));
-    cov_shift_kernel<__nv_bfloat16><<<L->n_kv_heads, FATHOM_D, 0, st>>>(static_cast<const __nv_bfloat16*>(K), L->n, shift);
-    cov_partial_tc_kernel<__nv_bfloat16><<<grid, TC_THREADS, CV_SMEM, st>>>(static_cast<const __nv_bfloat16*>(K), shift, partial,
-                                                                             partial_sum, L->n, ctx->dev_status);
-  }
-  FATHOM_CUDA_TRY(ctx, cudaGetLastError());
-  return FATHOM_OK;
+  return k_dtype == FATHOM_F32 ? launch_cov<float>(ctx, L, K, shift, partial, partial_sum, grid, st)
+                               : launch_cov<__nv_bfloat16>(ctx, L, K, shift, partial, partial_sum, grid, st);
 }
 
 extern "C" int fathom_selftest_wait_expiry(fathom_ctx* ctx, int tries, void* stream) {
