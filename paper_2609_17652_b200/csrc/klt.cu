@@ -211,9 +211,9 @@ var_partial_kernel(const T* __restrict__ K, long long n, float* __restrict__ par
   }
 }
 
-// A CTA per (16 channels, KV head): thread (channel, lane) merges tiles lane, lane + 64, ... and the 64 lanes are then
-// combined in lane order, so the result does not depend on scheduling.  (One CTA per KV head with 8 lanes per channel was a chain of
-// 2 x 128 dependent loads at n = 1M: 116 us, against 600 us for the pass over the keys; now 19 us.)
+// A CTA per (8 channels, KV head): thread (channel, lane) merges tiles lane, lane + 128, ... and the 128 lanes are then combined in a
+// fixed order, so the result does not depend on scheduling.  (One CTA per KV head with 8 lanes per channel was a chain of 2 x 128
+// dependent loads at n = 1M: 116 us, against 600 us for the pass over the keys; 16 channels a CTA and a division per tile: 18 us.)
 constexpr int VF_CHANNELS = 8, VF_LANES = 128;
 __global__ void __launch_bounds__(VF_CHANNELS * VF_LANES)
 var_final_kernel(const float* __restrict__ partial, int tiles, long long n, float* __restrict__ mean, float* __restrict__ var) {
