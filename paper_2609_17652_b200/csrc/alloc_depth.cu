@@ -19,7 +19,7 @@ constexpr int AD_SPLIT = 8;                        // threads per candidate
 constexpr int AD_THREADS = AD_CAND * AD_SPLIT;     // 512
 
 __global__ void __launch_bounds__(AD_THREADS)
-alloc_depth_kernel(const float* __restrict__ q, const float* __restrict__ var, int mode, int budget,
+alloc_depth_kernel(const float* q, const float* var, int mode, int budget,
                    int heads_per_plan, int G, uint8_t* __restrict__ depth) {
   __shared__ alignas(16) unsigned long long pri[NCAND];       // bit patterns of the (non-negative) priorities
   __shared__ int partial[AD_SPLIT][AD_CAND];

@@ -14,13 +14,13 @@ namespace {
 constexpr int BP_THREADS = 2 * FATHOM_D;
 constexpr int HALF = FATHOM_BLOCK / 2;                         // tokens per thread
 
-__device__ __forceinline__ float load_k(const float* p) { return __ldg(p); }
-__device__ __forceinline__ float load_k(const __nv_bfloat16* p) { return __bfloat162float(__ldg(p)); }
+__device__ __forceinline__ float load_k(const float* p) { return *p; }
+__device__ __forceinline__ float load_k(const __nv_bfloat16* p) { return __bfloat162float(*p); }
 
 // BLOCKS_PER_CTA: 8, or 1 for short sequences
 template <typename T, int BLOCKS_PER_CTA>
-__global__ void __launch_bounds__(BP_THREADS)
-build_planes_kernel(const T* __restrict__ K, uint32_t* __restrict__ planes32, uint16_t* __restrict__ scales,
+__global__ void __launch_bounds__(BP_THREADS, 4)
+build_planes_kernel(const T* K, uint32_t* __restrict__ planes32, uint16_t* __restrict__ scales,
                     long long n, long long nb, long long plane_stride, long long scale_stride) {
   constexpr int OUT_PITCH = FATHOM_NPLANES * BLOCKS_PER_CTA * 2 + 1;
   __shared__ float s_amax[2][2][FATHOM_D];                     // [parity of block][token half][channel]

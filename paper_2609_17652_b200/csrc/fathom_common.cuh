@@ -46,6 +46,9 @@ static inline size_t fathom_round_up(size_t x, size_t a) { return (x + a - 1) / 
 // must execute FATHOM_PDL_WAIT before it touches anything the previous kernels wrote; the wait returns when they have
 // completed and their writes are visible.  Both are no-ops in a normally launched kernel, and a kernel that never
 // releases simply serialises.  Every kernel of the decode step waits at its top, so completion is transitive.
+// What a dependent reads after its wait may have been written while it was resident already, so it must not be read as data that
+// stays constant for the kernel's lifetime (ld.global.nc, which the compiler may also move above the wait): no __ldg there, and no
+// __restrict__ on a pointer to const, which lets the compiler choose that load.
 #define FATHOM_PDL_WAIT() asm volatile("griddepcontrol.wait;" ::: "memory")
 #define FATHOM_PDL_RELEASE() asm volatile("griddepcontrol.launch_dependents;" ::: "memory")
 template <typename... P, typename... A>

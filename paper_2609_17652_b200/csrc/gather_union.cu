@@ -24,7 +24,7 @@ constexpr int LIST_THREADS = 1024;
 // Thread t owns `per` consecutive words (an odd multiple of four: 16-byte reads without bank conflicts), so that one block prefix
 // ranks the whole bitmap.
 __global__ void __launch_bounds__(LIST_THREADS)
-union_list_kernel(const int32_t* __restrict__ idx, int k, long long n, int G, int per, int32_t* __restrict__ ulist, int capacity,
+union_list_kernel(const int32_t* idx, int k, long long n, int G, int per, int32_t* __restrict__ ulist, int capacity,
                   int32_t* __restrict__ union_count, int32_t* __restrict__ idx_local) {
   extern __shared__ __align__(16) uint32_t s_bitmap[];        // [LIST_THREADS * per]
   __shared__ uint32_t s_warp[LIST_THREADS / 32];
@@ -41,7 +41,7 @@ union_list_kernel(const int32_t* __restrict__ idx, int k, long long n, int G, in
   auto clamped = [&](int32_t t) { return t < 0 ? 0 : ((long long)t >= n ? (int32_t)(n - 1) : t); };   // like in attention
 #pragma unroll 8
   for (int e = tid; e < picks; e += LIST_THREADS) {
-    const int32_t t = clamped(__ldg(my_idx + e));
+    const int32_t t = clamped(my_idx[e]);
     atomicOr(&s_bitmap[t >> 5], 1u << (t & 31));
   }
   __syncthreads();
@@ -75,7 +75,7 @@ union_list_kernel(const int32_t* __restrict__ idx, int k, long long n, int G, in
   }
   __syncthreads();
   for (int e = tid; e < picks; e += LIST_THREADS) {
-    const int32_t t = clamped(__ldg(my_idx + e));
+    const int32_t t = clamped(my_idx[e]);
     const int word = t >> 5, owner = word / per;
     uint32_t r = s_base[owner] + __popc(s_bitmap[word] & ((1u << (t & 31)) - 1u));
     for (int w = owner * per; w < word; ++w) r += __popc(s_bitmap[w]);
@@ -144,10 +144,8 @@ union_rank_kernel(const uint32_t* __restrict__ bitmap, long long words, uint32_t
 
 template <typename T>
 __global__ void __launch_bounds__(GU_THREADS)
-union_fetch_kernel(const T* __restrict__ Krows, const T* __restrict__ Vrows, long long n, const int32_t* __restrict__ ulist,
-                   const int32_t* __restrict__ union_count, int capacity, T* __restrict__ K_stage, T* __restrict__ V_stage,
-                   const int32_t* __restrict__ idx, int k, int G, int Hq, const uint32_t* __restrict__ bitmap,
-                   const uint32_t* __restrict__ word_rank, long long words, int32_t* __restrict__ idx_local) {
+union_fetch_kernel(const T* Krows, const T* Vrows, long long n, const int32_t* ulist, const int32_t* union_count, int capacity, T* __restrict__ K_stage, T* __restrict__ V_stage,
+                   const int32_t* idx, int k, int G, int Hq, const uint32_t* bitmap, const uint32_t* word_rank, long long words, int32_t* __restrict__ idx_local) {
   FATHOM_PDL_WAIT();                                          // the list comes from the previous kernel
   FATHOM_PDL_RELEASE();                                       // the attention may become resident where this kernel has finished
   constexpr int ROW_U4 = FATHOM_D * sizeof(T) / 16;           // 16-byte pieces per row: 16 (bf16) or 32 (fp32)
@@ -165,8 +163,8 @@ union_fetch_kernel(const T* __restrict__ Krows, const T* __restrict__ Vrows, lon
     const int r = r0 + (ROW_U4 < 32 ? lane / ROW_U4 : 0), piece = lane % ROW_U4;
     if (r < count) {
       const size_t src = (size_t)ulist[(size_t)kv * capacity + r] * FATHOM_D;
-      const uint4 a = __ldg(reinterpret_cast<const uint4*>(Kh + src) + piece);
-      const uint4 b = __ldg(reinterpret_cast<const uint4*>(Vh + src) + piece);
+      const uint4 a = reinterpret_cast<const uint4*>(Kh + src)[piece];
+      const uint4 b = reinterpret_cast<const uint4*>(Vh + src)[piece];
       reinterpret_cast<uint4*>(Ks + (size_t)r * FATHOM_D)[piece] = a;
       reinterpret_cast<uint4*>(Vs + (size_t)r * FATHOM_D)[piece] = b;
     }

@@ -96,7 +96,7 @@ rotate_keys_kernel(const T* __restrict__ K, const float* __restrict__ mean, cons
 // One fused multiply-add chain per output, as short as it is (128 steps); what took 10 us was loading the basis in groups of
 // eight, so the whole column is requested before the first step.
 __global__ void __launch_bounds__(FATHOM_D)
-rotate_query_kernel(const float* __restrict__ q, const float* __restrict__ basis, float* __restrict__ q_rot, int G) {
+rotate_query_kernel(const float* q, const float* basis, float* __restrict__ q_rot, int G) {
   __shared__ float s_q[FATHOM_D];
   FATHOM_PDL_WAIT();
   FATHOM_PDL_RELEASE();
@@ -104,7 +104,7 @@ rotate_query_kernel(const float* __restrict__ q, const float* __restrict__ basis
   const float* V = basis + (size_t)(h / G) * FATHOM_D * FATHOM_D + j;
   float v[FATHOM_D];
 #pragma unroll
-  for (int c = 0; c < FATHOM_D; ++c) v[c] = __ldg(V + c * FATHOM_D);
+  for (int c = 0; c < FATHOM_D; ++c) v[c] = V[c * FATHOM_D];
   s_q[j] = q[(size_t)h * FATHOM_D + j];
   __syncthreads();
   float acc = 0.0f;
@@ -216,7 +216,7 @@ var_partial_kernel(const T* __restrict__ K, long long n, float* __restrict__ par
 // dependent loads at n = 1M: 116 us, against 600 us for the pass over the keys; 16 channels a CTA and a division per tile: 18 us.)
 constexpr int VF_CHANNELS = 8, VF_LANES = 128;
 __global__ void __launch_bounds__(VF_CHANNELS * VF_LANES)
-var_final_kernel(const float* __restrict__ partial, int tiles, long long n, float* __restrict__ mean, float* __restrict__ var) {
+var_final_kernel(const float* partial, int tiles, long long n, float* __restrict__ mean, float* __restrict__ var) {
   __shared__ double s_acc[VF_LANES][VF_CHANNELS];
   __shared__ double s_mu[VF_CHANNELS];
   const int kv = blockIdx.y, cl = threadIdx.x % VF_CHANNELS, tl = threadIdx.x / VF_CHANNELS, c = blockIdx.x * VF_CHANNELS + cl;
@@ -275,7 +275,7 @@ var_final_kernel(const float* __restrict__ partial, int tiles, long long n, floa
 // at the end (read element by element along its columns it was a sector per element: 15 -> 6 us for 8 heads of 18 partials).
 constexpr int CF_TILE = 32;
 __global__ void __launch_bounds__(CF_TILE * CF_TILE)
-cov_final_tc_kernel(const float* __restrict__ partial, const float* __restrict__ partial_sum, const float* __restrict__ shift,
+cov_final_tc_kernel(const float* partial, const float* partial_sum, const float* shift,
                     int slots, long long n, float* __restrict__ mean, float* __restrict__ cov) {
   __shared__ double s_S[2][CF_TILE];                          // of the tile's rows, of its columns
   __shared__ double s_t[CF_TILE][CF_TILE + 1];

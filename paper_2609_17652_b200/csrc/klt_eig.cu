@@ -343,7 +343,7 @@ __device__ __forceinline__ void apply_sweeps(EigSmem& M, EigSmem& M0, Cluster& c
 }
 
 __global__ void __cluster_dims__(EIG_CLUSTER, 1, 1) __launch_bounds__(EIG_THREADS, 1)
-klt_eig_kernel(const float* __restrict__ cov, float* __restrict__ basis_out, float* __restrict__ eigenvalues) {
+klt_eig_kernel(const float* cov, float* basis_out, float* __restrict__ eigenvalues) {
   extern __shared__ __align__(16) unsigned char raw[];
   EigSmem& M = *reinterpret_cast<EigSmem*>(raw);
   cg::cluster_group cluster = cg::this_cluster();

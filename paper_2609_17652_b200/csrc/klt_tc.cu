@@ -197,9 +197,9 @@ __device__ __forceinline__ void unpack16(const uint4& u, float (&x)[8]) {
   for (int c = 0; c < 4; ++c) { x[2 * c] = __uint_as_float(w[c] << 16); x[2 * c + 1] = __uint_as_float(w[c] & 0xffff0000u); }
 }
 template <typename T> __device__ __forceinline__ float4 load_row4(const T* p);
-template <> __device__ __forceinline__ float4 load_row4<float>(const float* p) { return __ldg(reinterpret_cast<const float4*>(p)); }
+template <> __device__ __forceinline__ float4 load_row4<float>(const float* p) { return *reinterpret_cast<const float4*>(p); }
 template <> __device__ __forceinline__ float4 load_row4<__nv_bfloat16>(const __nv_bfloat16* p) {
-  const uint2 u = __ldg(reinterpret_cast<const uint2*>(p));
+  const uint2 u = *reinterpret_cast<const uint2*>(p);
   return make_float4(__uint_as_float(u.x << 16), __uint_as_float(u.x & 0xffff0000u), __uint_as_float(u.y << 16),
                      __uint_as_float(u.y & 0xffff0000u));
 }
@@ -572,7 +572,7 @@ __device__ __forceinline__ void umma_tf32_mn(uint32_t tmem_d, uint64_t a, uint64
 constexpr int SHIFT_KEYS = 64, SHIFT_GROUPS = 4;
 template <typename T>
 __global__ void __launch_bounds__(FATHOM_D * SHIFT_GROUPS)
-cov_shift_kernel(const T* __restrict__ K, long long n, float* __restrict__ shift) {
+cov_shift_kernel(const T* K, long long n, float* __restrict__ shift) {
   constexpr int EACH = SHIFT_KEYS / SHIFT_GROUPS;
   __shared__ float s_sum[SHIFT_GROUPS][FATHOM_D];
   FATHOM_PDL_WAIT();
@@ -593,7 +593,7 @@ cov_shift_kernel(const T* __restrict__ K, long long n, float* __restrict__ shift
 
 template <typename T>
 __global__ void __launch_bounds__(TC_THREADS, 1)
-cov_partial_tc_kernel(const T* __restrict__ K, const float* __restrict__ shift, float* __restrict__ partial,
+cov_partial_tc_kernel(const T* K, const float* shift, float* __restrict__ partial,
                       float* __restrict__ partial_sum, long long n, uint32_t* __restrict__ dev_status) {
   extern __shared__ unsigned char smem_raw[];
   unsigned char* sm = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);

@@ -213,7 +213,7 @@ scan_kernel(const __grid_constant__ ScanBatchOf<CAP> B, int G, int heads_per_pla
     float qa[NH];
 #pragma unroll
     for (int h = 0; h < NH; ++h) {
-      const float x = __ldg(B.q[it] + (size_t)(h0 + h) * FATHOM_D + tid);
+      const float x = *(const volatile float*)(B.q[it] + (size_t)(h0 + h) * FATHOM_D + tid);   // (a predecessor may have written it)
       M.q[h][tid] = x;
       qa[h] = fabsf(x);
     }

@@ -136,7 +136,7 @@ scan_simt_kernel(const __grid_constant__ ScanBatch B, int G, int heads_per_plan,
       const int j = M.row_ch[tid], p = M.row_pl[tid];
       const float pw = __int_as_float((130 - p) << 23);        // 2 * 8 * 2^-(p+1) = 2^(3-p), exact
 #pragma unroll
-      for (int h = 0; h < NH; ++h) M.qs[tid][h] = __ldg(B.q[it] + (size_t)(h0 + h) * FATHOM_D + j) * pw;
+      for (int h = 0; h < NH; ++h) M.qs[tid][h] = B.q[it][(size_t)(h0 + h) * FATHOM_D + j] * pw;
     }
   };
 
@@ -204,7 +204,7 @@ scan_simt_kernel(const __grid_constant__ ScanBatch B, int G, int heads_per_plan,
         const int j = M.row_ch[s0 + tid], p = M.row_pl[s0 + tid];
         const float pw = __int_as_float((130 - p) << 23);
 #pragma unroll
-        for (int h = 0; h < NH; ++h) M.qs[tid][h] = __ldg(B.q[item] + (size_t)(h0 + h) * FATHOM_D + j) * pw;
+        for (int h = 0; h < NH; ++h) M.qs[tid][h] = B.q[item][(size_t)(h0 + h) * FATHOM_D + j] * pw;
       }
       __syncthreads();
     }

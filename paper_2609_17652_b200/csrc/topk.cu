@@ -207,7 +207,7 @@ __device__ void find_threshold_bin(const uint32_t* __restrict__ h, uint32_t* __r
 constexpr int SAMPLE_THREADS = 1024;
 constexpr int SAMPLE_CLUSTER = 4;
 __global__ void __cluster_dims__(SAMPLE_CLUSTER, 1, 1) __launch_bounds__(SAMPLE_THREADS)
-topk_sample_kernel(const float* __restrict__ scores, long long sampled, long long chunk_stride, long long score_stride,
+topk_sample_kernel(const float* scores, long long sampled, long long chunk_stride, long long score_stride,
                    uint32_t* __restrict__ state, uint32_t want, uint32_t want_bound, uint32_t* __restrict__ cand_count,
                    uint32_t* __restrict__ cand_count2) {
   __shared__ uint32_t sh[FATHOM_TOPK_BINS];
@@ -228,13 +228,22 @@ topk_sample_kernel(const float* __restrict__ scores, long long sampled, long lon
   const float* row = scores + (size_t)head * (size_t)score_stride;
   // `sampled` whole chunks of 1024 scores, chunk_stride scores apart (16384: every 16th chunk of a score row; 1024: a
   // compact array of sampled scores); CTA `part` of the cluster takes every SAMPLE_CLUSTER-th group of 1024 float4
-#pragma unroll 4
-  for (long long v = (long long)part * SAMPLE_THREADS + threadIdx.x; v < sampled * 256; v += SAMPLE_CLUSTER * SAMPLE_THREADS) {
-    const float4 x = __ldg(reinterpret_cast<const float4*>(row + (v >> 8) * chunk_stride) + (v & 255));
-    atomicAdd(&sh[ordered_key(x.x) >> 20], 1u);
-    atomicAdd(&sh[ordered_key(x.y) >> 20], 1u);
-    atomicAdd(&sh[ordered_key(x.z) >> 20], 1u);
-    atomicAdd(&sh[ordered_key(x.w) >> 20], 1u);
+  constexpr int STRIDE = SAMPLE_CLUSTER * SAMPLE_THREADS, FLY = 4;            // loads in flight per thread
+  for (long long v0 = (long long)part * SAMPLE_THREADS + threadIdx.x; v0 < sampled * 256; v0 += FLY * STRIDE) {
+    float4 x[FLY];
+#pragma unroll
+    for (int u = 0; u < FLY; ++u) {
+      const long long v = v0 + u * STRIDE;
+      if (v < sampled * 256) x[u] = reinterpret_cast<const float4*>(row + (v >> 8) * chunk_stride)[v & 255];
+    }
+#pragma unroll
+    for (int u = 0; u < FLY; ++u) {
+      if (v0 + u * STRIDE >= sampled * 256) break;
+      atomicAdd(&sh[ordered_key(x[u].x) >> 20], 1u);
+      atomicAdd(&sh[ordered_key(x[u].y) >> 20], 1u);
+      atomicAdd(&sh[ordered_key(x[u].z) >> 20], 1u);
+      atomicAdd(&sh[ordered_key(x[u].w) >> 20], 1u);
+    }
   }
   __syncthreads();                                            // my histogram is complete
   cluster.barrier_wait(std::move(cleared));                   // (everyone arrived long ago: no wait in practice)
@@ -509,7 +518,7 @@ constexpr int FAST_EPT = 8;                                   // candidates per 
 // ROUNDS = 1: lists of up to 8192 candidates; 2: up to 16384 (a second round of loads once the length is known)
 template <int SMALL, int ROUNDS>
 __device__ __forceinline__ bool select_by_fine_histogram_rounds(
-    const float* __restrict__ cs, const int32_t* __restrict__ ci, uint32_t m, const float (&sc0)[FAST_EPT], const int32_t (&ix0)[FAST_EPT],
+    const float* cs, const int32_t* ci, uint32_t m, const float (&sc0)[FAST_EPT], const int32_t (&ix0)[FAST_EPT],
     uint32_t want, float lo, long long n, int k, int part,
     Forced F, unsigned char* s_dyn, uint32_t* s_fine, uint32_t* s_warp, int32_t* __restrict__ out, uint32_t* __restrict__ dev_status) {
   constexpr int EPT = FAST_EPT;
@@ -651,8 +660,8 @@ __device__ __forceinline__ bool select_by_fine_histogram_rounds(
 
 template <int SMALL>
 __device__ __forceinline__ bool select_by_fine_histogram(
-    const float* __restrict__ cs, const int32_t* __restrict__ ci, long long capacity, const uint32_t* __restrict__ count_ptr,
-    bool must_reach_want, uint32_t want, const uint32_t* __restrict__ lo_ptr, long long n, int k, int part,
+    const float* cs, const int32_t* ci, long long capacity, const uint32_t* count_ptr,
+    bool must_reach_want, uint32_t want, const uint32_t* lo_ptr, long long n, int k, int part,
     Forced F, unsigned char* s_dyn, uint32_t* s_fine, uint32_t* s_warp, int32_t* __restrict__ out, uint32_t* __restrict__ dev_status) {
   // ---- all loads in flight together (the candidate loads are speculative: the list's length is not known yet)
   const int tid = threadIdx.x;
@@ -685,13 +694,12 @@ __device__ __forceinline__ bool select_by_fine_histogram(
 constexpr int SORT_BUCKETS = 4096;
 template <bool DIRECT>
 __global__ void __launch_bounds__(FIN_THREADS)
-topk_select_kernel(const float* __restrict__ scores, long long n, long long score_stride, Forced F,
-                   const uint32_t* __restrict__ state, const int32_t* __restrict__ cand,
+topk_select_kernel(const float* scores, long long n, long long score_stride, Forced F, const uint32_t* state, const int32_t* cand,
                    uint32_t* __restrict__ bitmap, long long bitmap_words, int k, int32_t* __restrict__ idx_out,
                    uint32_t* __restrict__ dev_status, uint32_t* __restrict__ tile_count, int ntiles,
-                   const uint32_t* __restrict__ cand_count, long long cand_capacity, uint32_t want_direct, int bucket_shift,
-                   Gate gate, const float* __restrict__ collect_scores, long long collect_stride, float* __restrict__ collect_score_out,
-                   int32_t* __restrict__ collect_idx_out, int cache_entries, int lo_word, int parts, const uint32_t* __restrict__ cand_count_second) {
+                   const uint32_t* cand_count, long long cand_capacity, uint32_t want_direct, int bucket_shift,
+                   Gate gate, const float* collect_scores, long long collect_stride, float* collect_score_out, int32_t* collect_idx_out,
+                   int cache_entries, int lo_word, int parts, const uint32_t* cand_count_second) {
   constexpr int DIGIT_BITS = 11, DIGITS = 1 << DIGIT_BITS;    // radix of the candidate select
   constexpr int DPT = DIGITS / FIN_THREADS;                    // digits per thread in the suffix scan
   static_assert(FIN_THREADS == 1024, "one pair of s_diff words per lane; digits and ranges per thread");
@@ -766,7 +774,7 @@ topk_select_kernel(const float* __restrict__ scores, long long n, long long scor
 #pragma unroll
       for (int u = 0; u < 4; ++u) {
         const long long i = base + ((long long)u * FIN_THREADS + tid) * 4;
-        x[u] = i < n ? __ldg(reinterpret_cast<const float4*>(srow + i)) : make_float4(0.f, 0.f, 0.f, 0.f);
+        x[u] = i < n ? *reinterpret_cast<const float4*>(srow + i) : make_float4(0.f, 0.f, 0.f, 0.f);
       }
 #pragma unroll
       for (int u = 0; u < 4; ++u) {

@@ -107,7 +107,7 @@ __device__ __forceinline__ void find_bin(ResidentSmem& M, const uint32_t* hist, 
 
 template <int EPT>
 __global__ void __launch_bounds__(RT_THREADS, 2)
-topk_resident_kernel(const float* __restrict__ scores, int n, long long score_stride, int elig_lo, int elig_hi, int k, uint32_t want,
+topk_resident_kernel(const float* scores, int n, long long score_stride, int elig_lo, int elig_hi, int k, uint32_t want,
                      int by_maxima, uint32_t capacity, int32_t* __restrict__ idx_out, uint32_t* __restrict__ dev_status) {
   extern __shared__ __align__(16) unsigned char resident_smem[];
   ResidentSmem& M = *reinterpret_cast<ResidentSmem*>(resident_smem);
@@ -132,11 +132,11 @@ topk_resident_kernel(const float* __restrict__ scores, int n, long long score_st
     const float* src = row + wbase + 4 * lane;                // (score_stride is a multiple of 4: a float4 stays inside the row)
     if (wbase + 32 * EPT <= n) {                              // (uniform over the warp)
 #pragma unroll
-      for (int v = 0; v < V; ++v) *reinterpret_cast<float4*>(x + 4 * v) = __ldg(reinterpret_cast<const float4*>(src + 128 * v));
+      for (int v = 0; v < V; ++v) *reinterpret_cast<float4*>(x + 4 * v) = *reinterpret_cast<const float4*>(src + 128 * v);
     } else {
 #pragma unroll
       for (int v = 0; v < V; ++v)
-        *reinterpret_cast<float4*>(x + 4 * v) = token(4 * v) < n ? __ldg(reinterpret_cast<const float4*>(src + 128 * v)) : make_float4(NONE, NONE, NONE, NONE);
+        *reinterpret_cast<float4*>(x + 4 * v) = token(4 * v) < n ? *reinterpret_cast<const float4*>(src + 128 * v) : make_float4(NONE, NONE, NONE, NONE);
     }
     if (wbase < elig_lo || wbase + 32 * EPT > elig_hi) {
 #pragma unroll

@@ -77,3 +77,39 @@ def test_attention_over_few_rows(k, dtype):
     # logits below 12 in magnitude, each an fp32 sum of 128 products: their rounding, exponentiated, stays below 1e-5
     assert np.all(np.linalg.norm(out.cpu().numpy() - ref, axis=1) <= 2e-5 * np.linalg.norm(ref, axis=1))
     ctx.close()
+
+
+# every kernel of the chain may start while the one before it still writes; the buffers between them hold the step before's results
+def test_dependent_kernels_read_what_the_kernel_before_them_wrote():
+    from paper_2609_17652_b200 import binding as fb
+    n, Hkv, G, k, steps = 5003, 2, 4, 300, 12
+    Hq = Hkv * G
+    lay, staged = fb.make_layout(Hkv, Hq, n), fb.make_layout(Hkv, Hq, G * k)
+    ctx = fb.Context(0, max(fb.fathom_scratch_bytes(lay, k), fb.fathom_scratch_bytes(staged, k)))
+    g = torch.Generator(device="cuda").manual_seed(7)
+    K, V = (torch.randn(Hkv, n, 128, generator=g, device="cuda").to(torch.bfloat16) for _ in range(2))
+    # early steps take few distinct tokens, late ones many: a length or a list of the step before would show
+    scores = [torch.randn(Hq, lay.score_stride, generator=g, device="cuda") * t / steps for t in range(steps)]
+    shared = torch.randn(Hkv, 1, lay.score_stride, generator=g, device="cuda").expand(-1, G, -1).reshape(Hq, -1)
+    q = [torch.randn(Hq, 128, generator=g, device="cuda") for _ in range(steps)]
+    Ks, Vs = (torch.zeros(Hkv, G * k, 128, dtype=torch.bfloat16, device="cuda") for _ in range(2))
+    idx, local = (torch.zeros(Hq, k, dtype=torch.int32, device="cuda") for _ in range(2))
+    count, out = torch.zeros(Hkv, dtype=torch.int32, device="cuda"), torch.zeros(Hq, 128, device="cuda")
+    rows = [(shared + s).contiguous() for s in scores]
+    torch.cuda.synchronize()
+    seen = []
+    for s, x in zip(rows, q):
+        ctx.fathom_topk(lay, s, k, 0, 0, idx)
+        ctx.fathom_gather_union(lay, idx, k, K, V, Ks, Vs, local, count)
+        ctx.fathom_sparse_attend(staged, x, Ks, Vs, local, k, 1.0 / np.sqrt(128), out)
+        seen.append([t.clone() for t in (idx, local, count, out)])
+    for s, x, (i, l, c, o) in zip(rows, q, seen):
+        ref = O.topk(s[:, :n].double().cpu().numpy(), k, 0, 0)
+        assert np.array_equal(i.cpu().numpy(), ref)
+        for h in range(Hkv):
+            tokens = np.unique(ref[h * G:(h + 1) * G])
+            assert int(c[h]) == len(tokens) and np.array_equal(tokens[l[h * G:(h + 1) * G].cpu().numpy()], ref[h * G:(h + 1) * G])
+        exact = O.sparse_attend(x.cpu().numpy(), K.float().cpu().numpy(), V.float().cpu().numpy(), ref, 1.0 / np.sqrt(128))
+        # logits below 6 in magnitude, fp32 sums of 128 products
+        assert np.all(np.linalg.norm(o.cpu().numpy() - exact, axis=1) <= 2e-5 * np.linalg.norm(exact, axis=1))
+    ctx.close()
