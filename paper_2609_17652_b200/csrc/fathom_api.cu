@@ -28,13 +28,19 @@ fathom_topk_scratch fathom_carve_topk(void* base, int Hq, int64_t n, int k) {
   s.bitmap = reinterpret_cast<uint32_t*>(p + off);  off += fathom_round_up((size_t)Hq * (size_t)s.bitmap_words * 4, 256);
   s.cand = reinterpret_cast<int32_t*>(p + off);     off += fathom_round_up((size_t)Hq * (size_t)n * 4, 256);
   s.tile_count = reinterpret_cast<uint32_t*>(p + off); off += fathom_round_up((size_t)Hq * (size_t)((n + 8191) / 8192) * 4, 256);
-  s.cand_score = reinterpret_cast<float*>(p + off); off += fathom_round_up((size_t)Hq * (size_t)n * 4, 256);
+  const long long dense_stride = (n + 3) / 4 * 4;                           // a whole score row
+  s.cand_score = reinterpret_cast<float*>(p + off); off += fathom_round_up((size_t)Hq * (size_t)dense_stride * 4, 256);
   {
+    // Room for every 16th scan tile, whatever k: a context that serves a layout then serves every shorter one and every smaller k.
+    // Where the row is scanned whole the candidates' scores are not used, and the row lies there.
     const long long tile = fathom_scan_tile_tokens();
-    const int step = fathom_fused_tile_step(n, k);
-    const long long sampled = ((n + tile - 1) / tile + step - 1) / step;
-    s.sample_stride = step == 1 ? (long long)((n + 3) / 4 * 4) : sampled * tile;
-    s.sample = reinterpret_cast<float*>(p + off);   off += fathom_round_up((size_t)Hq * (size_t)s.sample_stride * 4, 256);
+    const long long sampled = ((n + tile - 1) / tile + 15) / 16 * tile;
+    s.sample = reinterpret_cast<float*>(p + off);   off += fathom_round_up((size_t)Hq * (size_t)(sampled < dense_stride ? sampled : dense_stride) * 4, 256);
+    s.sample_stride = sampled;
+    if (fathom_fused_tile_step(n, k) == 1) {
+      s.sample = s.cand_score;
+      s.sample_stride = dense_stride;
+    }
   }
   s.bytes = off;
   return s;

@@ -120,7 +120,7 @@ struct fathom_topk_scratch {
   int32_t* cand;         // [Hq][n] token indices of the threshold bin
   uint32_t* tile_count;  // [Hq][ceil(n / 8192)] selected tokens per filter tile, then their exclusive prefix
   float* cand_score;     // [Hq][n] scores of the fused path's candidates
-  float* sample;         // [Hq][sample_stride] scores of the sampled scan tiles (fused path)
+  float* sample;         // [Hq][sample_stride] scores of the sampled scan tiles (fused path); where all tiles are, the same memory as cand_score
   long long sample_stride;
   long long bitmap_words;
   size_t bytes;

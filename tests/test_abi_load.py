@@ -66,6 +66,23 @@ def test_scratch_bytes_and_host_side_rejection(fb):
     assert fb.lib.fathom_destroy(None) == 0
 
 
+@pytest.mark.parametrize("Hkv,Hq", [(1, 1), (8, 32), (8, 64)])
+def test_scratch_of_a_longer_session_serves_a_shorter_one(fb, Hkv, Hq):
+    """A program sizes its context for the longest session: the demand never falls as n or k grows, around the lengths at
+    which the selection changes its way in particular."""
+    lengths = sorted({1, 63, 64, 1000, 4096, 15360, 15361, 16384, 33001, 65536, 91136, 104448, 124928, 131071, 131072, 131073, 131200,
+                      150000, 180000, 262144, 262145, 278528, 278529, 500003, 524288, 540672, 540673, 1 << 20})
+    last_n = {}
+    for n in lengths:
+        last_k = 0
+        for k in (1, 64, 512, 2048, 4096, 8192, 16384):
+            if k > n:
+                break
+            need = fb.fathom_scratch_bytes(fb.make_layout(Hkv, Hq, n), k)
+            assert need >= last_k and need >= last_n.get(k, 0), (n, k)
+            last_k = last_n[k] = need
+
+
 def test_layer_budget_plan_host_function_matches_the_oracle(fb):
     """fathom_plan_layer_budgets is host code: compared here, level by level, with the oracle's greedy plan on random
     error tables (convex and not), uneven level spacing, ties and targets between two sums."""

@@ -36,6 +36,32 @@ def test_topk_of_rows_held_in_registers(n, k, n_sink, n_local, scores):
     ctx.close()
 
 
+# a context sized for one length serves every shorter one, over the lengths at which the selection changes its way
+@pytest.mark.parametrize("longest", [131073, 150001])
+def test_shorter_sessions_on_a_longer_sessions_context(longest):
+    from paper_2609_17652_b200 import binding as fb
+    Hq, k = 4, 64
+    ctx = fb.Context(0, fb.fathom_scratch_bytes(fb.make_layout(1, Hq, longest), k))
+    g = torch.Generator(device="cuda").manual_seed(longest)
+    for n in (longest, 131072, 104001, 33001, 64):
+        lay = fb.make_layout(1, Hq, n)
+        K = torch.randn(1, n, 128, generator=g, device="cuda")
+        q = torch.randn(Hq, 128, generator=g, device="cuda")
+        planes = torch.zeros(1, 128, 4, lay.plane_stride_words, dtype=torch.int64, device="cuda")
+        scales = torch.zeros(1, 128, lay.scale_stride, dtype=torch.int16, device="cuda")
+        depth = torch.zeros(1, 128, dtype=torch.uint8, device="cuda")
+        scores = torch.zeros(Hq, lay.score_stride, device="cuda")
+        idx, fused = (torch.full((Hq, k), -1, dtype=torch.int32, device="cuda") for _ in range(2))
+        ctx.fathom_build_planes(lay, K, planes, scales)
+        ctx.fathom_alloc_depth(lay, q, K.var(dim=1), fb.DEPTH_WATERFILL, 48, 4, depth)
+        ctx.fathom_scan(lay, planes, scales, q, depth, 4, scores)
+        ctx.fathom_topk(lay, scores, k, 0, 0, idx)
+        ctx.fathom_scan_topk(lay, planes, scales, q, depth, 4, k, 0, 0, fused)
+        assert np.array_equal(idx.cpu().numpy(), O.topk(scores[:, :n].double().cpu().numpy(), k, 0, 0)), n
+        assert torch.equal(idx, fused), n
+    ctx.close()
+
+
 # the longest sequence whose bitmap fits in shared memory and one token more; an odd length with picks in its first and last word
 @pytest.mark.parametrize("n,k", [(33, 33), (70001, 700), (52 * 1024 * 32, 2048), (52 * 1024 * 32 + 1, 2048)])
 def test_union_of_picks_on_both_sides_of_the_bitmap_limit(n, k):
