@@ -9,8 +9,9 @@
 #define PY_SSIZE_T_CLEAN
 #include <Python.h>
 
+#include <climits>
 #include <cstring>
-#include <vector>
+#include <memory>
 
 #include "fathom.h"
 
@@ -243,7 +244,17 @@ PyObject* m_fathom_scan_batch(PyObject* self, PyObject* const* args, Py_ssize_t 
   PyObject* seq = PySequence_Fast(got[0], "items must be a sequence");
   if (!seq) return nullptr;
   const Py_ssize_t n = PySequence_Fast_GET_SIZE(seq);
-  std::vector<fathom_scan_item> items((size_t)n);
+  if (n > INT_MAX) {
+    Py_DECREF(seq);
+    PyErr_SetString(PyExc_OverflowError, "too many items");
+    return nullptr;
+  }
+  struct Free { void operator()(void* p) const { PyMem_Free(p); } };
+  std::unique_ptr<fathom_scan_item[], Free> items(static_cast<fathom_scan_item*>(PyMem_Malloc((size_t)n * sizeof(fathom_scan_item))));
+  if (!items) {
+    Py_DECREF(seq);
+    return PyErr_NoMemory();
+  }
   bool ok = true;
   for (Py_ssize_t i = 0; i < n && ok; ++i) {
     PyObject* t = PySequence_Fast(PySequence_Fast_GET_ITEM(seq, i), "an item is (layout, planes, scales, q, depth, scores)");
@@ -271,7 +282,7 @@ PyObject* m_fathom_scan_batch(PyObject* self, PyObject* const* args, Py_ssize_t 
   if (!ok || !integer(got[1], &hpp) || !stream_of(got[2], &st)) return nullptr;
   fathom_ctx* ctx = reinterpret_cast<ContextObject*>(self)->ctx;
   int rc;
-  Py_BEGIN_ALLOW_THREADS rc = fathom_scan_batch(ctx, items.data(), (int)n, hpp, st);
+  Py_BEGIN_ALLOW_THREADS rc = fathom_scan_batch(ctx, items.get(), (int)n, hpp, st);
   Py_END_ALLOW_THREADS
   return finish(rc, ctx);
 }

@@ -3,6 +3,8 @@ and rejects bad arguments on the host before any launch."""
 import ctypes as C
 import os
 import re
+import subprocess
+import sys
 
 import pytest
 
@@ -81,6 +83,23 @@ def test_scratch_of_a_longer_session_serves_a_shorter_one(fb, Hkv, Hq):
             need = fb.fathom_scratch_bytes(fb.make_layout(Hkv, Hq, n), k)
             assert need >= last_k and need >= last_n.get(k, 0), (n, k)
             last_k = last_n[k] = need
+
+
+def test_a_batch_without_room_for_its_items_raises(fb):
+    """The call layer's item list of a large batch does not fit: a MemoryError, not the end of the process."""
+    code = """
+import resource
+from paper_2609_17652_b200 import binding as fb
+items = [(fb.make_layout(1, 1, 64), 16, 16, 16, 16, 16)] * 20_000_000
+used = int(open('/proc/self/statm').read().split()[0]) * resource.getpagesize()
+resource.setrlimit(resource.RLIMIT_AS, (used + (1 << 28), -1))       # 2 GB are asked for
+try:
+    fb._native.ContextCalls().fathom_scan_batch(items, 1, 0)
+except MemoryError:
+    print('refused')
+"""
+    run = subprocess.run([sys.executable, "-c", code], cwd=ROOT, capture_output=True, text=True)
+    assert run.returncode == 0 and run.stdout.strip() == "refused", run.stderr[-500:]
 
 
 def test_layer_budget_plan_host_function_matches_the_oracle(fb):
