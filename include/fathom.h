@@ -93,10 +93,11 @@ const char* fathom_strerror(int status);
 const char* fathom_last_cuda_error(const fathom_ctx* ctx);
 /* Copies the device status word to *status (host pointer) and clears it.  Synchronises `stream`. */
 int fathom_device_status(fathom_ctx* ctx, void* stream, uint32_t* status);
-/* Self-test of the bounded device-side waits (the paper has no counterpart): enqueues a one-warp kernel in which one
- * thread polls, at most `tries` (1 .. 4096) times, a barrier that nothing will ever complete - no copy or tensor-core
- * operation is outstanding - then sets FATHOM_DEV_WAIT_EXPIRED in the status word and returns.  The kernels that wait
- * on copies or tensor-core work take the same path when a wait runs out; the context stays usable afterwards. */
+/* Self-test of the bounded device-side waits (the paper has no counterpart): enqueues a one-warp kernel whose lanes poll,
+ * at most `tries` (1 .. 4096) times, a barrier that nothing will ever complete - no copy or tensor-core operation is
+ * outstanding - and then one for which only some of the lanes give up.  If the whole warp agrees that both waits ran out it
+ * sets FATHOM_DEV_WAIT_EXPIRED in the status word, and it returns either way.  The kernels that wait on copies or
+ * tensor-core work take the same path when a wait runs out; the context stays usable afterwards. */
 int fathom_selftest_wait_expiry(fathom_ctx* ctx, int tries, void* stream);
 /* Library version, major * 100 + minor. */
 int fathom_version(void);

@@ -138,16 +138,29 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, uint32_
   return false;
 }
 
-// The give-up path of the bounded wait, exercised on its own: one thread waits `tries` times on a barrier that nothing will
-// ever arrive on (no copy, no MMA, nothing asynchronous is outstanding), reports FATHOM_DEV_WAIT_EXPIRED and returns.
+// The same for a whole warp whose lanes all poll (each of them reads what has arrived): false in every lane if the limit ran out for
+// any.  A warp that disagreed would split at the next branch on the answer, and lanes that give up would leave the others in a
+// full-mask shuffle.
+__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, uint32_t tries = WAIT_TRIES) {
+  return __all_sync(0xffffffffu, mbar_wait(bar, parity, tries)) != 0;
+}
+
+// The give-up path of the bounded waits, exercised on its own (no copy, no MMA, nothing asynchronous is outstanding): one warp
+// waits `tries` times on a barrier that nothing will ever arrive on, and on one whose phase is complete with a limit that has run
+// out for its odd lanes.  If all lanes say that both waits gave up, FATHOM_DEV_WAIT_EXPIRED is reported.
 __global__ void wait_expiry_selftest_kernel(uint32_t* dev_status, uint32_t tries) {
-  __shared__ __align__(8) uint64_t bar;
-  const uint32_t b = (uint32_t)__cvta_generic_to_shared(&bar);
+  __shared__ __align__(8) uint64_t bars[2];
+  const uint32_t never = (uint32_t)__cvta_generic_to_shared(&bars[0]), complete = never + 8;
   if (threadIdx.x == 0) {
-    mbar_init(b, 1);
+    mbar_init(never, 1);
+    mbar_init(complete, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    if (!mbar_wait(b, 0, tries)) atomicOr(dev_status, FATHOM_DEV_WAIT_EXPIRED);
+    asm volatile("mbarrier.arrive.release.cta.shared::cta.b64 _, [%0];" :: "r"(complete) : "memory");
   }
+  __syncwarp();
+  const bool gave_up = !mbar_wait_warp(never, 0, tries), split = !mbar_wait_warp(complete, 0, threadIdx.x & 1 ? 0u : tries);
+  const bool all = __all_sync(0xffffffffu, gave_up && split) != 0;
+  if (threadIdx.x == 0 && all) atomicOr(dev_status, FATHOM_DEV_WAIT_EXPIRED);
 }
 
 __device__ __forceinline__ bool elect_one() {
@@ -251,7 +264,7 @@ rotate_tc_kernel(const T* __restrict__ K, const float* __restrict__ mean, const 
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = *s_tmem;
 
-  bool alive = true;                                          // false once a bounded wait ran out
+  bool alive = true;                                          // false once a bounded wait ran out; the same in all lanes of a warp
   // one lane polls for its warp
   auto wait = [&](uint32_t bar, uint32_t parity) {
     if (alive) {
@@ -328,7 +341,7 @@ rotate_tc_kernel(const T* __restrict__ K, const float* __restrict__ mean, const 
         unsigned char* group = sm + stage * STAGE_BYTES + warp * GROUP_BYTES;
         unsigned char* to = group + (c0 / HALF_CH) * 1024;
         float* factor = s_factor + (tcount % FACTORS) * TILE_M + warp * GROUP;
-        if (tcount < requested && !mbar_wait(bar_raw + 8 * (stage * GROUPS + warp), (tcount / STAGES) & 1u)) alive = false;
+        if (tcount < requested && !mbar_wait_warp(bar_raw + 8 * (stage * GROUPS + warp), (tcount / STAGES) & 1u)) alive = false;
         uint4 xr[LOADS];
 #pragma unroll
         for (int i = 0; i < LOADS; ++i) xr[i] = reinterpret_cast<const uint4*>(group)[i * 32 + lane];
@@ -381,8 +394,8 @@ rotate_tc_kernel(const T* __restrict__ K, const float* __restrict__ mean, const 
       for (long long t = 0; t < count; ++t, ++tcount) {
         const uint32_t buf = tcount & 1u, acc = tm + COL_ACC + buf * 128u;
         const uint32_t stage = tcount % STAGES, phase = (tcount / STAGES) & 1u;
-        if (alive && !mbar_wait(bar_acc_empty + 8 * buf, ((tcount >> 1) & 1u) ^ 1u)) alive = false;
-        if (alive && !ready && !mbar_wait(bar_full + 8 * stage, phase)) alive = false;
+        if (alive && !mbar_wait_warp(bar_acc_empty + 8 * buf, ((tcount >> 1) & 1u) ^ 1u)) alive = false;
+        if (alive && !ready && !mbar_wait_warp(bar_full + 8 * stage, phase)) alive = false;
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         const uint32_t slab = base + stage * STAGE_BYTES;
         if (elect_one()) {
@@ -402,7 +415,7 @@ rotate_tc_kernel(const T* __restrict__ K, const float* __restrict__ mean, const 
           umma_commit(bar_acc_full + 8 * buf);
           mbar_arrive(bar_acc_full + 8 * buf);
         }
-        ready = mbar_test(bar_full + 8 * ((tcount + 1) % STAGES), ((tcount + 1) / STAGES) & 1u);
+        ready = __all_sync(0xffffffffu, mbar_test(bar_full + 8 * ((tcount + 1) % STAGES), ((tcount + 1) / STAGES) & 1u)) != 0;
         __syncwarp();
       }
     } else {

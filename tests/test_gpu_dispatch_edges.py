@@ -139,3 +139,19 @@ def test_dependent_kernels_read_what_the_kernel_before_them_wrote():
         # logits below 6 in magnitude, fp32 sums of 128 products
         assert np.all(np.linalg.norm(o.cpu().numpy() - exact, axis=1) <= 2e-5 * np.linalg.norm(exact, axis=1))
     ctx.close()
+
+
+# limits on both sides of the point from which a wait sleeps between polls; part of the warp gives up before the rest
+@pytest.mark.parametrize("tries", [1, 64, 66, 4096])
+def test_a_warp_agrees_that_its_wait_ran_out(tries):
+    from paper_2609_17652_b200 import binding as fb
+    lay = fb.make_layout(1, 1, 300)
+    ctx = fb.Context(0, fb.fathom_scratch_bytes(lay, 64))
+    ctx.fathom_selftest_wait_expiry(tries)
+    assert ctx.fathom_device_status() == fb.DEV_WAIT_EXPIRED
+    K = torch.randn(1, 300, 128, device="cuda")
+    out = torch.zeros_like(K)
+    ctx.fathom_rotate_keys(lay, K, torch.zeros(1, 128, device="cuda"), torch.eye(128, device="cuda").unsqueeze(0).contiguous(), out)
+    # the identity moves no key: what is left out of head and tail of both operands is below 2^-21 of it
+    assert ctx.fathom_device_status() == 0 and torch.allclose(out, K, rtol=2.0 ** -21, atol=1e-9)
+    ctx.close()
