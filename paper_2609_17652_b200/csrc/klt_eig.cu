@@ -357,7 +357,7 @@ klt_eig_kernel(const float* cov, float* basis_out, float* __restrict__ eigenvalu
 
   FATHOM_PDL_WAIT();                                          // the covariance comes from the previous kernel
   FATHOM_PDL_RELEASE();
-  // ---- 1. fp32 sweeps; the accumulated basis goes through the output buffer to every CTA
+  // ---- 1. fp32 sweeps.  (The output is written when the covariance has been read for the last time: it may be the same buffer)
   if (part == 0) {
     float m = 0.0f;                                           // scaled by a power of two so that the largest diagonal element is near one
     for (int i = lane; i < N; i += 32) m = fmaxf(m, fabsf(C[i * N + i]));
@@ -369,8 +369,6 @@ klt_eig_kernel(const float* cov, float* basis_out, float* __restrict__ eigenvalu
     for (int e = tid; e < rows * N; e += EIG_THREADS) V[e] = (e >> 7) + first_row == (e & (N - 1)) ? 1.0f : 0.0f;
     __syncthreads();
     apply_sweeps(M, M0, cluster, V, rows);
-    __syncthreads();
-    for (int e = tid; e < rows * N; e += EIG_THREADS) basis[first_row * N + e] = V[e];
   }
   cluster.sync();
 
@@ -427,20 +425,34 @@ klt_eig_kernel(const float* cov, float* basis_out, float* __restrict__ eigenvalu
     __syncthreads();
   };
   auto as_is = [](int, int, double v) { return v; };
-  auto load_full = [&](const float* from) {                   // a 128 x 128 matrix of floats, all loads in flight together
-    constexpr int PER = (N * N / 4 + EIG_THREADS - 1) / EIG_THREADS;
-    float4 v[PER];
+  constexpr int FULL = (N * N / 4 + EIG_THREADS - 1) / EIG_THREADS;
+  auto store_full = [&](const float4 (&v)[FULL]) {
 #pragma unroll
-    for (int u = 0; u < PER; ++u)
-      if (tid + u * EIG_THREADS < N * N / 4) v[u] = __ldcg(reinterpret_cast<const float4*>(from) + tid + u * EIG_THREADS);
-#pragma unroll
-    for (int u = 0; u < PER; ++u) {
+    for (int u = 0; u < FULL; ++u) {
       const int e = 4 * (tid + u * EIG_THREADS);
       if (e < N * N) {
         double* to = X + (e >> 7) * LDX + (e & (N - 1));
         to[0] = v[u].x; to[1] = v[u].y; to[2] = v[u].z; to[3] = v[u].w;
       }
     }
+    __syncthreads();
+  };
+  auto load_covariance = [&]() {                              // all loads in flight together
+    float4 v[FULL];
+#pragma unroll
+    for (int u = 0; u < FULL; ++u)
+      if (tid + u * EIG_THREADS < N * N / 4) v[u] = __ldcg(reinterpret_cast<const float4*>(C) + tid + u * EIG_THREADS);
+    store_full(v);
+  };
+  auto load_basis = [&]() {                                   // the rows that the sweeps left in the other CTAs
+    float4 v[FULL];
+#pragma unroll
+    for (int u = 0; u < FULL; ++u) {
+      const int e = tid + u * EIG_THREADS, i = e / (N / 4);
+      if (e < N * N / 4) v[u] = reinterpret_cast<const float4*>(cluster.map_shared_rank(M.A, 1 + i / V_ROWS))[i % V_ROWS * (N / 4) + e % (N / 4)];
+    }
+    cluster.sync();                                           // (X lies where the rows do)
+    store_full(v);
   };
   auto gather = [&]() {                                       // X = the columns M.W of all CTAs, four CTAs' in flight together
     constexpr int PER = (N * COLS + EIG_THREADS - 1) / EIG_THREADS;
@@ -462,8 +474,7 @@ klt_eig_kernel(const float* cov, float* basis_out, float* __restrict__ eigenvalu
     }
     __syncthreads();
   };
-  load_full(basis);
-  __syncthreads();
+  load_basis();
   double worst = 0.0;                                         // the largest product of two tangents in a column
   for (int round = 0; round < MAX_FINISHES; ++round) {
     // one step squares the distance from orthonormal, 1e-6 after the fp32 sweeps; after a round it is the worst product
@@ -475,8 +486,7 @@ klt_eig_kernel(const float* cov, float* basis_out, float* __restrict__ eigenvalu
       gather();
       cluster.sync();                                         // (read by everyone before they are rewritten)
     }
-    load_full(C);
-    __syncthreads();
+    load_covariance();
     for (int e = tid; e < N * N; e += EIG_THREADS) {          // the symmetric part, exactly
       const int i = e >> 7, j = e & (N - 1);
       if (i < j) X[i * LDX + j] = X[j * LDX + i] = 0.5 * (X[i * LDX + j] + X[j * LDX + i]);

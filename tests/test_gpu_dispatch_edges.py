@@ -155,3 +155,25 @@ def test_a_warp_agrees_that_its_wait_ran_out(tries):
     # the identity moves no key: what is left out of head and tail of both operands is below 2^-21 of it
     assert ctx.fathom_device_status() == 0 and torch.allclose(out, K, rtol=2.0 ** -21, atol=1e-9)
     ctx.close()
+
+
+# the basis may replace the covariance: finished in fp64 rounds, and by the sweeps that go on where eigenvalues are close
+@pytest.mark.parametrize("spread", [100.0, 1e-5])
+def test_klt_basis_in_place(spread):
+    from paper_2609_17652_b200 import binding as fb
+    kv = 3
+    lay = fb.make_layout(kv, kv, 1000)
+    ctx = fb.Context(0, 0)
+    g = torch.Generator(device="cuda").manual_seed(3)
+    Q = torch.linalg.qr(torch.randn(kv, 128, 128, generator=g, device="cuda").double())[0]
+    cov = ((Q * (1.0 + spread * torch.linspace(0, 1, 128, device="cuda").double())) @ Q.transpose(1, 2)).float()
+    cov = (0.5 * (cov + cov.transpose(1, 2))).contiguous()
+    basis, eig = torch.zeros_like(cov), torch.zeros(kv, 128, device="cuda")
+    ctx.fathom_klt_basis(lay, cov, basis, eig)
+    again, eig_again = cov.clone(), torch.zeros_like(eig)
+    ctx.fathom_klt_basis(lay, again, again, eig_again)
+    assert torch.equal(again, basis) and torch.equal(eig_again, eig)
+    B = basis.double()
+    # directions are rounded to fp32 (where fp64 sweeps go on they apply their rotations in fp32: 2e-6 measured)
+    assert (B.transpose(1, 2) @ B - torch.eye(128, device="cuda").double()).norm() / np.sqrt(128 * kv) < 1e-5
+    ctx.close()
