@@ -10,7 +10,8 @@
 //           then read over the host link exactly once).
 // The fetch of an offloaded step is bound by the link; what was left to save is the time in which the link is idle: clearing,
 // marking and ranking a bitmap in global memory were three launches in front of it (12 us a session, now 5).  A sequence whose
-// bitmap does not fit in shared memory (more than 1.7 M tokens) still takes those.
+// bitmap does not fit in shared memory (more than 1.7 M tokens) still takes those, and so do picks in such numbers that one CTA
+// lists them more slowly than the whole chip marks them (list_in_one_cta).
 #include "fathom_common.cuh"
 
 namespace {
@@ -20,6 +21,11 @@ constexpr int RANK_THREADS = 1024;
 
 constexpr long long LIST_MAX_WORDS = 52 * 1024;              // bitmap words (32 tokens each) kept in shared memory: 208 KB
 constexpr int LIST_THREADS = 1024;
+
+// One CTA per KV head takes about a nanosecond a pick; the kernels over the whole chip take what their launches and their pass over
+// the bitmap cost.  8 KV heads, bf16 rows in device memory, us with one CTA / with the chip: 131,072 tokens, 2048 picks 8.4 / 12.0,
+// 8192 picks 18.5 / 17.3, 32,768 picks 80 / 62; 600,000 tokens, 8192 picks 27 / 33, 16,384 picks 51 / 46.
+static bool list_in_one_cta(long long picks, long long n, long long words) { return words <= LIST_MAX_WORDS && picks <= 4096 + n / 64; }
 
 // Thread t owns `per` consecutive words (an odd multiple of four: 16-byte reads without bank conflicts), so that one block prefix
 // ranks the whole bitmap.
@@ -212,7 +218,7 @@ extern "C" int fathom_gather_union(fathom_ctx* ctx, const fathom_layout* L, cons
   uint32_t* word_rank = reinterpret_cast<uint32_t*>(base + bm_bytes);
   int32_t* ulist = reinterpret_cast<int32_t*>(base + 2 * bm_bytes);
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  if (words <= LIST_MAX_WORDS) {
+  if (list_in_one_cta(cap_ll, L->n, words)) {
     const int per = (int)(((words + LIST_THREADS * 4 - 1) / (LIST_THREADS * 4)) | 1) * 4;
     static bool configured[64] = {};
     if (ctx->device < 0 || ctx->device >= 64 || !configured[ctx->device]) {

@@ -177,3 +177,26 @@ def test_klt_basis_in_place(spread):
     # directions are rounded to fp32 (where fp64 sweeps go on they apply their rotations in fp32: 2e-6 measured)
     assert (B.transpose(1, 2) @ B - torch.eye(128, device="cuda").double()).norm() / np.sqrt(128 * kv) < 1e-5
     ctx.close()
+
+
+# picks on both sides of the line between one CTA per KV head and the whole chip
+@pytest.mark.parametrize("n,k", [(20000, 1102), (20000, 1103), (70001, 4000)])
+def test_union_of_many_picks(n, k):
+    from paper_2609_17652_b200 import binding as fb
+    Hkv, G = 2, 4
+    r = np.random.default_rng(k)
+    idx = np.stack([np.sort(r.choice(n, k, replace=False)) for _ in range(Hkv * G)]).astype(np.int32)
+    lay = fb.make_layout(Hkv, Hkv * G, n)
+    ctx = fb.Context(0, fb.fathom_scratch_bytes(lay, k))
+    K = torch.randn(Hkv, n, 128, device="cuda")
+    Ks, Vs = (torch.zeros(Hkv, G * k, 128, device="cuda") for _ in range(2))
+    local = torch.full((Hkv * G, k), -1, dtype=torch.int32, device="cuda")
+    count = torch.zeros(Hkv, dtype=torch.int32, device="cuda")
+    ctx.fathom_gather_union(lay, torch.from_numpy(idx).cuda(), k, K, K, Ks, Vs, local, count)
+    for h in range(Hkv):
+        tokens = np.unique(idx[h * G:(h + 1) * G])
+        assert int(count[h]) == len(tokens)
+        assert np.array_equal(tokens[local[h * G:(h + 1) * G].cpu().numpy()], idx[h * G:(h + 1) * G])
+        rows = K[h][torch.from_numpy(tokens.astype(np.int64)).cuda()]
+        assert torch.equal(Ks[h, :len(tokens)], rows) and torch.equal(Vs[h, :len(tokens)], rows)
+    ctx.close()
