@@ -64,7 +64,9 @@ static_assert(2 * DEEP_WORDS + (MAX_KSTEPS - STAGE_KSTEPS) * 32 * 8 <= 2 * STAGE
 // into the CTA's four candidate lists (one shared-memory atomic per head); the lists go to the heads' global lists once,
 // when the CTA has scanned its last tile (one global atomic per head and CTA).
 constexpr int PARK_RING = 64;                                // parked groups per warp
-constexpr int CAND_LIST = 128;                               // candidates per head the CTA keeps; beyond that: straight to the global list
+constexpr int CAND_LIST = 512;                               // candidates the CTA keeps, shared out evenly to its heads; beyond that: straight to the global list,
+                                                             // with one atomic per warp, head and round (one per candidate: 500,003 tokens, 4096 of 32 heads
+                                                             // with a plan each, budget 48: 155 us instead of 102; 8192 of 32 heads, budget 16: 96 instead of 76)
 
 template <int MODE>
 struct alignas(16) Smem {
@@ -80,7 +82,7 @@ struct alignas(16) Smem {
   alignas(16) float4 park_lo[MODE == 2 ? WARPS * PARK_RING : 1];     // MODE 2: scores 0..3 of a parked group
   alignas(16) float4 park_hi[MODE == 2 ? WARPS * PARK_RING : 1];     //         scores 4..7
   uint32_t park_tok[MODE == 2 ? WARPS * PARK_RING : 1];       //         its first token (30 bits) and the head within the CTA (2 bits)
-  uint2 clist[MODE == 2 ? 4 * CAND_LIST : 1];                 // MODE 2: (score bits, token) per head
+  uint2 clist[MODE == 2 ? CAND_LIST : 1];                     // MODE 2: (score bits, token) per head
   alignas(16) uint2 bfr[STAGE_KSTEPS][32];                    // right operand of the first 96 rows: per 16 rows, the two B registers of every lane
   alignas(16) unsigned char words[2 * STAGE_WORDS];           // staged plane words, double buffered; deep plans: + the other rows' right operand
   alignas(16) unsigned char scale[2 * STAGE_SCALES];          // staged fp16 scales, double buffered
@@ -149,6 +151,7 @@ scan_kernel(const __grid_constant__ ScanBatchOf<CAP> B, int G, int heads_per_pla
   if ((int)blockIdx.x >= total) return;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   constexpr bool in_hbm = IN_HBM;
+  constexpr int HEAD_LIST = CAND_LIST / NH;
   const int gq = lane >> 2, t4 = lane & 3;                     // mma fragment coordinates: lane = (row group, column pair)
   const int h0 = blockIdx.y * NH;                              // first of the NH query heads of this CTA
   const int plan = h0 / heads_per_plan;                        // NH divides heads_per_plan: one plan per CTA
@@ -280,11 +283,11 @@ scan_kernel(const __grid_constant__ ScanBatchOf<CAP> B, int G, int heads_per_pla
     if (MODE != 2) return;
     __syncwarp();                                              // the parked groups are visible to the whole warp
     const uint32_t elo = M.elig[0], ehi = M.elig[1];
-    auto append = [&](uint32_t h, uint32_t pos, float val, uint32_t token) {
-      if (pos < (uint32_t)CAND_LIST) {
-        M.clist[h * CAND_LIST + pos] = make_uint2(__float_as_uint(val), token);
-      } else {                                                 // list full (only with a threshold far too low): straight to the global list
-        const uint32_t at = atomicAdd(&fz.cand_count[h0 + h], 1u);
+    auto append = [&](uint32_t h, uint32_t pos, float val, uint32_t token, uint32_t beyond) {
+      if (pos < (uint32_t)HEAD_LIST) {
+        M.clist[h * HEAD_LIST + pos] = make_uint2(__float_as_uint(val), token);
+      } else {                                                 // list full: straight to the global list, where a place has been reserved, or at one's own
+        const uint32_t at = beyond != 0xffffffffu ? beyond : atomicAdd(&fz.cand_count[h0 + h], 1u);
         if ((long long)at < fz.capacity) {
           fz.cand_score[(size_t)(h0 + h) * fz.capacity + at] = val;
           fz.cand_idx[(size_t)(h0 + h) * fz.capacity + at] = (int32_t)token;
@@ -312,17 +315,23 @@ scan_kernel(const __grid_constant__ ScanBatchOf<CAP> B, int G, int heads_per_pla
         if (h == (uint32_t)hh) rank = __popc(with & ((1u << lane) - 1u));
         if (lane == hh) tot = __popc(with);
       }
-      if (lane < 4 && tot) base = atomicAdd(&M.ccount[lane], tot);
+      uint32_t over = 0u;                                      // where those of my head that do not fit start in the global list
+      if (lane < 4 && tot) {
+        base = atomicAdd(&M.ccount[lane], tot);
+        const uint32_t fits = base < (uint32_t)HEAD_LIST ? min(tot, (uint32_t)HEAD_LIST - base) : 0u;
+        if (fits < tot) over = atomicAdd(&fz.cand_count[h0 + lane], tot - fits) - fits;
+      }
       base = __shfl_sync(0xffffffffu, base, (int)h);
+      over = __shfl_sync(0xffffffffu, over, (int)h);
       if (mask) {
         const uint32_t x = (uint32_t)__ffs((int)mask) - 1u;
         mask &= mask - 1u;
-        append(h, base + rank, score_at(x), tok + x);
+        append(h, base + rank, score_at(x), tok + x, over + rank);
       }
       while (mask) {                                           // a second candidate in one group of eight: rare
         const uint32_t x = (uint32_t)__ffs((int)mask) - 1u;
         mask &= mask - 1u;
-        append(h, atomicAdd(&M.ccount[h], 1u), score_at(x), tok + x);
+        append(h, atomicAdd(&M.ccount[h], 1u), score_at(x), tok + x, 0xffffffffu);
       }
     }
     parked = 0u;
@@ -556,7 +565,7 @@ scan_kernel(const __grid_constant__ ScanBatchOf<CAP> B, int G, int heads_per_pla
     sift();
     __syncthreads();
     if (tid < NH) {
-      const uint32_t c = min(M.ccount[tid], (uint32_t)CAND_LIST);
+      const uint32_t c = min(M.ccount[tid], (uint32_t)HEAD_LIST);
       M.ccount[tid] = c;
       M.cbase[tid] = c ? atomicAdd(&fz.cand_count[h0 + tid], c) : 0u;
     }
@@ -566,7 +575,7 @@ scan_kernel(const __grid_constant__ ScanBatchOf<CAP> B, int G, int heads_per_pla
       const uint32_t c = M.ccount[h], at = M.cbase[h];
       for (uint32_t e = tid; e < c; e += THREADS)
         if ((long long)(at + e) < fz.capacity) {
-          const uint2 it = M.clist[h * CAND_LIST + e];
+          const uint2 it = M.clist[h * HEAD_LIST + e];
           fz.cand_score[(size_t)(h0 + h) * fz.capacity + at + e] = __uint_as_float(it.x);
           fz.cand_idx[(size_t)(h0 + h) * fz.capacity + at + e] = (int32_t)it.y;
         }
@@ -680,7 +689,7 @@ int fathom_launch_scan_sample(const fathom_layout* L, const uint64_t* planes, co
   fathom_scan_fuse fz = {};
   fz.tile_step = tile_step;
   return dispatch_scan<1>(single_item(L, planes, scales, q, depth, sample, sample_stride, tile_step), L->n_kv_heads, L->n_q_heads,
-                          heads_per_plan, fz, false, st);
+                          heads_per_plan, fz, true, st);
 }
 
 int fathom_launch_scan_filter(const fathom_layout* L, const uint64_t* planes, const uint16_t* scales, const float* q,

@@ -200,3 +200,30 @@ def test_union_of_many_picks(n, k):
         rows = K[h][torch.from_numpy(tokens.astype(np.int64)).cuda()]
         assert torch.equal(Ks[h, :len(tokens)], rows) and torch.equal(Vs[h, :len(tokens)], rows)
     ctx.close()
+
+
+# one CTA per plan: its candidate lists run over (1200 of them for 512, 256 and 128 places a head)
+@pytest.mark.parametrize("heads_per_plan", [1, 2, 4])
+def test_fused_selection_with_more_candidates_than_a_cta_lists(heads_per_plan):
+    from paper_2609_17652_b200 import binding as fb
+    n, Hq, k = 140001, 4, 1200
+    lay = fb.make_layout(1, Hq, n)
+    ctx = fb.Context(0, fb.fathom_scratch_bytes(lay, k))
+    g = torch.Generator(device="cuda").manual_seed(heads_per_plan)
+    K, q = torch.randn(1, n, 128, generator=g, device="cuda"), torch.randn(Hq, 128, generator=g, device="cuda")
+    planes = torch.zeros(1, 128, 4, lay.plane_stride_words, dtype=torch.int64, device="cuda")
+    scales = torch.zeros(1, 128, lay.scale_stride, dtype=torch.int16, device="cuda")
+    depth = torch.zeros(Hq // heads_per_plan, 128, dtype=torch.uint8, device="cuda")
+    scores = torch.zeros(Hq, lay.score_stride, device="cuda")
+    fused = torch.full((Hq, k), -1, dtype=torch.int32, device="cuda")
+    ctx.fathom_build_planes(lay, K, planes, scales)
+    ctx.fathom_alloc_depth(lay, q, K.var(dim=1), fb.DEPTH_WATERFILL, 32, heads_per_plan, depth)
+    ctx.fathom_scan(lay, planes, scales, q, depth, heads_per_plan, scores)
+    fb.fathom_scan_set_ctas_per_plan(1)
+    try:
+        ctx.fathom_scan_topk(lay, planes, scales, q, depth, heads_per_plan, k, 4, 32, fused)
+    finally:
+        fb.fathom_scan_set_ctas_per_plan(0)
+    assert np.array_equal(fused.cpu().numpy(), O.topk(scores[:, :n].double().cpu().numpy(), k, 4, 32))
+    assert ctx.fathom_device_status() == 0
+    ctx.close()
