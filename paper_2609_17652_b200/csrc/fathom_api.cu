@@ -16,7 +16,7 @@ int fathom_check_layout(const fathom_layout* L) {
   return FATHOM_OK;
 }
 
-fathom_topk_scratch fathom_carve_topk(void* base, int Hq, int64_t n, int k) {
+fathom_topk_scratch fathom_carve_topk(void* base, int Hq, int64_t n) {
   fathom_topk_scratch s;
   char* p = static_cast<char*>(base);
   size_t off = 0;
@@ -28,20 +28,14 @@ fathom_topk_scratch fathom_carve_topk(void* base, int Hq, int64_t n, int k) {
   s.bitmap = reinterpret_cast<uint32_t*>(p + off);  off += fathom_round_up((size_t)Hq * (size_t)s.bitmap_words * 4, 256);
   s.cand = reinterpret_cast<int32_t*>(p + off);     off += fathom_round_up((size_t)Hq * (size_t)n * 4, 256);
   s.tile_count = reinterpret_cast<uint32_t*>(p + off); off += fathom_round_up((size_t)Hq * (size_t)((n + 8191) / 8192) * 4, 256);
-  const long long dense_stride = (n + 3) / 4 * 4;                           // a whole score row
-  s.cand_score = reinterpret_cast<float*>(p + off); off += fathom_round_up((size_t)Hq * (size_t)dense_stride * 4, 256);
-  {
-    // Room for every 16th scan tile, whatever k: a context that serves a layout then serves every shorter one and every smaller k.
-    // Where the row is scanned whole the candidates' scores are not used, and the row lies there.
-    const long long tile = fathom_scan_tile_tokens();
-    const long long sampled = ((n + tile - 1) / tile + 15) / 16 * tile;
-    s.sample = reinterpret_cast<float*>(p + off);   off += fathom_round_up((size_t)Hq * (size_t)(sampled < dense_stride ? sampled : dense_stride) * 4, 256);
-    s.sample_stride = sampled;
-    if (fathom_fused_tile_step(n, k) == 1) {
-      s.sample = s.cand_score;
-      s.sample_stride = dense_stride;
-    }
-  }
+  s.dense_stride = (n + 3) / 4 * 4;                                         // a whole score row
+  s.cand_score = reinterpret_cast<float*>(p + off); off += fathom_round_up((size_t)Hq * (size_t)s.dense_stride * 4, 256);
+  // Room for every 16th scan tile, whatever k: a context that serves a layout then serves every shorter one and every smaller k
+  // (a row that is scanned whole lies where the candidates' scores would).
+  const long long tile = fathom_scan_tile_tokens();
+  s.sample_stride = ((n + tile - 1) / tile + 15) / 16 * tile;
+  s.sample = reinterpret_cast<float*>(p + off);
+  off += fathom_round_up((size_t)Hq * (size_t)(s.sample_stride < s.dense_stride ? s.sample_stride : s.dense_stride) * 4, 256);
   s.bytes = off;
   return s;
 }
@@ -58,7 +52,7 @@ extern "C" {
 
 size_t fathom_scratch_bytes(const fathom_layout* L, int k) {
   if (fathom_check_layout(L) != FATHOM_OK || k < 1) return 0;
-  size_t a = fathom_carve_topk(nullptr, L->n_q_heads, L->n, k).bytes;
+  size_t a = fathom_carve_topk(nullptr, L->n_q_heads, L->n).bytes;
   size_t b = fathom_carve_attn(nullptr, L->n_q_heads, k).bytes;
   size_t c = fathom_union_scratch_bytes(L->n_kv_heads, L->n, (L->n_q_heads / L->n_kv_heads) * k);
   size_t e = fathom_calib_scratch_bytes(L->n_kv_heads, L->n);

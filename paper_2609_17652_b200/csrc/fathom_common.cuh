@@ -40,6 +40,17 @@ int fathom_check_layout(const fathom_layout* L);
 static inline int64_t fathom_nblocks(int64_t n) { return (n + FATHOM_BLOCK - 1) / FATHOM_BLOCK; }
 static inline bool fathom_aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 static inline size_t fathom_round_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
+// SMs of the current device; a B200's where there is none (calls that only plan)
+static inline int fathom_sm_count() {
+  static int sms[64] = {};
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 148;
+  if (!sms[dev]) {
+    int v = 0;
+    sms[dev] = cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && v > 0 ? v : 148;
+  }
+  return sms[dev];
+}
 
 // ---- programmatic dependent launch (sm_90+): a kernel launched with fathom_launch_dependent may become resident while
 // the previous kernel of the stream still runs (once every CTA of that kernel has passed FATHOM_PDL_RELEASE or exited) and
@@ -120,8 +131,8 @@ struct fathom_topk_scratch {
   int32_t* cand;         // [Hq][n] token indices of the threshold bin
   uint32_t* tile_count;  // [Hq][ceil(n / 8192)] selected tokens per filter tile, then their exclusive prefix
   float* cand_score;     // [Hq][n] scores of the fused path's candidates
-  float* sample;         // [Hq][sample_stride] scores of the sampled scan tiles (fused path); where all tiles are, the same memory as cand_score
-  long long sample_stride;
+  float* sample;         // [Hq][sample_stride] scores of the sampled scan tiles (fused path); where all tiles are scanned they take cand_score
+  long long sample_stride, dense_stride;   // (rows of cand_score: n or dense_stride apart, as candidates or as a score row)
   long long bitmap_words;
   size_t bytes;
 };
@@ -130,7 +141,7 @@ struct fathom_attn_scratch {
   int splits;
   size_t bytes;
 };
-fathom_topk_scratch fathom_carve_topk(void* base, int Hq, int64_t n, int k);
+fathom_topk_scratch fathom_carve_topk(void* base, int Hq, int64_t n);
 fathom_attn_scratch fathom_carve_attn(void* base, int Hq, int k);
 size_t fathom_union_scratch_bytes(int Hkv, long long n, int capacity);
 int fathom_launch_rotate_tc(fathom_ctx* ctx, const fathom_layout* L, const void* K, int k_dtype, const float* mean,

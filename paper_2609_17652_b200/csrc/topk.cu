@@ -3,9 +3,10 @@
 // All paths select on the order-preserving integer image of the fp32 score (-0 folded onto +0), and all give the
 // one set the definition fixes (ties to the lower token index), in ascending token order.
 //
-// Rows of up to 131,072 scores are held in registers by a cluster per head and selected in one kernel (topk_resident.cu).
+// Rows of up to 131,072 scores are held in registers by a cluster per head and selected in one kernel (topk_resident.cu), but for
+// large k and many heads (held_in_registers).
 //
-// Single pass (longer rows, when a sixteenth of the row holds enough of what is wanted): one read of the scores.
+// Single pass (other rows of at least 65,536, when a sixteenth of the row holds enough of what is wanted): one read of the scores.
 //   a. a cluster of four CTAs per head histograms every 16th 1024-score chunk (12 leading key bits, shared memory,
 //      merged through distributed shared memory) and finds two bins:
 //      the ESTIMATE, whose suffix count in the sample reaches the expected rank plus four standard deviations, and
@@ -206,7 +207,7 @@ __device__ void find_threshold_bin(const uint32_t* __restrict__ h, uint32_t* __r
 // estimated and the bound bin: no global histogram, no flush, no ticket.  For rows of up to a few million scores.
 constexpr int SAMPLE_THREADS = 1024;
 constexpr int SAMPLE_CLUSTER = 4;
-__global__ void __cluster_dims__(SAMPLE_CLUSTER, 1, 1) __launch_bounds__(SAMPLE_THREADS)
+__global__ void __cluster_dims__(SAMPLE_CLUSTER, 1, 1) __launch_bounds__(SAMPLE_THREADS, 2)
 topk_sample_kernel(const float* scores, long long sampled, long long chunk_stride, long long score_stride,
                    uint32_t* __restrict__ state, uint32_t want, uint32_t want_bound, uint32_t* __restrict__ cand_count,
                    uint32_t* __restrict__ cand_count2) {
@@ -228,7 +229,7 @@ topk_sample_kernel(const float* scores, long long sampled, long long chunk_strid
   const float* row = scores + (size_t)head * (size_t)score_stride;
   // `sampled` whole chunks of 1024 scores, chunk_stride scores apart (16384: every 16th chunk of a score row; 1024: a
   // compact array of sampled scores); CTA `part` of the cluster takes every SAMPLE_CLUSTER-th group of 1024 float4
-  constexpr int STRIDE = SAMPLE_CLUSTER * SAMPLE_THREADS, FLY = 4;            // loads in flight per thread
+  constexpr int STRIDE = SAMPLE_CLUSTER * SAMPLE_THREADS, FLY = 2;            // loads in flight per thread: 32 registers, two CTAs per SM
   for (long long v0 = (long long)part * SAMPLE_THREADS + threadIdx.x; v0 < sampled * 256; v0 += FLY * STRIDE) {
     float4 x[FLY];
 #pragma unroll
@@ -1184,6 +1185,27 @@ static bool single_pass_plan(long long n, int k, uint32_t want, uint32_t* rank_o
   return !force_two_pass() && want > 0 && chunks >= 64 && (long long)rank * 8 <= n_sample && (long long)k * 2 <= n_sample;
 }
 
+// Whether rows of n scores are held in registers (topk_resident.cu).  `scored`: the scores exist; else (the fused call) scanning and
+// selecting them densely stands against the sampled path, which scans a part of the row twice and takes five launches.
+// us held in registers / the other way (single pass where the row and k allow it, else two passes):
+//   131,072 scores  32 heads: k = 64 13.5 / 15.2, 2048 16.9 / 18.1, 3000 20.7 / 18.9, 4096 24.6 / 19.7; 8 heads: 3000 12.5 / 14.5;
+//                   64 heads: 512 23.6 / 24.7, 2048 29.6 / 26.3; 128 heads, 4096 (two waves): 74 / 56
+//   100,000 scores  32 heads, 16,384: 71 / 39; 40 heads, 8192: 44 / 48; 64 heads, 8192: 69 / 53
+//   65,536 scores   128 heads, 2048: 41 / 47
+//   33,001 scores   32 heads: 4096 21 / 32, 8192 35 / 32, 16,384 43 / 29; 8 heads: 16,384 18 / 26
+//   20,000 scores   16 heads, 16,384: 24 / 31
+// (scores of some thirty distinct values overflow the list and take radix rounds: 100,000 scores, 32 heads, k = 2048 55 / 31)
+static bool held_in_registers(long long n, int Hq, int k, uint32_t want, bool scored) {
+  if (n > FATHOM_TOPK_RESIDENT_MAX || force_two_pass()) return false;
+  const long long ctas = (long long)Hq * fathom_topk_resident_ctas(n), sms = fathom_sm_count();
+  uint32_t rank;
+  if (want > 8192) return (n <= 32768 ? 1 : 2) * ctas <= sms;  // its list overflows: radix rounds over the cluster
+  if (want > 4096) return 2 * ctas <= 5 * sms;                // (one CTA per SM)
+  if (n <= 65536) return true;
+  if (!scored || !single_pass_plan(n, k, want, &rank)) return ctas <= 4 * sms;
+  return want <= 512 || (want <= 2048 && 2 * ctas <= 5 * sms) || (want <= 3072 && 2 * ctas <= sms);
+}
+
 // log2 of the token range per counting-sort bucket of the direct select: the smallest that maps n tokens to SORT_BUCKETS
 static int bucket_shift_for(long long n) {
   int s = 0;
@@ -1230,15 +1252,14 @@ static int launch_direct_select(fathom_ctx* ctx, long long n, int Hq, int k, For
 
 static int run_dense_topk(fathom_ctx* ctx, const float* scores, long long n, long long score_stride, int Hq, int k,
                           Forced F, uint32_t want, const fathom_topk_scratch& S, int32_t* idx, cudaStream_t st) {
-  if (n <= FATHOM_TOPK_RESIDENT_MAX && !force_two_pass())
-    return fathom_launch_topk_resident(ctx, scores, n, score_stride, Hq, k, F, want, idx, st);
+  if (held_in_registers(n, Hq, k, want, true)) return fathom_launch_topk_resident(ctx, scores, n, score_stride, Hq, k, F, want, idx, st);
   const int ntiles = (int)((n + FILT_TILE - 1) / FILT_TILE);
   dim3 fgrid((unsigned)ntiles, (unsigned)Hq);
   Gate always = {nullptr, 0u, 0, 0};
   // Single pass when the row is long enough to estimate the threshold from every 16th 1024-score chunk.
   const long long chunks = n / 1024, sampled = (chunks + 15) / 16;           // whole chunks; chunks 0, 16, 32, .. are sampled
   uint32_t rank = 0;
-  const bool single = single_pass_plan(n, k, want, &rank);
+  const bool single = scores != S.cand_score && single_pass_plan(n, k, want, &rank);   // (the single pass writes candidates there)
   // histograms, per-head states and candidate counters are contiguous at the start of the arena; the sample
   // kernel keeps its histogram in shared memory
   // (the sample kernel writes every state word that path reads and clears the candidate counter: nothing to clear then)
@@ -1316,7 +1337,7 @@ extern "C" int fathom_topk(fathom_ctx* ctx, const fathom_layout* L, const float*
   F.local_begin = (n - n_local > F.sink_end) ? (n - n_local) : F.sink_end;
   const long long n_forced = F.sink_end + (n - F.local_begin);
   if (n_forced > k) return FATHOM_ERR_INVALID_ARG;
-  fathom_topk_scratch S = fathom_carve_topk(ctx->scratch, L->n_q_heads, n, k);
+  fathom_topk_scratch S = fathom_carve_topk(ctx->scratch, L->n_q_heads, n);
   if (S.bytes > ctx->scratch_bytes) return FATHOM_ERR_SCRATCH_TOO_SMALL;
   return run_dense_topk(ctx, scores, n, L->score_stride, L->n_q_heads, k, F, (uint32_t)(k - n_forced), S, idx,
                         static_cast<cudaStream_t>(stream));
@@ -1341,8 +1362,6 @@ int fathom_fused_tile_step(long long n, int k) {
   const long long sampled = (ntiles + 15) / 16;                       // tiles 0, 16, 32, ...
   const long long last_start = (sampled - 1) * 16 * tile;             // first token of the last sampled tile (< n)
   const long long valid = (sampled - 1) * tile + ((n - last_start) < tile ? (n - last_start) : tile);
-  // rows that the top-k holds in registers are scanned whole: one scan and one selection against the five kernels of the sampled path
-  if (n <= FATHOM_TOPK_RESIDENT_MAX && !force_two_pass()) return 1;
   return (ntiles >= 16 && valid >= 2LL * k) ? 16 : 1;
 }
 
@@ -1363,18 +1382,24 @@ extern "C" int fathom_scan_topk(fathom_ctx* ctx, const fathom_layout* L, const u
   F.local_begin = (n - n_local > F.sink_end) ? (n - n_local) : F.sink_end;
   const long long n_forced = F.sink_end + (n - F.local_begin);
   if (n_forced > k) return FATHOM_ERR_INVALID_ARG;
-  fathom_topk_scratch S = fathom_carve_topk(ctx->scratch, Hq, n, k);
+  fathom_topk_scratch S = fathom_carve_topk(ctx->scratch, Hq, n);
   if (S.bytes > ctx->scratch_bytes) return FATHOM_ERR_SCRATCH_TOO_SMALL;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   const uint32_t want = (uint32_t)(k - n_forced);
-  const int step = fathom_fused_tile_step(n, k);
+  const bool held = held_in_registers(n, Hq, k, want, false);
+  const int step = held ? 1 : fathom_fused_tile_step(n, k);
   const long long tile = fathom_scan_tile_tokens();
   const long long ntiles_scan = (n + tile - 1) / tile;
+  if (step == 1) {                                            // the whole row is scanned: where the candidates' scores would lie
+    S.sample = S.cand_score;
+    S.sample_stride = S.dense_stride;
+  }
 
   // ---- sample: scores of every `step`-th scan tile, compact
   rc = fathom_launch_scan_sample(L, planes, scales, q, depth, heads_per_plan, S.sample, S.sample_stride, step, st);
   if (rc != FATHOM_OK) return rc;
-  if (step == 1)                                              // short sequence: the sample is the whole score array
+  if (held) return fathom_launch_topk_resident(ctx, S.sample, n, S.sample_stride, Hq, k, F, want, idx, st);
+  if (step == 1)                                              // too short to sample: the sample is the whole score array
     return run_dense_topk(ctx, S.sample, n, S.sample_stride, Hq, k, F, want, S, idx, st);
 
   // ---- thresholds from a histogram of the sample.  Bound: the bin in which the sample's k-th largest score lies; at

@@ -409,7 +409,8 @@ topk_resident_kernel(const float* scores, int n, long long score_stride, int eli
 template <int EPT>
 cudaError_t launch(const float* scores, long long n, long long score_stride, int Hq, int k, Forced F, uint32_t want, int32_t* idx,
                    uint32_t* dev_status, int ctas, cudaStream_t st) {
-  // room for twice what is wanted (the bound lets through 1.05 to 1.5 times), as long as two CTAs fit on an SM
+  // room for twice what is wanted (the bound lets through 1.05 to 1.5 times), up to 16,384: 164 KB, one CTA per SM; two fit on an SM
+  // up to about 10,000
   const uint32_t room = 2u * want < 2048u ? 2048u : 2u * want;
   const uint32_t capacity = room < 16384u ? room : 16384u;
   const size_t smem = sizeof(ResidentSmem) + (size_t)capacity * 8;
@@ -443,13 +444,20 @@ cudaError_t launch(const float* scores, long long n, long long score_stride, int
 
 }  // namespace
 
+// as few tokens per thread as eight CTAs allow (at least 8: more CTAs cost barrier time), then as few CTAs as hold the row
+static int tokens_per_thread(long long n) {
+  const long long per_cta8 = RT_THREADS * 8;
+  return n <= MAX_CLUSTER * per_cta8 ? 8 : (n <= 2 * MAX_CLUSTER * per_cta8 ? 16 : 32);
+}
+int fathom_topk_resident_ctas(long long n) {
+  int ctas = 1;
+  while ((long long)ctas * RT_THREADS * tokens_per_thread(n) < n) ctas *= 2;
+  return ctas;
+}
+
 int fathom_launch_topk_resident(fathom_ctx* ctx, const float* scores, long long n, long long score_stride, int Hq, int k, Forced F,
                                 uint32_t want, int32_t* idx, cudaStream_t st) {
-  // as few tokens per thread as eight CTAs allow (at least 8: more CTAs cost barrier time), then as few CTAs as hold the row
-  const long long per_cta8 = RT_THREADS * 8;
-  const int ept = n <= MAX_CLUSTER * per_cta8 ? 8 : (n <= 2 * MAX_CLUSTER * per_cta8 ? 16 : 32);
-  int ctas = 1;
-  while ((long long)ctas * RT_THREADS * ept < n) ctas *= 2;
+  const int ept = tokens_per_thread(n), ctas = fathom_topk_resident_ctas(n);
   cudaError_t e;
   if (ept == 8) e = launch<8>(scores, n, score_stride, Hq, k, F, want, idx, ctx->dev_status, ctas, st);
   else if (ept == 16) e = launch<16>(scores, n, score_stride, Hq, k, F, want, idx, ctx->dev_status, ctas, st);

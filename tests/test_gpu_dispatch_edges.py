@@ -179,6 +179,29 @@ def test_klt_basis_in_place(spread):
     ctx.close()
 
 
+# (tokens, heads, k) on both sides of every line between the kernels of the selection, scores that exist and scores that do not
+@pytest.mark.parametrize("n,Hq,k", [(131072, 60, 548), (131072, 46, 600), (131072, 47, 600), (131072, 9, 3108), (131072, 9, 3109), (131072, 2, 16384),
+                                    (131073, 2, 16384), (33001, 9, 9000), (33001, 10, 9000), (20000, 18, 8300), (20000, 19, 8300), (70001, 75, 2100)])
+def test_selection_on_both_sides_of_its_lines(n, Hq, k):
+    from paper_2609_17652_b200 import binding as fb
+    lay = fb.make_layout(1, Hq, n)
+    ctx = fb.Context(0, fb.fathom_scratch_bytes(lay, k))
+    g = torch.Generator(device="cuda").manual_seed(n + Hq + k)
+    K, q = torch.randn(1, n, 128, generator=g, device="cuda"), torch.randn(Hq, 128, generator=g, device="cuda")
+    planes = torch.zeros(1, 128, 4, lay.plane_stride_words, dtype=torch.int64, device="cuda")
+    scales = torch.zeros(1, 128, lay.scale_stride, dtype=torch.int16, device="cuda")
+    depth, scores = torch.zeros(Hq, 128, dtype=torch.uint8, device="cuda"), torch.zeros(Hq, lay.score_stride, device="cuda")
+    idx, fused = (torch.full((Hq, k), -1, dtype=torch.int32, device="cuda") for _ in range(2))
+    ctx.fathom_build_planes(lay, K, planes, scales)
+    ctx.fathom_alloc_depth(lay, q, K.var(dim=1), fb.DEPTH_WATERFILL, 16, 1, depth)
+    ctx.fathom_scan(lay, planes, scales, q, depth, 1, scores)
+    ctx.fathom_topk(lay, scores, k, 4, 32, idx)
+    ctx.fathom_scan_topk(lay, planes, scales, q, depth, 1, k, 4, 32, fused)
+    assert np.array_equal(idx.cpu().numpy(), O.topk(scores[:, :n].double().cpu().numpy(), k, 4, 32))
+    assert torch.equal(idx, fused) and ctx.fathom_device_status() == 0
+    ctx.close()
+
+
 # picks on both sides of the line between one CTA per KV head and the whole chip
 @pytest.mark.parametrize("n,k", [(20000, 1102), (20000, 1103), (70001, 4000)])
 def test_union_of_many_picks(n, k):
