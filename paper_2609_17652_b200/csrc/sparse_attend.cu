@@ -289,13 +289,25 @@ cudaError_t launch_few(const float* q, const void* K, const void* V, const int32
 }
 
 // The kernel for k rows, the same for both entry points.  Beyond 1024 rows the gather is bound by memory, which the CTAs of 128 rows
-// fill better than clusters do.
+// fill better than clusters do.  Clusters that are not all resident at once lose more: the next one waits until a whole cluster has
+// left.  That costs more than they gain where the other kernel is at its best, with eight chunks (their triples are merged in one
+// round of loads, fewer of them one after the other), and with more than 128 heads.  Us with clusters / with CTAs of 128 rows: 1024 bf16 rows,
+// 48 heads 6.1 / 6.8, 64 heads 9.5 / 7.3, 128 heads 15.1 / 10.6; 1024 fp32 rows, 32 heads 6.1 / 7.6, 40 heads 10.2 / 8.5; 896 bf16
+// rows, 64 heads 8.6 / 10.4, 128 heads 14.0 / 13.9; 512 bf16 rows, 128 heads 9.3 / 8.8, 256 heads 15.5 / 12.2.
 constexpr int FEW_ROWS = FEW_CLUSTER * FEW_HW * 8;
+template <typename T>
+bool takes_clusters(int k, int Hq) {
+  if (k > FEW_ROWS) return false;
+  if (k <= FEW_ROWS - FATHOM_ATTN_CHUNK && Hq <= 128) return true;
+  const bool short_rows = k <= FEW_ROWS / 2;                  // (four rows per half-warp)
+  const int rows = short_rows ? 4 : 8, per_sm = sizeof(T) == 2 ? (short_rows ? 5 : 3) : (short_rows ? 4 : 2);   // by their registers: 48, 80; 62, 102
+  return (long long)Hq * ((k + FEW_HW * rows - 1) / (FEW_HW * rows)) <= (long long)per_sm * fathom_sm_count();
+}
 template <typename T>
 cudaError_t launch_attend(const float* q, const void* K, const void* V, const int32_t* idx, int k, long long n, int Hq, int G, float scale,
                           float* partial, int splits, unsigned int* tickets, float* out, cudaStream_t st) {
-  if (k <= FEW_ROWS / 2) return launch_few<T, 4>(q, K, V, idx, k, n, Hq, G, scale, out, st);
-  if (k <= FEW_ROWS) return launch_few<T, 8>(q, K, V, idx, k, n, Hq, G, scale, out, st);
+  if (takes_clusters<T>(k, Hq))
+    return (k <= FEW_ROWS / 2 ? launch_few<T, 4> : launch_few<T, 8>)(q, K, V, idx, k, n, Hq, G, scale, out, st);
   // (launched so that its CTAs may become resident while the selection kernel still runs)
   return fathom_launch_dependent(attend_partial_kernel<T>, dim3((unsigned)splits, (unsigned)Hq), dim3(AT_THREADS), 0, st, q, static_cast<const T*>(K),
                                  static_cast<const T*>(V), idx, k, n, G, scale, partial, splits, tickets, out);
