@@ -211,10 +211,14 @@ var_partial_kernel(const T* __restrict__ K, long long n, float* __restrict__ par
   }
 }
 
-// A CTA per (8 channels, KV head): thread (channel, lane) merges tiles lane, lane + 128, ... and the 128 lanes are then combined in a
-// fixed order, so the result does not depend on scheduling.  (One CTA per KV head with 8 lanes per channel was a chain of 2 x 128
-// dependent loads at n = 1M: 116 us, against 600 us for the pass over the keys; 16 channels a CTA and a division per tile: 18 us.)
-constexpr int VF_CHANNELS = 8, VF_LANES = 128;
+// A CTA per (VF_CHANNELS channels, KV head): thread (channel, lane) merges tiles lane, lane + VF_LANES, ... and the lanes are then
+// combined in a fixed order, so the result does not depend on scheduling.  Many tiles: 8 channels and 128 lanes (one CTA per KV
+// head with 8 lanes per channel was a chain of 2 x 128 dependent loads at n = 1M: 116 us, against 600 us for the pass over the
+// keys; 16 channels a CTA and a division per tile: 18 us).  Up to 16 tiles, or up to 64 where the heads' CTAs of 1024 threads are more
+// than the chip holds, 32 channels and 8 lanes: there starting and combining 128 lanes costs more than the shorter chain gives
+// (the whole call with 128 / with 8 lanes, bf16: 8192 tokens x 8 heads 11.5 / 10.5 us, x 32 heads 20.1 / 11.9; 33,001 tokens
+// x 8 heads 12.4 / 14.1, x 32 heads 54.3 / 48.3).
+template <int VF_CHANNELS, int VF_LANES>
 __global__ void __launch_bounds__(VF_CHANNELS * VF_LANES)
 var_final_kernel(const float* partial, int tiles, long long n, float* __restrict__ mean, float* __restrict__ var) {
   __shared__ double s_acc[VF_LANES][VF_CHANNELS];
@@ -222,21 +226,23 @@ var_final_kernel(const float* partial, int tiles, long long n, float* __restrict
   const int kv = blockIdx.y, cl = threadIdx.x % VF_CHANNELS, tl = threadIdx.x / VF_CHANNELS, c = blockIdx.x * VF_CHANNELS + cl;
   FATHOM_PDL_WAIT();
   const float* P = partial + (size_t)kv * tiles * 3 * FATHOM_D + c;
-  auto sum_lanes = [&]() {                                    // fixed order: sixteen sums of eight lanes, then their sum
-    constexpr int EACH = VF_LANES / 16;
+  auto sum_lanes = [&]() {                                    // fixed order: up to sixteen sums of EACH lanes, then their sum
+    constexpr int SUMS = VF_LANES < 16 ? VF_LANES : 16, EACH = VF_LANES / SUMS;
     __syncthreads();
-    if (tl < 16) {
-      double s = 0.0;
+    if (EACH > 1) {
+      if (tl < SUMS) {
+        double s = 0.0;
 #pragma unroll
-      for (int w = 0; w < EACH; ++w) s += s_acc[tl * EACH + w][cl];
-      s_acc[tl * EACH][cl] = s;
+        for (int w = 0; w < EACH; ++w) s += s_acc[tl * EACH + w][cl];
+        s_acc[tl * EACH][cl] = s;
+      }
+      __syncthreads();
     }
-    __syncthreads();
-    double s[16];
+    double s[SUMS];
 #pragma unroll
-    for (int w = 0; w < 16; ++w) s[w] = s_acc[w * EACH][cl];
+    for (int w = 0; w < SUMS; ++w) s[w] = s_acc[w * EACH][cl];
 #pragma unroll
-    for (int h = 8; h; h >>= 1)
+    for (int h = SUMS / 2; h; h >>= 1)
 #pragma unroll
       for (int w = 0; w < h; ++w) s[w] += s[w + h];
     return s[0];
@@ -269,22 +275,35 @@ var_final_kernel(const float* partial, int tiles, long long n, float* __restrict
   }
 }
 
+cudaError_t launch_var_final(const float* partial, int tiles, long long n, int Hkv, float* mean, float* var, bool dependent, cudaStream_t st) {
+  const bool few = tiles <= 16 || (tiles <= 64 && 16LL * Hkv > 2LL * fathom_sm_count());
+  const dim3 grid((unsigned)(FATHOM_D / (few ? 32 : 8)), (unsigned)Hkv), block(few ? 32 * 8 : 8 * 128);
+  auto kernel = few ? var_final_kernel<32, 8> : var_final_kernel<8, 128>;
+  if (dependent) return fathom_launch_dependent(kernel, grid, block, 0, st, partial, tiles, n, mean, var);
+  kernel<<<grid, block, 0, st>>>(partial, tiles, n, mean, var);
+  return cudaGetLastError();
+}
+
 // reduction of the tensor-core partials (fp64, slot order): S = sum_t sums[kv][t], mean = shift + S / n,
 // cov = (sum_t (P1 + P2 + P2^T) - S S^T / n) / (n - 1)  with the partials [kv][t][2][d][d] of the shifted keys
-// A CTA per 32 x 32 tile of the result, a thread per element; the transposed tile of P2 is summed where it lies and turned round once
-// at the end (read element by element along its columns it was a sector per element: 15 -> 6 us for 8 heads of 18 partials).
-constexpr int CF_TILE = 32;
-__global__ void __launch_bounds__(CF_TILE * CF_TILE)
+// A CTA per CF_TILE x CF_TILE tile of the result, GROUPS threads per element (each sums every GROUPS-th partial; their sums are added in
+// order); the transposed tile of P2 is summed where it lies and turned round once at the end (read element by element along its
+// columns it was a sector per element: 15 -> 6 us for 8 heads of 18 partials).  One thread per element of 32 x 32 where that fills
+// the chip; with few heads there are few CTAs and many partials each, and 16 x 16 with four threads per element are taken (the whole
+// calibration of 131,072 fp32 tokens: 1 head 71.5 -> 42.9 us, 2 heads 65.7 -> 52.8; 8192 tokens, 2 heads 34.9 -> 21.3).
+template <int CF_TILE, int GROUPS>
+__global__ void __launch_bounds__(CF_TILE * CF_TILE * GROUPS)
 cov_final_tc_kernel(const float* partial, const float* partial_sum, const float* shift,
                     int slots, long long n, float* __restrict__ mean, float* __restrict__ cov) {
+  constexpr int TILES = FATHOM_D / CF_TILE, CELLS = CF_TILE * CF_TILE;
   __shared__ double s_S[2][CF_TILE];                          // of the tile's rows, of its columns
   __shared__ double s_t[CF_TILE][CF_TILE + 1];
-  constexpr int TILES = FATHOM_D / CF_TILE;
+  __shared__ double s_part[GROUPS > 1 ? GROUPS - 1 : 1][GROUPS > 1 ? CELLS : 1][2];
   FATHOM_PDL_WAIT();
   FATHOM_PDL_RELEASE();
   const int kv = blockIdx.y, i0 = blockIdx.x / TILES * CF_TILE, j0 = blockIdx.x % TILES * CF_TILE;
-  const int x = threadIdx.x % CF_TILE, y = threadIdx.x / CF_TILE;
-  if (y < 2) {
+  const int cell = threadIdx.x % CELLS, group = threadIdx.x / CELLS, x = cell % CF_TILE, y = cell / CF_TILE;
+  if (group == 0 && y < 2) {
     const int c = (y ? j0 : i0) + x;
     double t = 0.0;
 #pragma unroll 8
@@ -296,14 +315,27 @@ cov_final_tc_kernel(const float* partial, const float* partial_sum, const float*
   const int here = (i0 + y) * FATHOM_D + j0 + x, there = (j0 + y) * FATHOM_D + i0 + x;
   double s = 0.0, turned = 0.0;
 #pragma unroll 6
-  for (int t = 0; t < slots; ++t) {
+  for (int t = group; t < slots; t += GROUPS) {
     const float* p1 = P + (size_t)t * 2 * FATHOM_D * FATHOM_D;
     const float* p2 = p1 + FATHOM_D * FATHOM_D;
     s += (double)p1[here] + (double)p2[here];
     turned += (double)p2[there];
   }
-  s_t[y][x] = turned;
+  if (GROUPS > 1) {
+    if (group > 0) {
+      s_part[group - 1][cell][0] = s;
+      s_part[group - 1][cell][1] = turned;
+    }
+    __syncthreads();
+    if (group == 0)
+      for (int h = 0; h < GROUPS - 1; ++h) {
+        s += s_part[h][cell][0];
+        turned += s_part[h][cell][1];
+      }
+  }
+  if (group == 0) s_t[y][x] = turned;
   __syncthreads();
+  if (group > 0) return;
   s += s_t[x][y];
   s -= s_S[0][y] * s_S[1][x] / (double)n;
   cov[(size_t)kv * FATHOM_D * FATHOM_D + here] = (float)(s / (double)(n > 1 ? n - 1 : 1));
@@ -348,7 +380,7 @@ extern "C" int fathom_channel_variance(fathom_ctx* ctx, const fathom_layout* L, 
     var_partial_kernel<float><<<dim3(mt, Hkv), KT_THREADS, 0, st>>>(static_cast<const float*>(K), n, part, mt);
   else
     var_partial_kernel<__nv_bfloat16><<<dim3(mt, Hkv), KT_THREADS, 0, st>>>(static_cast<const __nv_bfloat16*>(K), n, part, mt);
-  FATHOM_CUDA_TRY(ctx, fathom_launch_dependent(var_final_kernel, dim3(FATHOM_D / VF_CHANNELS, Hkv), dim3(VF_CHANNELS * VF_LANES), 0, st, part, mt, n, mean, var));
+  FATHOM_CUDA_TRY(ctx, launch_var_final(part, mt, n, Hkv, mean, var, true, st));
   return FATHOM_OK;
 }
 
@@ -377,9 +409,9 @@ extern "C" int fathom_calibrate(fathom_ctx* ctx, const fathom_layout* L, const v
     float* psum = reinterpret_cast<float*>(base + stats_partial_bytes(Hkv, n) + cov_bytes + fathom_round_up((size_t)Hkv * FATHOM_D * 4, 256));   // [Hkv][slots][d]
     rc = fathom_launch_cov_tc(ctx, L, K, k_dtype, var_tmp, pcov, psum, slots, st);
     if (rc != FATHOM_OK) return rc;
-    constexpr int TILES = FATHOM_D / CF_TILE;
-    FATHOM_CUDA_TRY(ctx, fathom_launch_dependent(cov_final_tc_kernel, dim3(TILES * TILES, Hkv), dim3(CF_TILE * CF_TILE), 0, st, pcov, psum, var_tmp, slots, n,
-                                                 mean, cov));
+    const bool few = 16LL * Hkv * 2 <= fathom_sm_count();               // fewer CTAs of 32 x 32 than half the SMs
+    FATHOM_CUDA_TRY(ctx, fathom_launch_dependent(few ? cov_final_tc_kernel<16, 4> : cov_final_tc_kernel<32, 1>, dim3(few ? 64 : 16, Hkv), dim3(1024), 0, st,
+                                                 pcov, psum, var_tmp, slots, n, mean, cov));
     return FATHOM_OK;
   }
   // plain fp32 kernels: (1) mean
@@ -387,7 +419,7 @@ extern "C" int fathom_calibrate(fathom_ctx* ctx, const fathom_layout* L, const v
     var_partial_kernel<float><<<dim3(mt, Hkv), KT_THREADS, 0, st>>>(static_cast<const float*>(K), n, part, mt);
   else
     var_partial_kernel<__nv_bfloat16><<<dim3(mt, Hkv), KT_THREADS, 0, st>>>(static_cast<const __nv_bfloat16*>(K), n, part, mt);
-  var_final_kernel<<<dim3(FATHOM_D / VF_CHANNELS, Hkv), VF_CHANNELS * VF_LANES, 0, st>>>(part, mt, n, mean, var_tmp);
+  FATHOM_CUDA_TRY(ctx, launch_var_final(part, mt, n, Hkv, mean, var_tmp, false, st));
   // (2) covariance partials
   int slots;
   {

@@ -209,10 +209,13 @@ __device__ __forceinline__ void unpack16(const uint4& u, float (&x)[8]) {
 #pragma unroll
   for (int c = 0; c < 4; ++c) { x[2 * c] = __uint_as_float(w[c] << 16); x[2 * c + 1] = __uint_as_float(w[c] & 0xffff0000u); }
 }
-template <typename T> __device__ __forceinline__ float4 load_row4(const T* p);
-template <> __device__ __forceinline__ float4 load_row4<float>(const float* p) { return *reinterpret_cast<const float4*>(p); }
-template <> __device__ __forceinline__ float4 load_row4<__nv_bfloat16>(const __nv_bfloat16* p) {
-  const uint2 u = *reinterpret_cast<const uint2*>(p);
+// four channels of a key, as loaded; converted where they are used (a conversion behind the load waited for it there, before the MMAs of
+// the stage were issued: calibration of 131,072 bf16 tokens x 8 heads 274 -> 146 us)
+template <typename T> struct Row4;
+template <> struct Row4<float> { using type = float4; };
+template <> struct Row4<__nv_bfloat16> { using type = uint2; };
+__device__ __forceinline__ float4 row4(const float4& r) { return r; }
+__device__ __forceinline__ float4 row4(const uint2& u) {
   return make_float4(__uint_as_float(u.x << 16), __uint_as_float(u.x & 0xffff0000u), __uint_as_float(u.y << 16),
                      __uint_as_float(u.y & 0xffff0000u));
 }
@@ -632,7 +635,6 @@ cov_partial_tc_kernel(const T* K, const float* shift, float* __restrict__ partia
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
   FATHOM_PDL_WAIT();                                          // the shift comes from the previous kernel
-  FATHOM_PDL_RELEASE();
   if (tid < FATHOM_D) s_mu[tid] = shift[(size_t)kv * FATHOM_D + tid];
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
@@ -643,12 +645,15 @@ cov_partial_tc_kernel(const T* K, const float* shift, float* __restrict__ partia
   const int q4 = tid & 31, kc = q4 >> 3, c4 = q4 & 7, tok0 = tid >> 5;      // token tok0 + 8 i
   const int x_off = kc * CV_SLAB + slab_offset_mn(tok0, c4);                 // + 1024 i (tokens 8 apart: eight rows further)
   const float4 mu = *reinterpret_cast<const float4*>(s_mu + 4 * q4);
-  float4 xr[8];
+  using Raw = typename Row4<T>::type;
+  Raw xr[8];
   auto load_stage = [&](long long st) {
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
       const long long t = st * CV_TOK + tok0 + 8 * i;
-      xr[i] = (st < s1 && t < n) ? load_row4<T>(Kh + (size_t)t * FATHOM_D + 4 * q4) : make_float4(mu.x, mu.y, mu.z, mu.w);
+      if constexpr (sizeof(T) == 4) xr[i] = mu;               // tokens past the end count as the shift: they add nothing
+      else xr[i] = Raw{};
+      if (st < s1 && t < n) xr[i] = *reinterpret_cast<const Raw*>(Kh + (size_t)t * FATHOM_D + 4 * q4);
     }
   };
   load_stage(s0);
@@ -660,8 +665,9 @@ cov_partial_tc_kernel(const T* K, const float* shift, float* __restrict__ partia
     const uint32_t bar_empty = buf ? bar_empty1 : bar_empty0;
     if (q >= 2 && alive && !mbar_wait(bar_empty, ((q >> 1) - 1) & 1)) alive = false;
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {                             // tokens past the end were loaded as the shift: they add nothing
-      const float a0 = xr[i].x - mu.x, a1 = xr[i].y - mu.y, a2 = xr[i].z - mu.z, a3 = xr[i].w - mu.w;
+    for (int i = 0; i < 8; ++i) {
+      const float4 x = sizeof(T) == 4 || st * CV_TOK + tok0 + 8 * i < n ? row4(xr[i]) : mu;
+      const float a0 = x.x - mu.x, a1 = x.y - mu.y, a2 = x.z - mu.z, a3 = x.w - mu.w;
       sum4.x += a0; sum4.y += a1; sum4.z += a2; sum4.w += a3;
       const float h0 = tf32_head(a0), h1 = tf32_head(a1), h2 = tf32_head(a2), h3 = tf32_head(a3);
       const int off = buf * 2 * CV_PART + x_off + i * 1024;
@@ -686,6 +692,9 @@ cov_partial_tc_kernel(const T* K, const float* shift, float* __restrict__ partia
       if (st == s1 - 1) umma_commit(bar_acc);
     }
   }
+  // (not before: CTAs of the merge that wait beside this one for the whole pass take issue slots from it - 131,072 bf16 tokens x 4 heads
+  // 150 -> 144 us; beside fp32 keys they do not fit)
+  FATHOM_PDL_RELEASE();
   // ---- per-channel sums of (x - shift): the eight threads of a channel quad (one per warp) are added in warp order
   {
     float4* red = reinterpret_cast<float4*>(s_stage);         // [8 warps][32 quads]

@@ -202,6 +202,29 @@ def test_selection_on_both_sides_of_its_lines(n, Hq, k):
     ctx.close()
 
 
+# statistics on both sides of the lines between their merges: 1, 64 and 65 tiles, few and many KV heads
+@pytest.mark.parametrize("kv,n", [(1, 3), (1, 1025), (4, 65536), (5, 65537), (9, 2000)])
+def test_statistics_merges(kv, n):
+    from paper_2609_17652_b200 import binding as fb
+    lay = fb.make_layout(kv, kv, n)
+    ctx = fb.Context(0, fb.fathom_scratch_bytes(lay, 1))
+    g = torch.Generator(device="cuda").manual_seed(n)
+    K = 2.0 * torch.randn(kv, n, 128, generator=g, device="cuda") + torch.randn(kv, 1, 128, generator=g, device="cuda")
+    mean, var, m2 = (torch.zeros(kv, 128, device="cuda") for _ in range(3))
+    cov = torch.zeros(kv, 128, 128, device="cuda")
+    ctx.fathom_channel_variance(lay, K, mean, var)
+    ctx.fathom_calibrate(lay, K, m2, cov)
+    X = K.double()
+    mu = X.mean(dim=1)
+    C = (X - mu.unsqueeze(1)).transpose(1, 2) @ (X - mu.unsqueeze(1)) / (n - 1)
+    v = torch.diagonal(C, dim1=1, dim2=2)
+    # variances: fp32 sums of 1024 tokens.  Covariances: an accumulator takes up to 65536 / 29 tokens, eight a step, and every step
+    # may round towards zero by 2^-23 of it: up to 283 * 2^-23 = 3.4e-5 (1.1e-5 measured)
+    assert (mean - mu).norm() < 1e-6 * mu.norm() and (m2 - mu).norm() < 1e-6 * mu.norm()
+    assert (var - v).norm() < 1e-5 * v.norm() and (cov - C).norm() < 5e-5 * C.norm()
+    ctx.close()
+
+
 # picks on both sides of the line between one CTA per KV head and the whole chip
 @pytest.mark.parametrize("n,k", [(20000, 1102), (20000, 1103), (70001, 4000)])
 def test_union_of_many_picks(n, k):
