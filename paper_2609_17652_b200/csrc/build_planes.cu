@@ -121,10 +121,9 @@ int launch_blocks(fathom_ctx* ctx, const fathom_layout* L, const T* K, uint64_t*
 // A CTA per block while that is less than one wave of CTAs (four of 64 registers x 256 threads are resident per SM): the partial
 // sectors it writes are few then, and the walk over eight blocks is a chain of eight load latencies (one head, 424 tokens of
 // fp32: 5.9 -> 2.9 us).
-constexpr long long SHORT_BLOCKS = 148 * 4;
 template <typename T>
 int launch_build(fathom_ctx* ctx, const fathom_layout* L, const T* K, uint64_t* planes, uint16_t* scales, cudaStream_t st) {
-  if (fathom_nblocks(L->n) * L->n_kv_heads <= SHORT_BLOCKS) return launch_blocks<T, 1>(ctx, L, K, planes, scales, st);
+  if (fathom_nblocks(L->n) * L->n_kv_heads <= 4LL * fathom_sm_count()) return launch_blocks<T, 1>(ctx, L, K, planes, scales, st);
   return launch_blocks<T, 8>(ctx, L, K, planes, scales, st);
 }
 

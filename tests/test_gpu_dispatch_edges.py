@@ -248,6 +248,23 @@ def test_union_of_many_picks(n, k):
     ctx.close()
 
 
+# eight CTAs per plan up to 18 plans and from 75 on, else four
+@pytest.mark.parametrize("plans", [1, 18, 19, 74, 75])
+@pytest.mark.parametrize("mode,budget", [("waterfill", 48), ("fixed_top_r", 16), ("uniform", 2)])
+def test_depths_of_few_and_many_plans(plans, mode, budget):
+    from paper_2609_17652_b200 import binding as fb
+    lay = fb.make_layout(1, plans, 100)
+    ctx = fb.Context(0, 0)
+    g = torch.Generator(device="cuda").manual_seed(plans)
+    q, var = torch.randn(plans, 128, generator=g, device="cuda"), torch.rand(1, 128, generator=g, device="cuda")
+    depth = torch.full((plans, 128), 9, dtype=torch.uint8, device="cuda")
+    code = dict(waterfill=fb.DEPTH_WATERFILL, fixed_top_r=fb.DEPTH_FIXED_TOP_R, uniform=fb.DEPTH_UNIFORM)[mode]
+    ctx.fathom_alloc_depth(lay, q, var, code, budget, 1, depth)
+    ref = O.alloc_depth(q.cpu().numpy(), var.cpu().numpy(), mode, budget, 1)
+    assert np.array_equal(depth.cpu().numpy(), ref)
+    ctx.close()
+
+
 # one CTA per plan: its candidate lists run over (1200 of them for 512, 256 and 128 places a head)
 @pytest.mark.parametrize("heads_per_plan", [1, 2, 4])
 def test_fused_selection_with_more_candidates_than_a_cta_lists(heads_per_plan):
