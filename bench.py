@@ -214,9 +214,10 @@ def run_ours(args):
     sm_scale = 1.0 / math.sqrt(d)
 
     stage_names = ["alloc_depth", "scan", "topk", "sparse_attend"]
-    topk_passes = fb.fathom_topk_passes(lay, k)                 # 1: sampled estimate + one collection pass; 2: histogram + filter
-    # single pass: sample histogram, collection, selection (3 kernels); two passes: histogram, filter, select, emit (4)
-    launches_per_step = {"alloc_depth": 1, "scan": 1, "topk": 3 if topk_passes == 1 else 4, "sparse_attend": 1}
+    topk_passes = fb.fathom_topk_passes(lay, k)                 # 1: held in registers, or sampled estimate + one collection pass; 2: histogram + filter
+    # rows held in registers: 1 kernel (counted for all rows that may be); single pass: sample histogram, collection, selection (3);
+    # two passes: histogram, filter, select, emit (4)
+    launches_per_step = {"alloc_depth": 1, "scan": 1, "topk": 4 if topk_passes == 2 else 1 if n <= 131072 else 3, "sparse_attend": 1}
 
     def stage(i, W, st, q=None, var=None, result=None):
         """Stage i of the decode step on layer store W: alloc_depth, scan, topk, sparse_attend (`result`: where the

@@ -175,19 +175,19 @@ int fathom_scan_set_ctas_per_plan(int ctas);
  *   scores  in   [Hq][score_stride] fp32 (finite)
  *   idx     out  [Hq][k] int32, ascending token indices
  * Uses the context scratch (fathom_scratch_bytes).
- * Rows of up to 131,072 scores are selected by one kernel that holds them in registers.  Longer rows are read once: a histogram of every 16th chunk
- * gives an estimated threshold bin (and a bound: the bin of the sample's own k-th largest score), one pass collects
- * the tokens above the estimate, and the exact selection runs among them, head by head.  A head that collected fewer
- * than it needs is served instead by a second launch, enqueued behind the first, in which the head's CTA collects
- * above the bound and selects; the decision is taken on the device and the result is the same either way.  Rows of
- * which more than a thirty-second is wanted take two passes (histogram of all scores, filter).
+ * Rows of up to 131,072 scores are selected by one kernel that holds them in registers, unless k and the number of
+ * heads make another way faster.  Other rows are read once: a histogram of every 16th chunk gives an estimated threshold
+ * bin (and a bound: the bin of the sample's own k-th largest score), one pass collects the tokens above the estimate,
+ * and the exact selection runs among them, head by head.  A head that collected fewer than it needs collects again in
+ * the selection's own launch, above the bound; the decision is taken on the device and the result is the same either
+ * way.  Rows of which more than a thirty-second is wanted take two passes (histogram of all scores, filter).
  * Environment: FATHOM_TOPK_PATH=two_pass (read once) always takes the two-pass selection. */
 #define FATHOM_MAX_K 16384
 int fathom_topk(fathom_ctx* ctx, const fathom_layout* layout, const float* scores, int k,
                 int n_sink, int n_local, int32_t* idx, void* stream);
-/* How many times fathom_topk reads the scores for these arguments at most (host only, no GPU work): 1 where at least 256
- * tokens are wanted of a row long enough to estimate their threshold from a sample, else 2; or a negative status for
- * arguments fathom_topk would reject. */
+/* How many times fathom_topk reads the scores for these arguments (host only, no GPU work): 1 where the rows are held in
+ * registers or their threshold is estimated from a sample (a head whose estimate fails reads its row once more), 2 where
+ * they take two passes; or a negative status for arguments fathom_topk would reject. */
 int fathom_topk_passes(const fathom_layout* layout, int k, int n_sink, int n_local);
 
 /* ---- (3+4) fused scan and top-k, scores never materialised — Sec. 9 Conclusion (fusing the scan with what follows it) ------
@@ -200,8 +200,8 @@ int fathom_topk_passes(const fathom_layout* layout, int k, int n_sink, int n_loc
  * standard deviations: ~6 times fewer candidates).  The scan runs with the estimate; if any head then holds fewer
  * candidates than it needs, a second scan with the bound, enqueued behind the first, does the work instead - the
  * decision is taken on the device, and the result never depends on how representative the sample is.
- * Sequences too short to sample (fewer than 16 tiles or fewer than 2 k sampled tokens) are scanned into scratch
- * and selected densely.  Uses the context scratch (fathom_scratch_bytes). */
+ * Sequences of up to 131,072 tokens (but for many heads), and longer ones that are too short to sample (fewer than 2 k
+ * sampled tokens), are scanned into scratch and selected densely instead.  Uses the context scratch (fathom_scratch_bytes). */
 int fathom_scan_topk(fathom_ctx* ctx, const fathom_layout* layout, const uint64_t* planes, const uint16_t* scales,
                      const float* q, const uint8_t* depth, int heads_per_plan, int k, int n_sink, int n_local,
                      int32_t* idx, void* stream);

@@ -1350,8 +1350,9 @@ extern "C" int fathom_topk_passes(const fathom_layout* L, int k, int n_sink, int
   const long long local_begin = (n - n_local > sink_end) ? (n - n_local) : sink_end;
   const long long n_forced = sink_end + (n - local_begin);
   if (n_forced > k) return FATHOM_ERR_INVALID_ARG;
+  const uint32_t want = (uint32_t)(k - n_forced);
   uint32_t rank;
-  return k - n_forced >= 256 && single_pass_plan(n, k, (uint32_t)(k - n_forced), &rank) ? 1 : 2;
+  return held_in_registers(n, L->n_q_heads, k, want, true) || single_pass_plan(n, k, want, &rank) ? 1 : 2;
 }
 
 // Tile step of the sample scan for (n, k): every 16th scan tile when that sample still holds at least 2 k tokens,

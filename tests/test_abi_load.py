@@ -138,9 +138,11 @@ def test_topk_pass_plan_and_rejections_of_the_newer_entry_points(fb):
     beyond the five calls are refused before any launch."""
     lay = fb.make_layout(8, 32, 1 << 20)
     assert fb.fathom_topk_passes(lay, 4096) == 1 and fb.fathom_topk_passes(lay, 4096, 4, 32) == 1
-    assert fb.fathom_topk_passes(lay, 64) == 2                       # too few winners to estimate from a sample
-    assert fb.fathom_topk_passes(fb.make_layout(8, 32, 40000), 2048) == 2     # too short to sample
+    assert fb.fathom_topk_passes(lay, 64) == 1                       # few winners: the sample's estimate has its margin
+    assert fb.fathom_topk_passes(fb.make_layout(8, 32, 40000), 2048) == 1     # held in registers
     assert fb.fathom_topk_passes(fb.make_layout(8, 32, 131072), 2048) == 1
+    assert fb.fathom_topk_passes(fb.make_layout(8, 32, 262144), 16384) == 2   # more than the sample can bound
+    assert fb.fathom_topk_passes(fb.make_layout(8, 32, 100000), 16384) == 2   # neither held nor sampled
     assert fb.lib.fathom_topk_passes(C.byref(lay), 0, 0, 0) < 0 and fb.lib.fathom_topk_passes(C.byref(lay), 10, 8, 8) < 0
     for call, nargs in (("fathom_scan_topk", 12), ("fathom_gather_union", 12), ("fathom_calibrate", 7), ("fathom_rotate_keys", 8),
                         ("fathom_rotate_query", 6), ("fathom_channel_variance", 7), ("fathom_build_planes_rotated", 9)):
