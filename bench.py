@@ -566,8 +566,8 @@ def run_ours(args):
 
 def session_kernels_leg(ctx, lay, L, stream, hbm_peak):
     """Times fathom_channel_variance, fathom_calibrate and fathom_rotate_keys on the bench's keys (L2 flushed before
-    each launch) and reports them against the HBM peak and, for the two contractions, the tf32 tensor peak
-    (measured bf16 peak x the nominal tf32 : bf16 ratio 1.1 : 2.25)."""
+    each launch) and reports them against the HBM peak and, for the two contractions, the tensor peak of their operands
+    (fp16: the measured bf16 peak; tf32: that x the nominal tf32 : bf16 ratio 1.1 : 2.25)."""
     Hkv, n, d = L.K.shape
     dev = L.K.device
     mean = torch.zeros((Hkv, d), device=dev); var = torch.zeros((Hkv, d), device=dev)
@@ -582,12 +582,12 @@ def session_kernels_leg(ctx, lay, L, stream, hbm_peak):
     }
     kbytes = float(L.K.numel() * L.K.element_size())
     alg_bytes = {"channel_variance": kbytes, "calibrate": kbytes, "rotate_keys": kbytes + 4.0 * K_rot.numel()}
-    products = {"calibrate": 2, "rotate_keys": 3}                  # tf32 products per multiply of the split operands
-    tf32_peak = None
+    products = {"calibrate": (2, "tf32"), "rotate_keys": (3, "fp16")}      # products per multiply of the split operands, their type
+    peak = None
     p = os.path.join(ROOT, "MEASURED_PEAKS.json")
     if os.path.exists(p):
         with open(p) as f:
-            tf32_peak = float(json.load(f)["bf16_tflops"]) * 1.1 / 2.25
+            peak = float(json.load(f)["bf16_tflops"])
     out = {}
     for nm, fn in calls.items():
         ts = []
@@ -602,12 +602,14 @@ def session_kernels_leg(ctx, lay, L, stream, hbm_peak):
         gbs = alg_bytes[nm] / (t_us * 1e-6) / 1e9
         r = {"us": round(t_us, 1), "algorithmic_bytes": alg_bytes[nm], "achieved_gbs": round(gbs, 1), "frac_of_hbm_peak": round(gbs / hbm_peak, 4)}
         if nm in products:
-            tf = products[nm] * 2.0 * n * Hkv * d * d / (t_us * 1e-6) / 1e12
-            r.update({"tensor_tflops_tf32": round(tf, 1), "tf32_peak_tflops": round(tf32_peak, 1) if tf32_peak else None,
-                      "frac_of_tf32_peak": round(tf / tf32_peak, 4) if tf32_peak else None})
+            times, operands = products[nm]
+            tf = times * 2.0 * n * Hkv * d * d / (t_us * 1e-6) / 1e12
+            top = peak * (1.1 / 2.25 if operands == "tf32" else 1.0) if peak else None
+            r.update({"tensor_operands": operands, "tensor_tflops": round(tf, 1), "tensor_peak_tflops": round(top, 1) if top else None,
+                      "frac_of_tensor_peak": round(tf / top, 4) if top else None})
         out[nm] = r
     out["note"] = ("once per session, not in the timed step; calibrate reads the keys once (covariance and sums of keys centred "
-                   "on a shift); the contractions run as tcgen05.mma on tf32 operands split in head and tail")
+                   "on a shift); the contractions run as tcgen05.mma on operands split in head and tail")
     return out
 
 

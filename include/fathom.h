@@ -248,17 +248,21 @@ int fathom_gather_union(fathom_ctx* ctx, const fathom_layout* layout, const int3
  *                        fathom_klt_basis turns the covariances into bases and eigenvalues.
  *                        Uses the context scratch.  FATHOM_CALIBRATE_PATH=simt: two passes in plain fp32 FMAs.
  *   fathom_rotate_keys:  K_rot [Hkv][n][d] fp32 = (K - mean) basis, basis [Hkv][d][d] row-major with the
- *                        directions in its columns; tensor cores, tf32 operands split in head and tail (three
- *                        products, fp32 accumulation, fixed order); FATHOM_ROTATE_PATH=simt: plain fp32 FMAs.
+ *                        directions in its columns; tensor cores, operands split in an fp16 head and tail after every
+ *                        key and every direction has been scaled by a power of two (three products, fp32
+ *                        accumulation, fixed order; 7e-7 of the norm of the rotated keys, and elements below 2^-18 of
+ *                        the largest of their key keep an absolute error of 2^-39 of that); FATHOM_ROTATE_PATH=simt:
+ *                        plain fp32 FMAs.
  *   fathom_rotate_query: q_rot [Hq][d] = q basis[h / G].
  * K is [Hkv][n][d], FATHOM_F32 or FATHOM_BF16, 16-byte aligned, like basis, cov and K_rot. */
 int fathom_calibrate(fathom_ctx* ctx, const fathom_layout* layout, const void* K, int k_dtype, float* mean,
                      float* cov, void* stream);
 /*   fathom_klt_basis:    basis [Hkv][d][d] (fp32, row-major, directions in its columns) and eigenvalues [Hkv][d] (fp32,
- *                        descending) of cov [Hkv][d][d] (its symmetric part is used): two-sided cyclic Jacobi in fp64, one
- *                        CTA per KV head, rotations accumulated in fp32, fixed order (bit-reproducible); every direction is
- *                        signed so that its largest component is positive.  About 6 ms for 8 KV heads, once per session.  The eigenvalues
- *                        are the `var` of fathom_alloc_depth for the rotated store. */
+ *                        descending) of cov [Hkv][d][d] (its symmetric part is used): two-sided cyclic Jacobi by eight CTAs
+ *                        per KV head, sweeps in fp32, finished in fp64 from the covariance itself (or by fp64 sweeps where
+ *                        eigenvalues are close), fixed order (bit-reproducible); every direction is signed so that its
+ *                        largest component is positive.  0.35 to 2 ms for 8 KV heads, once per session.  basis may be
+ *                        cov.  The eigenvalues are the `var` of fathom_alloc_depth for the rotated store. */
 int fathom_klt_basis(fathom_ctx* ctx, const fathom_layout* layout, const float* cov, float* basis, float* eigenvalues,
                      void* stream);
 int fathom_rotate_keys(fathom_ctx* ctx, const fathom_layout* layout, const void* K, int k_dtype,

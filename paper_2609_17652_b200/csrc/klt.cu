@@ -8,7 +8,8 @@
 //
 // This file holds the statistics kernels, the entry points and the plain-fp32 variants of rotation and covariance
 // (FATHOM_ROTATE_PATH=simt, FATHOM_CALIBRATE_PATH=simt); the default paths are the tcgen05 kernels of klt_tc.cu, which
-// split both operands into tf32 head and tail so that the rotated keys, which feed a quantiser, keep fp32 accuracy.
+// split both operands into a head and a tail (rotation: fp16, scaled; covariance: tf32) so that the rotated keys, which feed a quantiser,
+// keep fp32 accuracy.
 // The fp32 variants are the same register-tiled product  C[i][j] += P[t][i] * Q[t][j]  over a shared-memory panel:
 // 256 threads, each an 8 x 8 block of the 128 x 128 result (columns split 4 + 4 so that the 16-byte panel loads of
 // neighbouring lanes are contiguous), plain FMAs in a fixed order.
@@ -94,7 +95,7 @@ rotate_keys_kernel(const T* __restrict__ K, const float* __restrict__ mean, cons
 
 // ---- q' = q V ---------------------------------------------------------------------------------------------------
 // One fused multiply-add chain per output, as short as it is (128 steps); what took 10 us was loading the basis in groups of
-// eight, so the whole column is requested before the first step.
+// eight, so the whole column is requested before the first step (151 registers; 32 heads, calls behind one another: 4.5 -> 1.9 us).
 __global__ void __launch_bounds__(FATHOM_D)
 rotate_query_kernel(const float* q, const float* basis, float* __restrict__ q_rot, int G) {
   __shared__ float s_q[FATHOM_D];
@@ -447,7 +448,7 @@ extern "C" int fathom_rotate_keys(fathom_ctx* ctx, const fathom_layout* L, const
   if (k_dtype != FATHOM_F32 && k_dtype != FATHOM_BF16) return FATHOM_ERR_UNSUPPORTED;
   if (!fathom_aligned16(K) || !fathom_aligned16(basis) || !fathom_aligned16(K_rot)) return FATHOM_ERR_ALIGNMENT;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  // tensor cores (tf32 operands split in two, three products) unless FATHOM_ROTATE_PATH=simt asks for the plain fp32 kernel
+  // tensor cores (operands split in two, three products) unless FATHOM_ROTATE_PATH=simt asks for the plain fp32 kernel
   const char* path = getenv("FATHOM_ROTATE_PATH");
   if (!(path && strcmp(path, "simt") == 0)) return fathom_launch_rotate_tc(ctx, L, K, k_dtype, mean, basis, K_rot, st);
   const size_t smem = (size_t)2 * FATHOM_D * PANEL * sizeof(float);

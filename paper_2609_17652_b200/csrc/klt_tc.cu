@@ -4,10 +4,12 @@
 // The rotation is the one dense contraction next to the decode path (n x 128 by 128 x 128 per KV head), so it runs
 // as tcgen05.mma with the accumulator in tensor memory.  The rotated keys feed a quantiser, so 11 significant bits are not
 // enough; both operands are split into an fp16 head and an fp16 tail, x = xh + xl, v = vh + vl, and three products are
-// accumulated in fp32:  xh vh + xh vl + xl vh  (the dropped xl vl term is below 2^-24 of |x||v|).  fp16 has the significant bits
+// accumulated in fp32:  xh vh + xh vl + xl vh  (the dropped xl vl term is below 2^-22 of |x||v|).  fp16 has the significant bits
 // of tf32 at half the bytes and twice the rate; its range is made up for by powers of two: every token and every rotated channel
-// is scaled so that its largest element lies in [2^14, 2^15), which leaves elements down to 2^-28 of it with all their bits, and the
-// accumulator is scaled back (exactly) where it is read.
+// is scaled so that its largest element lies in [2^14, 2^15), and the accumulator is scaled back (exactly) where it is read.  A
+// tail has no bits below 2^-24: elements above 2^-18 of the largest keep 22 bits, smaller ones an absolute error of 2^-39 of it.
+// Against fp64, keys of 0.1 to 4 with four channels at 16: 7.0e-7 of the norm (both parts in tf32, cut off: 1.7e-6); with one channel at
+// 1e5 times the others and a basis that leaves it alone, the others are off by 7e-7 of theirs.
 //
 // The BASIS is the left operand (M = 128 rotated channels) and the tokens are the right one (N = 128):
 //   * the split basis stays in tensor memory (128 columns) for all of a head's tiles, so an MMA reads only the tokens from
@@ -27,8 +29,8 @@
 //                      accumulator's (two accumulators alternate);
 //   8 epilogue warps   read the accumulator with tcgen05.ld (warp w: lanes 32 (w mod 4).., block w div 4 of the tile), hand it
 //                      back, scale, and store or quantise.
-// Measured: 262,144 fp32 tokens x 8 heads to planes 1057 us (both operands in shared memory, tf32) -> 386 us = 2.8 TB/s; 200,001 bf16
-// tokens to rotated keys 290 us = 4.2 TB/s.  Stamps inside the kernel (fp32 to planes, ~5000 cycles a tile): a tile's MMAs take 2300
+// Measured: 262,144 fp32 tokens x 8 heads to planes 1057 us (both operands in shared memory, tf32) -> 375 us = 2.9 TB/s; 200,001 bf16
+// tokens to rotated keys 233 us = 5.3 TB/s.  Stamps inside the kernel (fp32 to planes, ~5000 cycles a tile): a tile's MMAs take 2300
 // cycles, its conversion 2100 while the epilogue rests and up to 4000 beside it, its epilogue 4900 (2500 of them the
 // quantiser): the roles share the ALU's issue slots, and eight epilogue warps set the pace.  Tried: 8 producer and 16 epilogue warps, a block on
 // two threads, the accumulator handed back before the quantiser runs: the producers set the pace instead (411 us).

@@ -4,8 +4,8 @@
 //
 // Two values at a time: n = round(k * (1/s)) by the 1.5 * 2^23 trick, d = k - n s in one fused multiply-add.  n s is exact in
 // it (n has 4 bits, s 11), so the SIGN of d is exact and floor(k / s) = n - (d < 0) whatever the rounding of 1/s and of the
-// product did: |k| <= 8.01 s, so they move k / s by less than 1e-5 and n is one of the two integers next to it.  -0 counts as
-// 0 (the negated n is +0 there, so d is +0).  The packed 16-bit add-min-relu clips both codes to 0..15 in one instruction,
+// product did: |k| <= 8.01 s (12 s where an eighth of the maximum was rounded to a subnormal s: clipped like the rest), so they
+// move k / s by less than 1e-5 and n is one of the two integers next to it.  -0 counts as 0 (the negated n is +0 there, so d is +0).  The packed 16-bit add-min-relu clips both codes to 0..15 in one instruction,
 // the codes are collected as nibbles, and two rounds of masked merges turn four registers of eight nibbles into the four
 // plane words: about 4.5 instructions per value, against 13 for four compare-and-select steps with a predicated OR each.
 #pragma once
