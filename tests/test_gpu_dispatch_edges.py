@@ -290,3 +290,53 @@ def test_fused_selection_with_more_candidates_than_a_cta_lists(heads_per_plan):
     assert np.array_equal(fused.cpu().numpy(), O.topk(scores[:, :n].double().cpu().numpy(), k, 4, 32))
     assert ctx.fathom_device_status() == 0
     ctx.close()
+
+
+# block maxima whose eighth is rounded to a subnormal fp16 (quotients of up to 12 steps), to the smallest one and to zero; one block per CTA and eight
+@pytest.mark.parametrize("n", [200, 40003])
+def test_planes_of_keys_with_subnormal_scales(n):
+    from paper_2609_17652_b200 import binding as fb
+    lay = fb.make_layout(1, 1, n)
+    ctx = fb.Context(0, fb.fathom_scratch_bytes(lay, 1))
+    g = torch.Generator(device="cuda").manual_seed(n)
+    K = torch.randn(1, n, 128, generator=g, device="cuda") * torch.exp2(torch.linspace(-26, -12, 128, device="cuda"))
+    planes = torch.zeros(1, 128, 4, lay.plane_stride_words, dtype=torch.int64, device="cuda")
+    scales = torch.zeros(1, 128, lay.scale_stride, dtype=torch.int16, device="cuda")
+    ctx.fathom_build_planes(lay, K, planes, scales)
+    ref_planes, ref_scales = O.build_planes(K.cpu().numpy())
+    nb = ref_planes.shape[-1]
+    assert (ref_scales.view(np.uint16) == 0).any() and (ref_scales.view(np.uint16) == 1).any()
+    assert np.array_equal(scales[..., :nb].cpu().numpy().view(np.uint16), ref_scales.view(np.uint16))
+    assert np.array_equal(planes[..., :nb].cpu().numpy().view(np.uint64), ref_planes)
+    # the rotation's own quantiser, against the same keys rotated first: the bits are the same
+    V = torch.linalg.qr(torch.randn(1, 128, 128, generator=g, device="cuda"))[0].contiguous()
+    mean, rotated = torch.zeros(1, 128, device="cuda"), torch.zeros_like(K)
+    again, scales_again = torch.zeros_like(planes), torch.zeros_like(scales)
+    ctx.fathom_rotate_keys(lay, K, mean, V, rotated)
+    ctx.fathom_build_planes(lay, rotated, planes, scales)
+    ctx.fathom_build_planes_rotated(lay, K, mean, V, again, scales_again)
+    assert torch.equal(again, planes) and torch.equal(scales_again, scales)
+    ctx.close()
+
+
+# one channel far above the others in every key, bases that mix it in and one that leaves it alone
+@pytest.mark.parametrize("far", [1e3, 1e5])
+@pytest.mark.parametrize("basis", ["random", "identity"])
+def test_rotation_of_keys_with_one_large_channel(far, basis):
+    from paper_2609_17652_b200 import binding as fb
+    n = 1000
+    lay = fb.make_layout(1, 1, n)
+    ctx = fb.Context(0, fb.fathom_scratch_bytes(lay, 1))
+    g = torch.Generator(device="cuda").manual_seed(int(far))
+    K = torch.randn(1, n, 128, generator=g, device="cuda")
+    K[..., 5] *= far
+    V = torch.eye(128, device="cuda").unsqueeze(0).contiguous() if basis == "identity" else torch.linalg.qr(torch.randn(1, 128, 128, generator=g, device="cuda"))[0].contiguous()
+    mean, out = torch.randn(1, 128, generator=g, device="cuda"), torch.zeros_like(K)
+    ctx.fathom_rotate_keys(lay, K, mean, V, out)
+    X = K.double() - mean.double()
+    magnitude = X.abs() @ V.double().abs()
+    # the difference from the mean rounded to fp32, three terms of 2^-22 for the parts that are left out, 24 accumulations of up to 2^-23
+    # each; 2^-39 of the largest for small elements
+    bound = (2.0 ** -24 + 3 * 2.0 ** -22 + 24 * 2.0 ** -23) * magnitude + 2.0 ** -39 * X.abs().amax(dim=2, keepdim=True) * V.double().abs().sum(dim=1, keepdim=True)
+    assert ((out.double() - X @ V.double()).abs() <= bound).all() and ctx.fathom_device_status() == 0
+    ctx.close()
