@@ -6,24 +6,23 @@
 // every CTA computes all 128 importances (thread = channel; fp64 with explicit round-to-nearest intrinsics,
 // no fused multiply-add, so the ranking is identical on every machine; no logarithm is evaluated) and ranks
 // the 64 candidates of its own 16 channels against all 512, eight threads per candidate (each counts over an
-// eighth of the others: the kernel is a latency chain, and the counting loop is its longest link).  Where that is more
-// than one CTA per SM the importances that every CTA computes again cost more than the shorter chain gives, and four
-// CTAs serve a plan: 24 plans 5.3 -> 5.2 us, 32 plans 7.0 -> 5.3, 64 plans 10.1 -> 9.7; with 128 plans eight are again
-// the better choice (15.9 against 17.2).
+// eighth of the others: the kernel is a latency chain, and the counting loop is its longest link).  Four CTAs per plan take
+// less time behind one another with 32 plans (5.3 us against 7.0), but the decode step more: 30.0 us against 25.1 with 8000
+// tokens, 34.7 against 33.2 with 40,000.
 // Non-negative doubles order like their bit patterns, so the comparisons run on 64-bit integers.
 #include "fathom_common.cuh"
 
 namespace {
 
 constexpr int NCAND = FATHOM_D * FATHOM_NPLANES;   // 512
-constexpr int AD_THREADS = 512;
+constexpr int CTAS_PER_PLAN = 8;
+constexpr int AD_CAND = NCAND / CTAS_PER_PLAN;     // 64 candidates ranked per CTA
+constexpr int AD_SPLIT = 8;                        // threads per candidate
+constexpr int AD_THREADS = AD_CAND * AD_SPLIT;     // 512
 
-template <int CTAS_PER_PLAN>
 __global__ void __launch_bounds__(AD_THREADS)
 alloc_depth_kernel(const float* q, const float* var, int mode, int budget,
                    int heads_per_plan, int G, uint8_t* __restrict__ depth) {
-  constexpr int AD_CAND = NCAND / CTAS_PER_PLAN;              // candidates ranked per CTA: 64 or 128
-  constexpr int AD_SPLIT = AD_THREADS / AD_CAND;              // threads per candidate: 8 or 4
   __shared__ alignas(16) unsigned long long pri[NCAND];       // bit patterns of the (non-negative) priorities
   __shared__ int partial[AD_SPLIT][AD_CAND];
   FATHOM_PDL_WAIT();
@@ -91,7 +90,7 @@ alloc_depth_kernel(const float* q, const float* var, int mode, int budget,
   }
   partial[share][cand] = rank;
   __syncthreads();
-  if (share == 0) {                                           // the first warps: one thread per candidate
+  if (share == 0) {                                           // the first two warps: one thread per candidate
     rank = 0;
 #pragma unroll
     for (int s = 0; s < AD_SPLIT; ++s) rank += partial[s][cand];
@@ -116,15 +115,7 @@ extern "C" int fathom_alloc_depth(fathom_ctx* ctx, const fathom_layout* L, const
   const int G = L->n_q_heads / L->n_kv_heads;
   if (heads_per_plan < 1 || G % heads_per_plan != 0) return FATHOM_ERR_INVALID_ARG;
   const int plans = L->n_q_heads / heads_per_plan;
-  const int sms = fathom_sm_count();
-  const bool wide = plans * 8LL <= sms || plans * 2LL > sms;
-  const dim3 grid(plans * (wide ? 8 : 4));
-  if (wide || (long long)grid.x <= sms) {
-    FATHOM_CUDA_TRY(ctx, fathom_launch_dependent(wide ? alloc_depth_kernel<8> : alloc_depth_kernel<4>, grid, dim3(AD_THREADS), 0,
-                                                 static_cast<cudaStream_t>(stream), q, var, mode, budget, heads_per_plan, G, depth));
-  } else {                                                    // CTAs that start where the kernel before ends lie four to an SM beside empty ones
-    alloc_depth_kernel<4><<<grid, AD_THREADS, 0, static_cast<cudaStream_t>(stream)>>>(q, var, mode, budget, heads_per_plan, G, depth);
-    FATHOM_CUDA_TRY(ctx, cudaGetLastError());
-  }
+  FATHOM_CUDA_TRY(ctx, fathom_launch_dependent(alloc_depth_kernel, dim3(plans * CTAS_PER_PLAN), dim3(AD_THREADS), 0,
+                                               static_cast<cudaStream_t>(stream), q, var, mode, budget, heads_per_plan, G, depth));
   return FATHOM_OK;
 }

@@ -248,7 +248,7 @@ def test_union_of_many_picks(n, k):
     ctx.close()
 
 
-# eight CTAs per plan up to 18 plans and from 75 on, else four
+# one plan, fewer CTAs than SMs, more
 @pytest.mark.parametrize("plans", [1, 18, 19, 74, 75])
 @pytest.mark.parametrize("mode,budget", [("waterfill", 48), ("fixed_top_r", 16), ("uniform", 2)])
 def test_depths_of_few_and_many_plans(plans, mode, budget):
