@@ -1,27 +1,35 @@
-// Top-k of rows of up to 131,072 scores in ONE kernel: a cluster of up to eight CTAs per head holds the row's keys in
+// Top-k of rows of up to 131,072 scores in ONE kernel: a cluster of up to eight CTAs per head holds the row's scores in
 // registers, so whatever the selection has to look at twice is not read twice, and nothing goes through global memory
-// between its steps.  What bounded such rows was the chain of launches (histogram, filter, select and emission with a memset
-// before them: 30 us for 32 heads of 33,001 scores; sample, collection and selection: 21 us at 131,072) and not the data.
+// between its steps.  What bounds such rows is not the data but the instructions that every warp executes once, at some nine
+// cycles each: 512 threads share out a few hundred candidates.  So a step takes as few instructions per warp as possible (a search
+// by one warp over two levels of counts, lists of tokens instead of places computed for every score, one candidate per thread from
+// then on).
 //
 // The order of a head's tokens is that of the 64-bit composite (key << 32 | ~token): larger score first, ties to the lower
-// token.  The steps, with a cluster barrier after 1, 2 and 3:
-//   1. coarse histogram (4096 bins, a thirty-second of an octave where scores usually lie) of the threads' MAXIMA: the bin that holds the want-th largest maximum is a
-//      bound - at least `want` tokens reach its lower edge - and a close one: for want = q groups of EPT tokens a share
-//      1 - (1 - q)^(1 / EPT) of the tokens reaches the want-th maximum.  Where `want` is most of the number of groups the
-//      histogram is of all tokens instead.  Every CTA adds its non-empty bins (a few dozen) to the histograms of all others
-//      through distributed shared memory and finds the bound for itself;
-//   2. the tokens that reach the bound are listed in token order in every CTA's shared memory;
-//   3. the cluster's first CTA pulls the lists, which makes one list in token order of little more than `want` members:
-//      fine histogram (2048 bins of 2^13 keys from the bound on), the members of the bin that the threshold splits (a few
-//      dozen) ranked against one another, and the chosen tokens written in ascending order by a prefix count.
-// (A first form merged whole histograms in every CTA, 64 KB of distributed shared memory each, and exchanged the split bin
-// and the counts as well: 8000 of 30,000 cycles went into the first merge alone, 21.5 us at 33,001 scores.)
-// A list that would not fit (heavy ties) is not pulled: radix rounds of 11 bits over the composites, the digits' counts pushed
-// like in step 1, decide the threshold, and every CTA writes its own tokens.
+// token.  The row is dealt to the CTAs in chunks of 128 tokens, one after the other, so that every CTA holds a sample of the
+// whole row.  There is ONE exchange:
+//   1. coarse histogram (4096 bins, a thirty-second of an octave where scores usually lie) of the maxima of the threads' groups of
+//      tokens, in the CTA's own shared memory: its own bound is the bin that holds the quota-th largest maximum, the quota being its
+//      share of `want` and four standard deviations more;
+//   2. the tokens that reach the CTA's bound are listed, and list, length and bound are written to every CTA of the cluster.  (Where
+//      the large scores lie side by side too many tokens reach what bounds their groups; the bound is then taken from the tokens);
+//   3. after the cluster barrier every CTA finds the want-th largest of all lists: fine histogram (2048 bins of 2^13 keys from the
+//      lowest bound on), the members of the bin that the threshold splits (a few) ranked against one another.  A threshold
+//      that reaches every CTA's bound is exact: all lists are complete down to it.  One that does not is still a bound of the whole
+//      row (`want` tokens reach it), and the lists are made once more with it;
+//   4. every CTA marks the chosen tokens of all lists in a bitmap of the row, whose prefix counts give its own list's tokens their
+//      places in the ascending output.
+// (A first form merged whole histograms in every CTA; a second one merged those of the maxima and let the first CTA pull the lists,
+// select and write alone: three cluster barriers, and seven of eight CTAs idle for 40 % of the time.  32 heads, back to back, second
+// form / this one: 131,072 scores, k = 2048 16.7 / 12.4 us; 65,536, k = 1024 13.4 / 8.6; 33,001, k = 512 12.3 / 7.7; one head of 4096, k = 64 5.8 / 4.3.)
+// A list that would not fit (heavy ties) is not copied: radix rounds of 11 bits over the composites, the digits' counts
+// pushed to all CTAs, decide the threshold.
 // The set is unique and the counts are integers: the result does not depend on any order of atomics.
 #include "topk_shared.cuh"
 
 #include <cooperative_groups.h>
+
+#include <cstddef>
 
 namespace cg = cooperative_groups;
 
@@ -32,7 +40,10 @@ constexpr int RT_WARPS = RT_THREADS / 32;
 constexpr int MAX_CLUSTER = 8;
 constexpr int COARSE = 4096;
 constexpr int FINE = 2048, FINE_SHIFT = 13;
+constexpr int SUPER = 32;                                     // bins of a histogram that are also counted together
 constexpr int SPLIT = 512;                                    // members of a split bin ranked by comparison
+constexpr int CHUNK = 128, MAX_CHUNKS = (int)(FATHOM_TOPK_RESIDENT_MAX / CHUNK);
+constexpr int MOST_LISTED = 16384;                            // over all lists of a cluster of several CTAs
 
 // Coarse bin of a score (monotone, -0 with +0) and its lower edge.  Magnitudes from 2^-16 to 2^16 have 32 bins per octave, the others
 // four: with the same eight everywhere (the 12 leading key bits) a head whose threshold fell to the upper end of a bin had twice
@@ -55,250 +66,258 @@ __device__ __forceinline__ float coarse_edge(uint32_t bin) {
 }
 
 struct ResidentSmem {
-  alignas(16) uint32_t mine[COARSE];                          // this CTA's counts; the selecting CTA's fine histogram; members of its split bin
-  alignas(16) uint32_t merged[COARSE];                        // the cluster's
-  uint32_t warp_sum[RT_WARPS];
-  uint32_t cta_count[MAX_CLUSTER];                            // listed (later: chosen) tokens per CTA, pushed by each of them
-  uint32_t found_bin, found_above, found_count, split_count;
+  alignas(16) uint32_t coarse[COARSE];                        // counts of this CTA's maxima; then members of the split bin and places of the chunks,
+                                                              // or the digits' counts, this CTA's and the cluster's
+  uint32_t coarse_super[COARSE / SUPER];
+  uint32_t fine[FINE];                                        // counts of the lists
+  uint32_t fine_super[FINE / SUPER];
+  alignas(16) uint32_t warp_sum[RT_WARPS];
+  uint2 seg[MAX_CLUSTER];                                     // length and bound of every CTA's list, written by each of them
+  uint32_t listed, found_bin, found_above, found_count, split_count;
   unsigned long long threshold;
-  unsigned long long list[1];                                 // [capacity] composites
+  alignas(16) unsigned long long list[1];                     // [ctas][capacity] composites, [capacity] tokens of this CTA's list, [chunks] uint4 of
+                                                              // chosen tokens of the whole row
 };
-static_assert(SPLIT * 8 <= (COARSE - FINE) * 4, "the members of the split bin lie behind the fine histogram");
+constexpr int COUNTS = COARSE + COARSE / SUPER + FINE + FINE / SUPER;
+static_assert(offsetof(ResidentSmem, warp_sum) == COUNTS * 4 && COUNTS % 4 == 0, "the counts lie side by side");
+static_assert(SPLIT * 8 + MAX_CHUNKS * 4 <= COARSE * 4, "the split bin and the places fit over the coarse counts");
 
-// Finds the largest of BINS bins whose suffix count reaches `rank` (> 0) and leaves bin, the count above it and its own count in M
-// (all threads may read them afterwards).  If there are fewer than `rank`: bin 0 with everything.
+// One warp: the largest bin whose suffix count reaches `rank` (> 0), the count above it and its own, in every lane.  If there are
+// fewer than `rank`: bin 0 with everything.
 template <int BINS>
-__device__ __forceinline__ void find_bin(ResidentSmem& M, const uint32_t* hist, uint32_t rank) {
-  constexpr int PER = BINS / RT_THREADS;                      // thread t owns bins BINS - 1 - PER t .. descending
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+__device__ __forceinline__ void search_bins(const uint32_t* bins, const uint32_t* super, uint32_t rank, uint32_t& bin, uint32_t& above, uint32_t& count) {
+  constexpr int PER = BINS / SUPER / 32;                      // lane l owns super bins BINS / SUPER - 1 - PER l .. descending
+  const int lane = threadIdx.x & 31;
   uint32_t c[PER], local = 0u;
 #pragma unroll
-  for (int v = 0; v < PER / 4; ++v) {
-    const uint4 x = *reinterpret_cast<const uint4*>(hist + BINS - PER * tid - 4 * v - 4);
-    c[4 * v] = x.w; c[4 * v + 1] = x.z; c[4 * v + 2] = x.y; c[4 * v + 3] = x.x;
-    local += x.x + x.y + x.z + x.w;
+  for (int u = 0; u < PER; ++u) {
+    c[u] = super[BINS / SUPER - 1 - PER * lane - u];
+    local += c[u];
   }
-  uint32_t incl = local;
+  auto inclusive = [&](uint32_t x) {
 #pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
-    if (lane >= o) incl += y;
-  }
-  if (lane == 31) M.warp_sum[warp] = incl;
-  __syncthreads();
-  uint32_t above = incl - local;
-#pragma unroll
-  for (int w = 0; w < RT_WARPS; ++w) above += w < warp ? M.warp_sum[w] : 0u;
-  if (above < rank && above + local >= rank) {
-    uint32_t run = above;
-#pragma unroll
-    for (int b = 0; b < PER; ++b) {
-      if (run < rank && run + c[b] >= rank) {
-        M.found_bin = (uint32_t)(BINS - 1 - (PER * tid + b));
-        M.found_above = run;
-        M.found_count = c[b];
-      }
-      run += c[b];
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+      if (lane >= o) x += y;
     }
+    return x;
+  };
+  uint32_t incl = inclusive(local);
+  const unsigned reach = __ballot_sync(0xffffffffu, incl >= rank);
+  if (reach == 0u) {
+    bin = above = 0u;
+    count = __shfl_sync(0xffffffffu, incl, 31);
+    return;
   }
-  if (tid == RT_THREADS - 1 && above + local < rank) { M.found_bin = 0u; M.found_above = 0u; M.found_count = above + local; }
+  uint32_t run = incl - local;
+  int u = 0;
+#pragma unroll
+  for (int x = 0; x < PER - 1; ++x)
+    if (u == x && run + c[x] < rank) { run += c[x]; u = x + 1; }
+  const int from = __ffs(reach) - 1;
+  run = __shfl_sync(0xffffffffu, run, from);
+  u = __shfl_sync(0xffffffffu, u, from);
+  const int first = (BINS / SUPER - 1 - PER * from - u) * SUPER;
+  const uint32_t mine = bins[first + SUPER - 1 - lane];
+  incl = run + inclusive(mine);
+  const int at = __ffs(__ballot_sync(0xffffffffu, incl >= rank)) - 1;
+  bin = (uint32_t)(first + SUPER - 1 - at);
+  count = __shfl_sync(0xffffffffu, mine, at);
+  above = __shfl_sync(0xffffffffu, incl, at) - count;
+}
+
+// All threads of the CTA, after a barrier that completes the counts: what search_bins finds, in M (with a barrier behind it).
+template <int BINS>
+__device__ __forceinline__ void find_bin(ResidentSmem& M, const uint32_t* bins, const uint32_t* super, uint32_t rank) {
+  if (threadIdx.x < 32) {
+    uint32_t bin, above, count;
+    search_bins<BINS>(bins, super, rank, bin, above, count);
+    if (threadIdx.x == 0) { M.found_bin = bin; M.found_above = above; M.found_count = count; }
+  }
   __syncthreads();
 }
 
+// groups: 1 = one group of tokens per thread, 2 = two, 4 = one per four tokens, 0 = every token a group
 template <int EPT>
 __global__ void __launch_bounds__(RT_THREADS, 2)
-topk_resident_kernel(const float* scores, int n, long long score_stride, int elig_lo, int elig_hi, int k, uint32_t want,
-                     int by_maxima, uint32_t capacity, int32_t* __restrict__ idx_out, uint32_t* __restrict__ dev_status) {
+topk_resident_kernel(const float* scores, int n, long long score_stride, int elig_lo, int elig_hi, int k, uint32_t want, uint32_t quota,
+                     int groups, uint32_t capacity, int32_t* __restrict__ idx_out, uint32_t* __restrict__ dev_status) {
   extern __shared__ __align__(16) unsigned char resident_smem[];
   ResidentSmem& M = *reinterpret_cast<ResidentSmem*>(resident_smem);
   cg::cluster_group cluster = cg::this_cluster();
   const int ctas = (int)cluster.num_blocks(), rank = (int)cluster.block_rank(), head = blockIdx.x / ctas;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  for (int b = tid; b < 2 * COARSE / 4; b += RT_THREADS) reinterpret_cast<uint4*>(M.mine)[b] = make_uint4(0u, 0u, 0u, 0u);
+  auto started = cluster.barrier_arrive();                    // (nothing is written to a CTA's shared memory before it runs)
+  const int chunks = (n + CHUNK - 1) / CHUNK;
+  uint32_t* own = reinterpret_cast<uint32_t*>(M.list + (size_t)ctas * capacity);             // (capacity is a multiple of 4)
+  uint4* bits = reinterpret_cast<uint4*>(own + capacity);
+  unsigned long long* split = reinterpret_cast<unsigned long long*>(M.coarse);
+  uint32_t* places = M.coarse + 2 * SPLIT;
+  for (int b = tid; b < COUNTS / 4; b += RT_THREADS) reinterpret_cast<uint4*>(M.coarse)[b] = make_uint4(0u, 0u, 0u, 0u);
+  for (int b = tid; b < chunks; b += RT_THREADS) bits[b] = make_uint4(0u, 0u, 0u, 0u);
+  if (tid == 0) M.listed = M.split_count = 0u;
   __syncthreads();
-  auto cleared = cluster.barrier_arrive();                    // my histograms are clear (others will add to one of them)
   FATHOM_PDL_WAIT();                                          // the scores come from the previous kernel
   FATHOM_PDL_RELEASE();                                       // the attention that follows may become resident now
 
-  // ---- my tokens: token(i) = wbase + 128 (i / 4) + 4 lane + i % 4: the warp's loads are runs of 512 bytes.  They are kept as scores
-  //      and compared as scores (a key is only formed for the few that matter); NaN stands for a token that is not eligible
+  // ---- my tokens: chunks warp ctas + rank, RT_WARPS ctas further on, .. of the row, 4 consecutive ones per lane.  They are kept as
+  //      scores and compared as scores (a key is only formed for the few that matter); NaN stands for a token that is not eligible
   constexpr int V = EPT / 4;
-  const int wbase = (rank * RT_WARPS + warp) * 32 * EPT;      // n <= 131072
+  const int chunk0 = warp * ctas + rank, chunk_step = RT_WARPS * ctas;        // n <= 131072
   const float* row = scores + (size_t)head * (size_t)score_stride;
   const float NONE = __uint_as_float(0x7fffffffu);
-  auto token = [&](int i) { return wbase + 128 * (i >> 2) + 4 * lane + (i & 3); };
+  auto token = [&](int i) { return (chunk0 + (i >> 2) * chunk_step) * CHUNK + 4 * lane + (i & 3); };
   float x[EPT];
-  {
-    const float* src = row + wbase + 4 * lane;                // (score_stride is a multiple of 4: a float4 stays inside the row)
-    if (wbase + 32 * EPT <= n) {                              // (uniform over the warp)
 #pragma unroll
-      for (int v = 0; v < V; ++v) *reinterpret_cast<float4*>(x + 4 * v) = *reinterpret_cast<const float4*>(src + 128 * v);
-    } else {
+  for (int v = 0; v < V; ++v)                                 // (score_stride is a multiple of 4: a float4 stays inside the row)
+    *reinterpret_cast<float4*>(x + 4 * v) = token(4 * v) < n ? *reinterpret_cast<const float4*>(row + token(4 * v)) : make_float4(NONE, NONE, NONE, NONE);
 #pragma unroll
-      for (int v = 0; v < V; ++v)
-        *reinterpret_cast<float4*>(x + 4 * v) = token(4 * v) < n ? *reinterpret_cast<const float4*>(src + 128 * v) : make_float4(NONE, NONE, NONE, NONE);
-    }
-    if (wbase < elig_lo || wbase + 32 * EPT > elig_hi) {
+  for (int v = 0; v < V; ++v) {
+    const int first = (chunk0 + v * chunk_step) * CHUNK;
+    if (first < elig_lo || first + CHUNK > elig_hi) {         // (uniform over the warp)
 #pragma unroll
-      for (int i = 0; i < EPT; ++i)
+      for (int i = 4 * v; i < 4 * v + 4; ++i)
         if (token(i) < elig_lo || token(i) >= elig_hi) x[i] = NONE;
     }
   }
-  auto composite = [&](int i) { return ((unsigned long long)ordered_key(x[i]) << 32) | (uint32_t)~(uint32_t)token(i); };
 
-  // the non-empty bins of my histogram are added to every CTA's merged one
-  auto push = [&](int bins) {
-    for (int b = tid; b < bins; b += RT_THREADS) {
-      const uint32_t c = M.mine[b];
-      if (c)
-        for (int r = 0; r < ctas; ++r) atomicAdd(cluster.map_shared_rank(M.merged, r) + b, c);
+  // ---- 1. my bound
+  auto count = [&](float m) {
+    if (m == m) {
+      const uint32_t b = coarse_bin(m);
+      atomicAdd(&M.coarse[b], 1u);
+      atomicAdd(&M.coarse_super[b / SUPER], 1u);
     }
   };
-
-  // ---- 1. a bound: its coarse bin
-  if (by_maxima) {
-    float m = x[0];
-#pragma unroll
-    for (int i = 1; i < EPT; ++i) m = fmaxf(m, x[i]);          // (a NaN is no maximum)
-    if (m == m) atomicAdd(&M.mine[coarse_bin(m)], 1u);
-  } else {
-#pragma unroll
-    for (int i = 0; i < EPT; ++i)
-      if (x[i] == x[i]) atomicAdd(&M.mine[coarse_bin(x[i])], 1u);
-  }
-  __syncthreads();
-  cluster.barrier_wait(std::move(cleared));                   // (everyone arrived long ago)
-  push(COARSE);
-  cluster.sync();
-  uint32_t base = 0u;                                         // candidates are the scores from bound on, whose key is base
   float bound = NONE;                                         // (nothing wanted: none)
-  if (want) {
-    find_bin<COARSE>(M, M.merged, want);
-    for (int b = tid; b < FINE; b += RT_THREADS) M.mine[b] = 0u;             // (everyone's counts have been pushed)
-    bound = M.found_bin == 0u ? -INFINITY : coarse_edge(M.found_bin);       // (bin 0: everything, see find_bin)
-    base = ordered_key(bound);
-  }
-
-  // ---- places of a set of my tokens (bit i of `set`) among the CTA's, in token order: the counts of a lane's 4-token runs are
-  //      prefix-summed over the warp four runs at a time (a byte each: at most 128), run totals and warp totals added
-  auto place = [&](uint32_t set, uint32_t (&at)[V]) -> uint32_t {
-    uint32_t total = 0u;
+  bool exact = false;                                         // the bound is as close as it gets
+  bool fits = quota <= capacity;                              // (a quota that no list holds: straight to the radix rounds)
+  if (want && fits) {
+    auto largest = [&](int i0, int i1) {
+      float m = x[i0];
 #pragma unroll
-    for (int g = 0; g < (V + 3) / 4; ++g) {
-      uint32_t c = 0u;
+      for (int i = i0 + 1; i < i1; ++i) m = fmaxf(m, x[i]);   // (a NaN is no maximum)
+      return m;
+    };
+    if (groups == 1) {
+      count(largest(0, EPT));
+    } else if (groups == 2) {
+      count(largest(0, EPT / 2));
+      count(largest(EPT / 2, EPT));
+    } else if (groups == 4) {
 #pragma unroll
-      for (int v = 4 * g; v < 4 * g + 4 && v < V; ++v) c |= (uint32_t)__popc((set >> (4 * v)) & 15u) << (8 * (v - 4 * g));
-      uint32_t incl = c;
+      for (int v = 0; v < V; ++v) count(largest(4 * v, 4 * v + 4));
+    } else {
 #pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += y;
-      }
-      const uint32_t last = __shfl_sync(0xffffffffu, incl, 31), before = incl - c;
-#pragma unroll
-      for (int v = 4 * g; v < 4 * g + 4 && v < V; ++v) {
-        at[v] = total + ((before >> (8 * (v - 4 * g))) & 255u);
-        total += (last >> (8 * (v - 4 * g))) & 255u;
-      }
-    }
-    __syncthreads();                                          // (warp_sum may still be read)
-    if (lane == 0) M.warp_sum[warp] = total;
-    __syncthreads();
-    uint32_t ahead = 0u, all = 0u;
-#pragma unroll
-    for (int w = 0; w < RT_WARPS; ++w) {
-      const uint32_t s = M.warp_sum[w];
-      ahead += w < warp ? s : 0u;
-      all += s;
-    }
-#pragma unroll
-    for (int v = 0; v < V; ++v) at[v] += ahead;
-    return all;
-  };
-
-  // ---- 2. the tokens that reach the bound
-  uint32_t set = 0u, at[V];
-#pragma unroll
-  for (int i = 0; i < EPT; ++i) set |= (x[i] >= bound ? 1u : 0u) << i;
-  const uint32_t listed = place(set, at);
-  if (listed <= capacity) {                                   // (uniform) as (score, token) pairs: keys are formed by the CTA that selects
-#pragma unroll
-    for (int v = 0; v < V; ++v) {
-      if ((set >> (4 * v)) & 15u) {
-        uint2* to = reinterpret_cast<uint2*>(M.list) + at[v];
-#pragma unroll
-        for (int c = 0; c < 4; ++c)
-          if ((set >> (4 * v + c)) & 1u) *to++ = make_uint2(__float_as_uint(x[4 * v + c]), (uint32_t)token(4 * v + c));
-      }
-    }
-  }
-  if (tid < ctas) cluster.map_shared_rank(M.cta_count, tid)[rank] = listed;
-  cluster.sync();
-  uint32_t total = 0u;
-  for (int r = 0; r < ctas; ++r) total += M.cta_count[r];
-  int32_t* out = idx_out + (size_t)head * k;
-  const uint32_t n_sink = (uint32_t)elig_lo, n_local = (uint32_t)(n - elig_hi);
-
-  if (total <= capacity) {                                    // (the same for the whole cluster)
-    auto fine = [&](uint32_t key) { return min((key - base) >> FINE_SHIFT, (uint32_t)(FINE - 1)); };
-    // ---- 3. the first CTA selects
-    if (rank == 0) {
-      uint32_t start[MAX_CLUSTER];                            // where each CTA's list starts in the joint one
-      start[0] = 0u;
-#pragma unroll
-      for (int r = 1; r < MAX_CLUSTER; ++r) start[r] = start[r - 1] + (r - 1 < ctas ? M.cta_count[r - 1] : 0u);
-      for (uint32_t e0 = 0u; e0 < total; e0 += RT_THREADS * 8) {
-        uint2 c[8];                                           // eight loads in flight
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
-          const uint32_t e = e0 + u * RT_THREADS + tid;
-          if (e < total) {
-            int r = 0;
-            uint32_t s = 0u;
-#pragma unroll
-            for (int y = 1; y < MAX_CLUSTER; ++y)
-              if (y < ctas && e >= start[y]) { r = y; s = start[y]; }
-            c[u] = reinterpret_cast<const uint2*>(cluster.map_shared_rank(M.list, r))[e - s];
-          }
-        }
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
-          const uint32_t e = e0 + u * RT_THREADS + tid;
-          if (e < total) {
-            const uint32_t key = ordered_key(__uint_as_float(c[u].x));
-            M.list[e] = ((unsigned long long)key << 32) | (uint32_t)~c[u].y;
-            atomicAdd(&M.mine[fine(key)], 1u);
-          }
-        }
-      }
-      if (tid == 0) M.split_count = 0u;
-    }
-    auto pulled = cluster.barrier_arrive();
-    if (rank != 0) {
-      cluster.barrier_wait(std::move(pulled));
-      return;
+      for (int i = 0; i < EPT; ++i) count(x[i]);
     }
     __syncthreads();
-    unsigned long long T = 0ull;                              // fewer than wanted (non-finite scores), or just as many: all of them
+    find_bin<COARSE>(M, M.coarse, M.coarse_super, quota);
+    bound = M.found_bin == 0u ? -INFINITY : coarse_edge(M.found_bin);         // (bin 0: everything, see search_bins)
+  }
+  cluster.barrier_wait(std::move(started));                   // (everyone arrived long ago)
+
+  // ---- every warp of a CTA works on one of the lists
+  const int per_list = RT_WARPS / ctas, my_list = warp / per_list;            // (ctas is a power of two, at most 8)
+  const uint32_t e_first = (uint32_t)(warp % per_list) * 32 + lane, e_step = (uint32_t)per_list * 32;
+  const unsigned long long* mine = M.list + (size_t)my_list * capacity;
+
+  unsigned long long T = 0ull;                                // the smallest composite that is selected
+  float least = -INFINITY;                                    // no smaller score is selected
+  while (fits) {
+    // ---- 2. the tokens that reach the bound, in any order
+    uint32_t listed;
+    for (;;) {
+      uint32_t set = 0u;
+#pragma unroll
+      for (int i = 0; i < EPT; ++i)
+        if (x[i] >= bound) set |= 1u << i;
+      if (set) {
+        uint32_t at = atomicAdd(&M.listed, (uint32_t)__popc(set));
+        do {
+          const int i = __ffs(set) - 1;
+          set &= set - 1u;
+          if (at < capacity) own[at] = (uint32_t)token(i);
+          ++at;
+        } while (set);
+      }
+      __syncthreads();
+      listed = M.listed;
+      if (listed <= capacity || exact) break;                 // (the same for the whole CTA)
+      // the large scores lie side by side, or in one bin: a bound that the quota of tokens, not of groups, reaches, to 2^10 keys
+      exact = true;
+      for (int b = tid; b < COARSE + COARSE / SUPER; b += RT_THREADS) M.coarse[b] = 0u;
+      __syncthreads();
+#pragma unroll
+      for (int i = 0; i < EPT; ++i)
+        if (x[i] >= bound) count(x[i]);
+      __syncthreads();
+      find_bin<COARSE>(M, M.coarse, M.coarse_super, quota);
+      const uint32_t bin = M.found_bin, rest = quota - M.found_above;
+      if (bin != 0u) {
+        const uint32_t edge = ordered_key(coarse_edge(bin));
+#pragma unroll
+        for (int i = 0; i < EPT; ++i)
+          if (x[i] >= bound && coarse_bin(x[i]) == bin) {
+            const uint32_t b = min((ordered_key(x[i]) - edge) >> 10, (uint32_t)(FINE - 1));
+            atomicAdd(&M.fine[b], 1u);
+            atomicAdd(&M.fine_super[b / SUPER], 1u);
+          }
+        __syncthreads();                                      // (found_bin and found_above have been read, too)
+        find_bin<FINE>(M, M.fine, M.fine_super, rest);
+        bound = fmaxf(bound, key_to_float(edge + (M.found_bin << 10)));
+      }
+      for (int b = tid; b < FINE + FINE / SUPER; b += RT_THREADS) M.fine[b] = 0u;
+      if (tid == 0) M.listed = 0u;
+      __syncthreads();
+    }
+    if (listed <= capacity) {
+      for (uint32_t e = tid; e < listed; e += RT_THREADS) {
+        const uint32_t t = own[e];
+        const unsigned long long c = ((unsigned long long)ordered_key(row[t]) << 32) | (uint32_t)~t;         // (the row's line is in the L1)
+        unsigned long long* to = M.list + (size_t)rank * capacity + e;
+#pragma unroll 1
+        for (int r = 0; r < ctas; ++r) *cluster.map_shared_rank(to, r) = c;
+      }
+    }
+    if (tid < ctas) *cluster.map_shared_rank(&M.seg[rank], tid) = make_uint2(listed, __float_as_uint(bound));
+    if (ctas > 1) cluster.sync();
+    else __syncthreads();
+
+    // ---- 3. the want-th largest of all lists
+    const uint2 theirs = lane < ctas ? M.seg[lane] : make_uint2(0u, __float_as_uint(bound));
+    const uint32_t their_key = ordered_key(__uint_as_float(theirs.y));
+    const uint32_t total = __reduce_add_sync(0xffffffffu, theirs.x);
+    const uint32_t base = __reduce_min_sync(0xffffffffu, their_key), top = __reduce_max_sync(0xffffffffu, their_key);   // keys of the lowest and the highest bound
+    const uint32_t count = __shfl_sync(0xffffffffu, theirs.x, my_list);
+    fits = !__any_sync(0xffffffffu, theirs.x > capacity);
+    if (total >= want) least = key_to_float(base);
+    if (!fits || !want) break;                                // (the same for the whole cluster, like every other way out)
+    T = 0ull;                                                 // fewer than wanted, or just as many: all of them
     if (total > want) {
-      find_bin<FINE>(M, M.mine, want);
+      auto fine = [&](uint32_t key) { return min((key - base) >> FINE_SHIFT, (uint32_t)(FINE - 1)); };
+      for (uint32_t e = e_first; e < count; e += e_step) {
+        const uint32_t b = fine((uint32_t)(mine[e] >> 32));
+        atomicAdd(&M.fine[b], 1u);
+        atomicAdd(&M.fine_super[b / SUPER], 1u);
+      }
+      __syncthreads();
+      find_bin<FINE>(M, M.fine, M.fine_super, want);
       const uint32_t bin = M.found_bin, members = M.found_count, need = want - M.found_above;
       T = (unsigned long long)(base + (bin << FINE_SHIFT)) << 32;
       if (need != members) {                                  // the bin is split: its members are ranked
-        unsigned long long* split = reinterpret_cast<unsigned long long*>(M.mine + FINE);
         if (members <= (uint32_t)SPLIT) {
-#pragma unroll 4
-          for (uint32_t e = tid; e < total; e += RT_THREADS) {
-            const unsigned long long c = M.list[e];
+          for (uint32_t e = e_first; e < count; e += e_step) {
+            const unsigned long long c = mine[e];
             if (fine((uint32_t)(c >> 32)) == bin) split[atomicAdd(&M.split_count, 1u)] = c;
           }
           __syncthreads();
-          for (uint32_t i = warp; i < members; i += RT_WARPS) {             // a warp per member, its lanes over the others
-            const unsigned long long mine = split[i];
+          for (uint32_t i = warp; i < members; i += RT_WARPS) {               // a warp per member, its lanes over the others
+            const unsigned long long c = split[i];
             uint32_t larger = 0u;
-            for (uint32_t j = lane; j < members; j += 32) larger += split[j] > mine;
+            for (uint32_t j = lane; j < members; j += 32) larger += split[j] > c;
             larger = __reduce_add_sync(0xffffffffu, larger);
-            if (lane == 0 && larger + 1u == need) M.threshold = mine;
+            if (lane == 0 && larger + 1u == need) M.threshold = c;
           }
           __syncthreads();
           T = M.threshold;
@@ -307,119 +326,192 @@ topk_resident_kernel(const float* scores, int n, long long score_stride, int eli
           uint32_t left = need;
           for (int hi = 64; hi > 0;) {
             const int lo = hi > 11 ? hi - 11 : 0;
-            for (int b = tid; b < FINE; b += RT_THREADS) M.mine[b] = 0u;
+            for (int b = tid; b < FINE + FINE / SUPER; b += RT_THREADS) M.fine[b] = 0u;
             __syncthreads();
-            for (uint32_t e = tid; e < total; e += RT_THREADS) {
-              const unsigned long long c = M.list[e];
-              if (fine((uint32_t)(c >> 32)) == bin && (hi == 64 || (c >> hi) == (prefix >> hi))) atomicAdd(&M.mine[(uint32_t)(c >> lo) & ((1u << (hi - lo)) - 1u)], 1u);
+            for (uint32_t e = e_first; e < count; e += e_step) {
+              const unsigned long long c = mine[e];
+              if (fine((uint32_t)(c >> 32)) == bin && (hi == 64 || (c >> hi) == (prefix >> hi))) {
+                const uint32_t digit = (uint32_t)(c >> lo) & ((1u << (hi - lo)) - 1u);
+                atomicAdd(&M.fine[digit], 1u);
+                atomicAdd(&M.fine_super[digit / SUPER], 1u);
+              }
             }
             __syncthreads();
-            find_bin<FINE>(M, M.mine, left);
+            find_bin<FINE>(M, M.fine, M.fine_super, left);
             prefix |= (unsigned long long)M.found_bin << lo;
             left -= M.found_above;
-            const bool whole = left == M.found_count;
-            __syncthreads();
             hi = lo;
-            if (whole) break;
+            if (left == M.found_count) break;
+            __syncthreads();                                  // (M.found_count has been read)
           }
           T = prefix;
         }
       }
     }
-    // ---- ascending output: a warp takes a slice of the list, 32 entries at a time
-    const uint32_t slice = ((total + RT_THREADS - 1) / RT_THREADS) * 32, s0 = warp * slice, s1 = min(total, s0 + slice);
-    uint32_t count = 0u;
-#pragma unroll 4
-    for (uint32_t e = s0; e < s1; e += 32) count += __popc(__ballot_sync(0xffffffffu, e + lane < s1 && M.list[e + lane] >= T));
-    if (lane == 0) M.warp_sum[warp] = count;
+    // complete: the threshold reaches every bound, or every CTA has listed all that it has
+    const uint32_t lowest = ordered_key(-INFINITY);
+    const uint32_t t_key = total > want ? (uint32_t)(T >> 32) : (total == want ? base : 0u);
+    if (t_key >= top || top == lowest) {
+      // ---- 4. the chosen tokens of the row
+      for (uint32_t e = e_first; e < count; e += e_step) {
+        const unsigned long long c = mine[e];
+        const uint32_t t = ~(uint32_t)c;
+        if (c >= T) atomicOr(reinterpret_cast<uint32_t*>(bits) + t / 32, 1u << (t & 31));
+      }
+      __syncthreads();
+      break;
+    }
+    // another round: `want` tokens reach the threshold (where fewer than `want` were listed nothing less than everything will do)
+    bound = total >= want ? key_to_float(max(t_key, lowest)) : -INFINITY;
+    exact = true;
+    if (ctas > 1) cluster.sync();                             // (nobody reads the old lists any more)
+    else __syncthreads();
+    for (int b = tid; b < FINE + FINE / SUPER; b += RT_THREADS) M.fine[b] = 0u;
+    if (tid == 0) M.listed = M.split_count = 0u;
     __syncthreads();
-    uint32_t pos = n_sink, chosen = 0u;
+  }
+
+  uint32_t chosen = 0u;                                       // without lists, bit i: token(i) is selected by its score
+  if (!fits) {
+    // ---- more candidates than a list holds: 11-bit digits of the composites, over the whole cluster
+    auto composite = [&](int i) { return ((unsigned long long)ordered_key(x[i]) << 32) | (uint32_t)~(uint32_t)token(i); };
+    uint32_t *counts = M.coarse, *all = M.coarse + FINE;      // this CTA's and the cluster's
+    uint32_t* all_super = M.coarse_super;
+    static_assert(2 * FINE <= COARSE, "both fit");
+    uint32_t left = want;
+    T = 0ull;
+    for (int hi = 64; hi > 0;) {
+      const int lo = hi > 11 ? hi - 11 : 0;
+      for (int b = tid; b < COARSE; b += RT_THREADS) M.coarse[b] = 0u;
+      cluster.sync();
 #pragma unroll
-    for (int w = 0; w < RT_WARPS; ++w) {
-      const uint32_t s = M.warp_sum[w];
-      pos += w < warp ? s : 0u;
-      chosen += s;
+      for (int i = 0; i < EPT; ++i) {
+        const unsigned long long c = composite(i);
+        if (x[i] >= least && (hi == 64 || (c >> hi) == (T >> hi))) atomicAdd(&counts[(uint32_t)(c >> lo) & ((1u << (hi - lo)) - 1u)], 1u);
+      }
+      __syncthreads();
+      for (int b = tid; b < FINE; b += RT_THREADS) {          // the non-empty bins are added to every CTA's counts of the cluster
+        const uint32_t c = counts[b];
+        if (c)
+          for (int r = 0; r < ctas; ++r) atomicAdd(cluster.map_shared_rank(all, r) + b, c);
+      }
+      cluster.sync();
+      {                                                       // four bins per thread, eight threads a super bin
+        static_assert(FINE == 4 * RT_THREADS && SUPER == 32, "every bin once");
+        const uint4 c = *reinterpret_cast<const uint4*>(all + 4 * tid);
+        uint32_t sum = c.x + c.y + c.z + c.w;
+#pragma unroll
+        for (int o = 1; o < 8; o <<= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+        if ((tid & 7) == 0) all_super[tid / 8] = sum;
+      }
+      __syncthreads();
+      find_bin<FINE>(M, all, all_super, left);
+      T |= (unsigned long long)M.found_bin << lo;
+      left -= M.found_above;
+      hi = lo;
+      if (left == M.found_count) break;
+      __syncthreads();                                        // (M.found_count has been read)
     }
-#pragma unroll 4
-    for (uint32_t e = s0; e < s1; e += 32) {
-      const unsigned long long c = e + lane < s1 ? M.list[e + lane] : 0ull;
-      const bool take = e + lane < s1 && c >= T;
-      const unsigned b = __ballot_sync(0xffffffffu, take);
-      if (take) out[pos + __popc(b & ((1u << lane) - 1u))] = (int32_t)~(uint32_t)c;
-      pos += __popc(b);
+#pragma unroll
+    for (int i = 0; i < EPT; ++i)
+      if (x[i] >= least && composite(i) >= T) chosen |= 1u << i;
+#pragma unroll
+    for (int v = 0; v < V; ++v) {                             // every warp tells all CTAs its chunks' tokens, eight lanes a word
+      uint32_t w = ((chosen >> (4 * v)) & 15u) << (4 * (lane & 7));
+#pragma unroll
+      for (int o = 1; o < 8; o <<= 1) w |= __shfl_xor_sync(0xffffffffu, w, o);
+      const int at = chunk0 + v * chunk_step;
+      if ((lane & 7) < ctas && at < chunks) *(cluster.map_shared_rank(reinterpret_cast<uint32_t*>(bits), lane & 7) + 4 * at + (lane >> 3)) = w;
     }
+    cluster.sync();                                           // (nobody touches another CTA's shared memory after this)
+  }
+
+  // ---- places: the exclusive prefix of the chunks' counts
+  uint32_t picked;                                            // tokens selected by score, of the whole row
+  {
+    static_assert(MAX_CHUNKS == 2 * RT_THREADS, "one or two chunks per thread");
+    auto ones = [](const uint4& w) { return (uint32_t)(__popc(w.x) + __popc(w.y) + __popc(w.z) + __popc(w.w)); };
+    const bool two = chunks > RT_THREADS;
+    const int c0 = two ? 2 * tid : tid;
+    uint32_t first = 0u, incl = 0u;
+    if (c0 < chunks) {
+      first = ones(bits[c0]);
+      incl = first + (two && c0 + 1 < chunks ? ones(bits[c0 + 1]) : 0u);
+    }
+    const uint32_t local = incl;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += y;
+    }
+    if (lane == 31) M.warp_sum[warp] = incl;
+    __syncthreads();
+    const uint32_t s = lane < RT_WARPS ? M.warp_sum[lane] : 0u;
+    picked = __reduce_add_sync(0xffffffffu, s);
+    const uint32_t before = __reduce_add_sync(0xffffffffu, lane < warp ? s : 0u) + incl - local;
+    if (c0 < chunks) {
+      places[c0] = before;
+      if (two) places[c0 + 1] = before + first;
+    }
+    __syncthreads();
+  }
+  int32_t* out = idx_out + (size_t)head * k;
+  const uint32_t n_sink = (uint32_t)elig_lo, n_local = (uint32_t)(n - elig_hi);
+  auto write = [&](uint32_t t) {
+    const uint4 w = bits[t / CHUNK];
+    const uint32_t part = t % CHUNK / 32, word = part == 0 ? w.x : (part == 1 ? w.y : (part == 2 ? w.z : w.w));
+    uint32_t pos = n_sink + places[t / CHUNK] + __popc(word & ((1u << (t & 31)) - 1u));
+    pos += part > 0 ? __popc(w.x) : 0;
+    pos += part > 1 ? __popc(w.y) : 0;
+    pos += part > 2 ? __popc(w.z) : 0;
+    if (pos < (uint32_t)k) out[pos] = (int32_t)t;
+  };
+  if (fits) {
+    const uint32_t count = M.seg[rank].x;
+    const unsigned long long* list = M.list + (size_t)rank * capacity;
+    for (uint32_t e = tid; e < count; e += RT_THREADS) {
+      const unsigned long long c = list[e];
+      if (c >= T) write(~(uint32_t)c);
+    }
+  } else {
+    for (uint32_t left = chosen; left; left &= left - 1u) write((uint32_t)token(__ffs(left) - 1));
+  }
+  if (rank == 0) {                                            // the forced tokens
     for (uint32_t e = tid; e < n_sink; e += RT_THREADS) out[e] = (int32_t)e;
-    for (uint32_t e = tid; e < n_local; e += RT_THREADS) out[n_sink + chosen + e] = (int32_t)(elig_hi + e);
-    const uint32_t filled = n_sink + chosen + n_local;
+    for (uint32_t e = tid; e < n_local; e += RT_THREADS) out[n_sink + picked + e] = (int32_t)(elig_hi + e);
+    const uint32_t filled = n_sink + picked + n_local;
     if (filled < (uint32_t)k) {                               // short selection (non-finite scores)
       if (tid == 0) atomicOr(dev_status, FATHOM_DEV_TOPK_SHORT);
       for (uint32_t e = filled + tid; e < (uint32_t)k; e += RT_THREADS) out[e] = n - 1;   // pad with the last token
     }
-    cluster.barrier_wait(std::move(pulled));
-    return;
-  }
-
-  // ---- more candidates than the list holds: 11-bit digits of their composites, over the whole cluster
-  unsigned long long T = 0ull;
-  uint32_t left = want;
-  for (int hi = 64; hi > 0;) {
-    const int lo = hi > 11 ? hi - 11 : 0;
-    for (int b = tid; b < 2 * COARSE / 4; b += RT_THREADS) reinterpret_cast<uint4*>(M.mine)[b] = make_uint4(0u, 0u, 0u, 0u);
-    cluster.sync();
-#pragma unroll
-    for (int i = 0; i < EPT; ++i) {
-      const unsigned long long c = composite(i);
-      if (x[i] >= bound && (hi == 64 || (c >> hi) == (T >> hi))) atomicAdd(&M.mine[(uint32_t)(c >> lo) & ((1u << (hi - lo)) - 1u)], 1u);
-    }
-    __syncthreads();
-    push(FINE);
-    cluster.sync();
-    find_bin<FINE>(M, M.merged, left);
-    T |= (unsigned long long)M.found_bin << lo;
-    left -= M.found_above;
-    const bool whole = left == M.found_count;
-    __syncthreads();
-    hi = lo;
-    if (whole) break;
-  }
-  uint32_t chosen = 0u;                                       // bit i: token(i), forced or reaching T
-#pragma unroll
-  for (int i = 0; i < EPT; ++i) {
-    const int t = token(i);
-    const bool forced = t < n && (t < elig_lo || t >= elig_hi);
-    chosen |= (forced || (x[i] >= bound && composite(i) >= T) ? 1u : 0u) << i;
-  }
-  const uint32_t own = place(chosen, at);
-  if (tid < ctas) cluster.map_shared_rank(M.cta_count, tid)[rank] = own;
-  cluster.sync();                                             // (nobody touches another CTA's shared memory after this)
-  uint32_t ahead = 0u;
-  for (int r = 0; r < rank; ++r) ahead += M.cta_count[r];
-#pragma unroll
-  for (int v = 0; v < V; ++v) {
-    uint32_t pos = ahead + at[v];
-#pragma unroll
-    for (int c = 0; c < 4; ++c)
-      if ((chosen >> (4 * v + c)) & 1u) {
-        if (pos < (uint32_t)k) out[pos] = token(4 * v + c);
-        ++pos;
-      }
   }
 }
+
+size_t resident_smem_bytes(int ctas, uint32_t capacity, long long n) {
+  return sizeof(ResidentSmem) + (size_t)capacity * ((size_t)ctas * 8 + 4) + (size_t)((n + CHUNK - 1) / CHUNK) * 16;
+}
+// the largest request: two CTAs with half of them each (a single CTA lists no more than it has tokens)
+constexpr int RESIDENT_SMEM_MOST = (int)sizeof(ResidentSmem) + MOST_LISTED * 8 + MOST_LISTED / 2 * 4 + MAX_CHUNKS * 16;
+static_assert(RESIDENT_SMEM_MOST <= 227 * 1024, "fits on an SM");
 
 template <int EPT>
 cudaError_t launch(const float* scores, long long n, long long score_stride, int Hq, int k, Forced F, uint32_t want, int32_t* idx,
                    uint32_t* dev_status, int ctas, cudaStream_t st) {
-  // room for twice what is wanted (the bound lets through 1.05 to 1.5 times), up to 16,384: 164 KB, one CTA per SM; two fit on an SM
-  // up to about 10,000
-  const uint32_t room = 2u * want < 2048u ? 2048u : 2u * want;
-  const uint32_t capacity = room < 16384u ? room : 16384u;
-  const size_t smem = sizeof(ResidentSmem) + (size_t)capacity * 8;
+  // a CTA's share of what is wanted, with four standard deviations of a sample's count: one head in thousands needs a second round
+  const double share = (double)want / ctas;
+  const uint32_t quota = ctas == 1 ? want : (uint32_t)(share + 4.0 * sqrt(share) + 8.0);
+  // room for 1.75 times the quota (the bound lets through 1.05 to 1.4 times), for 2048 at least and for 16,384 over all lists; two CTAs
+  // fit on an SM while k is at most some 4000
+  const uint32_t least = (uint32_t)(2048 / ctas), most = (uint32_t)(ctas == 1 ? RT_THREADS * EPT : MOST_LISTED / ctas);
+  uint32_t capacity = (7u * quota / 4u + 3u) & ~3u;
+  capacity = capacity < least ? least : (capacity > most ? most : capacity);
+  const size_t smem = resident_smem_bytes(ctas, capacity, n);
   static bool configured[64] = {};
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
   if (dev < 0 || dev >= 64 || !configured[dev]) {
-    e = cudaFuncSetAttribute(topk_resident_kernel<EPT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(sizeof(ResidentSmem) + 16384 * 8));
+    e = cudaFuncSetAttribute(topk_resident_kernel<EPT>, cudaFuncAttributeMaxDynamicSharedMemorySize, RESIDENT_SMEM_MOST);
     if (e != cudaSuccess) return e;
     if (dev >= 0 && dev < 64) configured[dev] = true;
   }
@@ -436,28 +528,45 @@ cudaError_t launch(const float* scores, long long n, long long score_stride, int
   attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 2;
-  // maxima bound the threshold closely while `want` leaves a quarter of the groups below it
-  const int by_maxima = 4LL * want <= 3LL * (n / EPT) ? 1 : 0;
+  // the largest groups of which the quota is at most a half: they bound the threshold closely and take the fewest atomics
+  const long long lanes = (n + 128LL * ctas - 1) / (128LL * ctas) * 32;       // four tokens each, of a CTA
+  const long long threads = lanes < RT_THREADS ? lanes : RT_THREADS, beyond = lanes - EPT / 8 * RT_THREADS;
+  const long long halves = threads + (beyond < 0 ? 0 : (beyond < RT_THREADS ? beyond : RT_THREADS));
+  const int groups = 2LL * quota <= threads ? 1 : (EPT > 8 && 2LL * quota <= halves ? 2 : (2LL * quota <= lanes ? 4 : 0));
   return cudaLaunchKernelEx(&cfg, topk_resident_kernel<EPT>, scores, (int)n, score_stride, (int)F.sink_end, (int)F.local_begin, k, want,
-                            by_maxima, capacity, idx, dev_status);
+                            quota, groups, capacity, idx, dev_status);
+}
+
+// The fewest tokens per thread (8, 16 or 32) with which all heads' clusters run at a CTA per SM, else with which they have the fewest CTAs:
+// more tokens cost a thread less than a second CTA's threads cost the SM.  Clusters of eight leave SMs of a GPC over, so they have to be
+// content with two thirds of the chip.  us with 8 / 16 / 32 tokens per thread:
+//   8 heads   20,000 scores, k = 1024 6.1 / 6.6 / 8.0; 65,536 scores - / 6.6 / 7.3        16 heads  20,000 scores 7.3 / 6.7 / 8.0
+//   32 heads  8000 scores, k = 1024 7.0 / 8.2 / 9.3; 20,000 scores 8.1 / 7.1 / 8.1; 65,536 scores - / 8.6 / 8.4
+//   64 heads  20,000 scores, k = 1024 15.5 / 8.4 / 8.2; 33,001 scores - / 16.2 / 9.8
+// Lists of eight CTAs for most of a short row are long: 1 head, 20,000 scores, k = 8192 17.6 / 13.7 / 17.4; 32 heads 47.6 / 15.4 / 19.2.
+int ctas_for(long long n, int per_thread) {
+  int ctas = 1;
+  while ((long long)ctas * RT_THREADS * per_thread < n) ctas *= 2;
+  return ctas;
+}
+int tokens_per_thread(long long n, int Hq, uint32_t want) {
+  int best = 0;
+  for (int per = want > 4096 ? 16 : 8; per <= 32; per *= 2) {
+    const int ctas = ctas_for(n, per);
+    if (ctas > MAX_CLUSTER) continue;
+    if ((ctas == MAX_CLUSTER ? 3LL : 2LL) * ctas * Hq <= 2LL * fathom_sm_count()) return per;
+    if (!best || ctas < ctas_for(n, best)) best = per;
+  }
+  return best;
 }
 
 }  // namespace
 
-// as few tokens per thread as eight CTAs allow (at least 8: more CTAs cost barrier time), then as few CTAs as hold the row
-static int tokens_per_thread(long long n) {
-  const long long per_cta8 = RT_THREADS * 8;
-  return n <= MAX_CLUSTER * per_cta8 ? 8 : (n <= 2 * MAX_CLUSTER * per_cta8 ? 16 : 32);
-}
-int fathom_topk_resident_ctas(long long n) {
-  int ctas = 1;
-  while ((long long)ctas * RT_THREADS * tokens_per_thread(n) < n) ctas *= 2;
-  return ctas;
-}
+int fathom_topk_resident_ctas(long long n, int Hq, uint32_t want) { return ctas_for(n, tokens_per_thread(n, Hq, want)); }
 
 int fathom_launch_topk_resident(fathom_ctx* ctx, const float* scores, long long n, long long score_stride, int Hq, int k, Forced F,
                                 uint32_t want, int32_t* idx, cudaStream_t st) {
-  const int ept = tokens_per_thread(n), ctas = fathom_topk_resident_ctas(n);
+  const int ept = tokens_per_thread(n, Hq, want), ctas = ctas_for(n, ept);
   cudaError_t e;
   if (ept == 8) e = launch<8>(scores, n, score_stride, Hq, k, F, want, idx, ctx->dev_status, ctas, st);
   else if (ept == 16) e = launch<16>(scores, n, score_stride, Hq, k, F, want, idx, ctx->dev_status, ctas, st);

@@ -36,6 +36,37 @@ def test_topk_of_rows_held_in_registers(n, k, n_sink, n_local, scores):
     ctx.close()
 
 
+# rows of which one CTA's chunks of 128 tokens hold more than its share: the lists are made a second time with the threshold of the
+# first, or do not fit; few and many heads (8, 16 and 32 scores per thread for the same length)
+@pytest.mark.parametrize("Hq,n,k,n_sink,n_local", [(2, 20000, 700, 0, 0), (40, 20000, 700, 4, 32), (33, 33001, 2048, 0, 2000), (2, 65536, 4096, 100, 0),
+                                                   (20, 131072, 512, 0, 0), (9, 8200, 4000, 0, 0), (20, 20000, 8192, 0, 0)])
+@pytest.mark.parametrize("scores", ["one CTA", "one CTA, few", "rising", "end", "infinite"])
+def test_topk_of_uneven_rows_held_in_registers(Hq, n, k, n_sink, n_local, scores):
+    from paper_2609_17652_b200 import binding as fb
+    lay = fb.make_layout(1, Hq, n)
+    ctx = fb.Context(0, fb.fathom_scratch_bytes(lay, k))
+    g = torch.Generator(device="cuda").manual_seed(n + k)
+    s = torch.randn(Hq, lay.score_stride, generator=g, device="cuda")
+    t = torch.arange(lay.score_stride, device="cuda")
+    if scores == "one CTA":
+        s += 50.0 * (t // 128 % 8 == 3)
+    elif scores == "one CTA, few":
+        s += 50.0 * ((t // 128 % 8 == 3) & (t % 128 < 5))
+    elif scores == "rising":
+        s += 1e-3 * t
+    elif scores == "end":
+        s += 50.0 * (t >= n - n // 16)
+    else:
+        s = torch.where(t // 128 % 4 == 1, -float("inf") * torch.ones_like(s), s)
+        s[:, n // 2:n // 2 + 9] = float("inf")
+    s[:, n:] = float("nan")
+    idx = torch.full((Hq, k), -1, dtype=torch.int32, device="cuda")
+    ctx.fathom_topk(lay, s, k, n_sink, n_local, idx)
+    assert np.array_equal(idx.cpu().numpy(), O.topk(s[:, :n].double().cpu().numpy(), k, n_sink, n_local))
+    assert ctx.fathom_device_status() == 0
+    ctx.close()
+
+
 # a context sized for one length serves every shorter one, over the lengths at which the selection changes its way
 @pytest.mark.parametrize("longest", [131073, 150001])
 def test_shorter_sessions_on_a_longer_sessions_context(longest):
