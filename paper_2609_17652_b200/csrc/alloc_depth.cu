@@ -2,29 +2,27 @@
 //
 // Eq. 4 at the smallest water line that fits the budget grants exactly the min(B, 4d) candidate planes
 // (channel j, plane m = 1..4) with the largest priority g_j 4^-m, so a candidate is granted when fewer than
-// B others rank before it (ties: lower channel, then lower plane).  Eight CTAs of 512 threads serve a plan:
-// every CTA computes all 128 importances (thread = channel; fp64 with explicit round-to-nearest intrinsics,
-// no fused multiply-add, so the ranking is identical on every machine; no logarithm is evaluated) and ranks
-// the 64 candidates of its own 16 channels against all 512, eight threads per candidate (each counts over an
-// eighth of the others: the kernel is a latency chain, and the counting loop is its longest link).  Four CTAs per plan take
-// less time behind one another with 32 plans (5.3 us against 7.0), but the decode step more: 30.0 us against 25.1 with 8000
-// tokens, 34.7 against 33.2 with 40,000.
-// Non-negative doubles order like their bit patterns, so the comparisons run on 64-bit integers.
+// B others rank before it (ties: lower channel, then lower plane).  The importances are formed in fp64 with explicit
+// round-to-nearest intrinsics and no fused multiply-add, so the ranking is identical on every machine; no logarithm is evaluated.
+//
+// Two channels are compared once for all their planes: non-negative doubles order like their bit patterns, dividing by 4 takes 2^53 off
+// the pattern, so with D = pattern(g_i) - pattern(g_j) the planes of i that rank before (j, m) are those up to m + floor(D / 2^53)
+// (D - 1 where j wins ties).  (Products and sums of squares of fp32 numbers are far from fp64's subnormals, so the quarters are exact.)
+// A warp per channel j, four channels i per lane, the four planes' counts summed by two warp reductions of packed halves.
+// Eight CTAs serve a plan, 16 channels each; every CTA computes all 128 importances (thread = channel).  The kernel is a latency chain: it
+// compared each of the 512 candidates with all others before, eight threads per candidate (back to back: one plan 2.9 -> 1.4 us, 8 plans 3.1 -> 1.6, 32 plans 6.8 -> 2.0).
 #include "fathom_common.cuh"
 
 namespace {
 
-constexpr int NCAND = FATHOM_D * FATHOM_NPLANES;   // 512
 constexpr int CTAS_PER_PLAN = 8;
-constexpr int AD_CAND = NCAND / CTAS_PER_PLAN;     // 64 candidates ranked per CTA
-constexpr int AD_SPLIT = 8;                        // threads per candidate
-constexpr int AD_THREADS = AD_CAND * AD_SPLIT;     // 512
+constexpr int AD_CHANNELS = FATHOM_D / CTAS_PER_PLAN;        // 16 channels ranked per CTA, a warp each
+constexpr int AD_THREADS = 32 * AD_CHANNELS;                 // 512
 
 __global__ void __launch_bounds__(AD_THREADS)
 alloc_depth_kernel(const float* q, const float* var, int mode, int budget,
                    int heads_per_plan, int G, uint8_t* __restrict__ depth) {
-  __shared__ alignas(16) unsigned long long pri[NCAND];       // bit patterns of the (non-negative) priorities
-  __shared__ int partial[AD_SPLIT][AD_CAND];
+  __shared__ long long order[FATHOM_D];                       // bit patterns of the (non-negative) importances
   FATHOM_PDL_WAIT();
   FATHOM_PDL_RELEASE();                                       // the scan that follows may become resident now
   const int plan = blockIdx.x / CTAS_PER_PLAN, part = blockIdx.x % CTAS_PER_PLAN;
@@ -38,7 +36,7 @@ alloc_depth_kernel(const float* q, const float* var, int mode, int budget,
     return;
   }
 
-  if (tid < FATHOM_D) {                                       // thread = channel: its four priorities
+  if (tid < FATHOM_D) {                                       // thread = channel
     const int j = tid;
     double acc = 0.0;
     const float* qj = q + (size_t)h0 * FATHOM_D + j;
@@ -56,47 +54,45 @@ alloc_depth_kernel(const float* q, const float* var, int mode, int budget,
     if (mode == FATHOM_DEPTH_WATERFILL) {
       const float v = var[(size_t)kv * FATHOM_D + j];
       add_heads([](double x) { return __dmul_rn(x, x); });    // Eq. 3
-      const double g = __dmul_rn(acc, (double)v);
-      pri[4 * j + 0] = (unsigned long long)__double_as_longlong(fabs(__dmul_rn(g, 0.25)));        // g_j 4^-m
-      pri[4 * j + 1] = (unsigned long long)__double_as_longlong(fabs(__dmul_rn(g, 0.0625)));
-      pri[4 * j + 2] = (unsigned long long)__double_as_longlong(fabs(__dmul_rn(g, 0.015625)));
-      pri[4 * j + 3] = (unsigned long long)__double_as_longlong(fabs(__dmul_rn(g, 0.00390625)));
+      const long long g = __double_as_longlong(fabs(__dmul_rn(acc, (double)v)));
+      // Patterns of the products of finite fp32 numbers have exponents from 576 to 1420; 512 less, they leave room for channels of no
+      // importance below: so far apart that all planes of one rank before all planes of the next
+      const long long low = -((long long)(j + 1) << 55), most = 1023LL << 52;
+      order[j] = g == 0 ? low : min(g - (512LL << 52), most);
     } else {                                                  // fixed top-r channels by sum_h |q_j|
       add_heads([](double x) { return fabs(x); });
-      const unsigned long long key = (unsigned long long)__double_as_longlong(acc);
-      pri[4 * j + 0] = key; pri[4 * j + 1] = key; pri[4 * j + 2] = key; pri[4 * j + 3] = key;
+      order[j] = __double_as_longlong(acc);
     }
   }
   __syncthreads();
 
-  const int cand = tid & (AD_CAND - 1), share = tid / AD_CAND;
-  const int id = part * AD_CAND + cand;                       // my candidate: channel id / 4, plane id % 4 + 1
-  const unsigned long long key = pri[id];
-  int rank = 0;
-  const int o0 = share * (NCAND / AD_SPLIT), o1 = o0 + NCAND / AD_SPLIT;
+  const int lane = tid & 31, j = part * AD_CHANNELS + (tid >> 5);
+  const long long mine = order[j];
   if (mode == FATHOM_DEPTH_WATERFILL) {
-#pragma unroll 8
-    for (int o = o0; o < o1; o += 2) {
-      const ulonglong2 p = *reinterpret_cast<const ulonglong2*>(&pri[o]);
-      rank += (p.x > key) || (p.x == key && o < id);
-      rank += (p.y > key) || (p.y == key && o + 1 < id);
-    }
-  } else {                                                    // rank channels only (one key per channel)
-#pragma unroll 8
-    for (int o = o0; o < o1; o += 4) {
-      const unsigned long long p = pri[o];
-      rank += (p > key) || (p == key && o < (id & ~3));
-    }
-  }
-  partial[share][cand] = rank;
-  __syncthreads();
-  if (share == 0) {                                           // the first two warps: one thread per candidate
-    rank = 0;
+    uint32_t before12 = 0u, before34 = 0u;                    // candidates that rank before planes 1 and 2, 3 and 4 of channel j
 #pragma unroll
-    for (int s = 0; s < AD_SPLIT; ++s) rank += partial[s][cand];
-    const bool granted = rank < budget;                       // fixed mode: all four planes of a chosen channel
-    const unsigned ball = __ballot_sync(0xffffffffu, granted);
-    if ((id & 3) == 0) out[id >> 2] = (uint8_t)__popc((ball >> (tid & 31)) & 0xFu);
+    for (int u = 0; u < FATHOM_D / 32; ++u) {
+      const int i = lane + 32 * u;
+      const int e = (int)((order[i] - mine - (i < j ? 0 : 1)) >> 53);        // (i = j: the planes above m)
+      auto planes = [&](int m) { return (uint32_t)min(max(m + e, 0), FATHOM_NPLANES); };
+      before12 += planes(1) | planes(2) << 16;
+      before34 += planes(3) | planes(4) << 16;
+    }
+    before12 = __reduce_add_sync(0xffffffffu, before12);      // (at most 512 each)
+    before34 = __reduce_add_sync(0xffffffffu, before34);
+    if (lane == 0) {
+      const uint32_t b = (uint32_t)budget;
+      out[j] = (uint8_t)(((before12 & 0xffffu) < b) + ((before12 >> 16) < b) + ((before34 & 0xffffu) < b) + ((before34 >> 16) < b));
+    }
+  } else {
+    uint32_t before = 0u;
+#pragma unroll
+    for (int u = 0; u < FATHOM_D / 32; ++u) {
+      const int i = lane + 32 * u;
+      before += order[i] > mine || (order[i] == mine && i < j);
+    }
+    before = __reduce_add_sync(0xffffffffu, before);
+    if (lane == 0) out[j] = before < (uint32_t)budget ? FATHOM_NPLANES : 0;  // all four planes of a chosen channel
   }
 }
 

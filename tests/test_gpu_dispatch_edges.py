@@ -371,3 +371,30 @@ def test_rotation_of_keys_with_one_large_channel(far, basis):
     bound = (2.0 ** -24 + 3 * 2.0 ** -22 + 24 * 2.0 ** -23) * magnitude + 2.0 ** -39 * X.abs().amax(dim=2, keepdim=True) * V.double().abs().sum(dim=1, keepdim=True)
     assert ((out.double() - X @ V.double()).abs() <= bound).all() and ctx.fathom_device_status() == 0
     ctx.close()
+
+
+# importances that are zero, equal, powers of four apart, and at the ends of what fp32 queries and variances give: every tie is decided by
+# channel and plane
+@pytest.mark.parametrize("budget", [0, 1, 5, 47, 130, 300, 509, 512, 600])
+@pytest.mark.parametrize("kind", ["zeros", "ties", "powers", "extremes"])
+def test_depths_of_tied_and_extreme_importances(kind, budget):
+    from paper_2609_17652_b200 import binding as fb
+    Hq, hpp = 4, 2
+    lay = fb.make_layout(1, Hq, 64)
+    ctx = fb.Context(0, fb.fathom_scratch_bytes(lay, 1))
+    rng = np.random.default_rng(budget)
+    q = np.ones((Hq, 128), np.float32)
+    if kind == "zeros":
+        var = np.where(rng.random(128) < 0.6, 0.0, rng.random(128))
+    elif kind == "ties":
+        var = rng.integers(1, 4, 128).astype(np.float64)
+    elif kind == "powers":
+        var = 4.0 ** rng.integers(-3, 4, 128) * rng.choice([1.0, 1.0, 2.0], 128)
+    else:
+        q *= rng.choice(np.array([1e-45, 1e-20, 1.0, 3.4e38], np.float32), (1, 128))
+        var = rng.choice([0.0, 1e-45, 1e-30, 1.0, 3.4e38], 128)
+    var = var.astype(np.float32)[None]
+    depth = torch.full((Hq // hpp, 128), 9, dtype=torch.uint8, device="cuda")
+    ctx.fathom_alloc_depth(lay, torch.from_numpy(q).cuda(), torch.from_numpy(var).cuda(), fb.DEPTH_WATERFILL, budget, hpp, depth)
+    assert np.array_equal(depth.cpu().numpy(), O.alloc_depth(q, var, "waterfill", budget, hpp))
+    ctx.close()
