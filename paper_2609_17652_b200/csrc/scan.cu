@@ -23,8 +23,8 @@
 // A tile is 16 blocks (1024 tokens) of one plan (NH query heads that share the planes read).  With the planes in device
 // memory the CTAs are persistent: gridDim.x CTAs per plan walk the tiles round-robin, build the plan's row list and right
 // operand once, and fetch the next stage's plane words and scales with asynchronous copies (cp.async; a row's words are
-// one contiguous run, Sec. 3.6) into the other half of a double buffer.  A stage is a tile and up to 96 rows; deeper plans take half
-// tiles in passes of up to 96 rows and carry the accumulators over the passes.  The right operand of all rows stays in shared memory.
+// one contiguous run, Sec. 3.6) into the other half of a double buffer.  A stage is a tile and up to 96 rows, or half a tile and up to
+// 160; deeper plans take half tiles in passes of up to 96 rows and carry the accumulators over the passes.  The right operand of all rows stays in shared memory.
 // With the planes in pinned host memory the grid is one CTA per tile, which keeps the requests on the host link sequential.
 // Only planes p < t_j and the scales of active channels are ever read.
 #include "scan_shared.cuh"
@@ -50,7 +50,7 @@ constexpr int CTAS_PER_SM = FATHOM_SCAN_CTAS_PER_SM;
 template <int TB>
 struct Geo {
   static constexpr int ROW_BYTES = 8 * TB + 16;               // pitch of a staged plane-word row
-  static constexpr int SCALE_ELEMS = 24;                      // pitch of a staged scale row, fp16 elements
+  static constexpr int SCALE_ELEMS = TB == 16 ? 24 : 8;       // pitch of a staged scale row, fp16 elements
 };
 constexpr int STAGE_WORDS = STAGE_ROWS * Geo<16>::ROW_BYTES;           // one buffer of staged plane words
 constexpr int STAGE_SCALES = STAGE_ROWS * Geo<16>::SCALE_ELEMS * 2;    // one buffer of staged scales
@@ -58,6 +58,11 @@ constexpr int STAGE_KSTEPS = STAGE_ROWS / 16;
 // deep plans stage half tiles, which leaves room for the right operand of their further rows behind the staged words
 constexpr int DEEP_WORDS = STAGE_ROWS * Geo<8>::ROW_BYTES;
 static_assert(2 * DEEP_WORDS + (MAX_KSTEPS - STAGE_KSTEPS) * 32 * 8 <= 2 * STAGE_WORDS, "room for the right operand of deep plans");
+// half tiles of up to 160 rows fit in one stage
+constexpr int HALF_KSTEPS = 10;
+constexpr int HALF_WORDS = 16 * HALF_KSTEPS * Geo<8>::ROW_BYTES;
+static_assert(2 * HALF_WORDS + (HALF_KSTEPS - STAGE_KSTEPS) * 32 * 8 <= 2 * STAGE_WORDS, "room for the right operand of their further rows");
+static_assert(16 * HALF_KSTEPS * Geo<8>::SCALE_ELEMS * 2 <= STAGE_SCALES, "room for their scales");
 
 // MODE 2.  A lane whose eight scores hold a candidate parks all eight in its warp's ring (three stores, no atomic, no
 // loop); when the ring may not take another round of 32, the warp sifts it with all lanes, one parked group per lane,
@@ -139,7 +144,8 @@ __device__ __forceinline__ void mma_tokens8(float (&acc)[4][4], uint32_t x0, uin
 //         (score, token) pairs appended to the head's candidate list.
 // grid = (CTAs per plan, groups of NH query heads); MODE 1 and 2 are launched with one item.
 // IN_HBM: every store of the launch lies in device memory (its rows are staged past the L1).
-template <int NH, int MODE, bool IN_HBM, int CAP>
+// UNIT: blocks that a CTA takes at a time, 16 (a tile) or 8.
+template <int NH, int MODE, bool IN_HBM, int CAP, int UNIT>
 __global__ void __launch_bounds__(THREADS, CTAS_PER_SM)
 scan_kernel(const __grid_constant__ ScanBatchOf<CAP> B, int G, int heads_per_plan, fathom_scan_fuse fz) {
   extern __shared__ __align__(16) unsigned char scan_smem[];   // sizeof(Smem<MODE>): more than the static limit in MODE 2
@@ -173,7 +179,8 @@ scan_kernel(const __grid_constant__ ScanBatchOf<CAP> B, int G, int heads_per_pla
   float hs = 1.0f, hs_tail = 0.0f;                             // E of my head and E 2^-11
 
   auto bfr_of = [&](int ks) {                                  // the right operand of 16 rows, [32 lanes]
-    return ks < STAGE_KSTEPS ? M.bfr[ks] : reinterpret_cast<uint2*>(M.words + 2 * DEEP_WORDS) + (ks - STAGE_KSTEPS) * 32;
+    return ks < STAGE_KSTEPS ? M.bfr[ks]
+                             : reinterpret_cast<uint2*>(M.words + (nrows <= 16 * HALF_KSTEPS ? 2 * HALF_WORDS : 2 * DEEP_WORDS)) + (ks - STAGE_KSTEPS) * 32;
   };
   // ---- right operand of all rows (made visible by the barrier that precedes the first stage's arithmetic): entry
   //      (kstep, lane, i) holds rows 16 kstep + 2 (lane & 3) + 8 i and the next one, column lane >> 2 = (head, part)
@@ -259,14 +266,14 @@ scan_kernel(const __grid_constant__ ScanBatchOf<CAP> B, int G, int heads_per_pla
   // first block of launch tile `tile` within its session
   auto first_block = [&](int tile) -> int {
     const int tl = tile - (item ? (int)B.tile_end[item - 1] : 0);
-    return tl * (MODE == 1 ? fz.tile_step : 1) * TILE_BLOCKS;
+    return tl * (MODE == 1 ? fz.tile_step : 1) * UNIT;
   };
 
   // a buffer's scale rows from `first` up to the next multiple of 16 (at least 16) hold 0, so that whatever the stale plane bytes of
   // those rows say they contribute +-0
-  auto clear_pad = [&](int first, int buf) {
+  auto clear_pad = [&](auto tbc, int first, int buf) {
     const int pad = max(16, (first + 15) & ~15) - first;
-    constexpr int WPR = Geo<16>::SCALE_ELEMS / 2;              // 32-bit words per scale row
+    constexpr int WPR = Geo<decltype(tbc)::value>::SCALE_ELEMS / 2;           // 32-bit words per scale row
     for (int e = tid; e < pad * WPR; e += THREADS) reinterpret_cast<uint32_t*>(M.scale + buf * STAGE_SCALES)[first * WPR + e] = 0u;
   };
 
@@ -385,12 +392,12 @@ scan_kernel(const __grid_constant__ ScanBatchOf<CAP> B, int G, int heads_per_pla
   // are worked eight at a time (byte k of the loaded words).  Tokens past the end of the sequence are computed from zeros or from
   // what pads the rows and never leave.
   struct Place { const unsigned char* wp; const uint16_t* sp; uint32_t tok0, dst0; };
-  auto place = [&](auto tbc, int g, int u, int buf) {
+  auto place = [&](auto tbc, int g, int u, int buf, int buf_words) {
     constexpr int TB = decltype(tbc)::value, BYTES = TB / 4;   // plane bytes per row and lane
     const int mine = warp * (TB / 4) + (gq * BYTES) / 8;       // my block of the stage
     const int off = (gq * BYTES) % 8;                          // where my bytes start in its words
     Place p;
-    p.wp = M.words + buf * (TB == 16 ? STAGE_WORDS : DEEP_WORDS) + (2 * t4) * Geo<TB>::ROW_BYTES + mine * 8 + off;
+    p.wp = M.words + buf * buf_words + (2 * t4) * Geo<TB>::ROW_BYTES + mine * 8 + off;
     p.sp = reinterpret_cast<const uint16_t*>(M.scale + buf * STAGE_SCALES) + (2 * t4) * Geo<TB>::SCALE_ELEMS + mine;
     p.tok0 = (uint32_t)(first_block(g) + u * TB + mine) * FATHOM_BLOCK + off * 8;           // my first token
     p.dst0 = MODE == 1 ? (uint32_t)g * (TILE_BLOCKS * FATHOM_BLOCK) + (uint32_t)(u * TB + mine) * FATHOM_BLOCK + off * 8 : p.tok0;
@@ -408,75 +415,102 @@ scan_kernel(const __grid_constant__ ScanBatchOf<CAP> B, int G, int heads_per_pla
     S[0] = __byte_perm(sk[0], sk[SE], 0x5410);
     S[1] = __byte_perm(sk[8 * SE], sk[9 * SE], 0x5410);
   };
-  // plans of up to 96 rows, NKS x 16 of them (the last 16 may be padded): a stage is a tile.  A thread copies the same 16-byte
-  // column of the same rows in every stage, so where they start is kept in registers.  The words and scales a lane reads are in
-  // registers before the first MMA, and so is the right operand of up to four steps (of more it would spill)
-  auto run_single = [&](auto nksc, int g, int end) {
-    constexpr int NKS = decltype(nksc)::value;
-    constexpr bool KEEP = NKS <= 4;
-    constexpr std::integral_constant<int, 16> T16{};
-    constexpr int SC = (16 * NKS + 63) / 64;                   // sweeps of 64 rows over the scales
-    static_assert(THREADS == 128, "16 rows of plane words and 64 of scales per sweep of the CTA");
-    const int c = tid & 7, cs = tid & 1;
-    uint32_t wo[NKS], so[SC];
+  // A stage holds all rows, NKS x 16 of them (the last 16 may be padded), of TB blocks: a tile of up to 96 rows, or half a tile of up to
+  // 160.  A thread copies the same 16-byte column of the same rows in every stage, so where they start is kept in registers.  Up to 96
+  // rows the words and scales a lane reads are in registers before the first MMA, and so is the right operand of up to four steps (of
+  // more it would spill); of more rows the accumulators of all the lane's tokens are kept and the rows walked once.  (In two passes of up to 96
+  // rows, with a barrier and copy offsets made anew for each, 136 rows took 127 us at 1,048,576 tokens, 8 plans, against 104, and 7.9 at 4096
+  // tokens against 4.7.)
+  auto run_single = [&](auto tbc, auto nksc, int g, int end) {
+    constexpr int TB = decltype(tbc)::value, NKS = decltype(nksc)::value, RB = Geo<TB>::ROW_BYTES, SE = Geo<TB>::SCALE_ELEMS;
+    constexpr int BYTES = TB / 4;                              // plane bytes per row and lane
+    constexpr bool KEEP = NKS <= 4, WALK = NKS > STAGE_KSTEPS;
+    constexpr int WC = TB / 2, WR = THREADS / WC, WS = (16 * NKS + WR - 1) / WR;          // columns of a row of words, rows and sweeps of the CTA over them
+    constexpr int SC = TB / 8, SR = THREADS / SC, SS = (16 * NKS + SR - 1) / SR;          // ... of the scales
+    constexpr int BUF = TB == 16 ? STAGE_WORDS : HALF_WORDS;
+    const int wc = tid % WC, wr = tid / WC, sc = tid % SC, sr = tid / SC;
+    uint32_t wo[WS], so[SS];
 #pragma unroll
-    for (int i = 0; i < NKS; ++i) wo[i] = (uint32_t)M.row_id[min((tid >> 3) + 16 * i, MAX_ROWS - 1)] * half_stride;
+    for (int i = 0; i < WS; ++i) wo[i] = (uint32_t)M.row_id[min(wr + WR * i, MAX_ROWS - 1)] * half_stride;
 #pragma unroll
-    for (int i = 0; i < SC; ++i) so[i] = (uint32_t)(M.row_id[min((tid >> 1) + 64 * i, MAX_ROWS - 1)] >> 2) * eighth_stride;
-    const bool last_row = (tid >> 3) + 16 * (NKS - 1) < nrows;
+    for (int i = 0; i < SS; ++i) so[i] = (uint32_t)(M.row_id[min(sr + SR * i, MAX_ROWS - 1)] >> 2) * eighth_stride;
     auto prefetch = [&](int blk0, int buf) {
       const int nblk = nb_item - blk0;                         // >= 1
-      const bool vw = 2 * c < nblk, vs = 8 * cs < nblk;
-      const uint4* words_src = planes_kv + (vw ? (blk0 >> 1) + c : 0);       // (nothing is read where there is no block)
-      const uint4* scales_src = scales_kv + (vs ? (blk0 >> 3) + cs : 0);
-      unsigned char* wd = M.words + buf * STAGE_WORDS + (tid >> 3) * Geo<16>::ROW_BYTES + c * 16;
-      unsigned char* sd = M.scale + buf * STAGE_SCALES + (tid >> 1) * (Geo<16>::SCALE_ELEMS * 2) + cs * 16;
+      const bool vw = 2 * wc < nblk, vs = 8 * sc < nblk;
+      const uint4* words_src = planes_kv + (vw ? (blk0 >> 1) + wc : 0);       // (nothing is read where there is no block)
+      const uint4* scales_src = scales_kv + (vs ? (blk0 >> 3) + sc : 0);
+      unsigned char* wd = M.words + buf * BUF + wr * RB + wc * 16;
+      unsigned char* sd = M.scale + buf * STAGE_SCALES + sr * (SE * 2) + sc * 16;
 #pragma unroll
-      for (int i = 0; i < NKS; ++i)
-        if (i < NKS - 1 || last_row) fathom_copy_async<16>(wd + i * (16 * Geo<16>::ROW_BYTES), words_src + wo[i], vw, in_hbm);
+      for (int i = 0; i < WS; ++i)
+        if ((!WALK && WR * (i + 1) <= 16 * (NKS - 1)) || wr + WR * i < nrows) fathom_copy_async<16>(wd + i * (WR * RB), words_src + wo[i], vw, in_hbm);
 #pragma unroll
-      for (int i = 0; i < SC; ++i)
-        if ((tid >> 1) + 64 * i < nrows) fathom_copy_async<16>(sd + i * (64 * Geo<16>::SCALE_ELEMS * 2), scales_src + so[i], vs, in_hbm);
+      for (int i = 0; i < SS; ++i)
+        if (sr + SR * i < nrows) fathom_copy_async<16>(sd + i * (SR * SE * 2), scales_src + so[i], vs, in_hbm);
       fathom_copies_commit();
     };
     prefetch(first_block(g), 0);                               // the first stage's rows are on their way ...
-    clear_pad(nrows, 0);
-    clear_pad(nrows, 1);
+    clear_pad(tbc, nrows, 0);
+    clear_pad(tbc, nrows, 1);
     fill_bfr();                                                // ... while the right operand is made
     const uint32_t n = (uint32_t)B.n[item];                    // n < 2^31
     uint2 bf[KEEP ? NKS : 1];
-    for (int buf = 0;; buf ^= 1) {
-      const int g_next = g + gridDim.x;
+    for (int u = 0, buf = 0;; buf ^= 1) {
+      int g_next = g, u_next = u + 1;                          // (of half tiles: the tile's second, where it has blocks)
+      if (TB == UNIT || u_next == UNIT / TB || first_block(g) + u_next * TB >= nb_item) {
+        u_next = 0;
+        g_next = g + gridDim.x;
+      }
       const bool more = g_next < end;
       fathom_copies_wait<0>();
       __syncthreads();                                         // this stage's words and scales are in place, and every warp has
                                                                // left the previous stage: its buffer may be refilled
-      if (more) prefetch(first_block(g_next), buf ^ 1);        // lands while this stage is scanned
-      const Place at = place(T16, g, 0, buf);
-      uint32_t w[NKS][4], S[NKS][2];
+      if (more) prefetch(first_block(g_next) + u_next * TB, buf ^ 1);         // lands while this stage is scanned
+      const Place at = place(tbc, g, u, buf, BUF);
+      if constexpr (WALK) {
+        float acc[BYTES][4][4];
+        auto step = [&](auto first, int ks, uint2 b) {
+          uint32_t w[4], S[2];
+          load_rows(tbc, at.wp + ks * (16 * RB), at.sp + ks * (16 * SE), w, S);
 #pragma unroll
-      for (int ks = 0; ks < NKS; ++ks) {
-        if (KEEP) bf[ks] = M.bfr[ks][lane];
-        load_rows(T16, at.wp + ks * (16 * Geo<16>::ROW_BYTES), at.sp + ks * (16 * Geo<16>::SCALE_ELEMS), w[ks], S[ks]);
-      }
+          for (int k = 0; k < BYTES; ++k)
+            mma_tokens8<decltype(first)::value>(acc[k], row_bytes(w[0], w[1], k), row_bytes(w[2], w[3], k), S[0], S[1], b);
+        };
+        step(std::true_type{}, 0, M.bfr[0][lane]);
 #pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        float acc[4][4];
+        for (int ks = 1; ks < STAGE_KSTEPS; ++ks) step(std::false_type{}, ks, M.bfr[ks][lane]);
+        const uint2* further = bfr_of(STAGE_KSTEPS) + lane;
+#pragma unroll 1
+        for (int ks = STAGE_KSTEPS; 16 * ks < nrows; ++ks, further += 32) step(std::false_type{}, ks, *further);
+#pragma unroll
+        for (int k = 0; k < BYTES; ++k) finish(acc[k], at.tok0 + 8 * k, at.dst0 + 8 * k, n);
+      } else {
+        uint32_t w[NKS][4], S[NKS][2];
 #pragma unroll
         for (int ks = 0; ks < NKS; ++ks) {
-          const uint32_t x0 = row_bytes(w[ks][0], w[ks][1], k), x1 = row_bytes(w[ks][2], w[ks][3], k);
-          const uint2 b = KEEP ? bf[KEEP ? ks : 0] : M.bfr[ks][lane];
-          if (ks == 0) mma_tokens8<true>(acc, x0, x1, S[ks][0], S[ks][1], b);
-          else mma_tokens8<false>(acc, x0, x1, S[ks][0], S[ks][1], b);
+          if (KEEP) bf[ks] = M.bfr[ks][lane];
+          load_rows(tbc, at.wp + ks * (16 * RB), at.sp + ks * (16 * SE), w[ks], S[ks]);
         }
-        finish(acc, at.tok0 + 8 * k, at.dst0 + 8 * k, n);
+#pragma unroll
+        for (int k = 0; k < BYTES; ++k) {
+          float acc[4][4];
+#pragma unroll
+          for (int ks = 0; ks < NKS; ++ks) {
+            const uint32_t x0 = row_bytes(w[ks][0], w[ks][1], k), x1 = row_bytes(w[ks][2], w[ks][3], k);
+            const uint2 b = KEEP ? bf[KEEP ? ks : 0] : M.bfr[ks][lane];
+            if (ks == 0) mma_tokens8<true>(acc, x0, x1, S[ks][0], S[ks][1], b);
+            else mma_tokens8<false>(acc, x0, x1, S[ks][0], S[ks][1], b);
+          }
+          finish(acc, at.tok0 + 8 * k, at.dst0 + 8 * k, n);
+        }
       }
       if (MODE == 2 && (++stages & 3u) == 0u) sift();          // (every warp of the CTA at the same stages)
       if (!more) return;
       g = g_next;
+      u = u_next;
     }
   };
-  // plans of more than 96 rows: the accumulators of the lane's tokens are carried over the passes of a half tile (those of a whole
+  // plans of more than 160 rows: the accumulators of the lane's tokens are carried over the passes of a half tile (those of a whole
   // tile, 64 registers, would spill)
   auto run_passes = [&](int g, int end) {
     constexpr std::integral_constant<int, 8> tbc{};
@@ -497,7 +531,7 @@ scan_kernel(const __grid_constant__ ScanBatchOf<CAP> B, int G, int heads_per_pla
       unsigned char* sd = M.scale + buf * STAGE_SCALES;
       for (int r = tid; r < sc; r += THREADS)
         fathom_copy_async<16>(sd + r * (Geo<TB>::SCALE_ELEMS * 2), scales_kv + (blk0 >> 3) + (uint32_t)(M.row_id[s0 + r] >> 2) * eighth_stride, true, in_hbm);
-      clear_pad(sc, buf);
+      clear_pad(tbc, sc, buf);
       fathom_copies_commit();
     };
     prefetch(g, 0, 0, 0);
@@ -508,7 +542,7 @@ scan_kernel(const __grid_constant__ ScanBatchOf<CAP> B, int G, int heads_per_pla
       if (pass_next == npass) {
         pass_next = 0;
         u_next = u + 1;
-        if (u_next * TB >= TILE_BLOCKS || first_block(g) + u_next * TB >= nb_item) { u_next = 0; g_next = g + gridDim.x; }
+        if (u_next * TB >= UNIT || first_block(g) + u_next * TB >= nb_item) { u_next = 0; g_next = g + gridDim.x; }
       }
       const bool more = g_next < end;
       fathom_copies_wait<0>();
@@ -520,7 +554,7 @@ scan_kernel(const __grid_constant__ ScanBatchOf<CAP> B, int G, int heads_per_pla
 #pragma unroll
           for (int j = 0; j < 4; ++j) acc[k][j][0] = acc[k][j][1] = acc[k][j][2] = acc[k][j][3] = 0.0f;
       }
-      const Place at = place(tbc, g, u, buf);
+      const Place at = place(tbc, g, u, buf, DEEP_WORDS);
       const int ks0 = pass * (rows_stage >> 4), nks = (min(rows_stage, nrows - pass * rows_stage) + 15) >> 4;
 #pragma unroll 2
       for (int ks = 0; ks < nks; ++ks) {
@@ -550,13 +584,15 @@ scan_kernel(const __grid_constant__ ScanBatchOf<CAP> B, int G, int heads_per_pla
     if (MODE == 2) my_thr = M.thr[myh];
     const int end = min(total, (int)B.tile_end[item]);
     const int nks = (nrows + 15) >> 4;
-    if (nks > STAGE_KSTEPS) run_passes(g, end);
-    else if (nks <= 1) run_single(std::integral_constant<int, 1>{}, g, end);
-    else if (nks == 2) run_single(std::integral_constant<int, 2>{}, g, end);
-    else if (nks == 3) run_single(std::integral_constant<int, 3>{}, g, end);
-    else if (nks == 4) run_single(std::integral_constant<int, 4>{}, g, end);
-    else if (nks == 5) run_single(std::integral_constant<int, 5>{}, g, end);
-    else run_single(std::integral_constant<int, 6>{}, g, end);
+    auto shallow = [&](auto nksc) { run_single(std::integral_constant<int, UNIT>{}, nksc, g, end); };
+    if (nks <= 1) shallow(std::integral_constant<int, 1>{});
+    else if (nks == 2) shallow(std::integral_constant<int, 2>{});
+    else if (nks == 3) shallow(std::integral_constant<int, 3>{});
+    else if (nks == 4) shallow(std::integral_constant<int, 4>{});
+    else if (nks == 5) shallow(std::integral_constant<int, 5>{});
+    else if (nks == 6) shallow(std::integral_constant<int, 6>{});
+    else if (nks <= HALF_KSTEPS) run_single(std::integral_constant<int, 8>{}, std::integral_constant<int, HALF_KSTEPS>{}, g, end);
+    else run_passes(g, end);
     g += (end - g + (int)gridDim.x - 1) / (int)gridDim.x * (int)gridDim.x;      // my first tile of a later session
   }
   if (MODE == 2) {
@@ -583,17 +619,14 @@ scan_kernel(const __grid_constant__ ScanBatchOf<CAP> B, int G, int heads_per_pla
   }
 }
 
-template <int NH, int MODE, int CAP>
-int launch_scan(const ScanBatchOf<CAP>& B, int Hkv, int Hq, int heads_per_plan, const fathom_scan_fuse& fz, bool dependent,
-                cudaStream_t st) {
-  const long long tiles = B.tile_end[B.items - 1];
-  if (tiles <= 0) return FATHOM_OK;
+template <int NH, int MODE, int CAP, int UNIT>
+int launch_units(const ScanBatchOf<CAP>& B, int Hkv, int Hq, int heads_per_plan, const fathom_scan_fuse& fz, bool host, bool dependent,
+                 cudaStream_t st) {
   const int plans = Hq / NH;
-  bool host = false;                                          // any store of the launch in pinned host memory
-  for (int i = 0; i < B.items; ++i) host = host || fathom_planes_in_host_memory(B.planes[i]);
-  dim3 grid((unsigned)fathom_scan_grid_ctas(tiles, plans, host, CTAS_PER_SM), (unsigned)plans);
+  dim3 grid((unsigned)fathom_scan_grid_ctas(B.tile_end[B.items - 1], plans, host, CTAS_PER_SM), (unsigned)plans);
   constexpr size_t smem = sizeof(Smem<MODE>);                 // dynamic: MODE 2 needs more than the static limit
-  auto kernel = host ? scan_kernel<NH, MODE, false, CAP> : scan_kernel<NH, MODE, true, CAP>;
+  auto kernel = scan_kernel<NH, MODE, true, CAP, UNIT>;
+  if (UNIT == TILE_BLOCKS && host) kernel = scan_kernel<NH, MODE, false, CAP, TILE_BLOCKS>;
   if (smem > 48 * 1024) {
     static bool configured[64][2] = {};
     int dev = 0;
@@ -610,6 +643,31 @@ int launch_scan(const ScanBatchOf<CAP>& B, int Hkv, int Hq, int heads_per_plan, 
   }
   kernel<<<grid, THREADS, smem, st>>>(B, Hq / Hkv, heads_per_plan, fz);
   return FATHOM_OK;
+}
+
+template <int NH, int MODE, int CAP>
+int launch_scan(const ScanBatchOf<CAP>& B, int Hkv, int Hq, int heads_per_plan, const fathom_scan_fuse& fz, bool dependent, cudaStream_t st) {
+  const long long tiles = B.tile_end[B.items - 1];
+  if (tiles <= 0) return FATHOM_OK;
+  bool host = false;                                          // any store of the launch in pinned host memory
+  for (int i = 0; i < B.items; ++i) host = host || fathom_planes_in_host_memory(B.planes[i]);
+  // Half tiles as the CTAs' units where an SM has room for each of them alone, and where, over more than one wave of whole tiles, the busiest
+  // CTA then has a tenth fewer blocks.  (Budget 48, back to back, whole / half: one plan, 4096 tokens 3.5 / 3.0 us, 65,536 3.5 / 3.1; 8 plans,
+  // 16,384 tokens 3.6 / 3.8, 100,000 8.2 / 7.4, 262,144 13.6 / 12.8, budget 32 12.9 / 10.6.)
+  if constexpr (MODE == 0 && CAP == 1) {
+    const int plans = Hq / NH;
+    if (!host && fathom_scan_ctas_override() == 0) {
+      ScanBatchOf<CAP> U = B;
+      const long long halves = (fathom_nblocks(B.n[0]) + TILE_BLOCKS / 2 - 1) / (TILE_BLOCKS / 2);
+      const long long x16 = fathom_scan_grid_ctas(tiles, plans, false, CTAS_PER_SM), x8 = fathom_scan_grid_ctas(halves, plans, false, CTAS_PER_SM);
+      const bool alone = halves * plans <= fathom_sm_count(), waves = tiles > x16;
+      if (alone || (waves && (halves + x8 - 1) / x8 * 10 <= (tiles + x16 - 1) / x16 * 2 * 9)) {
+        U.tile_end[0] = halves;
+        return launch_units<NH, MODE, CAP, TILE_BLOCKS / 2>(U, Hkv, Hq, heads_per_plan, fz, false, dependent, st);
+      }
+    }
+  }
+  return launch_units<NH, MODE, CAP, TILE_BLOCKS>(B, Hkv, Hq, heads_per_plan, fz, host, dependent, st);
 }
 
 // FATHOM_SCAN_PATH=simt (read once) selects the CUDA-core kernel of scan_simt.cu for every scan of the process

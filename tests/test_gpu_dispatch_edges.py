@@ -398,3 +398,62 @@ def test_depths_of_tied_and_extreme_importances(kind, budget):
     ctx.fathom_alloc_depth(lay, torch.from_numpy(q).cuda(), torch.from_numpy(var).cuda(), fb.DEPTH_WATERFILL, budget, hpp, depth)
     assert np.array_equal(depth.cpu().numpy(), O.alloc_depth(q, var, "waterfill", budget, hpp))
     ctx.close()
+
+
+# rows at the edges of a stage (16 each; 96 of a tile, 160 of half a tile), half tiles alone on their SMs, whole tiles, half tiles over several waves; tails
+# of a block and of a unit
+@pytest.mark.parametrize("rows", [15, 17, 96, 97, 113, 144, 159, 160, 161, 255])
+@pytest.mark.parametrize("Hkv,n", [(1, 40), (1, 1100), (2, 9000), (2, 33001)])
+def test_scan_rows_and_units(Hkv, n, rows):
+    from paper_2609_17652_b200 import binding as fb
+    from tests._pipeline import score_tolerance
+    Hq, hpp = 4 * Hkv, 4
+    lay = fb.make_layout(Hkv, Hq, n)
+    ctx = fb.Context(0, 0)
+    g = torch.Generator(device="cuda").manual_seed(rows)
+    K = torch.randn(Hkv, n, 128, generator=g, device="cuda") * torch.exp(2 * torch.rand(Hkv, 1, 128, generator=g, device="cuda"))
+    q = torch.randn(Hq, 128, generator=g, device="cuda")
+    planes = torch.zeros(Hkv, 128, 4, lay.plane_stride_words, dtype=torch.int64, device="cuda")
+    scales = torch.zeros(Hkv, 128, lay.scale_stride, dtype=torch.int16, device="cuda")
+    depth = torch.zeros(Hkv, 128, dtype=torch.uint8, device="cuda")
+    scores, walked = (torch.full((Hq, lay.score_stride), -7.0, device="cuda") for _ in range(2))
+    ctx.fathom_build_planes(lay, K, planes, scales)
+    ctx.fathom_alloc_depth(lay, q, K.var(dim=1), fb.DEPTH_WATERFILL, rows, hpp, depth)
+    assert (depth.sum(dim=1) == rows).all()
+    ctx.fathom_scan(lay, planes, scales, q, depth, hpp, scores)
+    fb.fathom_scan_set_ctas_per_plan(2)                              # whole tiles, several per CTA
+    try:
+        ctx.fathom_scan(lay, planes, scales, q, depth, hpp, walked)
+    finally:
+        fb.fathom_scan_set_ctas_per_plan(0)
+    assert torch.equal(scores, walked) and (scores[:, n:] == -7.0).all()
+    m = min(n, 1100)                                                 # the oracle's share: the first blocks
+    nb = (m + 63) // 64
+    ref = O.scan(planes[..., :nb].cpu().numpy().view(np.uint64), scales[..., :nb].cpu().numpy().view(np.float16), q.cpu().numpy(), depth.cpu().numpy(), m, hpp)
+    assert np.all(np.abs(scores[:, :m].cpu().numpy() - ref) <= score_tolerance(ref))
+    ctx.close()
+
+
+# half tiles over several waves of CTAs give what whole tiles give
+@pytest.mark.parametrize("n", [100001, 262144])
+@pytest.mark.parametrize("budget", [16, 48, 136])
+def test_scan_of_half_tiles_over_waves(n, budget):
+    from paper_2609_17652_b200 import binding as fb
+    Hkv, Hq, hpp = 8, 16, 2
+    lay = fb.make_layout(Hkv, Hq, n)
+    ctx = fb.Context(0, 0)
+    g = torch.Generator(device="cuda").manual_seed(budget)
+    q, var = torch.randn(Hq, 128, generator=g, device="cuda"), torch.rand(Hkv, 128, generator=g, device="cuda")
+    planes = torch.randint(-2 ** 62, 2 ** 62, (Hkv, 128, 4, lay.plane_stride_words), generator=g, device="cuda")
+    scales = torch.rand(Hkv, 128, lay.scale_stride, generator=g, device="cuda").half().view(torch.int16)
+    depth = torch.zeros(Hkv, 128, dtype=torch.uint8, device="cuda")
+    scores, walked = (torch.full((Hq, lay.score_stride), -7.0, device="cuda") for _ in range(2))
+    ctx.fathom_alloc_depth(lay, q, var, fb.DEPTH_WATERFILL, budget, hpp, depth)
+    ctx.fathom_scan(lay, planes, scales, q, depth, hpp, scores)
+    fb.fathom_scan_set_ctas_per_plan(30)
+    try:
+        ctx.fathom_scan(lay, planes, scales, q, depth, hpp, walked)
+    finally:
+        fb.fathom_scan_set_ctas_per_plan(0)
+    assert torch.equal(scores, walked) and (scores[:, n:] == -7.0).all()
+    ctx.close()
