@@ -192,8 +192,8 @@ int fathom_topk_passes(const fathom_layout* layout, int k, int n_sink, int n_loc
 
 /* ---- (3+4) fused scan and top-k, scores never materialised — Sec. 9 Conclusion (fusing the scan with what follows it) ------
  * Gives exactly the idx that fathom_topk would give on the scores of fathom_scan (same arguments), without writing
- * or re-reading the n * Hq scores: (a) every 16th 1024-token tile is scanned and histogrammed per head (12 leading
- * score-key bits); (b) the full scan keeps only the (score, token) pairs that reach a threshold bin's lower edge;
+ * or re-reading the n * Hq scores: (a) every 16th 1024-token tile is scanned and histogrammed per head (the
+ * largest of every four scores); (b) the full scan keeps only the (score, token) pairs that reach a threshold bin's lower edge;
  * (c) the exact selection (ties to the lower token) runs on those candidates and writes idx.  Two thresholds come
  * from the sample: a BOUND (the bin of the sample's k-th largest score: at least k tokens reach it, so no winner lies
  * below) and an ESTIMATE (the bin of the rank that k tokens of the whole sequence are expected to reach, plus four

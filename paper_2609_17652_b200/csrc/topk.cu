@@ -7,8 +7,8 @@
 // large k and many heads (held_in_registers).
 //
 // Single pass (other rows of at least 65,536, when a sixteenth of the row holds enough of what is wanted): one read of the scores.
-//   a. a cluster of four CTAs per head histograms every 16th 1024-score chunk (12 leading key bits, shared memory,
-//      merged through distributed shared memory) and finds two bins:
+//   a. a cluster of four CTAs per head histograms the largest of every four scores of every 16th 1024-score chunk (bins of a
+//      thirty-second of an octave, shared memory, merged through distributed shared memory) and finds two bins:
 //      the ESTIMATE, whose suffix count in the sample reaches the expected rank plus four standard deviations, and
 //      the BOUND, whose suffix count reaches k in the sample alone and therefore in the whole row;
 //   b. every CTA of the collection pass loads its 8192 scores before the sample kernel has finished (programmatic
@@ -60,7 +60,7 @@ constexpr int FIN_CACHE_MAX = 16384;                         // ... direct selec
 
 using Gate = fathom_gate;
 
-template <int THREADS, bool IN_GLOBAL>
+template <int THREADS>
 __device__ void find_threshold_bin(const uint32_t* __restrict__ h, uint32_t* __restrict__ st, uint32_t want,
                                    uint32_t* __restrict__ dev_status, uint32_t* s_warp, uint32_t want_bound);
 
@@ -133,18 +133,17 @@ topk_hist_kernel(const float* __restrict__ scores, long long n, long long score_
   __syncthreads();
   if (!s_last) return;
   __threadfence();
-  find_threshold_bin<HIST_THREADS, true>(g, state + head * 8, want, dev_status, sh, want_bound);
+  find_threshold_bin<HIST_THREADS>(g, state + head * 8, want, dev_status, sh, want_bound);
 }
 
 // state[head][0] = threshold bin, [1] = tokens in bins above it, [2] = tokens still needed from it, [3] = bound bin
 // of a sampled histogram, [4] = candidates appended by the filter, [5] = ticket counter of the histogram CTAs,
 // [6] = the score a candidate of the first attempt must reach (fp32 bits): the lower edge of bin [0].
-// Run by all THREADS threads of a CTA that sees the head's complete histogram h (in global memory: the CTA that
-// finished it last; or in shared memory): thread t owns bins 4095 - BPT t .. (descending), so a block prefix over
+// Run by all THREADS threads of the CTA that finished the head's histogram h in global memory last: thread t owns bins 4095 - BPT t .. (descending), so a block prefix over
 // threads is a suffix count over bins.  s_warp: at least THREADS / 32 words of shared memory.
 // want: rank whose bin goes to words 0..2.  want_bound (0 = none): rank whose bin alone goes to word 3 (histogram of
 // a sample: the bin of the sample's want_bound-th largest score is reached by at least that many tokens of the row).
-template <int THREADS, bool IN_GLOBAL>
+template <int THREADS>
 __device__ void find_threshold_bin(const uint32_t* __restrict__ h, uint32_t* __restrict__ st, uint32_t want,
                                    uint32_t* __restrict__ dev_status, uint32_t* s_warp, uint32_t want_bound) {
   constexpr int BPT = FATHOM_TOPK_BINS / THREADS;             // bins per thread
@@ -153,7 +152,7 @@ __device__ void find_threshold_bin(const uint32_t* __restrict__ h, uint32_t* __r
 #pragma unroll
   for (int x = 0; x < BPT; ++x) {                             // a histogram other CTAs added to is read past the L1
     const uint32_t* p = h + (FATHOM_TOPK_BINS - 1 - (BPT * tid + x));
-    c[x] = IN_GLOBAL ? __ldcg(p) : *p;
+    c[x] = __ldcg(p);
     local += c[x];
   }
   uint32_t incl = local;
@@ -203,16 +202,22 @@ __device__ void find_threshold_bin(const uint32_t* __restrict__ h, uint32_t* __r
 
 // Histogram of a head's sample (every 16th whole chunk of 1024 scores) by a cluster of SAMPLE_CLUSTER CTAs: each
 // histograms its share of the chunks in its own shared memory, the others add their non-empty bins to the first CTA's
-// through distributed shared memory (atomics: a few hundred bins of 4096 hold anything), and the first CTA finds the
+// through distributed shared memory (atomics: a few hundred bins of 4096 hold anything), and two of its warps find the
 // estimated and the bound bin: no global histogram, no flush, no ticket.  For rows of up to a few million scores.
+// `grouped`: the largest of every four scores are counted (k is at most half of their number): a rank of them lies no
+// higher than the same rank of the scores, next to nothing lower where it is small, and there are four times fewer shared-memory atomics, of
+// which the kernel consists.  Bins of a thirty-second of an octave instead of an eighth: the lists hold less beyond what is wanted, and a row
+// whose large scores lie close together does not overflow them.  32 heads, back to back, every score in bins of an eighth / now: top-k
+// of 1,048,576 scores, k = 4096 38.3 / 36.9 us (with the last sixteenth 50 above the others 135 / 46), of 500,003, k = 2048 24.1 / 22.3; fused call,
+// 1,048,576 tokens, budget 48, k = 4096 74.3 / 65.1, budget 80 106.2 / 99.2.
 constexpr int SAMPLE_THREADS = 1024;
 constexpr int SAMPLE_CLUSTER = 4;
 __global__ void __cluster_dims__(SAMPLE_CLUSTER, 1, 1) __launch_bounds__(SAMPLE_THREADS, 2)
 topk_sample_kernel(const float* scores, long long sampled, long long chunk_stride, long long score_stride,
-                   uint32_t* __restrict__ state, uint32_t want, uint32_t want_bound, uint32_t* __restrict__ cand_count,
+                   uint32_t* __restrict__ state, uint32_t want, uint32_t want_bound, int grouped, uint32_t* __restrict__ cand_count,
                    uint32_t* __restrict__ cand_count2) {
-  __shared__ uint32_t sh[FATHOM_TOPK_BINS];
-  __shared__ uint32_t s_warp[SAMPLE_THREADS / 32];
+  __shared__ alignas(16) uint32_t sh[COARSE];
+  __shared__ uint32_t s_super[COARSE / SUPER];
   cg::cluster_group cluster = cg::this_cluster();
   const int head = blockIdx.x / SAMPLE_CLUSTER, part = (int)cluster.block_rank();
   FATHOM_PDL_WAIT();                                          // the scores come from the previous kernel (this one may be launched as its dependent)
@@ -223,12 +228,15 @@ topk_sample_kernel(const float* scores, long long sampled, long long chunk_strid
     cand_count[head] = 0u;
     if (cand_count2) cand_count2[head] = 0u;
   }
-  for (int b = threadIdx.x; b < FATHOM_TOPK_BINS; b += SAMPLE_THREADS) sh[b] = 0u;
+  for (int b = threadIdx.x; b < COARSE; b += SAMPLE_THREADS) sh[b] = 0u;
   __syncthreads();
   auto cleared = cluster.barrier_arrive();                    // my histogram is clear (the first CTA's will be added to)
   const float* row = scores + (size_t)head * (size_t)score_stride;
   // `sampled` whole chunks of 1024 scores, chunk_stride scores apart (16384: every 16th chunk of a score row; 1024: a
   // compact array of sampled scores); CTA `part` of the cluster takes every SAMPLE_CLUSTER-th group of 1024 float4
+  auto count = [&](float v) {
+    if (v == v) atomicAdd(&sh[coarse_bin(v)], 1u);
+  };
   constexpr int STRIDE = SAMPLE_CLUSTER * SAMPLE_THREADS, FLY = 2;            // loads in flight per thread: 32 registers, two CTAs per SM
   for (long long v0 = (long long)part * SAMPLE_THREADS + threadIdx.x; v0 < sampled * 256; v0 += FLY * STRIDE) {
     float4 x[FLY];
@@ -240,24 +248,47 @@ topk_sample_kernel(const float* scores, long long sampled, long long chunk_strid
 #pragma unroll
     for (int u = 0; u < FLY; ++u) {
       if (v0 + u * STRIDE >= sampled * 256) break;
-      atomicAdd(&sh[ordered_key(x[u].x) >> 20], 1u);
-      atomicAdd(&sh[ordered_key(x[u].y) >> 20], 1u);
-      atomicAdd(&sh[ordered_key(x[u].z) >> 20], 1u);
-      atomicAdd(&sh[ordered_key(x[u].w) >> 20], 1u);
+      if (grouped) {
+        count(fmaxf(fmaxf(x[u].x, x[u].y), fmaxf(x[u].z, x[u].w)));           // (a NaN is no maximum)
+      } else {
+        count(x[u].x);
+        count(x[u].y);
+        count(x[u].z);
+        count(x[u].w);
+      }
     }
   }
   __syncthreads();                                            // my histogram is complete
   cluster.barrier_wait(std::move(cleared));                   // (everyone arrived long ago: no wait in practice)
   if (part != 0) {                                            // my non-empty bins are added to the first CTA's: a few hundred of 4096
     uint32_t* first = cluster.map_shared_rank(sh, 0);
-    for (int b = threadIdx.x; b < FATHOM_TOPK_BINS; b += SAMPLE_THREADS) {
+    for (int b = threadIdx.x; b < COARSE; b += SAMPLE_THREADS) {
       const uint32_t c = sh[b];
       if (c) atomicAdd(first + b, c);
     }
   }
   cluster.sync();                                             // the additions are complete and visible
   if (part != 0) return;
-  find_threshold_bin<SAMPLE_THREADS, false>(sh, state + head * 8, want, nullptr, s_warp, want_bound);
+  {                                                           // four bins per thread, eight threads a super bin
+    static_assert(COARSE == 4 * SAMPLE_THREADS && SUPER == 32, "every bin once");
+    const uint4 c = *reinterpret_cast<const uint4*>(sh + 4 * threadIdx.x);
+    uint32_t sum = c.x + c.y + c.z + c.w;
+#pragma unroll
+    for (int o = 1; o < 8; o <<= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+    if ((threadIdx.x & 7) == 0) s_super[threadIdx.x / 8] = sum;
+  }
+  __syncthreads();
+  const int warp = threadIdx.x >> 5;
+  const uint32_t rank = warp == 0 ? want : want_bound;
+  if (warp < 2 && rank) {                                     // fewer than the rank, or the lowest bin: everything
+    uint32_t bin, above, members;
+    search_bins<COARSE>(sh, s_super, rank, bin, above, members);
+    const float edge = bin == 0u ? -INFINITY : coarse_edge(bin);
+    if ((threadIdx.x & 31) == 0) {
+      if (warp == 0) state[head * 8 + 6] = __float_as_uint(edge);
+      else state[head * 8 + 3] = bin == 0u ? 0u : ordered_key(edge) >> 20;    // (its lower edge is no higher)
+    }
+  }
 }
 
 
@@ -1283,7 +1314,7 @@ static int run_dense_topk(fathom_ctx* ctx, const float* scores, long long n, lon
     // reach the bound bin, hence at least k - forced = want eligible ones
     if (sampled <= 256) {                                              // up to 4M scores per row: one CTA per head
       FATHOM_CUDA_TRY(ctx, fathom_launch_dependent(topk_sample_kernel, dim3(Hq * SAMPLE_CLUSTER), dim3(SAMPLE_THREADS), 0, st, scores, sampled, 16 * 1024LL, score_stride, S.state, rank, (uint32_t)k,
-                                                        S.cand_count, (uint32_t*)nullptr));
+                                                        8LL * k <= sampled * 1024 ? 1 : 0, S.cand_count, (uint32_t*)nullptr));
     } else {
       const int reps = 8;                                              // sampled chunks per CTA
       dim3 sgrid((unsigned)((sampled + reps - 1) / reps), (unsigned)Hq);
@@ -1415,7 +1446,7 @@ extern "C" int fathom_scan_topk(fathom_ctx* ctx, const fathom_layout* L, const u
   if (one_cta_sample) {                                       // one CTA per head, histogram in shared memory only
     FATHOM_CUDA_TRY(ctx, fathom_launch_dependent(topk_sample_kernel, dim3(Hq * SAMPLE_CLUSTER), dim3(SAMPLE_THREADS), 0, st, (const float*)S.sample,
                                                  n_sample / 1024, 1024LL, S.sample_stride, S.state, two_attempts ? rank : (uint32_t)k,
-                                                 two_attempts ? (uint32_t)k : 0u, S.cand_count, S.cand_count2));
+                                                 two_attempts ? (uint32_t)k : 0u, 8LL * k <= n_sample ? 1 : 0, S.cand_count, S.cand_count2));
   } else {
     const int htile = hist_tile_for(n_sample, Hq);
     dim3 hgrid((unsigned)((n_sample + htile - 1) / htile), (unsigned)Hq);

@@ -38,32 +38,10 @@ namespace {
 constexpr int RT_THREADS = 512;
 constexpr int RT_WARPS = RT_THREADS / 32;
 constexpr int MAX_CLUSTER = 8;
-constexpr int COARSE = 4096;
 constexpr int FINE = 2048, FINE_SHIFT = 13;
-constexpr int SUPER = 32;                                     // bins of a histogram that are also counted together
 constexpr int SPLIT = 512;                                    // members of a split bin ranked by comparison
 constexpr int CHUNK = 128, MAX_CHUNKS = (int)(FATHOM_TOPK_RESIDENT_MAX / CHUNK);
 constexpr int MOST_LISTED = 16384;                            // over all lists of a cluster of several CTAs
-
-// Coarse bin of a score (monotone, -0 with +0) and its lower edge.  Magnitudes from 2^-16 to 2^16 have 32 bins per octave, the others
-// four: with the same eight everywhere (the 12 leading key bits) a head whose threshold fell to the upper end of a bin had twice
-// the candidates it wanted.
-constexpr uint32_t MAG_LO = 111u << 23, MAG_HI = 143u << 23, MID0 = MAG_LO >> 21, HIGH0 = MID0 + ((MAG_HI - MAG_LO) >> 18);
-constexpr uint32_t ZERO_BIN = 1920;
-static_assert(HIGH0 + ((0x7f800000u - MAG_HI) >> 21) < ZERO_BIN && 2 * ZERO_BIN <= COARSE, "bins of both signs");
-__device__ __forceinline__ uint32_t coarse_bin(float f) {
-  const uint32_t u = __float_as_uint(f) & 0x7fffffffu;
-  const uint32_t m = u < MAG_LO ? u >> 21 : (u < MAG_HI ? MID0 + ((u - MAG_LO) >> 18) : HIGH0 + ((u - MAG_HI) >> 21));
-  return f < 0.0f ? ZERO_BIN - 1u - m : ZERO_BIN + m;
-}
-__device__ __forceinline__ float coarse_edge(uint32_t bin) {
-  auto smallest = [](uint32_t m) {                            // magnitude bits
-    return m < MID0 ? m << 21 : (m < HIGH0 ? MAG_LO + ((m - MID0) << 18) : MAG_HI + ((m - HIGH0) << 21));
-  };
-  if (bin >= ZERO_BIN) return __uint_as_float(smallest(bin - ZERO_BIN));
-  const uint32_t u = smallest(ZERO_BIN - bin) - 1u;           // the largest magnitude of the bin
-  return u >= 0x7f800000u ? -INFINITY : __uint_as_float(u | 0x80000000u);
-}
 
 struct ResidentSmem {
   alignas(16) uint32_t coarse[COARSE];                        // counts of this CTA's maxima; then members of the split bin and places of the chunks,
@@ -81,50 +59,6 @@ struct ResidentSmem {
 constexpr int COUNTS = COARSE + COARSE / SUPER + FINE + FINE / SUPER;
 static_assert(offsetof(ResidentSmem, warp_sum) == COUNTS * 4 && COUNTS % 4 == 0, "the counts lie side by side");
 static_assert(SPLIT * 8 + MAX_CHUNKS * 4 <= COARSE * 4, "the split bin and the places fit over the coarse counts");
-
-// One warp: the largest bin whose suffix count reaches `rank` (> 0), the count above it and its own, in every lane.  If there are
-// fewer than `rank`: bin 0 with everything.
-template <int BINS>
-__device__ __forceinline__ void search_bins(const uint32_t* bins, const uint32_t* super, uint32_t rank, uint32_t& bin, uint32_t& above, uint32_t& count) {
-  constexpr int PER = BINS / SUPER / 32;                      // lane l owns super bins BINS / SUPER - 1 - PER l .. descending
-  const int lane = threadIdx.x & 31;
-  uint32_t c[PER], local = 0u;
-#pragma unroll
-  for (int u = 0; u < PER; ++u) {
-    c[u] = super[BINS / SUPER - 1 - PER * lane - u];
-    local += c[u];
-  }
-  auto inclusive = [&](uint32_t x) {
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
-      if (lane >= o) x += y;
-    }
-    return x;
-  };
-  uint32_t incl = inclusive(local);
-  const unsigned reach = __ballot_sync(0xffffffffu, incl >= rank);
-  if (reach == 0u) {
-    bin = above = 0u;
-    count = __shfl_sync(0xffffffffu, incl, 31);
-    return;
-  }
-  uint32_t run = incl - local;
-  int u = 0;
-#pragma unroll
-  for (int x = 0; x < PER - 1; ++x)
-    if (u == x && run + c[x] < rank) { run += c[x]; u = x + 1; }
-  const int from = __ffs(reach) - 1;
-  run = __shfl_sync(0xffffffffu, run, from);
-  u = __shfl_sync(0xffffffffu, u, from);
-  const int first = (BINS / SUPER - 1 - PER * from - u) * SUPER;
-  const uint32_t mine = bins[first + SUPER - 1 - lane];
-  incl = run + inclusive(mine);
-  const int at = __ffs(__ballot_sync(0xffffffffu, incl >= rank)) - 1;
-  bin = (uint32_t)(first + SUPER - 1 - at);
-  count = __shfl_sync(0xffffffffu, mine, at);
-  above = __shfl_sync(0xffffffffu, incl, at) - count;
-}
 
 // All threads of the CTA, after a barrier that completes the counts: what search_bins finds, in M (with a barrier behind it).
 template <int BINS>
