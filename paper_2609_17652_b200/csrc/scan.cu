@@ -392,14 +392,14 @@ scan_kernel(const __grid_constant__ ScanBatchOf<CAP> B, int G, int heads_per_pla
   // are worked eight at a time (byte k of the loaded words).  Tokens past the end of the sequence are computed from zeros or from
   // what pads the rows and never leave.
   struct Place { const unsigned char* wp; const uint16_t* sp; uint32_t tok0, dst0; };
-  auto place = [&](auto tbc, int g, int u, int buf, int buf_words) {
+  auto place = [&](auto tbc, int g, int u, int blk0, int buf, int buf_words) {     // blk0: the stage's first block
     constexpr int TB = decltype(tbc)::value, BYTES = TB / 4;   // plane bytes per row and lane
     const int mine = warp * (TB / 4) + (gq * BYTES) / 8;       // my block of the stage
     const int off = (gq * BYTES) % 8;                          // where my bytes start in its words
     Place p;
     p.wp = M.words + buf * buf_words + (2 * t4) * Geo<TB>::ROW_BYTES + mine * 8 + off;
     p.sp = reinterpret_cast<const uint16_t*>(M.scale + buf * STAGE_SCALES) + (2 * t4) * Geo<TB>::SCALE_ELEMS + mine;
-    p.tok0 = (uint32_t)(first_block(g) + u * TB + mine) * FATHOM_BLOCK + off * 8;           // my first token
+    p.tok0 = (uint32_t)(blk0 + mine) * FATHOM_BLOCK + off * 8;                               // my first token
     p.dst0 = MODE == 1 ? (uint32_t)g * (TILE_BLOCKS * FATHOM_BLOCK) + (uint32_t)(u * TB + mine) * FATHOM_BLOCK + off * 8 : p.tok0;
     return p;
   };
@@ -428,6 +428,11 @@ scan_kernel(const __grid_constant__ ScanBatchOf<CAP> B, int G, int heads_per_pla
     constexpr int WC = TB / 2, WR = THREADS / WC, WS = (16 * NKS + WR - 1) / WR;          // columns of a row of words, rows and sweeps of the CTA over them
     constexpr int SC = TB / 8, SR = THREADS / SC, SS = (16 * NKS + SR - 1) / SR;          // ... of the scales
     constexpr int BUF = TB == 16 ? STAGE_WORDS : HALF_WORDS;
+    // half tiles of one session's whole-tile launch are dealt out one by one all the same: the shares are even to a half tile (decode step, 136
+    // rows, 500,003 tokens 98.7 -> 96.6 us; a plan per head, 262,144 tokens 145.6 -> 141.0)
+    constexpr bool SINGLY = TB < UNIT && MODE == 0 && CAP == 1;
+    const int last = SINGLY ? (nb_item + TB - 1) / TB : end;
+    auto block_of = [&](int g, int u) { return SINGLY ? g * TB : first_block(g) + u * TB; };
     const int wc = tid % WC, wr = tid / WC, sc = tid % SC, sr = tid / SC;
     uint32_t wo[WS], so[SS];
 #pragma unroll
@@ -449,7 +454,7 @@ scan_kernel(const __grid_constant__ ScanBatchOf<CAP> B, int G, int heads_per_pla
         if (sr + SR * i < nrows) fathom_copy_async<16>(sd + i * (SR * SE * 2), scales_src + so[i], vs, in_hbm);
       fathom_copies_commit();
     };
-    prefetch(first_block(g), 0);                               // the first stage's rows are on their way ...
+    prefetch(block_of(g, 0), 0);                               // the first stage's rows are on their way ...
     clear_pad(tbc, nrows, 0);
     clear_pad(tbc, nrows, 1);
     fill_bfr();                                                // ... while the right operand is made
@@ -457,16 +462,16 @@ scan_kernel(const __grid_constant__ ScanBatchOf<CAP> B, int G, int heads_per_pla
     uint2 bf[KEEP ? NKS : 1];
     for (int u = 0, buf = 0;; buf ^= 1) {
       int g_next = g, u_next = u + 1;                          // (of half tiles: the tile's second, where it has blocks)
-      if (TB == UNIT || u_next == UNIT / TB || first_block(g) + u_next * TB >= nb_item) {
+      if (SINGLY || TB == UNIT || u_next == UNIT / TB || first_block(g) + u_next * TB >= nb_item) {
         u_next = 0;
         g_next = g + gridDim.x;
       }
-      const bool more = g_next < end;
+      const bool more = g_next < last;
       fathom_copies_wait<0>();
       __syncthreads();                                         // this stage's words and scales are in place, and every warp has
                                                                // left the previous stage: its buffer may be refilled
-      if (more) prefetch(first_block(g_next) + u_next * TB, buf ^ 1);         // lands while this stage is scanned
-      const Place at = place(tbc, g, u, buf, BUF);
+      if (more) prefetch(block_of(g_next, u_next), buf ^ 1);   // lands while this stage is scanned
+      const Place at = place(tbc, g, u, block_of(g, u), buf, BUF);
       if constexpr (WALK) {
         float acc[BYTES][4][4];
         auto step = [&](auto first, int ks, uint2 b) {
@@ -554,7 +559,7 @@ scan_kernel(const __grid_constant__ ScanBatchOf<CAP> B, int G, int heads_per_pla
 #pragma unroll
           for (int j = 0; j < 4; ++j) acc[k][j][0] = acc[k][j][1] = acc[k][j][2] = acc[k][j][3] = 0.0f;
       }
-      const Place at = place(tbc, g, u, buf, DEEP_WORDS);
+      const Place at = place(tbc, g, u, first_block(g) + u * TB, buf, DEEP_WORDS);
       const int ks0 = pass * (rows_stage >> 4), nks = (min(rows_stage, nrows - pass * rows_stage) + 15) >> 4;
 #pragma unroll 2
       for (int ks = 0; ks < nks; ++ks) {
@@ -651,17 +656,18 @@ int launch_scan(const ScanBatchOf<CAP>& B, int Hkv, int Hq, int heads_per_plan, 
   if (tiles <= 0) return FATHOM_OK;
   bool host = false;                                          // any store of the launch in pinned host memory
   for (int i = 0; i < B.items; ++i) host = host || fathom_planes_in_host_memory(B.planes[i]);
-  // Half tiles as the CTAs' units where an SM has room for each of them alone, and where, over more than one wave of whole tiles, the busiest
-  // CTA then has a tenth fewer blocks.  (Budget 48, back to back, whole / half: one plan, 4096 tokens 3.5 / 3.0 us, 65,536 3.5 / 3.1; 8 plans,
-  // 16,384 tokens 3.6 / 3.8, 100,000 8.2 / 7.4, 262,144 13.6 / 12.8, budget 32 12.9 / 10.6.)
+  // Half tiles as the CTAs' units where all of them are resident at once, and where, over several waves of whole tiles, the busiest
+  // CTA then has a tenth fewer blocks.  (Decode steps on stores that no cache holds, whole / half, 8 KV and 32 query heads, budget 48: 8192 tokens 15.7 /
+  // 15.3 us, 16,384 16.5 / 16.1, 33,001 20.8 / 20.3, 100,000 36.5 / 35.9, but 200,000 45.8 / 46.1, 500,003 60.5 / 63.2; two heads per plan, 16,384
+  // tokens 17.7 / 16.6; one head 33,001 16.0 / 15.4; a plan per head 8192 17.5 / 16.5, 33,001 24.1 / 24.5.)
   if constexpr (MODE == 0 && CAP == 1) {
     const int plans = Hq / NH;
     if (!host && fathom_scan_ctas_override() == 0) {
       ScanBatchOf<CAP> U = B;
       const long long halves = (fathom_nblocks(B.n[0]) + TILE_BLOCKS / 2 - 1) / (TILE_BLOCKS / 2);
       const long long x16 = fathom_scan_grid_ctas(tiles, plans, false, CTAS_PER_SM), x8 = fathom_scan_grid_ctas(halves, plans, false, CTAS_PER_SM);
-      const bool alone = halves * plans <= fathom_sm_count(), waves = tiles > x16;
-      if (alone || (waves && (halves + x8 - 1) / x8 * 10 <= (tiles + x16 - 1) / x16 * 2 * 9)) {
+      const bool resident = halves == x8, waves = tiles > x16;
+      if (resident || (waves && (halves + x8 - 1) / x8 * 10 <= (tiles + x16 - 1) / x16 * 2 * 9)) {
         U.tile_end[0] = halves;
         return launch_units<NH, MODE, CAP, TILE_BLOCKS / 2>(U, Hkv, Hq, heads_per_plan, fz, false, dependent, st);
       }
