@@ -421,12 +421,22 @@ topk_resident_kernel(const float* scores, int n, long long score_stride, int eli
   }
 }
 
-size_t resident_smem_bytes(int ctas, uint32_t capacity, long long n) {
+constexpr uint32_t most_listed(int ctas, int per_thread) { return ctas == 1 ? (uint32_t)(RT_THREADS * per_thread) : (uint32_t)(MOST_LISTED / ctas); }
+constexpr size_t resident_smem_bytes(int ctas, uint32_t capacity, long long n) {
   return sizeof(ResidentSmem) + (size_t)capacity * ((size_t)ctas * 8 + 4) + (size_t)((n + CHUNK - 1) / CHUNK) * 16;
 }
-// the largest request: two CTAs with half of them each (a single CTA lists no more than it has tokens)
-constexpr int RESIDENT_SMEM_MOST = (int)sizeof(ResidentSmem) + MOST_LISTED * 8 + MOST_LISTED / 2 * 4 + MAX_CHUNKS * 16;
-static_assert(RESIDENT_SMEM_MOST <= 227 * 1024, "fits on an SM");
+// the most that a launch with that many scores per thread may ask for: full lists, and the longest row that its CTAs hold (one CTA of 32 scores per
+// thread, which may list them all, takes more than two that share the lists)
+constexpr size_t resident_smem_most(int per_thread) {
+  size_t most = 0;
+  for (int ctas = 1; ctas <= MAX_CLUSTER; ctas *= 2) {
+    const long long held = (long long)ctas * RT_THREADS * per_thread;
+    const size_t bytes = resident_smem_bytes(ctas, most_listed(ctas, per_thread), held < FATHOM_TOPK_RESIDENT_MAX ? held : FATHOM_TOPK_RESIDENT_MAX);
+    most = bytes > most ? bytes : most;
+  }
+  return most;
+}
+static_assert(resident_smem_most(8) <= 227 * 1024 && resident_smem_most(16) <= 227 * 1024 && resident_smem_most(32) <= 227 * 1024, "fits on an SM");
 
 template <int EPT>
 cudaError_t launch(const float* scores, long long n, long long score_stride, int Hq, int k, Forced F, uint32_t want, int32_t* idx,
@@ -436,7 +446,7 @@ cudaError_t launch(const float* scores, long long n, long long score_stride, int
   const uint32_t quota = ctas == 1 ? want : (uint32_t)(share + 4.0 * sqrt(share) + 8.0);
   // room for 1.75 times the quota (the bound lets through 1.05 to 1.4 times), for 2048 at least and for 16,384 over all lists; two CTAs
   // fit on an SM while k is at most some 4000
-  const uint32_t least = (uint32_t)(2048 / ctas), most = (uint32_t)(ctas == 1 ? RT_THREADS * EPT : MOST_LISTED / ctas);
+  const uint32_t least = (uint32_t)(2048 / ctas), most = most_listed(ctas, EPT);
   uint32_t capacity = (7u * quota / 4u + 3u) & ~3u;
   capacity = capacity < least ? least : (capacity > most ? most : capacity);
   const size_t smem = resident_smem_bytes(ctas, capacity, n);
@@ -445,7 +455,7 @@ cudaError_t launch(const float* scores, long long n, long long score_stride, int
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
   if (dev < 0 || dev >= 64 || !configured[dev]) {
-    e = cudaFuncSetAttribute(topk_resident_kernel<EPT>, cudaFuncAttributeMaxDynamicSharedMemorySize, RESIDENT_SMEM_MOST);
+    e = cudaFuncSetAttribute(topk_resident_kernel<EPT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)resident_smem_most(EPT));
     if (e != cudaSuccess) return e;
     if (dev >= 0 && dev < 64) configured[dev] = true;
   }

@@ -212,7 +212,8 @@ def test_klt_basis_in_place(spread):
 
 # (tokens, heads, k) on both sides of every line between the kernels of the selection, scores that exist and scores that do not
 @pytest.mark.parametrize("n,Hq,k", [(131072, 60, 548), (131072, 46, 600), (131072, 47, 600), (131072, 9, 3108), (131072, 9, 3109), (131072, 2, 16384),
-                                    (131073, 2, 16384), (33001, 9, 9000), (33001, 10, 9000), (20000, 18, 8300), (20000, 19, 8300), (70001, 75, 2100)])
+                                    (131073, 2, 16384), (33001, 9, 9000), (33001, 10, 9000), (20000, 18, 8300), (20000, 19, 8300), (70001, 75, 2100),
+                                    (16384, 96, 16384), (16384, 128, 12000), (8769, 148, 8769), (16384, 149, 12000)])
 def test_selection_on_both_sides_of_its_lines(n, Hq, k):
     from paper_2609_17652_b200 import binding as fb
     lay = fb.make_layout(1, Hq, n)
