@@ -428,9 +428,10 @@ scan_kernel(const __grid_constant__ ScanBatchOf<CAP> B, int G, int heads_per_pla
     constexpr int WC = TB / 2, WR = THREADS / WC, WS = (16 * NKS + WR - 1) / WR;          // columns of a row of words, rows and sweeps of the CTA over them
     constexpr int SC = TB / 8, SR = THREADS / SC, SS = (16 * NKS + SR - 1) / SR;          // ... of the scales
     constexpr int BUF = TB == 16 ? STAGE_WORDS : HALF_WORDS;
-    // half tiles of one session's whole-tile launch are dealt out one by one all the same: the shares are even to a half tile (decode step, 136
-    // rows, 500,003 tokens 98.7 -> 96.6 us; a plan per head, 262,144 tokens 145.6 -> 141.0)
-    constexpr bool SINGLY = TB < UNIT && MODE == 0 && CAP == 1;
+    // half tiles of one device-resident session's whole-tile launch are dealt out one by one all the same: the shares are even to a half tile
+    // (decode step, 136 rows, 500,003 tokens 98.7 -> 96.6 us; a plan per head, 262,144 tokens 145.6 -> 141.0).  Over the host link a CTA takes its
+    // tile's halves one after the other: they are the two ends of the same lines (136 rows, 8192 tokens, 8 plans 46.8 -> 39.5 us)
+    constexpr bool SINGLY = TB < UNIT && MODE == 0 && CAP == 1 && IN_HBM;
     const int last = SINGLY ? (nb_item + TB - 1) / TB : end;
     auto block_of = [&](int g, int u) { return SINGLY ? g * TB : first_block(g) + u * TB; };
     const int wc = tid % WC, wr = tid / WC, sc = tid % SC, sr = tid / SC;

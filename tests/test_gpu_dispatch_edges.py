@@ -458,3 +458,46 @@ def test_scan_of_half_tiles_over_waves(n, budget):
         fb.fathom_scan_set_ctas_per_plan(0)
     assert torch.equal(scores, walked) and (scores[:, n:] == -7.0).all()
     ctx.close()
+
+
+# plans that fit one stage of half tiles only, and deeper ones: over the host link, and in a batch whose sessions end in a first half or in a second one,
+# with CTAs that cross from one session to the next
+@pytest.mark.parametrize("budget", [97, 136, 160, 161])
+@pytest.mark.parametrize("host,ctas", [(False, None), (False, 3), (True, None)])
+def test_deep_plans_of_several_sessions(budget, host, ctas):
+    from paper_2609_17652_b200 import binding as fb
+    from tests._pipeline import score_tolerance
+    Hkv, Hq, hpp = 2, 8, 4
+    ctx = fb.Context(0, 0)
+    g = torch.Generator(device="cuda").manual_seed(budget)
+    items, alone = [], []
+    for n in (3000, 512, 4609, 64, 1536, 40):
+        lay = fb.make_layout(Hkv, Hq, n)
+        q, var = torch.randn(Hq, 128, generator=g, device="cuda"), torch.rand(Hkv, 128, generator=g, device="cuda")
+        K = torch.randn(Hkv, n, 128, generator=g, device="cuda")
+        planes = torch.zeros(Hkv, 128, 4, lay.plane_stride_words, dtype=torch.int64, device="cuda")
+        scales = torch.zeros(Hkv, 128, lay.scale_stride, dtype=torch.int16, device="cuda")
+        depth = torch.zeros(Hkv, 128, dtype=torch.uint8, device="cuda")
+        scores, single = (torch.full((Hq, lay.score_stride), -7.0, device="cuda") for _ in range(2))
+        ctx.fathom_build_planes(lay, K, planes, scales)
+        ctx.fathom_alloc_depth(lay, q, var, fb.DEPTH_WATERFILL, budget, hpp, depth)
+        ctx.fathom_scan(lay, planes, scales, q, depth, hpp, single)
+        if host:
+            planes, scales = (torch.empty(t.shape, dtype=t.dtype, pin_memory=True).copy_(t) for t in (planes, scales))
+            again = torch.full_like(single, -7.0)
+            ctx.fathom_scan(lay, planes, scales, q, depth, hpp, again)
+            assert torch.equal(again, single), n
+        items.append((lay, planes, scales, q, depth, scores))
+        alone.append(single)
+    fb.fathom_scan_set_ctas_per_plan(ctas or 0)
+    try:
+        ctx.fathom_scan_batch(items, hpp)
+    finally:
+        fb.fathom_scan_set_ctas_per_plan(0)
+    for (lay, planes, scales, q, depth, scores), single in zip(items, alone):
+        assert torch.equal(scores, single), lay.n
+        planes, scales, n = planes.cpu().numpy(), scales.cpu().numpy(), lay.n
+        nb = (n + 63) // 64
+        ref = O.scan(planes[..., :nb].view(np.uint64), scales[..., :nb].view(np.float16), q.cpu().numpy(), depth.cpu().numpy(), n, hpp)
+        assert np.all(np.abs(scores[:, :n].cpu().numpy() - ref) <= score_tolerance(ref))
+    ctx.close()
