@@ -8,6 +8,8 @@
 // Two channels are compared once for all their planes: non-negative doubles order like their bit patterns, dividing by 4 takes 2^53 off
 // the pattern, so with D = pattern(g_i) - pattern(g_j) the planes of i that rank before (j, m) are those up to m + floor(D / 2^53)
 // (D - 1 where j wins ties).  (Products and sums of squares of fp32 numbers are far from fp64's subnormals, so the quarters are exact.)
+// Infinite and NaN importances rank before all finite ones, by their patterns and then by channel, all planes of a channel together (their
+// quarters are no smaller).
 // A warp per channel j, four channels i per lane, the four planes' counts summed by two warp reductions of packed halves.
 // Eight CTAs serve a plan, 16 channels each; every CTA computes all 128 importances (thread = channel).  The kernel is a latency chain: it
 // compared each of the 512 candidates with all others before, eight threads per candidate (back to back: one plan 2.9 -> 1.4 us, 8 plans 3.1 -> 1.6, 32 plans 6.8 -> 2.0).
@@ -18,6 +20,15 @@ namespace {
 constexpr int CTAS_PER_PLAN = 8;
 constexpr int AD_CHANNELS = FATHOM_D / CTAS_PER_PLAN;        // 16 channels ranked per CTA, a warp each
 constexpr int AD_THREADS = 32 * AD_CHANNELS;                 // 512
+constexpr long long FIRST_NONFINITE = 928LL << 52;           // where the patterns of infinity and NaN are moved to
+
+// Bit pattern without its sign.  (The sign is taken off an integer in which the compiler does not see a double: it would make that a floating-point
+// absolute value, which leaves a NaN its sign.)
+__device__ __forceinline__ long long magnitude(double x) {
+  long long b;
+  asm("mov.b64 %0, %1;" : "=l"(b) : "d"(x));
+  return b & 0x7fffffffffffffffLL;
+}
 
 __global__ void __launch_bounds__(AD_THREADS)
 alloc_depth_kernel(const float* q, const float* var, int mode, int budget,
@@ -54,14 +65,15 @@ alloc_depth_kernel(const float* q, const float* var, int mode, int budget,
     if (mode == FATHOM_DEPTH_WATERFILL) {
       const float v = var[(size_t)kv * FATHOM_D + j];
       add_heads([](double x) { return __dmul_rn(x, x); });    // Eq. 3
-      const long long g = __double_as_longlong(fabs(__dmul_rn(acc, (double)v)));
+      const long long g = magnitude(__dmul_rn(acc, (double)v));
       // Patterns of the products of finite fp32 numbers have exponents from 576 to 1420; 512 less, they leave room for channels of no
-      // importance below: so far apart that all planes of one rank before all planes of the next
-      const long long low = -((long long)(j + 1) << 55), most = 1023LL << 52;
-      order[j] = g == 0 ? low : min(g - (512LL << 52), most);
+      // importance below: so far apart that all planes of one rank before all planes of the next.  The other patterns are moved to where
+      // no plane of a finite channel comes near them and no difference overflows
+      const long long low = -((long long)(j + 1) << 55), nonfinite = 2047LL << 52;
+      order[j] = g == 0 ? low : (g < nonfinite ? g - (512LL << 52) : g - nonfinite + FIRST_NONFINITE);
     } else {                                                  // fixed top-r channels by sum_h |q_j|
       add_heads([](double x) { return fabs(x); });
-      order[j] = __double_as_longlong(acc);
+      order[j] = magnitude(acc);
     }
   }
   __syncthreads();
@@ -73,7 +85,9 @@ alloc_depth_kernel(const float* q, const float* var, int mode, int budget,
 #pragma unroll
     for (int u = 0; u < FATHOM_D / 32; ++u) {
       const int i = lane + 32 * u;
-      const int e = (int)((order[i] - mine - (i < j ? 0 : 1)) >> 53);        // (i = j: the planes above m)
+      const long long d = order[i] - mine - (i < j ? 0 : 1);
+      int e = (int)(d >> 53);                                 // (i = j: the planes above m)
+      if (mine >= FIRST_NONFINITE && i != j) e = d >= 0 ? FATHOM_NPLANES : -FATHOM_NPLANES;       // (uniform over the warp)
       auto planes = [&](int m) { return (uint32_t)min(max(m + e, 0), FATHOM_NPLANES); };
       before12 += planes(1) | planes(2) << 16;
       before34 += planes(3) | planes(4) << 16;

@@ -401,6 +401,41 @@ def test_depths_of_tied_and_extreme_importances(kind, budget):
     ctx.close()
 
 
+# infinite importances, and ones that are no number (an infinite query times no variance): before all others, one channel after the other
+@pytest.mark.parametrize("budget", [1, 4, 6, 17, 60, 300, 512])
+@pytest.mark.parametrize("kind", ["infinite", "no number"])
+def test_depths_of_importances_that_are_not_finite(kind, budget):
+    from paper_2609_17652_b200 import binding as fb
+    lay = fb.make_layout(1, 2, 64)
+    ctx = fb.Context(0, fb.fathom_scratch_bytes(lay, 1))
+    rng = np.random.default_rng(budget)
+    q, var = rng.standard_normal((2, 128)).astype(np.float32), rng.random((1, 128)).astype(np.float32)
+    far = np.sort(rng.choice(128, 12, replace=False))                # channels of an infinite query; among them some of no variance
+    q[0, far[1:]], var[0, far[0]], q[1, 127 - far[0]] = np.inf, np.inf, 3.4e38
+    odd = far[2:9:3] if kind == "no number" else far[:0]
+    var[0, odd] = 0.0
+    var[0, (far[-1] + 1) % 128] = 0.0
+    depth = torch.full((1, 128), 9, dtype=torch.uint8, device="cuda")
+    ctx.fathom_alloc_depth(lay, torch.from_numpy(q).cuda(), torch.from_numpy(var).cuda(), fb.DEPTH_WATERFILL, budget, 2, depth)
+    with np.errstate(invalid="ignore"):
+        g = O.importance(q, var, 2)[0]
+    assert np.array_equal(np.flatnonzero(np.isnan(g)), odd) and np.isinf(g).any()
+    ref, left = np.zeros(128, np.uint8), budget
+    for j in odd:
+        ref[j] = min(4, left)
+        left -= int(ref[j])
+    rest = np.setdiff1d(np.arange(128), odd)
+    ref[rest] = O.waterfill_depths(g[rest], left)
+    assert np.array_equal(depth.cpu().numpy()[0], ref)
+    # channels by the sum of magnitudes
+    q[1, odd] = np.nan
+    ctx.fathom_alloc_depth(lay, torch.from_numpy(q).cuda(), None, fb.DEPTH_FIXED_TOP_R, min(budget, 128), 2, depth)
+    w = np.abs(q.astype(np.float64)).sum(axis=0)
+    first = sorted(range(128), key=lambda j: (not np.isnan(w[j]), 0.0 if np.isnan(w[j]) else -w[j], j))[:min(budget, 128)]
+    assert np.array_equal(np.flatnonzero(depth.cpu().numpy()[0] == 4), np.sort(first)) and set(np.unique(depth.cpu().numpy())) <= {0, 4}
+    ctx.close()
+
+
 # rows at the edges of a stage (16 each; 96 of a tile, 160 of half a tile), half tiles alone on their SMs, whole tiles, half tiles over several waves; tails
 # of a block and of a unit
 @pytest.mark.parametrize("rows", [15, 17, 96, 97, 113, 144, 159, 160, 161, 255])
