@@ -1218,18 +1218,18 @@ static bool single_pass_plan(long long n, int k, uint32_t want, uint32_t* rank_o
 
 // Whether rows of n scores are held in registers (topk_resident.cu).
 // us held in registers / the other way (single pass where the row and k allow it, else two passes):
-//   131,072 scores  32 heads: k = 64 7.8 / 14.8, 2048 11.9 / 18.0, 3000 15.4 / 18.8, 4096 16.8 / 19.7; 40 heads: 2048 20.9 / 23.0, 3000 26.0 / 24.4;
-//                   128 heads: 2048 44 / 47, 3000 56 / 50
-//   100,000 scores  k = 8192: 16 heads 29 / 38, 32 heads 47 / 44; k = 16,384: 8 heads 36 / 30
-//   65,536 scores   k = 4096: 32 heads 14 / 33, 128 heads 33 / 52; k = 8192: 64 heads 37 / 51, 128 heads 74 / 64
-//   33,001 scores   k = 8192: 32 heads 18 / 30, 64 heads 35 / 36, 128 heads 69 / 46; k = 16,384: 32 heads 19 / 29, 64 heads 32 / 33
-// (scores of some thirty distinct values overflow the lists and take radix rounds: 100,000 scores, 32 heads, k = 2048 32 / 31)
-static bool held_in_registers(long long n, int Hq, uint32_t want) {
+//   up to 65,536 scores  33,001, k = 64: 32 heads 6.3 / 34; 128 heads, k = 16,384: 39 / 55; 65,536, 148 heads: k = 8192 69 / 77, 16,384 67 / 73
+//   131,072 scores  32 heads: k = 64 7.8 / 14, 2048 12 / 18, 4096 17 / 19; 40 heads: 3000 26 / 24, 4096 29 / 25; 128 heads: 2048 43 / 47; 148 heads: 1024 44 / 48,
+//                   2048 52 / 52; k = 8192: 32 heads 39 / 49, 40 heads 49 / 53, 64 heads 66 / 61
+//   70,000 scores   148 heads: 1024 43 / 43, 2048 50 / 46; two passes, k = 4096: 64 heads 32 / 51, 128 heads 61 / 63; k = 8192: 40 heads 41 / 51, 64 heads 52 / 57
+static bool held_in_registers(long long n, int Hq, int k, uint32_t want) {
   if (n > FATHOM_TOPK_RESIDENT_MAX || force_two_pass()) return false;
-  const long long ctas = (long long)Hq * fathom_topk_resident_ctas(n, Hq, want), sms = fathom_sm_count();
-  if (want > 8192) return n <= 65536 && ctas <= sms;          // no list holds its quota: radix rounds over the cluster
-  if (want > 4096) return ctas <= (n <= 65536 ? 2 : 1) * sms;
-  return n <= 65536 || want <= 2048 || ctas <= 2 * sms;
+  if (n <= 65536) return true;
+  const long long ctas = (long long)Hq * fathom_topk_resident_ctas(n, Hq), sms = fathom_sm_count();
+  uint32_t rank;
+  if (want > 4096) return ctas <= 3 * sms;
+  if (want > 2048 && single_pass_plan(n, k, want, &rank)) return ctas <= 2 * sms;
+  return want <= 1024 || ctas <= 7 * sms;
 }
 
 // log2 of the token range per counting-sort bucket of the direct select: the smallest that maps n tokens to SORT_BUCKETS
@@ -1278,7 +1278,7 @@ static int launch_direct_select(fathom_ctx* ctx, long long n, int Hq, int k, For
 
 static int run_dense_topk(fathom_ctx* ctx, const float* scores, long long n, long long score_stride, int Hq, int k,
                           Forced F, uint32_t want, const fathom_topk_scratch& S, int32_t* idx, cudaStream_t st) {
-  if (held_in_registers(n, Hq, want)) return fathom_launch_topk_resident(ctx, scores, n, score_stride, Hq, k, F, want, idx, st);
+  if (held_in_registers(n, Hq, k, want)) return fathom_launch_topk_resident(ctx, scores, n, score_stride, Hq, k, F, want, idx, st);
   const int ntiles = (int)((n + FILT_TILE - 1) / FILT_TILE);
   dim3 fgrid((unsigned)ntiles, (unsigned)Hq);
   Gate always = {nullptr, 0u, 0, 0};
@@ -1378,7 +1378,7 @@ extern "C" int fathom_topk_passes(const fathom_layout* L, int k, int n_sink, int
   if (n_forced > k) return FATHOM_ERR_INVALID_ARG;
   const uint32_t want = (uint32_t)(k - n_forced);
   uint32_t rank;
-  return held_in_registers(n, L->n_q_heads, want) || single_pass_plan(n, k, want, &rank) ? 1 : 2;
+  return held_in_registers(n, L->n_q_heads, k, want) || single_pass_plan(n, k, want, &rank) ? 1 : 2;
 }
 
 // Tile step of the sample scan for (n, k): every 16th scan tile when that sample still holds at least 2 k tokens,
@@ -1413,7 +1413,7 @@ extern "C" int fathom_scan_topk(fathom_ctx* ctx, const fathom_layout* L, const u
   if (S.bytes > ctx->scratch_bytes) return FATHOM_ERR_SCRATCH_TOO_SMALL;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   const uint32_t want = (uint32_t)(k - n_forced);
-  const bool held = held_in_registers(n, Hq, want);
+  const bool held = held_in_registers(n, Hq, k, want);
   const int step = held ? 1 : fathom_fused_tile_step(n, k);
   const long long tile = fathom_scan_tile_tokens();
   const long long ntiles_scan = (n + tile - 1) / tile;

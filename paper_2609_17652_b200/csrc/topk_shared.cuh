@@ -90,6 +90,6 @@ struct Forced { long long sink_end, local_begin; };          // eligible tokens:
 
 // Rows that a cluster of CTAs can hold in registers (topk_resident.cu)
 constexpr long long FATHOM_TOPK_RESIDENT_MAX = 131072;
-int fathom_topk_resident_ctas(long long n, int Hq, uint32_t want);          // CTAs per head
+int fathom_topk_resident_ctas(long long n, int Hq);           // CTAs per head
 int fathom_launch_topk_resident(fathom_ctx* ctx, const float* scores, long long n, long long score_stride, int Hq, int k, Forced F,
                                 uint32_t want, int32_t* idx, cudaStream_t st);
