@@ -197,8 +197,8 @@ int fathom_topk_passes(const fathom_layout* layout, int k, int n_sink, int n_loc
  * (c) the exact selection (ties to the lower token) runs on those candidates and writes idx.  Two thresholds come
  * from the sample: a BOUND (the bin of the sample's k-th largest score: at least k tokens reach it, so no winner lies
  * below) and an ESTIMATE (the bin of the rank that k tokens of the whole sequence are expected to reach, plus four
- * standard deviations: ~6 times fewer candidates).  The scan runs with the estimate; if any head then holds fewer
- * candidates than it needs, a second scan with the bound, enqueued behind the first, does the work instead - the
+ * standard deviations or more: ~6 times fewer candidates).  The scan runs with the estimate; the heads that then hold fewer
+ * candidates than they need are scanned again with the bound, by a launch enqueued behind the first - the
  * decision is taken on the device, and the result never depends on how representative the sample is.
  * Sequences of up to 131,072 tokens (but for many heads), and longer ones that are too short to sample (fewer than 2 k
  * sampled tokens), are scanned into scratch and selected densely instead.  Uses the context scratch (fathom_scratch_bytes). */

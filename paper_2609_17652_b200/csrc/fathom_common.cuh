@@ -78,31 +78,24 @@ static inline cudaError_t fathom_launch_dependent(void (*kernel)(P...), dim3 gri
 }
 
 // ---- pieces shared by scan.cu and topk.cu for the fused scan + selection (fathom_scan_topk) -------------------
-// A launch that belongs to one of two alternative continuations decides on the device whether it runs.  A first
-// attempt collects, per head, the tokens above an ESTIMATED threshold; it goes on only if every head collected at
-// least `want` of them.  Otherwise the second attempt, enqueued behind it with a threshold that is a guaranteed
-// bound, does the work.  The host enqueues both and never synchronises.
+// A first attempt collects, per head, the tokens above an ESTIMATED threshold.  The heads of which it collected fewer than `want`
+// are scanned again by a second attempt, enqueued behind it, with a threshold that is a guaranteed bound; what that collects replaces
+// those heads' lists.  The host enqueues both and never synchronises.
 struct fathom_gate {
   const uint32_t* counts;       // [heads] candidates the first attempt collected per head
   uint32_t want;
-  int heads;
-  int mode;                     // 0: always run; 1: only if every head collected enough; 2: only if some head did not;
-                                // 5: always run - the kernel itself looks at its head's count and picks its input
+  int mode;                     // 0: all heads; 2: only heads of which the first attempt collected too few;
+                                // 3, 5: all heads - the selection looks at its head's count and picks its input
 };
-// Called by every thread of the CTA at the top of a gated kernel.
-__device__ __forceinline__ bool fathom_gate_open(const fathom_gate& g) {
-  if (g.mode == 0 || g.mode == 5) return true;
-  bool ok = true;
-  for (int h = threadIdx.x; h < g.heads; h += blockDim.x) ok = ok && (__ldcg(g.counts + h) >= g.want);
-  const bool all_ok = __syncthreads_and(ok) != 0;
-  return g.mode == 1 ? all_ok : !all_ok;
+__device__ __forceinline__ bool fathom_gate_wants(const fathom_gate& g, int head) {
+  return g.mode != 2 || __ldcg(g.counts + head) < g.want;
 }
 
 struct fathom_scan_fuse {       // extra arguments of the sampling / filtering scan variants
   int tile_step;                // sample: scan every tile_step-th tile
   const uint32_t* state;        // filter: [Hq][8] (pointer already offset to the word to read): a threshold bin, or,
   int state_is_score;           //         if state_is_score, the fp32 bits of the score a candidate must reach
-  fathom_gate gate;             // filter: whether this launch runs at all
+  fathom_gate gate;             // filter: which heads this launch is for
   long long sink_end, local_begin;   // filter: eligible tokens are sink_end <= i < local_begin
   float* cand_score;            // filter: [Hq][capacity] scores of the candidates
   int32_t* cand_idx;            // filter: [Hq][capacity] their tokens
@@ -123,8 +116,8 @@ int fathom_launch_scan_filter(const fathom_layout* L, const uint64_t* planes, co
 
 struct fathom_topk_scratch {
   uint32_t* hist;        // [Hq][FATHOM_TOPK_BINS]
-  uint32_t* state;       // [Hq][8]: 0 threshold bin, 1 count above it, 2 needed from it, 3 bound bin (sampled paths),
-                         //          4 candidates written, 5 tickets
+  uint32_t* state;       // [Hq][8]: 0 threshold bin, 1 count above it, 2 needed from it (two passes, and samples of very long rows), 3 bound bin
+                         //          (sampled paths), 4 candidates written, 5 tickets, 6 score that a candidate has to reach
   uint32_t* cand_count;  // [Hq] candidates collected above an estimated threshold (single-pass top-k, fused path)
   uint32_t* cand_count2; // [Hq] candidates of the second attempt (threshold that is a bound, not an estimate)
   uint32_t* bitmap;      // [Hq][bitmap_words] selection bitmap, token i at bit (i % 32) of word i / 32

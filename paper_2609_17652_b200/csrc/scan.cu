@@ -152,7 +152,6 @@ scan_kernel(const __grid_constant__ ScanBatchOf<CAP> B, int G, int heads_per_pla
   Smem<MODE>& M = *reinterpret_cast<Smem<MODE>*>(scan_smem);
 
   FATHOM_PDL_WAIT();                                          // depths (and thresholds) come from the previous kernels
-  if (MODE == 2 && !fathom_gate_open(fz.gate)) return;         // second attempt of the fused selection: may have nothing to do
   const int total = (int)B.tile_end[B.items - 1];              // tiles of this launch (tile and block indices fit 32 bits)
   if ((int)blockIdx.x >= total) return;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -160,6 +159,8 @@ scan_kernel(const __grid_constant__ ScanBatchOf<CAP> B, int G, int heads_per_pla
   constexpr int HEAD_LIST = CAND_LIST / NH;
   const int gq = lane >> 2, t4 = lane & 3;                     // mma fragment coordinates: lane = (row group, column pair)
   const int h0 = blockIdx.y * NH;                              // first of the NH query heads of this CTA
+  // second attempt of the fused selection: may have nothing to do
+  if (MODE == 2 && fz.gate.mode == 2 && !__syncthreads_or(fathom_gate_wants(fz.gate, h0 + tid % NH))) return;
   const int plan = h0 / heads_per_plan;                        // NH divides heads_per_plan: one plan per CTA
   const int kv = h0 / G;
   const int myh = t4 < NH ? t4 : 0;                            // the head whose scores this lane receives (lanes t4 >= NH: none)
@@ -171,7 +172,8 @@ scan_kernel(const __grid_constant__ ScanBatchOf<CAP> B, int G, int heads_per_pla
     M.elig[1] = (uint32_t)hi;
   }
   if (MODE == 2 && tid < NH)                                   // read after the barriers of the first item's row list
-    M.thr[tid] = fz.state_is_score ? __uint_as_float(fz.state[(h0 + tid) * 8]) : fathom_bin_lower_edge(fz.state[(h0 + tid) * 8]);
+    M.thr[tid] = !fathom_gate_wants(fz.gate, h0 + tid) ? __uint_as_float(0x7fc00000u)              // (nothing reaches a NaN)
+               : fz.state_is_score ? __uint_as_float(fz.state[(h0 + tid) * 8]) : fathom_bin_lower_edge(fz.state[(h0 + tid) * 8]);
 
   int item = -1, nrows = 0, nb_item = 0;
   uint32_t half_stride = 0, eighth_stride = 0;                 // rows of plane words and of scales in 16-byte units, and my KV head's first

@@ -93,18 +93,20 @@ scan_simt_kernel(const __grid_constant__ ScanBatch B, int G, int heads_per_plan,
   constexpr int QS_ROWS = (int)(sizeof(M.qs) / sizeof(M.qs[0]));
 
   FATHOM_PDL_WAIT();                                          // depths (and thresholds) come from the previous kernels
-  if (MODE == 2 && !fathom_gate_open(fz.gate)) return;         // second attempt of the fused selection: may have nothing to do
   const int total = (int)B.tile_end[B.items - 1];              // tiles of this launch (tile and block indices fit 32 bits)
   int g = blockIdx.x;                                          // my current tile of the launch
   if (g >= total) return;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int h0 = blockIdx.y * NH;                              // first of the NH query heads of this CTA
+  // second attempt of the fused selection: may have nothing to do
+  if (MODE == 2 && fz.gate.mode == 2 && !__syncthreads_or(fathom_gate_wants(fz.gate, h0 + tid % NH))) return;
   const int plan = h0 / heads_per_plan;                        // NH divides heads_per_plan: one plan per CTA
   const int kv = h0 / G;
   const int beta = lane >> 3, oct = lane & 7;                  // lane = (block of the warp, octet of its tokens)
   const int myb = warp * WB + beta;                            // my block within the tile
   if (MODE == 2 && tid < NH)                                   // read after the barriers of the first item's row list
-    M.thr[tid] = fz.state_is_score ? __uint_as_float(fz.state[(h0 + tid) * 8]) : fathom_bin_lower_edge(fz.state[(h0 + tid) * 8]);
+    M.thr[tid] = !fathom_gate_wants(fz.gate, h0 + tid) ? __uint_as_float(0x7fc00000u)              // (nothing reaches a NaN)
+               : fz.state_is_score ? __uint_as_float(fz.state[(h0 + tid) * 8]) : fathom_bin_lower_edge(fz.state[(h0 + tid) * 8]);
 
   int item = -1, nrows = 0, npass = 1;
 

@@ -760,17 +760,9 @@ topk_select_kernel(const float* scores, long long n, long long score_stride, For
   }
   FATHOM_PDL_WAIT();                                          // the candidates come from the previous kernel
   FATHOM_PDL_RELEASE();                                       // the attention that follows may become resident now
-  // gate mode 3: one launch serves both attempts of the fused path - the first attempt's lists if every head holds what
-  // it needs, else the lists the second filtering scan has written over them (counted in cand_count_second; their
-  // threshold was a bin, so the general way)
-  bool second = false;
-  if (gate.mode == 3) {
-    bool ok = true;
-    for (int h = tid; h < gate.heads; h += FIN_THREADS) ok = ok && (__ldcg(gate.counts + h) >= gate.want);
-    second = __syncthreads_and(ok) == 0;
-  } else if (!fathom_gate_open(gate)) {
-    return;
-  }
+  // gate mode 3: one launch serves both attempts of the fused path - the first attempt's list if it holds what the head needs, else the
+  // list the second filtering scan has written over it (counted in cand_count_second; its threshold was a bin, so the general way)
+  const bool second = gate.mode == 3 && __ldcg(gate.counts + head) < gate.want;
   if (second) cand_count = cand_count_second;
   if (counted) {
     if (!second &&
@@ -1249,12 +1241,11 @@ static int direct_cache_entries(int k) {
 static size_t direct_select_smem(int k) { return (size_t)direct_cache_entries(k) * 8 + (size_t)SORT_BUCKETS * 4 + (size_t)2 * k * 4; }
 
 // The two attempts of a sampled path on the candidates collected above the estimated bin (counts in S.cand_count)
-// and above the bound bin (S.cand_count2): the first runs if every head collected `want`, the second otherwise.
-// gate_mode 3: both attempts of the fused path in one launch (after both filtering scans): the first lists if every head
-// collected `want`, else the second.
-// gate_mode 0: a single attempt whose threshold is a bound (candidates counted in S.cand_count); 1 / 2: first and second
-// attempt of the fused path (all heads together, second list counted in S.cand_count2); 5: the single-pass top-k, head
-// by head in one launch - a head that collected too few collects again itself, above the bound bin, from `scores`.
+// and above the bound bin (S.cand_count2).
+// gate_mode 3: both attempts of the fused path in one launch (after both filtering scans), the first list of a head that collected
+// `want`, else the second.
+// gate_mode 0: a single attempt whose threshold is a bound (candidates counted in S.cand_count); 5: the single-pass top-k - a head that
+// collected too few collects again itself, above the bound bin, from `scores`.
 static int launch_direct_select(fathom_ctx* ctx, long long n, int Hq, int k, Forced F, uint32_t want, const fathom_topk_scratch& S,
                                 int32_t* idx, int gate_mode, cudaStream_t st, const float* scores = nullptr, long long score_stride = 0) {
   static bool attr_set[64] = {};
@@ -1262,16 +1253,16 @@ static int launch_direct_select(fathom_ctx* ctx, long long n, int Hq, int k, For
     FATHOM_CUDA_TRY(ctx, cudaFuncSetAttribute(topk_select_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 216 * 1024));
     attr_set[ctx->device] = true;
   }
-  Gate g = {S.cand_count, want, Hq, gate_mode};
-  const int lo_word = gate_mode == 2 ? -1 : 6;                // state word with the score the candidates had to reach (-1: a bin, no short way)
+  Gate g = {S.cand_count, want, gate_mode};
+  const int lo_word = 6;                                      // state word with the score the candidates had to reach
   const size_t smem = direct_select_smem(k);
   // the short way: a known score threshold, tokens that fit in 21 bits, a part's bitmap within the shared memory
-  const bool counted = lo_word >= 0 && n <= FAST_MAX_TOKENS && fast_select_groups(n) <= FAST_MAXU && (size_t)fast_select_bytes(n) <= smem;
+  const bool counted = n <= FAST_MAX_TOKENS && fast_select_groups(n) <= FAST_MAXU && (size_t)fast_select_bytes(n) <= smem;
   const int parts = counted ? FAST_PARTS : 1;
   FATHOM_CUDA_TRY(ctx, fathom_launch_dependent(
       topk_select_kernel<true>, dim3(Hq * parts), dim3(FIN_THREADS), smem, st, (const float*)S.cand_score, n, 0LL, F,
       (const uint32_t*)S.state, (const int32_t*)S.cand, (uint32_t*)nullptr, 0LL, k, idx, ctx->dev_status, (uint32_t*)nullptr, 0,
-      (const uint32_t*)(gate_mode == 2 ? S.cand_count2 : S.cand_count), n, want, bucket_shift_for(n), g,
+      (const uint32_t*)S.cand_count, n, want, bucket_shift_for(n), g,
       (const float*)(gate_mode == 5 ? scores : nullptr), score_stride, S.cand_score, S.cand, direct_cache_entries(k), lo_word, parts, (const uint32_t*)(gate_mode == 3 ? S.cand_count2 : nullptr)));
   return FATHOM_OK;
 }
@@ -1281,7 +1272,7 @@ static int run_dense_topk(fathom_ctx* ctx, const float* scores, long long n, lon
   if (held_in_registers(n, Hq, k, want)) return fathom_launch_topk_resident(ctx, scores, n, score_stride, Hq, k, F, want, idx, st);
   const int ntiles = (int)((n + FILT_TILE - 1) / FILT_TILE);
   dim3 fgrid((unsigned)ntiles, (unsigned)Hq);
-  Gate always = {nullptr, 0u, 0, 0};
+  Gate always = {nullptr, 0u, 0};
   // Single pass when the row is long enough to estimate the threshold from every 16th 1024-score chunk.
   const long long chunks = n / 1024, sampled = (chunks + 15) / 16;           // whole chunks; chunks 0, 16, 32, .. are sampled
   uint32_t rank = 0;
@@ -1465,14 +1456,14 @@ extern "C" int fathom_scan_topk(fathom_ctx* ctx, const fathom_layout* L, const u
   fz.cand_idx = S.cand;
   fz.cand_count = S.cand_count;
   fz.capacity = n;
-  fz.gate = fathom_gate{nullptr, 0u, 0, 0};
+  fz.gate = fathom_gate{nullptr, 0u, 0};
   rc = fathom_launch_scan_filter(L, planes, scales, q, depth, heads_per_plan, fz, st);
   if (rc != FATHOM_OK) return rc;
-  if (two_attempts) {                                         // stands by: runs only if some head's estimate was too high
+  if (two_attempts) {                                         // stands by, for heads whose estimate was too high
     fz.state = S.state + 3;
     fz.state_is_score = 0;
     fz.cand_count = S.cand_count2;
-    fz.gate = fathom_gate{S.cand_count, want, Hq, 2};
+    fz.gate = fathom_gate{S.cand_count, want, 2};
     rc = fathom_launch_scan_filter(L, planes, scales, q, depth, heads_per_plan, fz, st);
     if (rc != FATHOM_OK) return rc;
   }

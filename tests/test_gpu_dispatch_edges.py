@@ -324,6 +324,32 @@ def test_fused_selection_with_more_candidates_than_a_cta_lists(heads_per_plan):
     ctx.close()
 
 
+# keys alike over runs: samples of whole tiles miss some heads' largest scores, and those heads alone are scanned again; with and without scores that exist
+@pytest.mark.parametrize("run", [32, 1024])
+@pytest.mark.parametrize("n,k,heads_per_plan", [(140001, 300, 4), (140001, 1000, 1), (300032, 4096, 2)])
+def test_selection_where_some_heads_samples_miss(n, k, heads_per_plan, run):
+    from paper_2609_17652_b200 import binding as fb
+    Hkv, Hq = 2, 8
+    lay = fb.make_layout(Hkv, Hq, n)
+    ctx = fb.Context(0, fb.fathom_scratch_bytes(lay, k))
+    g = torch.Generator(device="cuda").manual_seed(run + k)
+    K, q = torch.randn(Hkv, n, 128, generator=g, device="cuda"), torch.randn(Hq, 128, generator=g, device="cuda")
+    K[0] = 0.3 * K[0] + torch.randn(n // run + 1, 128, generator=g, device="cuda").repeat_interleave(run, dim=0)[:n]
+    planes = torch.zeros(Hkv, 128, 4, lay.plane_stride_words, dtype=torch.int64, device="cuda")
+    scales = torch.zeros(Hkv, 128, lay.scale_stride, dtype=torch.int16, device="cuda")
+    depth = torch.zeros(Hq // heads_per_plan, 128, dtype=torch.uint8, device="cuda")
+    scores = torch.zeros(Hq, lay.score_stride, device="cuda")
+    idx, fused = (torch.full((Hq, k), -1, dtype=torch.int32, device="cuda") for _ in range(2))
+    ctx.fathom_build_planes(lay, K, planes, scales)
+    ctx.fathom_alloc_depth(lay, q, K.var(dim=1), fb.DEPTH_WATERFILL, 48, heads_per_plan, depth)
+    ctx.fathom_scan(lay, planes, scales, q, depth, heads_per_plan, scores)
+    ctx.fathom_topk(lay, scores, k, 4, 32, idx)
+    ctx.fathom_scan_topk(lay, planes, scales, q, depth, heads_per_plan, k, 4, 32, fused)
+    assert np.array_equal(idx.cpu().numpy(), O.topk(scores[:, :n].double().cpu().numpy(), k, 4, 32))
+    assert torch.equal(idx, fused) and ctx.fathom_device_status() == 0
+    ctx.close()
+
+
 # block maxima whose eighth is rounded to a subnormal fp16 (quotients of up to 12 steps), to the smallest one and to zero; one block per CTA and eight
 @pytest.mark.parametrize("n", [200, 40003])
 def test_planes_of_keys_with_subnormal_scales(n):
