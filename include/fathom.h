@@ -176,8 +176,8 @@ int fathom_scan_set_ctas_per_plan(int ctas);
  *   idx     out  [Hq][k] int32, ascending token indices
  * Uses the context scratch (fathom_scratch_bytes).
  * Rows of up to 131,072 scores are selected by one kernel that holds them in registers, unless k and the number of
- * heads make another way faster.  Other rows are read once: a histogram of every 16th chunk gives an estimated threshold
- * bin (and a bound: the bin of the sample's own k-th largest score), one pass collects the tokens above the estimate,
+ * heads make another way faster.  Other rows are read once: a histogram of a line in every 512 scores gives an estimated threshold
+ * bin (and a bound: the bin of the k-th largest that was counted), one pass collects the tokens above the estimate,
  * and the exact selection runs among them, head by head.  A head that collected fewer than it needs collects again in
  * the selection's own launch, above the bound; the decision is taken on the device and the result is the same either
  * way.  Rows of which more than a thirty-second is wanted take two passes (histogram of all scores, filter).
@@ -193,9 +193,9 @@ int fathom_topk_passes(const fathom_layout* layout, int k, int n_sink, int n_loc
 /* ---- (3+4) fused scan and top-k, scores never materialised — Sec. 9 Conclusion (fusing the scan with what follows it) ------
  * Gives exactly the idx that fathom_topk would give on the scores of fathom_scan (same arguments), without writing
  * or re-reading the n * Hq scores: (a) every 16th 1024-token tile is scanned and histogrammed per head (the
- * largest of every four scores); (b) the full scan keeps only the (score, token) pairs that reach a threshold bin's lower edge;
+ * largest of every four or two scores where that leaves at least 2 k of them, else all); (b) the full scan keeps only the (score, token) pairs that reach a threshold bin's lower edge;
  * (c) the exact selection (ties to the lower token) runs on those candidates and writes idx.  Two thresholds come
- * from the sample: a BOUND (the bin of the sample's k-th largest score: at least k tokens reach it, so no winner lies
+ * from the sample: a BOUND (the bin of the k-th largest that was counted: at least k tokens reach it, so no winner lies
  * below) and an ESTIMATE (the bin of the rank that k tokens of the whole sequence are expected to reach, plus four
  * standard deviations or more: ~6 times fewer candidates).  The scan runs with the estimate; the heads that then hold fewer
  * candidates than they need are scanned again with the bound, by a launch enqueued behind the first - the

@@ -7,7 +7,7 @@
 // large k and many heads (held_in_registers).
 //
 // Single pass (other rows of at least 65,536, when a sixteenth of the row holds enough of what is wanted): one read of the scores.
-//   a. a cluster of four CTAs per head histograms the largest of every four scores of every 16th 1024-score chunk (bins of a
+//   a. a cluster of four CTAs per head histograms the largest of every four scores of a sample, a line in every 512 scores (bins of a
 //      thirty-second of an octave, shared memory, merged through distributed shared memory) and finds two bins:
 //      the ESTIMATE, whose suffix count in the sample reaches the expected rank plus four standard deviations, and
 //      the BOUND, whose suffix count reaches k in the sample alone and therefore in the whole row;
@@ -200,21 +200,25 @@ __device__ void find_threshold_bin(const uint32_t* __restrict__ h, uint32_t* __r
   if (want_bound) search(want_bound, true);
 }
 
-// Histogram of a head's sample (every 16th whole chunk of 1024 scores) by a cluster of SAMPLE_CLUSTER CTAs: each
-// histograms its share of the chunks in its own shared memory, the others add their non-empty bins to the first CTA's
+// Histogram of a head's sample (a sixteenth of its scores) by a cluster of SAMPLE_CLUSTER CTAs: each
+// histograms its share of the pieces in its own shared memory, the others add their non-empty bins to the first CTA's
 // through distributed shared memory (atomics: a few hundred bins of 4096 hold anything), and two of its warps find the
 // estimated and the bound bin: no global histogram, no flush, no ticket.  For rows of up to a few million scores.
-// `grouped`: the largest of every four scores are counted (k is at most half of their number): a rank of them lies no
-// higher than the same rank of the scores, next to nothing lower where it is small, and there are four times fewer shared-memory atomics, of
+// `group`: the largest of every four or two neighbouring scores are counted (k is at most half of their number): a rank of them lies no
+// higher than the same rank of the scores, next to nothing lower where it is small, and there are fewer shared-memory atomics, of
 // which the kernel consists.  Bins of a thirty-second of an octave instead of an eighth: the lists hold less beyond what is wanted, and a row
 // whose large scores lie close together does not overflow them.  32 heads, back to back, every score in bins of an eighth / now: top-k
-// of 1,048,576 scores, k = 4096 38.3 / 36.9 us (with the last sixteenth 50 above the others 135 / 46), of 500,003, k = 2048 24.1 / 22.3; fused call,
-// 1,048,576 tokens, budget 48, k = 4096 74.3 / 65.1, budget 80 106.2 / 99.2.
+// of 1,048,576 scores, k = 4096 37.8 / 36.5 us (with the last sixteenth 50 above the others 135 / 46), of 500,003, k = 2048 24.5 / 23.4; fused call,
+// 1,048,576 tokens, budget 48, k = 4096 73.6 / 66.
+// A sample consists of lines (32 scores), one in every 512 scores: neighbours' scores are alike where keys are, and of a sample of whole chunks of 1024
+// scores the largest were often missing, whole chunks of them (scores alike over runs of 1024 tokens, 1,048,576 scores, k = 4096: 381 us against 47 now;
+// with all of a thread's loads in flight together independent scores take no longer than in chunks).
 constexpr int SAMPLE_THREADS = 1024;
 constexpr int SAMPLE_CLUSTER = 4;
+constexpr int SAMPLE_PIECE = 32;                              // scores side by side in a sample
 __global__ void __cluster_dims__(SAMPLE_CLUSTER, 1, 1) __launch_bounds__(SAMPLE_THREADS, 2)
-topk_sample_kernel(const float* scores, long long sampled, long long chunk_stride, long long score_stride,
-                   uint32_t* __restrict__ state, uint32_t want, uint32_t want_bound, int grouped, uint32_t* __restrict__ cand_count,
+topk_sample_kernel(const float* scores, int pieces, long long piece_stride, long long score_stride,
+                   uint32_t* __restrict__ state, uint32_t want, uint32_t want_bound, int group, uint32_t* __restrict__ cand_count,
                    uint32_t* __restrict__ cand_count2) {
   __shared__ alignas(16) uint32_t sh[COARSE];
   __shared__ uint32_t s_super[COARSE / SUPER];
@@ -232,29 +236,35 @@ topk_sample_kernel(const float* scores, long long sampled, long long chunk_strid
   __syncthreads();
   auto cleared = cluster.barrier_arrive();                    // my histogram is clear (the first CTA's will be added to)
   const float* row = scores + (size_t)head * (size_t)score_stride;
-  // `sampled` whole chunks of 1024 scores, chunk_stride scores apart (16384: every 16th chunk of a score row; 1024: a
-  // compact array of sampled scores); CTA `part` of the cluster takes every SAMPLE_CLUSTER-th group of 1024 float4
+  // `pieces` lines of SAMPLE_PIECE scores, one in every piece_stride, not always at the same place of it (keys may have a period); CTA `part` of
+  // the cluster takes every SAMPLE_CLUSTER-th group of 1024 float4
   auto count = [&](float v) {
     if (v == v) atomicAdd(&sh[coarse_bin(v)], 1u);
   };
-  constexpr int STRIDE = SAMPLE_CLUSTER * SAMPLE_THREADS, FLY = 2;            // loads in flight per thread: 32 registers, two CTAs per SM
-  for (long long v0 = (long long)part * SAMPLE_THREADS + threadIdx.x; v0 < sampled * 256; v0 += FLY * STRIDE) {
+  constexpr int STRIDE = SAMPLE_CLUSTER * SAMPLE_THREADS, FLY = 4, PER_PIECE = SAMPLE_PIECE / 4;          // loads in flight per thread: 32 registers (two CTAs per SM), and all of a million tokens
+  const int vectors = pieces * PER_PIECE, start = part * SAMPLE_THREADS + threadIdx.x, p = start / PER_PIECE;
+  static_assert(STRIDE / PER_PIECE % 256 == 0, "a thread's pieces lie at the same place of theirs");
+  const long long place = ((5 * p + (p >> 4)) % 16 * (int)(piece_stride / SAMPLE_PIECE)) >> 4, step = STRIDE / PER_PIECE * piece_stride;
+  const float* at = row + p * piece_stride + place * SAMPLE_PIECE + start % PER_PIECE * 4;
+  for (int v0 = start; v0 < vectors; v0 += FLY * STRIDE, at += FLY * step) {
     float4 x[FLY];
 #pragma unroll
-    for (int u = 0; u < FLY; ++u) {
-      const long long v = v0 + u * STRIDE;
-      if (v < sampled * 256) x[u] = reinterpret_cast<const float4*>(row + (v >> 8) * chunk_stride)[v & 255];
-    }
+    for (int u = 0; u < FLY; ++u)
+      if (v0 + u * STRIDE < vectors) x[u] = *reinterpret_cast<const float4*>(at + u * step);
 #pragma unroll
     for (int u = 0; u < FLY; ++u) {
-      if (v0 + u * STRIDE >= sampled * 256) break;
-      if (grouped) {
-        count(fmaxf(fmaxf(x[u].x, x[u].y), fmaxf(x[u].z, x[u].w)));           // (a NaN is no maximum)
+      if (v0 + u * STRIDE >= vectors) break;
+      const float4 s = x[u];
+      if (group == 4) {                                       // (a NaN is no maximum)
+        count(fmaxf(fmaxf(s.x, s.y), fmaxf(s.z, s.w)));
+      } else if (group == 2) {
+        count(fmaxf(s.x, s.y));
+        count(fmaxf(s.z, s.w));
       } else {
-        count(x[u].x);
-        count(x[u].y);
-        count(x[u].z);
-        count(x[u].w);
+        count(s.x);
+        count(s.y);
+        count(s.z);
+        count(s.w);
       }
     }
   }
@@ -518,7 +528,7 @@ __device__ __forceinline__ uint32_t block_exclusive_scan(uint32_t v, uint32_t* s
 // share a head without talking to one another: each loads all the candidates and finds the threshold itself, then
 // emits the chosen tokens of its own quarter of the sequence.
 // The candidates (at most 16 per thread, loaded once, kept in registers as bin and token) are counted in a fine
-// histogram of the key's distance from lo's key (2048 bins of 2^13 keys: 16 bins of the 12-bit histogram lo came from;
+// histogram of the key's distance from lo's key (2048 bins of 2^13 keys: 64 bins of a thirty-second of an octave;
 // the last bin takes everything beyond).  Its suffix counts give the bin b that holds the wanted-th largest candidate;
 // candidates in bins above b are chosen at once, the few dozen members of b are listed and ranked against one another
 // on the composite (key << 32 | ~token).  A chosen token of the CTA's own quarter is set in a bitmap in shared memory,
@@ -1187,12 +1197,21 @@ static int hist_tile_for(long long n, int Hq) {
   return (int)tile;
 }
 
-// Rank in a sample of n_sample of n tokens whose score is, with a margin of four standard deviations of the
-// sampling count, low enough that `want` tokens of the whole sequence reach it.
-static uint32_t estimate_rank(uint32_t want, long long n_sample, long long n) {
-  const double expect = (double)want * (double)n_sample / (double)n;
-  return (uint32_t)(expect + 4.0 * sqrt(expect) + 16.0);
+// How many neighbouring sampled scores are counted by their largest: 4 or 2, where k is at most half of the groups, else 1.
+static int sample_group(int k, long long n_sample) { return 8LL * k <= n_sample ? 4 : (4LL * k <= n_sample ? 2 : 1); }
+
+// Rank in a sample of n_sample of n tokens whose score is low enough that `want` tokens of the whole sequence reach it, with a margin of four
+// standard deviations of the sampling count.  Neighbours' scores are alike where keys are: the samples then count as fewer than they are, for which
+// the groups' largest leave room; without groups the margin is twice as wide, unless that gives lists beyond the 8192 that the selection loads at once.
+// (Rows of 200,000 scores alike over runs of 64 tokens, k = 4096, with the scan: 148 us with four, 144 with six, 36 with eight deviations.)
+static uint32_t estimate_rank(uint32_t want, int k, long long n_sample, long long n) {
+  const double expect = (double)want * (double)n_sample / (double)n, deviation = sqrt(expect);
+  const double wide = expect + 8.0 * deviation + 16.0, narrow = expect + 4.0 * deviation + 16.0;
+  return (uint32_t)(sample_group(k, n_sample) == 1 && wide * (double)n <= 7500.0 * (double)n_sample ? wide : narrow);
 }
+
+// Distance of a row's sampled pieces; each starts on a 32-byte sector.
+static long long sample_piece_stride(long long n, long long pieces) { return n / pieces & ~7LL; }
 
 static bool force_two_pass() {
   static const bool v = [] { const char* e = getenv("FATHOM_TOPK_PATH"); return e && strcmp(e, "two_pass") == 0; }();
@@ -1203,7 +1222,7 @@ static bool force_two_pass() {
 static bool single_pass_plan(long long n, int k, uint32_t want, uint32_t* rank_out) {
   const long long chunks = n / 1024, sampled = (chunks + 15) / 16;           // whole chunks; chunks 0, 16, 32, .. are sampled
   const long long n_sample = sampled * 1024;
-  const uint32_t rank = estimate_rank(want, n_sample, n) + (uint32_t)(k - want);
+  const uint32_t rank = estimate_rank(want, k, n_sample, n) + (uint32_t)(k - want);
   *rank_out = rank;
   return !force_two_pass() && want > 0 && chunks >= 64 && (long long)rank * 8 <= n_sample && (long long)k * 2 <= n_sample;
 }
@@ -1304,8 +1323,9 @@ static int run_dense_topk(fathom_ctx* ctx, const float* scores, long long n, lon
     // the sample histogram counts forced tokens too, so both ranks allow for all of them: at least k sampled tokens
     // reach the bound bin, hence at least k - forced = want eligible ones
     if (sampled <= 256) {                                              // up to 4M scores per row: one CTA per head
-      FATHOM_CUDA_TRY(ctx, fathom_launch_dependent(topk_sample_kernel, dim3(Hq * SAMPLE_CLUSTER), dim3(SAMPLE_THREADS), 0, st, scores, sampled, 16 * 1024LL, score_stride, S.state, rank, (uint32_t)k,
-                                                        8LL * k <= sampled * 1024 ? 1 : 0, S.cand_count, (uint32_t*)nullptr));
+      FATHOM_CUDA_TRY(ctx, fathom_launch_dependent(topk_sample_kernel, dim3(Hq * SAMPLE_CLUSTER), dim3(SAMPLE_THREADS), 0, st, scores,
+                                                   (int)(sampled * (1024 / SAMPLE_PIECE)), sample_piece_stride(n, sampled * (1024 / SAMPLE_PIECE)), score_stride, S.state, rank,
+                                                   (uint32_t)k, sample_group(k, sampled * 1024), S.cand_count, (uint32_t*)nullptr));
     } else {
       const int reps = 8;                                              // sampled chunks per CTA
       dim3 sgrid((unsigned)((sampled + reps - 1) / reps), (unsigned)Hq);
@@ -1432,12 +1452,12 @@ extern "C" int fathom_scan_topk(fathom_ctx* ctx, const fathom_layout* L, const u
   Forced none;
   none.sink_end = 0;
   none.local_begin = n_sample;
-  const uint32_t rank = estimate_rank(want, n_sample, n) + (uint32_t)n_forced;
+  const uint32_t rank = estimate_rank(want, k, n_sample, n) + (uint32_t)n_forced;
   const bool two_attempts = !force_two_pass() && want >= 256 && (long long)rank * 2 <= k;
   if (one_cta_sample) {                                       // one CTA per head, histogram in shared memory only
     FATHOM_CUDA_TRY(ctx, fathom_launch_dependent(topk_sample_kernel, dim3(Hq * SAMPLE_CLUSTER), dim3(SAMPLE_THREADS), 0, st, (const float*)S.sample,
-                                                 n_sample / 1024, 1024LL, S.sample_stride, S.state, two_attempts ? rank : (uint32_t)k,
-                                                 two_attempts ? (uint32_t)k : 0u, 8LL * k <= n_sample ? 1 : 0, S.cand_count, S.cand_count2));
+                                                 (int)(n_sample / SAMPLE_PIECE), (long long)SAMPLE_PIECE, S.sample_stride, S.state, two_attempts ? rank : (uint32_t)k,
+                                                 two_attempts ? (uint32_t)k : 0u, sample_group(k, n_sample), S.cand_count, S.cand_count2));
   } else {
     const int htile = hist_tile_for(n_sample, Hq);
     dim3 hgrid((unsigned)((n_sample + htile - 1) / htile), (unsigned)Hq);
