@@ -210,9 +210,13 @@ def test_klt_basis_in_place(spread):
     ctx.close()
 
 
-# (tokens, heads, k) on both sides of every line between the kernels of the selection, scores that exist and scores that do not
-@pytest.mark.parametrize("n,Hq,k", [(131072, 60, 548), (131072, 46, 600), (131072, 47, 600), (131072, 9, 3108), (131072, 9, 3109), (131072, 2, 16384),
-                                    (131073, 2, 16384), (33001, 9, 9000), (33001, 10, 9000), (20000, 18, 8300), (20000, 19, 8300), (70001, 75, 2100),
+# (tokens, heads, k, 36 of them forced) on both sides of every line between the kernels of the selection, scores that exist and scores that do not: the
+# longest row in registers; heads for large, middling and small k; 1, 2, 4 and 8 CTAs of 8, 16 and 32 scores per thread, by lists and without; lists of two
+# sevenths of a row, of 9000, and of CTAs that cannot share an SM
+@pytest.mark.parametrize("n,Hq,k", [(131072, 2, 16384), (131073, 2, 16384), (65536, 149, 1100), (65537, 55, 4133), (65537, 56, 4133), (131072, 37, 2085), (131072, 38, 2085),
+                                    (65537, 129, 1061), (65537, 130, 1061), (65537, 130, 1060), (8000, 80, 300), (8000, 80, 8000), (16000, 40, 300), (16000, 40, 9000),
+                                    (30000, 14, 300), (30000, 14, 12000), (16000, 80, 300), (30000, 40, 300), (30000, 40, 12000), (60000, 14, 300), (60000, 14, 16000),
+                                    (4096, 3, 1206), (4096, 3, 1207), (131072, 2, 9036), (131072, 2, 9037), (33001, 40, 4700), (33001, 40, 5200),
                                     (16384, 96, 16384), (16384, 128, 12000), (8769, 148, 8769), (16384, 149, 12000)])
 def test_selection_on_both_sides_of_its_lines(n, Hq, k):
     from paper_2609_17652_b200 import binding as fb
