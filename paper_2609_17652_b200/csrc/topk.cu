@@ -138,7 +138,8 @@ topk_hist_kernel(const float* __restrict__ scores, long long n, long long score_
 
 // state[head][0] = threshold bin, [1] = tokens in bins above it, [2] = tokens still needed from it, [3] = bound bin
 // of a sampled histogram, [4] = candidates appended by the filter, [5] = ticket counter of the histogram CTAs,
-// [6] = the score a candidate of the first attempt must reach (fp32 bits): the lower edge of bin [0].
+// [6] = the score a candidate of the first attempt must reach (fp32 bits): the lower edge of bin [0].  (topk_sample_kernel, whose bins are finer,
+// writes words 3 and 6 alone.)
 // Run by all THREADS threads of the CTA that finished the head's histogram h in global memory last: thread t owns bins 4095 - BPT t .. (descending), so a block prefix over
 // threads is a suffix count over bins.  s_warp: at least THREADS / 32 words of shared memory.
 // want: rank whose bin goes to words 0..2.  want_bound (0 = none): rank whose bin alone goes to word 3 (histogram of
