@@ -1239,6 +1239,7 @@ static bool held_in_registers(long long n, int Hq, int k, uint32_t want) {
   if (n <= 65536) return true;
   const long long ctas = (long long)Hq * fathom_topk_resident_ctas(n, Hq), sms = fathom_sm_count();
   uint32_t rank;
+  if (want > 8192) return ctas <= sms;                        // (fathom_topk_passes states two passes for more)
   if (want > 4096) return ctas <= 3 * sms;
   if (want > 2048 && single_pass_plan(n, k, want, &rank)) return ctas <= 2 * sms;
   return want <= 1024 || ctas <= 7 * sms;
